@@ -85,10 +85,13 @@ __device__ __forceinline__ PairInfo bytepair_info(const PairTable& t, u32 a, u32
 
 // Asks for [p, p + bytes) to be brought into L2, spread over the whole grid (no result, nothing waits for it).
 // Used by a kernel while it waits for its predecessor: the tables it is about to probe at random are fetched
-// with idle bandwidth, so that after a cold start its dependent loads find them in L2.
+// with idle bandwidth, so that after a cold start its dependent loads find them in L2.  A grid that would have to issue
+// more than two lines per thread leaves it: so small a text probes a few hundred slots of a table of tens of thousands
+// of lines, and walking the table took longer than the whole call (2 KB of text with a 16 MB table: 75 us of 90).
 __device__ __forceinline__ void grid_prefetch_l2(const void* p, size_t bytes) {
     const char* c = reinterpret_cast<const char*>(p);
     const size_t lines = (bytes + 127) / 128, stride = (size_t)gridDim.x * blockDim.x;
+    if (lines > 2 * stride) return;
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < lines; i += stride)
         asm volatile("prefetch.global.L2 [%0];" ::"l"(c + i * 128));
 }
