@@ -14,6 +14,7 @@
 #include "unicode_table.inc"
 
 #include <climits>
+#include <memory>
 #include <mutex>
 #include <cstdio>
 #include <cstring>
@@ -25,7 +26,30 @@
 #include <vector>
 #include <algorithm>
 
+// Device and pinned memory of the sessions of one vocabulary.  A session's arrays are one allocation, and the memory of a
+// freed session is kept for the next one (at most POOL_ARENAS of them, POOL_BYTES in all; given back by
+// tt_vocab_free): fifteen cudaMalloc and cudaFree calls per session took 2 to 15 ms, more than the 17 tokenizations of
+// a conversation.  Sessions share ownership, so that one that outlives its vocabulary still frees what it holds.
+struct SessionHost;
+struct SessionArena { char* dev = nullptr; size_t bytes = 0; int device = 0; SessionHost* host = nullptr; };
+struct SessionPool {
+    static constexpr size_t POOL_ARENAS = 8, POOL_BYTES = (size_t)512 << 20;
+    std::mutex mu;
+    std::vector<SessionArena> kept;
+    bool closed = false;
+    static void destroy(SessionArena& a) { cudaFree(a.dev); if (a.host) cudaFreeHost(a.host); a = SessionArena{}; }
+    bool get(size_t bytes, SessionArena& out);
+    void put(SessionArena a);
+    void close() {
+        std::lock_guard<std::mutex> lk(mu);
+        closed = true;
+        for (SessionArena& a : kept) destroy(a);
+        kept.clear();
+    }
+};
+
 struct tt_vocab {
+    std::shared_ptr<SessionPool> sessions = std::make_shared<SessionPool>();
     int pattern = 0;
     int device = 0;
     int sm_count = 148;
@@ -87,6 +111,7 @@ extern "C" size_t tt_class_table(uint8_t* out, size_t cap) {
 
 extern "C" void tt_vocab_free(tt_vocab* v) {
     if (!v) return;
+    v->sessions->close();
     cudaFree(v->d_slots); cudaFree(v->d_bytepair); cudaFree(v->d_ext_id); cudaFree(v->d_cls); cudaFree(v->d_lit_entries); cudaFree(v->d_lit_blob); cudaFree(v->d_tokslots); cudaFree(v->d_longslots); cudaFree(v->d_longblob); cudaFree(v->d_meta);
     cudaFree(v->d_text); cudaFree(v->d_ids); cudaFree(v->d_count); cudaFree(v->d_status); cudaFree(v->d_ws);
     if (v->h_text) cudaFreeHost(v->h_text);
@@ -917,8 +942,39 @@ extern "C" int tt_encode_static(const tt_vocab* v, const uint8_t* text, size_t l
 }
 
 // ---- sessions: incremental repair on append (paper Sec. 3.3) ------------------------------------------
+// What one copy brings back to the host: scalars of the session in device memory, and their image in pinned memory.
+struct SessionScalars { RepairDecision dec; long long ntok, fcount; int32_t fstatus, sstatus; };
+struct SessionHost { SessionScalars s; };
+
+bool SessionPool::get(size_t bytes, SessionArena& out) {
+    int device = 0;
+    if (cudaGetDevice(&device) != cudaSuccess) { cudaGetLastError(); return false; }
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        size_t best = kept.size();
+        for (size_t i = 0; i < kept.size(); i++)                 // the smallest one that is large enough, not wastefully so
+            if (kept[i].device == device && kept[i].bytes >= bytes && kept[i].bytes / 4 <= bytes && (best == kept.size() || kept[i].bytes < kept[best].bytes)) best = i;
+        if (best < kept.size()) { out = kept[best]; kept.erase(kept.begin() + (ptrdiff_t)best); return true; }
+    }
+    out.bytes = bytes; out.device = device;
+    if (cudaMalloc(&out.dev, bytes) != cudaSuccess) { cudaGetLastError(); out.dev = nullptr; return false; }
+    if (cudaMallocHost(&out.host, sizeof(SessionHost)) != cudaSuccess) { cudaGetLastError(); cudaFree(out.dev); out = SessionArena{}; return false; }
+    return true;
+}
+void SessionPool::put(SessionArena a) {
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        size_t total = a.bytes;
+        for (const SessionArena& k : kept) total += k.bytes;
+        if (!closed && kept.size() < POOL_ARENAS && total <= POOL_BYTES) { kept.push_back(a); return; }
+    }
+    destroy(a);
+}
+
 struct tt_session {
     const tt_vocab* v = nullptr;
+    std::shared_ptr<SessionPool> pool;
+    SessionArena arena;
     size_t cap = 0;                       // bytes of text the session can hold
     size_t len = 0;                       // bytes stored
     uint32_t window_chars = 512;
@@ -928,20 +984,24 @@ struct tt_session {
     int32_t *d_ids = nullptr, *d_off = nullptr;                 // cached records; d_off[ntok] = len
     int32_t *d_fids = nullptr, *d_foff = nullptr, *d_fchar = nullptr;   // fresh records / scratch of the span export
     u8* d_eq = nullptr;
-    long long *d_ntok = nullptr, *d_fcount = nullptr;
-    int32_t *d_fstatus = nullptr, *d_sstatus = nullptr;
-    RepairDecision* d_dec = nullptr;
-    struct Host { RepairDecision dec; long long ntok; int32_t fstatus, sstatus; }* h = nullptr;   // pinned
+    SessionScalars* d_sc = nullptr;
+    SessionScalars* h = nullptr;                                        // pinned
     void *d_ws = nullptr, *d_sws = nullptr;
     size_t ws_bytes = 0, sws_bytes = 0;
 };
 
 extern "C" void tt_session_free(tt_session* s) {
     if (!s) return;
-    cudaFree(s->d_text); cudaFree(s->d_ids); cudaFree(s->d_off); cudaFree(s->d_fids); cudaFree(s->d_foff); cudaFree(s->d_fchar);
-    cudaFree(s->d_eq); cudaFree(s->d_ntok); cudaFree(s->d_fcount); cudaFree(s->d_fstatus); cudaFree(s->d_sstatus);
-    cudaFree(s->d_dec); cudaFree(s->d_ws); cudaFree(s->d_sws);
-    if (s->h) cudaFreeHost(s->h);
+    if (s->arena.dev) {
+        // copies out of the session, or kernels of the caller that read its view, may still be running on some stream; the
+        // memory is handed on only when they are through (as cudaFree would wait for them)
+        int dev = s->arena.device;
+        cudaGetDevice(&dev);
+        if (dev != s->arena.device) cudaSetDevice(s->arena.device);
+        if (cudaDeviceSynchronize() == cudaSuccess) s->pool->put(s->arena);
+        else { cudaGetLastError(); SessionPool::destroy(s->arena); cudaGetLastError(); }
+        if (dev != s->arena.device) cudaSetDevice(dev);
+    }
     delete s;
 }
 
@@ -950,19 +1010,30 @@ extern "C" int tt_session_create(const tt_vocab* v, size_t max_bytes, tt_session
     if (!v || !out || max_bytes == 0 || max_bytes >= (size_t)INT32_MAX - 64 || v->meta_n == 0) return TT_ERR_ARG;
     tt_session* s = new (std::nothrow) tt_session();
     if (!s) return TT_ERR_CUDA;
-    s->v = v; s->cap = max_bytes;
+    s->v = v; s->cap = max_bytes; s->pool = v->sessions;
     s->ws_bytes = tt_workspace_bytes(v, max_bytes, 1);
     s->sws_bytes = tt_spans_workspace_bytes(v, max_bytes);
     const size_t n1 = max_bytes + 1;
-    bool ok = cudaMalloc(&s->d_text, max_bytes + 64) == cudaSuccess && cudaMalloc(&s->d_ids, n1 * 4) == cudaSuccess &&
-              cudaMalloc(&s->d_off, n1 * 4) == cudaSuccess && cudaMalloc(&s->d_fids, n1 * 4) == cudaSuccess &&
-              cudaMalloc(&s->d_foff, n1 * 4) == cudaSuccess && cudaMalloc(&s->d_fchar, n1 * 4) == cudaSuccess &&
-              cudaMalloc(&s->d_eq, n1) == cudaSuccess && cudaMalloc(&s->d_ntok, 8) == cudaSuccess &&
-              cudaMalloc(&s->d_fcount, 8) == cudaSuccess && cudaMalloc(&s->d_fstatus, 4) == cudaSuccess &&
-              cudaMalloc(&s->d_sstatus, 4) == cudaSuccess && cudaMalloc(&s->d_dec, sizeof(RepairDecision)) == cudaSuccess &&
-              cudaMalloc(&s->d_ws, s->ws_bytes) == cudaSuccess && cudaMalloc(&s->d_sws, s->sws_bytes) == cudaSuccess &&
-              cudaMallocHost(&s->h, sizeof(tt_session::Host)) == cudaSuccess;
-    ok = ok && cudaMemset(s->d_ntok, 0, 8) == cudaSuccess && cudaMemset(s->d_off, 0, 4) == cudaSuccess;
+    size_t off = 0;
+    char* base = nullptr;
+    auto take = [&](size_t bytes) { const size_t o = off; off = align_up(off + bytes, 256); return base + o; };
+    auto carve_all = [&]() {
+        off = 0;
+        s->d_sc = (SessionScalars*)take(sizeof(SessionScalars));
+        s->d_text = (u8*)take(max_bytes + 64);
+        s->d_ids = (int32_t*)take(n1 * 4); s->d_off = (int32_t*)take(n1 * 4);
+        s->d_fids = (int32_t*)take(n1 * 4); s->d_foff = (int32_t*)take(n1 * 4); s->d_fchar = (int32_t*)take(n1 * 4);
+        s->d_eq = (u8*)take(n1);
+        s->d_ws = take(s->ws_bytes); s->d_sws = take(s->sws_bytes);
+    };
+    carve_all();
+    if (!s->pool->get(off, s->arena)) { delete s; return TT_ERR_CUDA; }
+    base = s->arena.dev;
+    carve_all();
+    s->h = &s->arena.host->s;
+    // no record yet: count 0, off[0] = 0.  (Waited for: the session may be used from any stream.)
+    const bool ok = cudaMemset(s->d_sc, 0, sizeof(SessionScalars)) == cudaSuccess && cudaMemset(s->d_off, 0, 4) == cudaSuccess &&
+                    cudaStreamSynchronize(nullptr) == cudaSuccess;
     if (!ok) { cudaGetLastError(); tt_session_free(s); return TT_ERR_CUDA; }
     *out = s;
     return TT_OK;
@@ -979,7 +1050,7 @@ extern "C" int tt_session_view(const tt_session* s, const int32_t** ids_dev, con
     if (!s) return TT_ERR_ARG;
     if (ids_dev) *ids_dev = s->d_ids;
     if (off_dev) *off_dev = s->d_off;
-    if (count_dev) *count_dev = (const int64_t*)s->d_ntok;
+    if (count_dev) *count_dev = (const int64_t*)&s->d_sc->ntok;
     if (len_bytes) *len_bytes = s->len;
     return TT_OK;
 }
@@ -987,9 +1058,10 @@ extern "C" int tt_session_view(const tt_session* s, const int32_t** ids_dev, con
 // Tokenizes text[from, new_len) into (ids, off, count) with offsets relative to `from`.
 static int session_tokenize(tt_session* s, size_t from, size_t new_len, cudaStream_t st, int32_t* ids, int32_t* off, long long* count) {
     const size_t n = new_len - from;
-    int rc = encode_impl(s->v, s->d_text + from, n, nullptr, 1, st, ids, s->cap, (int64_t*)count, nullptr, s->d_fstatus, s->d_ws);
+    int rc = encode_impl(s->v, s->d_text + from, n, nullptr, 1, st, ids, s->cap, (int64_t*)count, nullptr, &s->d_sc->fstatus, s->d_ws);
     if (rc != TT_OK) return rc;
-    return tt_spans(s->v, ids, (const int64_t*)count, s->cap, n, st, off, s->d_fchar, s->d_sstatus, s->d_sws, s->sws_bytes);
+    // (n bytes hold at most n tokens: the span kernels' grid follows the window, not the session's capacity)
+    return tt_spans(s->v, ids, (const int64_t*)count, n, n, st, off, s->d_fchar, &s->d_sc->sstatus, s->d_sws, s->sws_bytes);
 }
 
 // The host keeps the last bytes of the stored text, as many as the widest window of the protocol can span (five
@@ -1024,20 +1096,20 @@ extern "C" int tt_session_append(tt_session* s, const uint8_t* text, size_t len,
         if (left > 0 || ws == s->tail_base) ws = 0;           // the window reaches the start of the text (or beyond what the host kept: more work, same ids)
         local.attempts = attempt + 1;
         if (ws == 0) break;                                   // the window is the whole text
-        int rc = session_tokenize(s, ws, new_len, st, s->d_fids, s->d_foff, s->d_fcount);
+        int rc = session_tokenize(s, ws, new_len, st, s->d_fids, s->d_foff, &s->d_sc->fcount);
         if (rc != TT_OK) return fail(rc);
         RepairParams P;
-        P.ids = s->d_ids; P.off = s->d_off; P.ntok = s->d_ntok;
-        P.fids = s->d_fids; P.foff = s->d_foff; P.fchar = s->d_fchar; P.fcount = s->d_fcount;
-        P.fstatus = s->d_fstatus; P.sstatus = s->d_sstatus; P.text = s->d_text;
+        P.ids = s->d_ids; P.off = s->d_off; P.ntok = &s->d_sc->ntok;
+        P.fids = s->d_fids; P.foff = s->d_foff; P.fchar = s->d_fchar; P.fcount = &s->d_sc->fcount;
+        P.fstatus = &s->d_sc->fstatus; P.sstatus = &s->d_sc->sstatus; P.text = s->d_text;
         P.ws = (long long)ws; P.old_len = (long long)old_len; P.new_len = (long long)new_len;
         P.cls = s->v->d_cls; P.cls_bytes = s->v->cls_bytes; P.max_tok_chars = (int)s->v->max_token_chars;
-        P.eq = s->d_eq; P.dec = s->d_dec;
+        P.eq = s->d_eq; P.dec = &s->d_sc->dec;
         k_repair_decide<<<1, 256, 0, st>>>(P);
         const size_t fresh_max = new_len - ws;
         const int grid = (int)((fresh_max + 255) / 256 < (size_t)s->v->sm_count * 4 ? (fresh_max + 255) / 256 : (size_t)s->v->sm_count * 4);
         k_repair_apply<<<grid, 256, 0, st>>>(P);
-        if (cudaMemcpyAsync(&s->h->dec, s->d_dec, sizeof(RepairDecision), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        if (cudaMemcpyAsync(&s->h->dec, &s->d_sc->dec, sizeof(RepairDecision), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
             cudaStreamSynchronize(st) != cudaSuccess) { cudaGetLastError(); return fail(TT_ERR_CUDA); }
         const RepairDecision d = s->h->dec;
         if (d.status != TT_OK) return fail(d.status);          // e.g. the appended text is not valid UTF-8: nothing changed
@@ -1050,21 +1122,24 @@ extern "C" int tt_session_append(tt_session* s, const uint8_t* text, size_t len,
         }
     }
     if (local.attempts == 0) local.attempts = 1;
-    // full tokenization straight into the session's records (into the fresh buffers first, so that an error
-    // leaves the session as it was)
-    int rc = session_tokenize(s, 0, new_len, st, s->d_fids, s->d_foff, s->d_fcount);
+    // full tokenization: into the records themselves where there are none yet (count 0 whatever happens), else into the
+    // fresh buffers first, so that an error leaves the session as it was
+    const bool direct = old_len == 0;
+    long long* const count = direct ? &s->d_sc->ntok : &s->d_sc->fcount;
+    int rc = session_tokenize(s, 0, new_len, st, direct ? s->d_ids : s->d_fids, direct ? s->d_off : s->d_foff, count);
     if (rc != TT_OK) return fail(rc);
-    if (cudaMemcpyAsync(&s->h->ntok, s->d_fcount, 8, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaMemcpyAsync(&s->h->fstatus, s->d_fstatus, 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaMemcpyAsync(&s->h->sstatus, s->d_sstatus, 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+    if (cudaMemcpyAsync(s->h, s->d_sc, sizeof(SessionScalars), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess) { cudaGetLastError(); return fail(TT_ERR_CUDA); }
-    if (s->h->fstatus != TT_OK) return fail(s->h->fstatus);
-    if (s->h->sstatus != TT_OK) return fail(s->h->sstatus);
-    const size_t nt = (size_t)s->h->ntok;
-    if (cudaMemcpyAsync(s->d_ids, s->d_fids, nt * 4, cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
+    const int bad = s->h->fstatus != TT_OK ? s->h->fstatus : s->h->sstatus;
+    if (bad != TT_OK) {
+        if (direct) cudaMemsetAsync(&s->d_sc->ntok, 0, 8, st);
+        return fail(bad);
+    }
+    const size_t nt = (size_t)(direct ? s->h->ntok : s->h->fcount);
+    if (!direct && (cudaMemcpyAsync(s->d_ids, s->d_fids, nt * 4, cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
         cudaMemcpyAsync(s->d_off, s->d_foff, (nt + 1) * 4, cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
-        cudaMemcpyAsync(s->d_ntok, s->d_fcount, 8, cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess) { cudaGetLastError(); return fail(TT_ERR_CUDA); }
+        cudaMemcpyAsync(&s->d_sc->ntok, &s->d_sc->fcount, 8, cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
+        cudaStreamSynchronize(st) != cudaSuccess)) { cudaGetLastError(); return fail(TT_ERR_CUDA); }
     s->len = new_len; session_keep_tail(s, text, len);
     local.window_chars = 0; local.window_start = 0; local.run_tokens = 0; local.splice_byte = 0;
     local.n_tokens = (int64_t)nt; local.status = TT_OK;
@@ -1080,7 +1155,7 @@ extern "C" int tt_session_copy(const tt_session* s, int32_t* ids_out, size_t ids
     const size_t n = s->len < ids_cap ? s->len : ids_cap;
     if (ids_out && n) CK(cudaMemcpyAsync(ids_out, s->d_ids, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
     if (off_out) CK(cudaMemcpyAsync(off_out, s->d_off, (n + 1) * sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
-    CK(cudaMemcpyAsync(count_out, s->d_ntok, sizeof(int64_t), cudaMemcpyDeviceToDevice, st));
+    CK(cudaMemcpyAsync(count_out, &s->d_sc->ntok, sizeof(int64_t), cudaMemcpyDeviceToDevice, st));
     return TT_OK;
 }
 
