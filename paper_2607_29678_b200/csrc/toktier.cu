@@ -450,7 +450,7 @@ static size_t carve(TTWorkspace* w, void* base, size_t max_len, size_t max_docs)
     char* p;
     p = take(sizeof(TTHeader));                 if (w) w->hdr = (TTHeader*)p;
     p = take((padded / 32 + 4) * sizeof(u32));  if (w) w->docmask = (u32*)p;
-    p = take(nchunks * sizeof(u16));            if (w) w->startmask = (u16*)p;
+    p = take((padded / 32 + 4) * sizeof(u32));  if (w) w->startmask = (u32*)p;
     p = take((ntiles + 1) * sizeof(u32));       if (w) w->tile_cnt = (u32*)p;
     p = take((ntiles + 1) * sizeof(u32));       if (w) w->tile_first = (u32*)p;
     p = take((ntiles + 1) * sizeof(u32));       if (w) w->tile_last = (u32*)p;
@@ -490,14 +490,13 @@ extern "C" size_t tt_workspace_bytes(const tt_vocab* v, size_t max_len, size_t m
 #define CK(x) do { if ((x) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; } } while (0)
 
 // One instance of the first kernel per pattern (the pattern's rules are compiled in), chosen here.
-template <bool FUSED, int MINB>
+template <bool FUSED, int NT, int MINB>
 static void launch_pretok(int grid, cudaStream_t st, const PretokParams& P, const FrontParams& F) {
-    const size_t smem = TT_PRETOK_SMEM_BYTES;
     switch (P.pattern) {
-    case TT_PATTERN_O200K:     k_pretok<FUSED, MINB, TT_PATTERN_O200K><<<grid, TT_TILE_CHUNKS, smem, st>>>(P, F); break;
-    case TT_PATTERN_CL100K_N1: k_pretok<FUSED, MINB, TT_PATTERN_CL100K_N1><<<grid, TT_TILE_CHUNKS, smem, st>>>(P, F); break;
-    case TT_PATTERN_CUTS:      if constexpr (!FUSED) k_pretok<false, MINB, TT_PATTERN_CUTS><<<grid, TT_TILE_CHUNKS, smem, st>>>(P, F); break;
-    default:                   k_pretok<FUSED, MINB, TT_PATTERN_CL100K><<<grid, TT_TILE_CHUNKS, smem, st>>>(P, F); break;
+    case TT_PATTERN_O200K:     k_pretok<FUSED, NT, MINB, TT_PATTERN_O200K><<<grid, NT, 0, st>>>(P, F); break;
+    case TT_PATTERN_CL100K_N1: k_pretok<FUSED, NT, MINB, TT_PATTERN_CL100K_N1><<<grid, NT, 0, st>>>(P, F); break;
+    case TT_PATTERN_CUTS:      if constexpr (!FUSED) k_pretok<false, NT, MINB, TT_PATTERN_CUTS><<<grid, NT, 0, st>>>(P, F); break;
+    default:                   k_pretok<FUSED, NT, MINB, TT_PATTERN_CL100K><<<grid, NT, 0, st>>>(P, F); break;
     }
 }
 
@@ -516,7 +515,8 @@ static int run_pretok(const tt_vocab* v, const uint8_t* text, size_t len, const 
     }
     P.lo = shift; P.hi = shift + (long long)len;
     P.nchunks = (P.hi + TT_CHUNK - 1) / TT_CHUNK;
-    P.ntiles = (int)((P.nchunks + TT_TILE_CHUNKS - 1) / TT_TILE_CHUNKS);
+    P.nwords = (P.hi + TT_WORD - 1) / TT_WORD;
+    P.ntiles = (int)((P.nwords + TT_TILE_WORDS - 1) / TT_TILE_WORDS);
     P.pattern = v->pattern; P.epoch = next_epoch();
     P.docmask = nullptr; P.litstart = nullptr; P.litin = nullptr;
     P.startmask = w.startmask; P.tile_cnt = w.tile_cnt; P.tile_first = w.tile_first; P.want_prefix = piece_off_dst != nullptr; P.hdr = w.hdr;
@@ -549,9 +549,9 @@ static int run_pretok(const tt_vocab* v, const uint8_t* text, size_t len, const 
         // stages A and B: span starts into cutmask (with the caller's document starts); stage C: pattern 0 with
         // those cuts as its document boundaries
         PretokParams C1 = P;
-        C1.pattern = TT_PATTERN_CUTS; C1.startmask = reinterpret_cast<u16*>(w.cutmask);
+        C1.pattern = TT_PATTERN_CUTS; C1.startmask = w.cutmask;
         C1.want_prefix = 0; C1.litstart = nullptr; C1.litin = nullptr;
-        launch_pretok<false, PRETOK_CTAS_REQUEST>(grid, st, C1, FrontParams{});
+        launch_pretok<false, PRETOK_THREADS_REQUEST, PRETOK_CTAS_REQUEST>(grid, st, C1, FrontParams{});
         P.pattern = TT_PATTERN_CL100K; P.docmask = w.cutmask;
     }
     if (fused) {
@@ -559,11 +559,11 @@ static int run_pretok(const tt_vocab* v, const uint8_t* text, size_t len, const 
         F.tile_last = w.tile_last; F.tile_tok = w.tile_tok; F.tile_q = w.tile_q; F.tile_long = w.tile_long; F.piece_off16 = w.piece_off16;
         F.piece_cnt = w.piece_cnt; F.q = w.q; F.toktab = v->toktab; F.longtab = v->longtab; F.ext_id = v->d_ext_id;
         F.wq = P.ntiles > MERGE_SR_MAX_TILES ? w.wq : nullptr;
-        if (bulk) launch_pretok<true, PRETOK_CTAS_BULK>(grid, st, P, F);
-        else launch_pretok<true, PRETOK_CTAS_REQUEST>(grid, st, P, F);
-    } else launch_pretok<false, PRETOK_CTAS_REQUEST>(grid, st, P, FrontParams{});
+        if (bulk) launch_pretok<true, PRETOK_THREADS_BULK, PRETOK_CTAS_BULK>(grid, st, P, F);
+        else launch_pretok<true, PRETOK_THREADS_REQUEST, PRETOK_CTAS_REQUEST>(grid, st, P, F);
+    } else launch_pretok<false, PRETOK_THREADS_REQUEST, PRETOK_CTAS_REQUEST>(grid, st, P, FrontParams{});
     if (piece_off_dst)
-        k_compact<<<grid, TT_TILE_CHUNKS, 0, st>>>(w.startmask, w.tile_cnt, P.nchunks, P.ntiles, shift, (long long)len,
+        k_compact<<<grid, TT_TILE_WORDS, 0, st>>>(w.startmask, w.tile_cnt, P.nwords, P.ntiles, shift, (long long)len,
                                                    piece_off_dst, w.hdr, P.epoch);
     CK(cudaGetLastError());
     return TT_OK;

@@ -21,13 +21,13 @@ typedef uint32_t u32;
 typedef uint64_t u64;
 
 // ---- geometry of the pre-tokenization pass -------------------------------------------------
-// A chunk is one aligned 16-byte vector load; a tile is what one CTA classifies per iteration.
+// A chunk is one aligned 16-byte vector load, a word the 32 bytes that one thread classifies and evaluates (a mask word has
+// a bit for each), a tile what one CTA takes per iteration.
 constexpr int TT_CHUNK = 16;
-#ifndef TT_TILE_CHUNKS_DEF
-#define TT_TILE_CHUNKS_DEF 128
-#endif
-constexpr int TT_TILE_CHUNKS = TT_TILE_CHUNKS_DEF;        // = threads per CTA
-constexpr int TT_TILE_BYTES = TT_CHUNK * TT_TILE_CHUNKS; // 2 KiB of text per tile
+constexpr int TT_WORD = 32;
+constexpr int TT_TILE_WORDS = 64;
+constexpr int TT_TILE_BYTES = TT_WORD * TT_TILE_WORDS;    // 2 KiB of text per tile
+constexpr int TT_TILE_CHUNKS = TT_TILE_BYTES / TT_CHUNK;
 constexpr int TT_GROUP_TILES = 256;              // bulk text: token totals are also kept per group of 256 tiles
 constexpr int TT_TILE_QCAP = TT_TILE_BYTES / 2;  // unsettled pieces of <= 256 bytes a tile can have (each has >= 2 bytes)
 constexpr int TT_TILE_LONGCAP = 8;               // pieces of > 256 bytes that lie inside one tile
@@ -107,7 +107,7 @@ __device__ __forceinline__ void hdr_set_status(TTHeader* h, unsigned long long e
 struct TTWorkspace {
     TTHeader* hdr;
     u32* docmask;      // bit per text byte: first byte of a document (batch only)
-    u16* startmask;    // bit per text byte: first byte of a piece, one u16 per chunk (tt_pretokenize and the cut pass only)
+    u32* startmask;    // bit per text byte: first byte of a piece (tt_pretokenize and the cut pass only)
     u32* tile_cnt;     // (tt_pretokenize: then the exclusive prefix, ntiles + 1)
     u32* tile_first;
     u32* tile_last;
