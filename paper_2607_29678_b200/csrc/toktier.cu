@@ -57,6 +57,7 @@ struct tt_vocab {
     uint4* d_slots = nullptr;
     u64* d_bytepair = nullptr;
     int32_t* d_ext_id = nullptr;
+    u16* d_tok_len = nullptr;            // bytes of every internal token, 65,535 = at least that many
     u8* d_cls = nullptr;
     int cls_bytes = 0;
     PairTable tab{};
@@ -112,7 +113,7 @@ extern "C" size_t tt_class_table(uint8_t* out, size_t cap) {
 extern "C" void tt_vocab_free(tt_vocab* v) {
     if (!v) return;
     v->sessions->close();
-    cudaFree(v->d_slots); cudaFree(v->d_bytepair); cudaFree(v->d_ext_id); cudaFree(v->d_cls); cudaFree(v->d_lit_entries); cudaFree(v->d_lit_blob); cudaFree(v->d_tokslots); cudaFree(v->d_longslots); cudaFree(v->d_longblob); cudaFree(v->d_meta);
+    cudaFree(v->d_slots); cudaFree(v->d_bytepair); cudaFree(v->d_ext_id); cudaFree(v->d_tok_len); cudaFree(v->d_cls); cudaFree(v->d_lit_entries); cudaFree(v->d_lit_blob); cudaFree(v->d_tokslots); cudaFree(v->d_longslots); cudaFree(v->d_longblob); cudaFree(v->d_meta);
     cudaFree(v->d_text); cudaFree(v->d_ids); cudaFree(v->d_count); cudaFree(v->d_status); cudaFree(v->d_ws);
     if (v->h_text) cudaFreeHost(v->h_text);
     if (v->h_ids) cudaFreeHost(v->h_ids);
@@ -219,8 +220,8 @@ static int build_token_table(tt_vocab* v, const tt_merge* merges, size_t n_merge
         Q.hdr = d_hdr; Q.epoch = next_epoch(); Q.tab = v->tab;
         Q.toktab.slots = nullptr; Q.toktab.mask = 0; Q.toktab.shift = 0;      // no table yet: every piece is merged
         Q.longtab = LongTable{}; Q.litstart = nullptr;
-        Q.ext_id = v->d_ext_id; Q.piece_cnt = d_cnt; Q.stage = d_stage; Q.pairbuf = nullptr; Q.tile_tok = d_tt; Q.grp_tok = nullptr; Q.wq = nullptr; Q.gq = nullptr; Q.gq_x[0] = Q.gq_x[1] = Q.gq_x[2] = nullptr; Q.lq = nullptr;
-        k_merge<<<v->sm_count * MERGE_CTAS_PER_SM, MERGE_THREADS, MERGE_SMEM_BYTES>>>(Q);
+        Q.ext_id = v->d_ext_id; Q.piece_cnt = d_cnt; Q.stage = d_stage; Q.pairbuf = nullptr; Q.tile_tok = d_tt; Q.grp_tok = nullptr; Q.wq = nullptr; Q.gq = nullptr; Q.gq_x[0] = Q.gq_x[1] = Q.gq_x[2] = nullptr; Q.lq = nullptr; Q.tok_len = nullptr;
+        k_merge<<<v->sm_count * MERGE_CTAS_PER_SM, MERGE_THREADS, MERGE_SMEM_REQUEST>>>(Q);
         ok = cudaGetLastError() == cudaSuccess && cudaDeviceSynchronize() == cudaSuccess;
     }
     ok = ok && cudaMemcpy(cnt.data(), d_cnt, cnt.size() * sizeof(u32), cudaMemcpyDeviceToHost) == cudaSuccess;
@@ -412,18 +413,24 @@ extern "C" int tt_vocab_load_ex(const tt_merge* merges, size_t n_merges, const i
     ok = ok && cudaMemcpy(v->d_cls, cls.data(), v->cls_bytes, cudaMemcpyHostToDevice) == cudaSuccess;
     if (!ok) { cudaGetLastError(); tt_vocab_free(v); return TT_ERR_CUDA; }
     v->tab.slots = v->d_slots; v->tab.bytepair = v->d_bytepair; v->tab.mask = mask; v->tab.shift = shift;
-    if (cudaFuncSetAttribute(k_merge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MERGE_SMEM_BYTES) != cudaSuccess ||
+    if (cudaFuncSetAttribute(k_merge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MERGE_SMEM_REQUEST) != cudaSuccess ||
         cudaFuncSetAttribute(k_merge_bulk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MERGE_SMEM_BYTES) != cudaSuccess) { cudaGetLastError(); tt_vocab_free(v); return TT_ERR_CUDA; }
     { const int rc = build_token_table(v, merges, n_merges, ext_id); if (rc != TT_OK) { tt_vocab_free(v); return rc; } }
     {   // byte length and number of non-continuation bytes of every token, indexed by the caller's id
         std::vector<uint2> in(256 + n_merges);
         for (int b = 0; b < 256; b++) in[b] = make_uint2(1u, (b & 0xC0) != 0x80 ? 1u : 0u);
+        std::vector<u16> tok_len(in.size());
         int32_t max_ext = 0;
         for (int32_t e : ext_id) max_ext = e > max_ext ? e : max_ext;
         for (size_t r = 0; r < n_merges; r++) {
             const uint2 L = in[internal[merges[r].left]], R = in[internal[merges[r].right]];
             in[256 + r] = make_uint2(L.x + R.x, L.y + R.y);
             if (in[256 + r].y > v->max_token_chars) v->max_token_chars = in[256 + r].y;
+        }
+        for (size_t i = 0; i < in.size(); i++) tok_len[i] = (u16)(in[i].x < 65535u ? in[i].x : 65535u);
+        if (cudaMalloc(&v->d_tok_len, tok_len.size() * sizeof(u16)) != cudaSuccess ||
+            cudaMemcpy(v->d_tok_len, tok_len.data(), tok_len.size() * sizeof(u16), cudaMemcpyHostToDevice) != cudaSuccess) {
+            cudaGetLastError(); tt_vocab_free(v); return TT_ERR_CUDA;
         }
         if (max_ext < (1 << 24)) {
             std::vector<uint2> meta((size_t)max_ext + 1, make_uint2(0, 0));
@@ -464,15 +471,15 @@ static size_t carve(TTWorkspace* w, void* base, size_t max_len, size_t max_docs)
     // the global lists of bulk text: only where a text can have more tiles than a request's job search covers (any
     // alignment of the text counted in)
     const bool bulk_lists = (15 + max_len + TT_TILE_BYTES - 1) / TT_TILE_BYTES > (size_t)MERGE_SR_MAX_TILES;
-    if (w) { w->wq = nullptr; w->gq = nullptr; w->lq = nullptr; for (int c = 0; c < TT_SHORT_CLASSES - 1; c++) w->gq_x[c] = nullptr; }
+    if (w) { w->wq = nullptr; w->gq = nullptr; for (int c = 0; c < TT_SHORT_CLASSES - 1; c++) w->gq_x[c] = nullptr; }
     if (bulk_lists) {
         p = take((max_len / 33 + 64) * sizeof(u64));             if (w) w->wq = (u64*)p;
         p = take((max_len / 2 + 64) * sizeof(u64));              if (w) w->gq = (u64*)p;
         for (int c = 1; c < TT_SHORT_CLASSES; c++) {              // a piece of class c has more bytes than class c - 1 allows
             p = take((max_len / (tt_short_class_max(c - 1) + 1) + 64) * sizeof(u64));   if (w) w->gq_x[c - 1] = (u64*)p;
         }
-        p = take((max_len / 257 + 16) * sizeof(uint4));          if (w) w->lq = (uint4*)p;
     }
+    p = take((max_len / 257 + 16) * sizeof(uint4));              if (w) w->lq = (uint4*)p;
     p = take((max_len + 1) * sizeof(int32_t));  if (w) w->stage = (int32_t*)p;
     p = take((max_len + 1) * sizeof(u64));      if (w) w->pairbuf = (u64*)p;
     p = take(padded + 16);                      if (w) w->cand = (u8*)p;
@@ -583,12 +590,12 @@ static int check_common(const tt_vocab* v, const void* text, size_t len, void* w
 // signalled, and wait inside the kernel (cudaGridDependencySynchronize) until the predecessor's memory
 // is complete.  Only the launch latency is hidden; the data dependence is unchanged.
 template <typename Params>
-static cudaError_t launch_after(void (*kernel)(const Params), int grid, int block, cudaStream_t st, const Params& p, size_t smem = 0) {
+static cudaError_t launch_after(void (*kernel)(const Params), int grid, int block, cudaStream_t st, const Params& p, size_t smem = 0, bool early = true) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3((unsigned)block); cfg.dynamicSmemBytes = smem; cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[0].val.programmaticStreamSerializationAllowed = early ? 1 : 0;
     cfg.attrs = attr; cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, p);
 }
@@ -630,14 +637,14 @@ static int encode_impl(const tt_vocab* v, const uint8_t* text, size_t len, const
     Q.ext_id = v->d_ext_id; Q.piece_cnt = w.piece_cnt; Q.stage = w.stage; Q.pairbuf = w.pairbuf; Q.tile_tok = w.tile_tok;
     Q.grp_tok = PP.ntiles > MERGE_SR_MAX_TILES ? w.grp_tok : nullptr;   // group totals only where k_scatter's CTAs would otherwise sum thousands of tiles each
     Q.wq = big ? w.wq : nullptr; Q.gq = big ? w.gq : nullptr;
-    for (int c = 0; c < TT_SHORT_CLASSES - 1; c++) Q.gq_x[c] = big ? w.gq_x[c] : nullptr; Q.lq = big ? w.lq : nullptr;
+    for (int c = 0; c < TT_SHORT_CLASSES - 1; c++) Q.gq_x[c] = big ? w.gq_x[c] : nullptr;
+    Q.lq = w.lq; Q.tok_len = v->d_tok_len;
     if (big) {                                                               // bulk text: closing pieces and the global lists first
         const int cgrid = (PP.ntiles + CLOSING_THREADS - 1) / CLOSING_THREADS;
         if (ev) k_closing<<<cgrid, CLOSING_THREADS, 0, st>>>(Q);
         else CK(launch_after(k_closing, cgrid, CLOSING_THREADS, st, Q));
     }
-    if (ev) { if (big) k_merge_bulk<<<merge_grid, MERGE_THREADS, MERGE_SMEM_BYTES, st>>>(Q); else k_merge<<<merge_grid, MERGE_THREADS, MERGE_SMEM_BYTES, st>>>(Q); }
-    else CK(launch_after(big ? k_merge_bulk : k_merge, merge_grid, MERGE_THREADS, st, Q, MERGE_SMEM_BYTES));
+    CK(launch_after(big ? k_merge_bulk : k_merge, merge_grid, MERGE_THREADS, st, Q, big ? MERGE_SMEM_BYTES : MERGE_SMEM_REQUEST, ev == nullptr));
     MARK(2);
     ScatterParams S;
     S.shift = PP.lo; S.hi = PP.hi; S.ntiles = PP.ntiles; S.tile_cnt = w.tile_cnt; S.tile_tok = w.tile_tok; S.grp_tok = Q.grp_tok; S.piece_off16 = w.piece_off16;

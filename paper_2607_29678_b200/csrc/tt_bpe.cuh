@@ -203,12 +203,12 @@ __device__ __forceinline__ u32 select_bit(u32 mask, u32 j) {
 
 // ---- warp merge rounds with at most 32 tokens: one token per lane, no shared memory -----------------------
 // t = token of position `lane`, p = (rank, cl, cr) of the pair (lane, lane + 1) or none, m = token count.
-// Runs rounds to the fixpoint, stages the tokens (caller's ids) at stage[a ...] and returns their count.
+// Runs rounds to the fixpoint, hands token j of the result to out(j, token) and returns their count.
 // A round: Q marks a pair identical to the pair on its left (t t t); a pair that is not Q heads a run; a head
 // may go if its left guard holds or it has the round's minimum rank; a pair goes if its run's head may go, it
 // lies an even number of places behind the head and its right guard holds (or it has the minimum rank).
-__device__ __forceinline__ u32 warp_merge_reg_rounds(u32 t, PairInfo p, u32 m, u32 a, const PairTable& tab,
-                                                     const int32_t* __restrict__ ext_id, int32_t* __restrict__ stage, int lane) {
+template <class Out>
+__device__ __forceinline__ u32 warp_merge_reg_rounds(u32 t, PairInfo p, u32 m, const PairTable& tab, int lane, Out out) {
     const u32 FULL = 0xFFFFFFFFu, lt = (1u << lane) - 1, le = lt | (1u << lane);
     u32 r = p.r, cl = p.cl, cr = p.cr;
     if ((u32)lane + 1 >= m) r = cl = cr = TT_RANK_INF;      // the last token has no pair
@@ -246,17 +246,17 @@ __device__ __forceinline__ u32 warp_merge_reg_rounds(u32 t, PairInfo p, u32 m, u
         if ((u32)lane + 1 >= m) r = cl = cr = TT_RANK_INF;
         else if (r == RK_STALE) { const PairInfo q = pair_probe(tab, t, tn); r = q.r; cl = q.cl; cr = q.cr; }
     }
-    if ((u32)lane < m) stage[a + lane] = ext_id[t];
+    if ((u32)lane < m) out((u32)lane, t);
     return m;
 }
 
 // A piece of up to 32 bytes.
-__device__ __forceinline__ u32 warp_merge_reg(const u8* __restrict__ text, u32 a, u32 n, const PairTable& tab,
-                                              const int32_t* __restrict__ ext_id, int32_t* __restrict__ stage, int lane) {
+template <class Out>
+__device__ __forceinline__ u32 warp_merge_reg(const u8* __restrict__ text, u32 a, u32 n, const PairTable& tab, int lane, Out out) {
     const u32 t = (u32)lane < n ? text[a + lane] : 0;
     const u32 tn = __shfl_down_sync(0xFFFFFFFFu, t, 1);
     const PairInfo p = ((u32)lane + 1 < n) ? bytepair_info(tab, t, tn) : pair_none();
-    return warp_merge_reg_rounds(t, p, n, a, tab, ext_id, stage, lane);
+    return warp_merge_reg_rounds(t, p, n, tab, lane, out);
 }
 
 // ---- warp merge, 33..32 E bytes: E tokens per lane, compaction through shared memory ------------------------
@@ -264,10 +264,9 @@ __device__ __forceinline__ u32 warp_merge_reg(const u8* __restrict__ text, u32 a
 // words (token, rank, cl, cr by position).  Each round the survivors are written to their new positions in
 // the other copy and read back (one warp barrier); ranks next to a merge are marked stale and probed again,
 // the probed guards go to the current copy, from which the next round reads its neighbours' values.
-template <int E>
+template <int E, class Out>
 __device__ __forceinline__ u32 warp_merge_perm(u32* buf /* 2 * 4 * 32 E words of this warp */, const u8* __restrict__ text,
-                                               u32 a, u32 n, const PairTable& tab, const int32_t* __restrict__ ext_id,
-                                               int32_t* __restrict__ stage, int lane) {
+                                               u32 a, u32 n, const PairTable& tab, int lane, Out out) {
     constexpr u32 N = 32 * E;
     const u32 FULL = 0xFFFFFFFFu, lt = (1u << lane) - 1, le = lt | (1u << lane);
     u32 t[E], r[E];
@@ -297,7 +296,7 @@ __device__ __forceinline__ u32 warp_merge_perm(u32* buf /* 2 * 4 * 32 E words of
         __syncwarp();                                   // the guards written after the probes are visible
         if (m <= 32) {                                  // cheaper rounds from here on
             PairInfo p; p.r = r[0]; p.cl = cb[2 * N + lane]; p.cr = cb[3 * N + lane];
-            return warp_merge_reg_rounds(t[0], p, m, a, tab, ext_id, stage, lane);
+            return warp_merge_reg_rounds(t[0], p, m, tab, lane, out);
         }
         const int nch = (int)((m + 31) >> 5);
         u32 sel[E];
@@ -361,7 +360,7 @@ __device__ __forceinline__ u32 warp_merge_perm(u32* buf /* 2 * 4 * 32 E words of
 #pragma unroll
     for (int j = 0; j < E; j++) {
         const u32 k = j * 32 + lane;
-        if (k < m) stage[a + k] = ext_id[t[j]];
+        if (k < m) out(k, t[j]);
     }
     return m;
 }
@@ -706,6 +705,7 @@ __device__ u32 cta_merge_long(const u8* __restrict__ text, u32 a, u32 n, const P
 // never settled by the first kernel (its end is the next piece start, which another CTA finds): k_merge
 // settles it, looking the end up in tile_first of the following tiles.
 __device__ __forceinline__ u32 tile_queue_entry(u32 off, u32 idx, u32 n) { return off | (idx << 11) | ((n - 1) << 22); }
+constexpr u32 TQ_MAY_LONG = 0x80000000u;              // tile_q: the tile allows for a piece of more than 256 bytes (see k_pretok)
 constexpr u32 TQ_NS_MASK = 0x7FFu, TQ_NW_SHIFT = 11, TQ_NW_MASK = 0x7Fu, TQ_NL_SHIFT = 18, TQ_NL_MASK = 0xFu;
 
 struct PieceParams {
@@ -734,7 +734,9 @@ struct PieceParams {
     u64* wq;                   // bulk text: the warp-class pieces of all tiles (tile << 32 | queue entry), else null
     u64* gq;                   // bulk text: the short pieces of all tiles, gathered by k_closing (tile << 32 | queue entry),
     u64* gq_x[3];              // one list per length class (tt_short_class_max); gq is the first
-    uint4* lq;                 // bulk text: the long pieces of all tiles, listed by k_closing (text offset, bytes, piece slot, 0)
+    uint4* lq;                 // long pieces (text offset, bytes, piece slot, state): of all tiles, listed by k_closing (bulk text), or those
+                               // that k_merge hands to the whole grid (a request)
+    const u16* tok_len;        // bytes of every internal token (65,535 = that many or more)
 };
 
 // ---- K4, second half: the merges ------------------------------------------------------------------------------
@@ -804,20 +806,12 @@ __device__ __forceinline__ bool piece_in_range(const PieceParams& P, u32 a, u32 
 __device__ __forceinline__ void warp_merge_piece(const PieceParams& P, const u8* __restrict__ text, u32 a, u32 n, u32 slot, u64* wbuf, int lane) {
     if (!piece_in_range(P, a, n, slot, 1u) || n < 2 || n > (u32)TT_WARP_PIECE_MAX) { if (n < 2 || n > (u32)TT_WARP_PIECE_MAX) hdr_selfcheck_failed(P.hdr, P.epoch, 2u, a, n, slot, 0u); return; }
     u32* const pbuf = reinterpret_cast<u32*>(wbuf);
-    const u32 m = n <= LANE_MAX ? warp_merge_reg(text, a, n, P.tab, P.ext_id, P.stage, lane)
-                : n <= 64 ? warp_merge_perm<2>(pbuf, text, a, n, P.tab, P.ext_id, P.stage, lane)
-                : n <= 128 ? warp_merge_perm<4>(pbuf, text, a, n, P.tab, P.ext_id, P.stage, lane)
-                           : warp_merge_perm<WCH>(pbuf, text, a, n, P.tab, P.ext_id, P.stage, lane);
+    const auto out = [&](u32 j, u32 t) { P.stage[a + j] = P.ext_id[t]; };
+    const u32 m = n <= LANE_MAX ? warp_merge_reg(text, a, n, P.tab, lane, out)
+                : n <= 64 ? warp_merge_perm<2>(pbuf, text, a, n, P.tab, lane, out)
+                : n <= 128 ? warp_merge_perm<4>(pbuf, text, a, n, P.tab, lane, out)
+                           : warp_merge_perm<WCH>(pbuf, text, a, n, P.tab, lane, out);
     if (lane == 0) piece_done(P, slot, m);
-}
-
-// Exclusive prefix over the lanes of a 64-bit value holding two counts (low 32 bits, high 32 bits); *total = warp sum.
-__device__ __forceinline__ u64 warp_exscan_u64(u64 v, int lane, u64* total) {
-    u64 x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) { const u64 t = __shfl_up_sync(0xFFFFFFFFu, x, o); if (lane >= o) x += t; }
-    *total = __shfl_sync(0xFFFFFFFFu, x, 31);
-    return x - v;
 }
 
 // ---- bulk text only: the closing pieces, and one list per length class for the whole text ---------------------
@@ -899,41 +893,434 @@ k_closing(const PieceParams P) {
     }
 }
 
-// Long pieces of the tiles [t_lo, t_hi) (at most MERGE_THREADS of them), a whole CTA each.  Called by all threads
-// of the CTA with the records of tile t_lo + tid in nl / np / last / c_end / closing_long.
-__device__ void cta_long_pieces(const PieceParams& P, const u8* __restrict__ text, int t_lo, int t_hi, u32 nl, u32 np, u32 last, u32 c_end,
-                                bool closing_long, u64* s_buf, u32* sc, uint4* s_long, u32* s_nlong) {
-    const int tid = threadIdx.x;
-    for (int k = 0; k < MERGE_THREADS && t_lo + k < t_hi; k++) {      // block-uniform; tile after tile, so that the shared list cannot overflow
-        if (!__syncthreads_or(tid == k && (nl != 0 || closing_long))) continue;
-        if (tid == k) {
-            const int t = t_lo + k;
-            u32 cnt = 0;
-            for (u32 j = 0; j < nl && j < (u32)TT_TILE_LONGCAP; j++) {
-                const u32 idx = P.tile_long[(size_t)t * TT_TILE_LONGCAP + j];
-                const u32 o = P.piece_off16[(size_t)t * TT_TILE_BYTES + idx], o2 = P.piece_off16[(size_t)t * TT_TILE_BYTES + idx + 1];
-                s_long[cnt++] = make_uint4((u32)((long long)t * TT_TILE_BYTES + o - P.shift), o2 - o, (u32)t * TT_TILE_BYTES + idx, 0u);
-            }
-            if (closing_long) {
-                const u32 st = (u32)t * TT_TILE_BYTES + last;
-                s_long[cnt++] = make_uint4((u32)((long long)st - P.shift), c_end - st, (u32)t * TT_TILE_BYTES + np - 1, 0u);
-            }
-            *s_nlong = cnt;
+// ---- long pieces --------------------------------------------------------------------------------------------------
+// A piece of more than 256 bytes used to be merged by one CTA, round after round over the whole piece: 0.8 ms for the 64 KB
+// blank runs of the 3M-char case, 45 ms for 64 KB of letters, with the rest of the GPU idle.  Now it is cut into windows.
+//
+// Why that is exact.  Call two tokens compatible if the byte string of the two together encodes to exactly these two.  A
+// token sequence is the encoding of its byte string if and only if all its neighbours are compatible:
+//   * If they are, look at the first merge of the sequential run on the whole string that crosses a boundary between two
+//     of the tokens u, v.  Until then every merge lay inside a token, so the merges inside u and v were those of the run
+//     on "u v" alone, in the same order (the lowest rank, leftmost, of the whole string is also that of the part it lies
+//     in).  The run on "u v" alone would therefore make the crossing merge too, and u, v would not be compatible.
+//   * Conversely the final run never crossed u | v, so the run on "u v" alone makes the same merges and ends with u, v.
+// A window's encoding is a run of compatible neighbours.  Where the encodings of two overlapping windows share one token
+// (same bytes, same place), the first one up to and including it, followed by the second one behind it, is again a run
+// of compatible neighbours, whatever either window made of the rest.  So the windows are encoded independently, each by
+// a warp, and joined at a shared token of every overlap; only if some overlap has none (a run of one character whose
+// tokens stand at different phases in the two windows) the piece is merged as a whole by one CTA.
+constexpr u32 LWIN = 256, LSTEP = 192;                 // bytes of a window (what a warp merges) and distance of their starts
+constexpr u32 LQ_WINDOWS = 1, LQ_DONE = 2, LQ_FALLBACK = 3;       // states of an entry of lq
+constexpr int LQ_CHUNK = 256;
+constexpr int TT_RUNS = 32;                            // runs of one token that a warp keeps, one per lane
+struct LongShared {
+    uint4 q[LQ_CHUNK]; u32 pre[LQ_CHUNK + 1];          // a stretch of lq and the windows before each of its pieces
+    u32 ticket;
+    u32 nruns, rpos[TT_RUNS], rtok[2 * TT_RUNS], rcnt[2 * TT_RUNS];   // a piece of few byte runs (cta_run_piece)
+};
+__device__ __forceinline__ u32 long_windows(u32 n) { return n <= LWIN ? 1u : (n - LWIN + LSTEP - 1) / LSTEP + 1u; }
+
+// The grid works through the steps below by tickets: a step's tasks are taken one by one by whichever CTA or warp comes,
+// and a CTA waits before the next step until every task that was taken has been done.  So a CTA only ever waits for CTAs
+// that are running: one that starts late, or never gets its place while others run, is not needed and finds nothing left
+// to do.  Every wait is bounded.  step: 0 pieces found, 1 windows, 2 counts, 3 places, 4 ids.
+__device__ __forceinline__ u32 warp_take(u32* counter, int lane) {
+    u32 t = 0;
+    if (lane == 0) t = atomicAdd(counter, 1u);
+    return __shfl_sync(0xFFFFFFFFu, t, 0);
+}
+__device__ __forceinline__ u32 cta_take(u32* counter, u32* s_word) {
+    __syncthreads();
+    if (threadIdx.x == 0) *s_word = atomicAdd(counter, 1u);
+    __syncthreads();
+    return *s_word;
+}
+__device__ __noinline__ bool long_wait(const PieceParams& P, int step, u32 tasks) {          // all `tasks` tasks of the step are done
+    bool ok = true;
+    if (threadIdx.x == 0) {
+        u32 seen = 0, tries = 0;
+        for (;;) {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&P.hdr->long_done[step]) : "memory");
+            if (seen >= tasks) break;
+            if ((++tries & 1023u) == 0 && hdr_status(P.hdr, P.epoch) != 0) { ok = false; break; }     // (a CTA that found an error does not come)
+            if (tries > 10000000u) { ok = false; hdr_selfcheck_failed(P.hdr, P.epoch, 8u, seen, tasks, (u32)step, blockIdx.x); break; }
+            __nanosleep(64);
         }
-        __syncthreads();
-        const u32 cnt = *s_nlong;
-        for (u32 e = 0; e < cnt; e++) {                               // block-uniform
-            const uint4 q = s_long[e];
-            __syncthreads();
-            if (!piece_in_range(P, q.x, q.y, q.z, 3u)) continue;
-            if (tid == 0) { u32 v = 0; sc[SCR_FLAG] = piece_settled_without_merge(P, text, q.x, q.y, v) ? 1u : 0u; sc[SCR_VALUE] = v; }
-            __syncthreads();
-            if (sc[SCR_FLAG]) { if (tid == 0) { P.piece_cnt[q.z] = sc[SCR_VALUE]; atomicAdd(&P.tile_tok[q.z / TT_TILE_BYTES], 1u); } continue; }
-            const u32 m = cta_merge_long(text, q.x, q.y, P.tab, P.ext_id, P.stage, P.pairbuf + q.x, s_buf, sc);
-            if (tid == 0) piece_done(P, q.z, m);
+    }
+    return __syncthreads_and(ok);
+}
+__device__ __forceinline__ void long_did(const PieceParams& P, int step, u32 tasks) {         // one thread, after its group's last write
+    __threadfence();
+    atomicAdd(&P.hdr->long_done[step], tasks);
+}
+
+// A piece that is a few runs of one byte each -- 64 KB of blanks, a ruler of equals signs -- is merged as runs: (token, how often),
+// a lane each.  The round of the lowest rank (x, y) turns every run of x (if x = y) into half as many new tokens, with the
+// odd one left at the end, or takes one token from the end of a run of x and one from the start of the run of y behind
+// it.  A run of 2^k bytes takes k rounds whatever its tokens' lengths are, where rounds over its positions took 0.4 ms
+// for 50 KB and windows would see tokens of thousands of bytes only in part.  Returns false if the piece has (or
+// comes to have) more than 32 runs; then nothing is done.  Called by the whole CTA.
+__device__ __noinline__ bool cta_run_piece(const PieceParams& P, const u8* __restrict__ text, u32 a, u32 n, u32 slot, LongShared& LS) {
+    const u32 tid = threadIdx.x, T = blockDim.x, FULL = 0xFFFFFFFFu;
+    const u8* const p = text + a;
+    volatile u32* const nruns = &LS.nruns;
+    __syncthreads();
+    if (tid == 0) *nruns = 0;
+    __syncthreads();
+    // where the byte changes
+    const auto change = [&](u32 pos) { if (*nruns < 2u * TT_RUNS) { const u32 k = atomicAdd(&LS.nruns, 1u); if (k < (u32)TT_RUNS) LS.rpos[k] = pos; } };
+    const u32 skew = (u32)(4 - ((uintptr_t)p & 3)) & 3, nw = (n - skew) / 4;
+    const u32* const w = reinterpret_cast<const u32*>(p + skew);
+    if (tid >= 1 && tid < skew && p[tid] != p[tid - 1]) change(tid);
+    if (tid < (n - skew) % 4) { const u32 q = skew + 4 * nw + tid; if (p[q] != p[q - 1]) change(q); }
+    for (u32 i0 = tid; i0 < nw && *nruns < 2u * TT_RUNS; i0 += 8 * T) {
+        u32 x[8], y[8];
+#pragma unroll
+        for (int u = 0; u < 8; u++) {
+            const u32 i = i0 + u * T;
+            x[u] = i < nw ? w[i] : 0u;
+            y[u] = i < nw ? (i ? w[i - 1] >> 24 : skew ? (u32)p[skew - 1] : x[u] & 0xFFu) : 0u;      // the byte before the word
+        }
+#pragma unroll
+        for (int u = 0; u < 8; u++) {
+            const u32 d = x[u] ^ ((x[u] << 8) | y[u]);
+            if (d) for (u32 k = 0; k < 4; k++) if ((d >> (8 * k)) & 0xFFu) change(skew + 4 * (i0 + u * T) + k);
         }
     }
     __syncthreads();
+    const u32 changes = *nruns;
+    __syncthreads();
+    if (changes >= (u32)TT_RUNS) return false;
+    if (tid < 32) {
+        const u32 lane = tid;
+        u32 m = changes + 1;
+        // runs in order
+        const u32 mine = lane < changes ? LS.rpos[lane] : 0xFFFFFFFFu;
+        u32 before = 0;
+        for (int i = 0; i < 32; i++) { const u32 o = __shfl_sync(FULL, mine, i); before += o < mine; }
+        __syncwarp();
+        if (lane < changes) LS.rcnt[before + 1] = mine;              // start of run `before` + 1
+        if (lane == 0) LS.rcnt[0] = 0;
+        __syncwarp();
+        u32 cnt = 0, tok = 0;
+        if (lane < m) { const u32 s = LS.rcnt[lane]; cnt = (lane + 1 < m ? LS.rcnt[lane + 1] : n) - s; tok = p[s]; }
+        __syncwarp();
+        bool ok = true;
+        for (u32 round = 0;; round++) {
+            if (round > 4096) { ok = false; break; }
+            // ranks of the pair inside the run and of the pair with the next run
+            const u32 tn = __shfl_down_sync(FULL, tok, 1);
+            u32 rs = TT_RANK_INF, rb = TT_RANK_INF;
+            if (lane < m && cnt >= 2) rs = pair_probe(P.tab, tok, tok).r;
+            if (lane + 1 < m) rb = pair_probe(P.tab, tok, tn).r;
+            const u32 mn = __reduce_min_sync(FULL, min(rs, rb));
+            if (mn == TT_RANK_INF) break;
+            const bool self = rs == mn, cut = rb == mn;
+            const u32 prev = __shfl_up_sync(FULL, (u32)cut, 1);
+            const u32 k = lane < m ? cnt - ((lane > 0 && prev) ? 1u : 0u) - (cut ? 1u : 0u) : 0u;     // (self and cut exclude each other: a rank is one pair)
+            // what becomes of the run, in order: (t0, k0), (t1, k1)
+            u32 t0 = tok, k0 = k, t1 = 256u + mn, k1 = cut ? 1u : 0u;
+            if (self) { t0 = 256u + mn; k0 = cnt >> 1; t1 = tok; k1 = cnt & 1; }
+            const u32 c = (k0 ? 1u : 0u) + (k1 ? 1u : 0u);
+            u32 at = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) { const u32 v = __shfl_up_sync(FULL, at, o); if (lane >= (u32)o) at += v; }
+            const u32 total = __shfl_sync(FULL, at, 31);
+            at -= c;
+            if (k0) { LS.rtok[at] = t0; LS.rcnt[at] = k0; at++; }
+            if (k1) { LS.rtok[at] = t1; LS.rcnt[at] = k1; }
+            __syncwarp();
+            // neighbours of one token become one run: a lane looks at elements 2 lane and 2 lane + 1
+            const u32 e0 = 2 * lane, e1 = e0 + 1;
+            const u32 a0 = e0 < total ? LS.rtok[e0] : 0xFFFFFFFFu, a1 = e1 < total ? LS.rtok[e1] : 0xFFFFFFFFu;
+            const u32 n0 = e0 < total ? LS.rcnt[e0] : 0u, n1 = e1 < total ? LS.rcnt[e1] : 0u;
+            u32 ap = __shfl_up_sync(FULL, a1, 1);
+            if (lane == 0) ap = 0xFFFFFFFEu;
+            const bool h0 = e0 < total && a0 != ap, h1 = e1 < total && a1 != a0;
+            u32 hd = (h0 ? 1u : 0u) + (h1 ? 1u : 0u);
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) { const u32 v = __shfl_up_sync(FULL, hd, o); if (lane >= (u32)o) hd += v; }
+            m = __shfl_sync(FULL, hd, 31);
+            if (m > 32) { ok = false; break; }
+            __syncwarp();
+            LS.rcnt[lane] = 0;
+            __syncwarp();
+            const u32 i1 = hd - 1, i0 = i1 - (h1 ? 1u : 0u);          // runs of the two elements
+            if (e0 < total) { if (h0) LS.rtok[i0] = a0; atomicAdd(&LS.rcnt[i0], n0); }
+            if (e1 < total) { if (h1) LS.rtok[i1] = a1; atomicAdd(&LS.rcnt[i1], n1); }
+            __syncwarp();
+            tok = lane < m ? LS.rtok[lane] : 0u; cnt = lane < m ? LS.rcnt[lane] : 0u;
+            __syncwarp();
+        }
+        if (ok) {
+            u32 end = lane < m ? cnt : 0u;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) { const u32 v = __shfl_up_sync(FULL, end, o); if (lane >= (u32)o) end += v; }
+            LS.rtok[lane] = tok; LS.rcnt[lane] = end;                  // (lanes beyond the runs: no token, the same end)
+        }
+        if (lane == 0) *nruns = ok ? m : 0u;
+    }
+    __syncthreads();
+    const u32 m = *nruns;
+    if (m == 0) return false;
+    const u32 total = LS.rcnt[m - 1];
+    for (u32 r = 0; r < m; r++) {
+        const int32_t id = P.ext_id[LS.rtok[r]];
+        for (u32 j = (r ? LS.rcnt[r - 1] : 0u) + tid; j < LS.rcnt[r]; j += T) P.stage[a + j] = id;
+    }
+    if (tid == 0) piece_done(P, slot, total);
+    __syncthreads();
+    return true;
+}
+
+// The part of lq that starts at c0, with the number of windows before each of its pieces; returns how many there are.
+__device__ u32 long_chunk(const PieceParams& P, u32 c0, u32 nl, LongShared& LS, u32* sc) {
+    const u32 tid = threadIdx.x;
+    __syncthreads();
+    uint4 q = make_uint4(0, 0, 0, 0);
+    if (tid < (u32)LQ_CHUNK && c0 + tid < nl) q = __ldcg(&P.lq[c0 + tid]);
+    u32 total;
+    const u32 ex = cta_excl_sum_scan(q.w == LQ_WINDOWS ? long_windows(q.y) : 0u, sc, &total);
+    if (tid < (u32)LQ_CHUNK) { LS.q[tid] = q; LS.pre[tid] = ex; }
+    __syncthreads();
+    return total;
+}
+__device__ __forceinline__ uint4 long_find(const LongShared& LS, u32 w, u32& k) {      // piece and number of window w of the chunk
+    u32 lo = 0, hi = LQ_CHUNK;                           // the last piece with at most w windows before it
+    while (hi - lo > 1) { const u32 mid = (lo + hi) >> 1; if (LS.pre[mid] <= w) lo = mid; else hi = mid; }
+    k = w - LS.pre[lo];
+    return LS.q[lo];
+}
+
+// The windows' results stand at the byte positions of their tokens, two words per position: even windows in the first, odd
+// ones in the second (a window overlaps its neighbours only).  Entry = token + 1 where a token begins, else 0.
+__device__ __forceinline__ u32* long_at(const PieceParams& P, u32 a, u32 pos, u32 k) { return reinterpret_cast<u32*>(P.pairbuf + a + pos) + (k & 1); }
+// A word per window that no window's result uses: 64 bytes into window k, in the words of the other windows.
+__device__ __forceinline__ u32* long_word(const PieceParams& P, u32 a, u32 k) { return long_at(P, a, k * LSTEP + 64, k + 1); }
+
+__device__ __noinline__ void long_window(const PieceParams& P, const u8* __restrict__ text, uint4 q, u32 k, u64* wbuf, int lane) {
+    u32* const buf = reinterpret_cast<u32*>(wbuf);
+    const u32 s = k * LSTEP, size = min(LWIN, q.y - s);
+    if (k == 0 && lane == 0) P.piece_cnt[q.z] = 0u;      // (set to 1 where two windows do not meet)
+    const u32 m = warp_merge_perm<WCH>(buf, text, q.x + s, size, P.tab, lane, [&](u32 j, u32 t) { buf[j] = t; });
+    __syncwarp();
+    u32 t[8], len[8], sum = 0;                           // eight neighbouring tokens per lane
+#pragma unroll
+    for (int j = 0; j < 8; j++) { const u32 i = lane * 8 + j; t[j] = i < m ? buf[i] : 0u; len[j] = i < m ? (u32)P.tok_len[t[j]] : 0u; sum += len[j]; }
+    u32 pos = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const u32 x = __shfl_up_sync(0xFFFFFFFFu, pos, o); if (lane >= o) pos += x; }
+    pos -= sum;
+    u32* const arr = buf + 512;
+#pragma unroll
+    for (int j = 0; j < 8; j++) arr[j * 32 + lane] = 0u;
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 8; j++) { if (lane * 8 + j < m && pos < LWIN) arr[pos] = t[j] + 1u; pos += len[j]; }
+    __syncwarp();
+    for (u32 p = lane; p < size; p += 32) *long_at(P, q.x, s + p, k) = arr[p];
+    __syncwarp();
+}
+// Where windows k and k + 1 share a token (offset in the piece), 0xFFFFFFFF: nowhere.
+__device__ __forceinline__ u32 long_seam(const PieceParams& P, uint4 q, u32 k, int lane) {
+    const u32 from = (k + 1) * LSTEP, to = min(k * LSTEP + LWIN, q.y);
+    u32 hit[2];
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+        const u32 p = from + h * 32 + lane;
+        u32 x = 0, y = 1;
+        if (p < to) { x = __ldcg(long_at(P, q.x, p, k)); y = __ldcg(long_at(P, q.x, p, k + 1)); }
+        hit[h] = __ballot_sync(0xFFFFFFFFu, x != 0 && x == y);
+    }
+    return hit[0] ? from + (u32)__ffs(hit[0]) - 1 : hit[1] ? from + 32 + (u32)__ffs(hit[1]) - 1 : 0xFFFFFFFFu;
+}
+__device__ __forceinline__ void long_span(const PieceParams& P, uint4 q, u32 k, int lane, u32& left, u32& right) {     // window k decides [left, right)
+    left = k ? long_seam(P, q, k - 1, lane) : 0u;
+    right = k + 1 < long_windows(q.y) ? long_seam(P, q, k, lane) : q.y;
+}
+
+__device__ __forceinline__ u32 long_count(const PieceParams& P, uint4 q, u32 k, u32 left, u32 right, int lane) {       // tokens of window k in [left, right)
+    u32 cnt = 0;
+    for (u32 p0 = left; p0 < right; p0 += 32) cnt += __popc(__ballot_sync(0xFFFFFFFFu, p0 + lane < right && __ldcg(long_at(P, q.x, p0 + lane, k)) != 0));
+    return cnt;
+}
+__device__ __forceinline__ void long_write(const PieceParams& P, uint4 q, u32 k, u32 left, u32 right, u32 at, int lane) {   // ... to the piece's places from `at` on
+    for (u32 p0 = left; p0 < right; p0 += 32) {
+        const u32 v = p0 + lane < right ? __ldcg(long_at(P, q.x, p0 + lane, k)) : 0u;
+        const u32 b = __ballot_sync(0xFFFFFFFFu, v != 0);
+        if (v && at < q.y) P.stage[q.x + at + __popc(b & ((1u << lane) - 1))] = P.ext_id[v - 1];
+        at += __popc(b);
+    }
+}
+
+// A piece of at most as many windows as the CTA has warps is the CTA's own: nobody waits for it.
+constexpr u32 LONG_CTA_MAX = (MERGE_WARPS - 1) * LSTEP + LWIN;
+__device__ __noinline__ void cta_window_piece(const PieceParams& P, const u8* __restrict__ text, uint4 q, u64* s_buf, u32* sc) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const u32 nw = long_windows(q.y), k = (u32)wid;
+    __syncthreads();
+    if (k < nw) long_window(P, text, q, k, s_buf + wid * WARP_SMEM_WORDS, lane);
+    __syncthreads();
+    u32 left = 0, right = 0, cnt = 0;
+    if (k < nw) long_span(P, q, k, lane, left, right);
+    const bool meet = left != 0xFFFFFFFFu && right != 0xFFFFFFFFu;
+    if (meet) cnt = long_count(P, q, k, left, right, lane);
+    if (lane == 0) sc[wid] = cnt;
+    u32 total = 0;
+    if (__syncthreads_and(meet)) {
+        u32 at = 0;
+        for (int w = 0; w < MERGE_WARPS; w++) { const u32 c = sc[w]; total += c; if (w < wid) at += c; }
+        long_write(P, q, k, left, right, at, lane);
+    } else total = cta_merge_long(text, q.x, q.y, P.tab, P.ext_id, P.stage, P.pairbuf + q.x, s_buf, sc);
+    if (threadIdx.x == 0) piece_done(P, q.z, total);
+    __syncthreads();
+}
+// What a CTA does with a long piece that it comes upon; false: the piece is for the whole grid.
+__device__ __forceinline__ bool cta_long_piece(const PieceParams& P, const u8* __restrict__ text, uint4 q, u64* s_buf, u32* sc, LongShared& LS) {
+    if (cta_run_piece(P, text, q.x, q.y, q.z, LS)) return true;
+    if (q.y > LONG_CTA_MAX) return false;
+    cta_window_piece(P, text, q, s_buf, sc);
+    return true;
+}
+
+// The pieces of lq in state LQ_WINDOWS, once the `found` tasks that look for long pieces are done.  Called by every CTA.
+__device__ __noinline__ void long_phase(const PieceParams& P, const u8* __restrict__ text, u32 found, u64* s_buf, u32* sc, LongShared& LS) {
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    if (!long_wait(P, 0, found)) return;
+    const u32 nl = *reinterpret_cast<volatile u32*>(&P.hdr->nq_long);
+    if (nl == 0) return;
+    u64* const wbuf = s_buf + wid * WARP_SMEM_WORDS;
+    // f(piece, window) for the windows of the list, by tickets of step `step`; returns the number of windows
+    auto each_window = [&](int step, auto f) {
+        u32 base = 0, mine = 0, t = warp_take(&P.hdr->long_take[step], lane);
+        for (u32 c0 = 0; c0 < nl; c0 += LQ_CHUNK) {
+            const u32 total = long_chunk(P, c0, nl, LS, sc);
+            while (t - base < total) { u32 k; const uint4 q = long_find(LS, t - base, k); f(q, k); mine++; t = warp_take(&P.hdr->long_take[step], lane); }
+            base += total;
+        }
+        __syncwarp();
+        if (lane == 0 && mine) long_did(P, step, mine);
+        return base;
+    };
+    const u32 nwin = each_window(1, [&](const uint4& q, u32 k) { long_window(P, text, q, k, wbuf, lane); });
+    if (!long_wait(P, 1, nwin)) return;
+    // how many tokens each window contributes
+    each_window(2, [&](const uint4& q, u32 k) {
+        u32 left, right;
+        long_span(P, q, k, lane, left, right);
+        if (left == 0xFFFFFFFFu || right == 0xFFFFFFFFu) { if (lane == 0) P.piece_cnt[q.z] = 1u; return; }
+        const u32 cnt = long_count(P, q, k, left, right, lane);
+        if (lane == 0) *long_word(P, q.x, k) = cnt;
+    });
+    if (!long_wait(P, 2, nwin)) return;
+    // a CTA per piece: the places of the windows' tokens
+    {
+        u32 mine = 0;
+        for (u32 e; (e = cta_take(&P.hdr->long_take[3], &LS.ticket)) < nl;) {     // block-uniform
+            mine++;
+            const uint4 q = __ldcg(&P.lq[e]);
+            if (q.w != LQ_WINDOWS) continue;
+            const u32 bad = __ldcg(&P.piece_cnt[q.z]);
+            __syncthreads();
+            if (bad) { if (tid == 0) P.lq[e].w = LQ_FALLBACK; continue; }
+            const u32 nw = long_windows(q.y);
+            u32 carry = 0;
+            for (u32 k0 = 0; k0 < nw; k0 += blockDim.x) {
+                const u32 k = k0 + tid;
+                u32 total;
+                const u32 ex = cta_excl_sum_scan(k < nw ? __ldcg(long_word(P, q.x, k)) : 0u, sc, &total);
+                if (k < nw) *long_word(P, q.x, k) = carry + ex;
+                carry += total;
+                __syncthreads();
+            }
+            if (tid == 0) piece_done(P, q.z, carry);
+        }
+        __syncthreads();
+        if (tid == 0 && mine) long_did(P, 3, mine);
+    }
+    if (!long_wait(P, 3, nl)) return;
+    // the ids
+    each_window(4, [&](const uint4& q, u32 k) {
+        u32 left, right;
+        long_span(P, q, k, lane, left, right);
+        long_write(P, q, k, left, right, __ldcg(long_word(P, q.x, k)), lane);
+    });
+    // windows that do not meet: the piece as a whole (nobody waits any more)
+    for (u32 e; (e = cta_take(&P.hdr->long_take[5], &LS.ticket)) < nl;) {         // block-uniform
+        const uint4 q = __ldcg(&P.lq[e]);
+        if (q.w != LQ_FALLBACK) continue;
+        const u32 m = cta_merge_long(text, q.x, q.y, P.tab, P.ext_id, P.stage, P.pairbuf + q.x, s_buf, sc);
+        if (tid == 0) piece_done(P, q.z, m);
+    }
+    __syncthreads();
+}
+
+// A request: the long pieces of one tile, by one thread; f(piece) for each.
+template <class F>
+__device__ __forceinline__ void tile_long_pieces(const PieceParams& P, int t, u32 tq, u32 np, u32 last, u32 next, F f) {
+    const u32 nl = (tq >> TQ_NL_SHIFT) & TQ_NL_MASK;
+    for (u32 j = 0; j < nl && j < (u32)TT_TILE_LONGCAP; j++) {
+        const u32 idx = P.tile_long[(size_t)t * TT_TILE_LONGCAP + j];
+        const u32 o = P.piece_off16[(size_t)t * TT_TILE_BYTES + idx], o2 = P.piece_off16[(size_t)t * TT_TILE_BYTES + idx + 1];
+        f(make_uint4((u32)((long long)t * TT_TILE_BYTES + o - P.shift), o2 - o, (u32)t * TT_TILE_BYTES + idx, 0u));
+    }
+    if (np) {
+        const u32 st = (u32)t * TT_TILE_BYTES + last, n = (next != TT_NONE ? (u32)(t + 1) * TT_TILE_BYTES + next : closing_piece_end(P, t)) - st;
+        if (n > (u32)TT_WARP_PIECE_MAX) f(make_uint4((u32)((long long)st - P.shift), n, (u32)t * TT_TILE_BYTES + np - 1, 0u));
+    }
+}
+// The long pieces of the list LS.q[0 .. cnt), by the whole CTA.
+__device__ __noinline__ void cta_long_list(const PieceParams& P, const u8* __restrict__ text, u32 cnt, u64* s_buf, u32* sc, LongShared& LS) {
+    const int tid = threadIdx.x;
+    for (u32 e = 0; e < cnt; e++) {                                   // block-uniform
+        const uint4 q = LS.q[e];
+        __syncthreads();
+        if (!piece_in_range(P, q.x, q.y, q.z, 3u)) continue;
+        if (tid == 0) { u32 v = 0; sc[SCR_FLAG] = piece_settled_without_merge(P, text, q.x, q.y, v) ? 1u : 0u; sc[SCR_VALUE] = v; }
+        __syncthreads();
+        if (sc[SCR_FLAG]) { if (tid == 0) { P.piece_cnt[q.z] = sc[SCR_VALUE]; atomicAdd(&P.tile_tok[q.z / TT_TILE_BYTES], 1u); } continue; }
+        const bool done = cta_long_piece(P, text, q, s_buf, sc, LS);
+        if (tid == 0 && !done) P.lq[atomicAdd(&P.hdr->nq_long, 1u)] = make_uint4(q.x, q.y, q.z, LQ_WINDOWS);
+    }
+    __syncthreads();
+}
+// A request: looks for its long pieces.  Without one for the whole grid, the CTA merges those of every gridDim.x-th tile and
+// nobody waits for it; with one, the tiles go by tickets, LONG_FIND each, so that all of them are looked at by the CTAs
+// that run.  Returns whether there are long pieces (1) and some for the grid (2); every CTA comes to the same answer.
+constexpr int LONG_FIND = 8;
+__device__ __forceinline__ u32 long_find_tasks(const PieceParams& P) { return (u32)(P.ntiles + LONG_FIND - 1) / LONG_FIND; }
+__device__ __noinline__ u32 cta_find_long(const PieceParams& P, const u8* __restrict__ text, u64* s_buf, u32* sc, LongShared& LS) {
+    const int tid = threadIdx.x;
+    if (tid == 0) LS.pre[0] = 0;
+    __syncthreads();
+    bool any = false, grid = false;
+    for (int t = tid; t < P.ntiles; t += MERGE_THREADS) {
+        const u32 next = t + 1 < P.ntiles ? P.tile_first[t + 1] : TT_NONE;
+        tile_long_pieces(P, t, P.tile_q[t], P.tile_cnt[t], P.tile_last[t], next, [&](uint4 q) {
+            any = true; grid |= q.y > LONG_CTA_MAX;
+            if (t % (int)gridDim.x == (int)blockIdx.x) { const u32 k = atomicAdd(&LS.pre[0], 1u); if (k < (u32)LQ_CHUNK) LS.q[k] = q; }
+        });
+    }
+    // (a share of more than 256 long pieces: by tickets too)
+    grid |= P.ntiles > (int)gridDim.x * (LQ_CHUNK / (TT_TILE_LONGCAP + 1));
+    if (!__syncthreads_or(any)) return 0;
+    if (!__syncthreads_or(grid)) { cta_long_list(P, text, LS.pre[0], s_buf, sc, LS); return 1; }
+    const u32 tasks = long_find_tasks(P);
+    u32 mine = 0;
+    for (u32 task; (task = cta_take(&P.hdr->long_take[0], &LS.ticket)) < tasks;) {
+        mine++;
+        if (tid == 0) LS.pre[0] = 0;
+        __syncthreads();
+        const int t = (int)task * LONG_FIND + tid;
+        static_assert(LONG_FIND * (TT_TILE_LONGCAP + 1) <= LQ_CHUNK, "the long pieces of a task");
+        if (tid < LONG_FIND && t < P.ntiles)
+            tile_long_pieces(P, t, P.tile_q[t], P.tile_cnt[t], P.tile_last[t], t + 1 < P.ntiles ? P.tile_first[t + 1] : TT_NONE, [&](uint4 q) { LS.q[atomicAdd(&LS.pre[0], 1u)] = q; });
+        __syncthreads();
+        cta_long_list(P, text, LS.pre[0], s_buf, sc, LS);
+    }
+    __syncthreads();
+    if (tid == 0 && mine) long_did(P, 0, mine);
+    return 2;
 }
 
 // Bulk text: the last CTA of k_merge to finish sums the token counts of every group of 256 tiles for k_scatter (a
@@ -959,20 +1346,24 @@ __device__ __forceinline__ void merge_group_totals(const PieceParams& P, u32* s_
     }
 }
 
-// Bulk text (k_closing has gathered the lists): long pieces a CTA each, warp-class pieces a warp each by index,
-// short pieces 32 of one length class at a time by ticket, a thread each.
-__device__ void merge_bulk_lists(const PieceParams& P, const u8* __restrict__ text, u64* s_buf, u32* sc, u32* s_warps_done) {
+// Bulk text (k_closing has gathered the lists): long pieces a CTA each where that is quick, else window by window with the
+// whole grid, warp-class pieces a warp each by index, short pieces 32 of one length class at a time by ticket, a thread each.
+__device__ void merge_bulk_lists(const PieceParams& P, const u8* __restrict__ text, u64* s_buf, u32* sc, LongShared& LS, u32* s_warps_done) {
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const u32 FULL = 0xFFFFFFFFu;
     const u32 nl = P.hdr->nq_long, nw = P.hdr->nwq, ns = P.hdr->nq_short;
-    for (u32 e = blockIdx.x; e < nl; e += gridDim.x) {                // block-uniform
-        const uint4 q = P.lq[e];
+    if (nl) {
+        u32 mine = 0;
+        for (u32 e; (e = cta_take(&P.hdr->long_take[0], &LS.ticket)) < nl;) {     // block-uniform
+            mine++;
+            const uint4 q = P.lq[e];
+            u32 state = LQ_DONE;
+            if (piece_in_range(P, q.x, q.y, q.z, 3u) && !cta_long_piece(P, text, q, s_buf, sc, LS)) state = LQ_WINDOWS;
+            if (tid == 0) P.lq[e].w = state;
+        }
         __syncthreads();
-        if (!piece_in_range(P, q.x, q.y, q.z, 3u)) continue;
-        const u32 m = cta_merge_long(text, q.x, q.y, P.tab, P.ext_id, P.stage, P.pairbuf + q.x, s_buf, sc);
-        if (tid == 0) piece_done(P, q.z, m);
+        if (tid == 0 && mine) long_did(P, 0, mine);
     }
-    if (nl > blockIdx.x) __syncthreads();
     u64* wbuf = s_buf + wid * WARP_SMEM_WORDS;
     const u32 W = gridDim.x * MERGE_WARPS, gw = (u32)wid * gridDim.x + blockIdx.x;
     for (u32 j = gw; j < nw; j += W) {                                // bounded by the list length
@@ -1012,6 +1403,7 @@ __device__ void merge_bulk_lists(const PieceParams& P, const u8* __restrict__ te
         }
         __syncwarp();
     }
+    if (nl) long_phase(P, text, nl, s_buf, sc, LS);
     merge_group_totals(P, s_warps_done);
 }
 
@@ -1021,6 +1413,7 @@ k_merge_bulk(const __grid_constant__ PieceParams P) {
     extern __shared__ __align__(16) u64 s_buf[];              // MERGE_SMEM_BYTES
     __shared__ u32 sc[SCR_WORDS];
     __shared__ u32 s_warps_done;
+    __shared__ LongShared LS;
     cudaTriggerProgrammaticLaunchCompletion();               // k_scatter may be placed; it waits for this grid's memory itself
     grid_prefetch_l2(P.tab.slots, ((size_t)P.tab.mask + 1) * 2 * sizeof(uint4));
     grid_prefetch_l2(P.tab.bytepair, 65536 * sizeof(u64));
@@ -1028,164 +1421,133 @@ k_merge_bulk(const __grid_constant__ PieceParams P) {
     cudaGridDependencySynchronize();                         // k_closing's lists are complete from here on
     __syncthreads();
     if (hdr_status(P.hdr, P.epoch) != 0) return;
-    merge_bulk_lists(P, P.base + P.shift, s_buf, sc, &s_warps_done);
+    merge_bulk_lists(P, P.base + P.shift, s_buf, sc, LS, &s_warps_done);
+}
+
+// Where a request's unsettled pieces stand, for the job search of k_merge: exclusive prefixes of the tiles' counts of short
+// and of warp-class pieces, in shared memory behind the warps' buffers (an entry is one tile up to 2,048 tiles).  The CTA
+// scans them once with one 16-byte load per thread; every warp then finds its jobs by bisection.  (Each warp summing the
+// counts of all tiles for itself took 1.6 us at 489 tiles, 13 at 1,400 and 24 at 1,900.)
+constexpr int MERGE_ENTRIES = MERGE_SR_MAX_TILES;
+struct MergeIndex { u32 pre_s[MERGE_ENTRIES + 1], pre_w[MERGE_ENTRIES + 1]; u64 wtot[MERGE_WARPS]; };
+constexpr size_t MERGE_SMEM_REQUEST = MERGE_SMEM_BYTES + sizeof(MergeIndex);
+static_assert(4 * MERGE_THREADS >= MERGE_ENTRIES, "four entries per thread");
+
+// Returns whether any tile allows for a piece of more than 256 bytes.
+__device__ __forceinline__ bool merge_index(const PieceParams& P, int unit, int entries, MergeIndex& X) {
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    u32 c[4] = {0, 0, 0, 0}, flags = 0;                           // per entry: short pieces (low half), warp-class pieces
+    u64 mine = 0;
+    if (4 * tid < entries) {
+        if (unit == 1) {
+            const uint4 v = *reinterpret_cast<const uint4*>(P.tile_q + 4 * tid);
+            c[0] = v.x; c[1] = v.y; c[2] = v.z; c[3] = v.w;
+        }
+#pragma unroll
+        for (int h = 0; h < 4; h++) {
+            u32 s = 0, w = 0;
+            for (int u = 0; u < unit; u++) {
+                const int t = (4 * tid + h) * unit + u;
+                if (t < P.ntiles) { const u32 q = unit == 1 ? c[h] : P.tile_q[t]; s += q & TQ_NS_MASK; w += (q >> TQ_NW_SHIFT) & TQ_NW_MASK; flags |= q; }
+            }
+            c[h] = s | (w << 16);
+            mine += (u64)s | ((u64)w << 32);
+        }
+    }
+    u64 x = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) { const u64 t = __shfl_up_sync(0xFFFFFFFFu, x, o); if (lane >= o) x += t; }
+    if (lane == 31) X.wtot[wid] = x;
+    __syncthreads();
+    u64 before = x - mine;
+    for (int w = 0; w < wid; w++) before += X.wtot[w];
+    if (4 * tid < entries) {
+        u32 s = (u32)before, w = (u32)(before >> 32);
+#pragma unroll
+        for (int h = 0; h < 4; h++) if (4 * tid + h <= entries) { X.pre_s[4 * tid + h] = s; X.pre_w[4 * tid + h] = w; s += c[h] & 0xFFFFu; w += c[h] >> 16; }
+        if (4 * tid + 4 >= entries) { X.pre_s[entries] = s; X.pre_w[entries] = w; }       // (entries behind the last one count nothing)
+    }
+    return __syncthreads_or(flags >> 31);
+}
+// The last entry with at most k pieces before it.
+__device__ __forceinline__ u32 merge_find(const u32* pre, u32 entries, u32 k) {
+    u32 lo = 0, hi = entries;
+    while (hi - lo > 1) { const u32 mid = (lo + hi) >> 1; if (pre[mid] <= k) lo = mid; else hi = mid; }
+    return lo;
 }
 
 __global__ void __launch_bounds__(MERGE_THREADS, MERGE_CTAS_PER_SM)
 k_merge(const __grid_constant__ PieceParams P) {
-    extern __shared__ __align__(16) u64 s_buf[];              // MERGE_SMEM_BYTES
+    extern __shared__ __align__(16) u64 s_buf[];              // MERGE_SMEM_REQUEST
     __shared__ u32 sc[SCR_WORDS];
-    __shared__ uint4 s_long[TT_TILE_LONGCAP + 2];             // the long pieces of one tile
-    __shared__ u32 s_nlong;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    __shared__ LongShared LS;
+    MergeIndex& X = *reinterpret_cast<MergeIndex*>(s_buf + MERGE_WARPS * WARP_SMEM_WORDS);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const u32 FULL = 0xFFFFFFFFu;
     cudaTriggerProgrammaticLaunchCompletion();               // k_scatter may be placed; it waits for this grid's memory itself
     grid_prefetch_l2(P.tab.slots, ((size_t)P.tab.mask + 1) * 2 * sizeof(uint4));
     grid_prefetch_l2(P.tab.bytepair, 65536 * sizeof(u64));
     cudaGridDependencySynchronize();                         // the first kernel's per-tile records are complete from here on
-    if (hdr_status(P.hdr, P.epoch) != 0) return;
+    const int status = hdr_status(P.hdr, P.epoch);
+    const int unit = (P.ntiles + MERGE_ENTRIES - 1) / MERGE_ENTRIES, entries = (P.ntiles + unit - 1) / unit;   // tiles per entry: 1 for a request
+    const bool may_long = merge_index(P, unit, entries, X);
+    if (status != 0) return;
     const u8* text = P.base + P.shift;
-    // ---- records of this CTA's share of the tiles (long pieces, a whole CTA each; a request settles them after
-    // its short pieces, bulk text before); the loads go out next to those of the job search below
-    const int per = (P.ntiles + (int)gridDim.x - 1) / (int)gridDim.x;
-    const int t_lo = (int)blockIdx.x * per, t_hi = min(P.ntiles, t_lo + per);
-    u32 a_nl = 0, a_np = 0, a_last = 0, a_next = TT_NONE;
-    {
-        const int t = t_lo + tid;
-        if (t < t_hi) {
-            a_nl = (P.tile_q[t] >> TQ_NL_SHIFT) & TQ_NL_MASK; a_np = P.tile_cnt[t]; a_last = P.tile_last[t];
-            if (t + 1 < P.ntiles) a_next = P.tile_first[t + 1];
-        }
-    }
+    const u32 longs = may_long ? cta_find_long(P, text, s_buf, sc, LS) : 0u;
     u64* wbuf = s_buf + wid * WARP_SMEM_WORDS;
     const u32 W = gridDim.x * MERGE_WARPS, gw = (u32)wid * gridDim.x + blockIdx.x;   // numbered across the CTAs first
-    const bool big = false;                                       // (bulk text took the lists above)
-    // job search of a request: every lane sums the counts of a stretch of tiles, kept as 16 sums of `unit` tiles
-    // (short pieces in the low half, warp-class pieces in the high half of a word)
-    const int unit = (P.ntiles + 511) / 512;                      // 1..4 tiles per register
-    const int tb = lane * 16 * unit;
-    u32 part[16];
-    u32 my_s = 0, my_w = 0;
-    if (!big) {
-        if (unit == 1) {                                          // up to 512 tiles: sixteen counts per lane, four vector loads
-            const uint4* src = reinterpret_cast<const uint4*>(P.tile_q + tb);
-            uint4 v[4];
-#pragma unroll
-            for (int g = 0; g < 4; g++) v[g] = tb + 4 * g < P.ntiles ? src[g] : make_uint4(0, 0, 0, 0);
-#pragma unroll
-            for (int g = 0; g < 16; g++) {
-                const uint4 x = v[g >> 2];
-                const u32 q = (g & 3) == 0 ? x.x : (g & 3) == 1 ? x.y : (g & 3) == 2 ? x.z : x.w;
-                part[g] = tb + g < P.ntiles ? (q & TQ_NS_MASK) | (((q >> TQ_NW_SHIFT) & TQ_NW_MASK) << 16) : 0u;
-            }
-        } else {
-#pragma unroll
-            for (int g = 0; g < 16; g++) {
-                u32 s1 = 0;
-                for (int u = 0; u < unit; u++) {
-                    const int t = tb + g * unit + u;
-                    if (t < P.ntiles) { const u32 q = P.tile_q[t]; s1 += (q & TQ_NS_MASK) | (((q >> TQ_NW_SHIFT) & TQ_NW_MASK) << 16); }
-                }
-                part[g] = s1;
-            }
-        }
-#pragma unroll
-        for (int g = 0; g < 16; g++) { my_s += part[g] & 0xFFFFu; my_w += part[g] >> 16; }
-    }
-    // the closing piece of tile t_lo + tid: is it long?
-    bool closing_long = false;
-    u32 c_end = 0;
-    if (a_np) {
-        const int t = t_lo + tid;
-        c_end = (t + 1 >= P.ntiles) ? (u32)P.hi : a_next != TT_NONE ? (u32)(t + 1) * TT_TILE_BYTES + a_next : closing_piece_end(P, t);
-        closing_long = c_end - ((u32)t * TT_TILE_BYTES + a_last) > (u32)TT_WARP_PIECE_MAX;
-    }
-    bool tickets = big;                                           // short pieces by tickets (bulk) or job by job (a request)
-    if (!big) {
-        u32 bs = my_s, bw = my_w;                                     // exclusive prefixes over the lanes
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const u32 x = __shfl_up_sync(FULL, bs, o), y = __shfl_up_sync(FULL, bw, o);
-            if (lane >= o) { bs += x; bw += y; }
-        }
-        const u32 NS = __shfl_sync(FULL, bs, 31), NW = __shfl_sync(FULL, bw, 31), NT = (u32)P.ntiles;
-        bs -= my_s; bw -= my_w;
+    const u32 NS = X.pre_s[entries], NW = X.pre_w[entries], NT = (u32)P.ntiles;
 #ifndef TT_SHORT_WARP_FACTOR
 #define TT_SHORT_WARP_FACTOR 12u
 #endif
-        // Measured crossover (1 M to 8 M chars of Unicode-heavy prose, 15 K to 120 K unsettled pieces): a warp per piece
-        // wins up to about 17 pieces per warp of the grid.
-        tickets = NS + NT > TT_SHORT_WARP_FACTOR * W;
-        const u32 J = tickets ? NW : NW + NT + NS;                    // with tickets only the warp-class pieces go job by job
-        for (u32 j = gw; j < J; j += W) {                             // bounded by the number of jobs
-            u32 a, n, slot;
-            if (j >= NW && j < NW + NT) {                             // the closing piece of tile j - NW
-                const int t = (int)(j - NW);
-                const u32 np = P.tile_cnt[t];
-                if (np == 0) continue;
-                const u32 st = (u32)t * TT_TILE_BYTES + P.tile_last[t];
-                n = closing_piece_end(P, t) - st;
-                if (n > (u32)TT_WARP_PIECE_MAX) continue;             // settled by a CTA below
-                a = (u32)((long long)st - P.shift); slot = (u32)t * TT_TILE_BYTES + np - 1;
-                u32 v;
-                if (piece_settled_without_merge(P, text, a, n, v)) {  // every lane computes the same
-                    if (lane == 0) { P.piece_cnt[slot] = v; atomicAdd(&P.tile_tok[t], 1u); }
-                    continue;
-                }
-            } else {
-                // the k-th queued piece of its class: the lane whose stretch holds it finds the tile
-                const bool wclass = j < NW;
-                const u32 k = wclass ? j : j - NW - NT;
-                const int sh = wclass ? 16 : 0;
-                const u32 owner = 31u - (u32)__clz(__ballot_sync(FULL, (wclass ? bw : bs) <= k) | 1u);
-                u32 found = 0;                                        // tile << 11 | rank within the tile
-                if ((u32)lane == owner) {
-                    u32 r = k - (wclass ? bw : bs);
-                    int g = 0;
-#pragma unroll
-                    for (int gg = 0; gg < 15; gg++) {
-                        const u32 c = (part[gg] >> sh) & 0xFFFFu;
-                        if (g == gg && r >= c) { r -= c; g = gg + 1; }
-                    }
-                    int t = tb + g * unit;
-                    for (int u = 0; u + 1 < unit; u++) {
-                        const u32 q = t < P.ntiles ? P.tile_q[t] : 0u;
-                        const u32 c = wclass ? (q >> TQ_NW_SHIFT) & TQ_NW_MASK : q & TQ_NS_MASK;
-                        if (r < c) break;
-                        r -= c; t++;
-                    }
-                    found = ((u32)t << 11) | r;
-                }
-                found = __shfl_sync(FULL, found, owner);
-                const u32 t = found >> 11, r = found & 2047u;
-                const u32 e = P.q[(size_t)t * TT_TILE_QCAP + (wclass ? (u32)TT_TILE_QCAP - 1 - r : r)];
-                n = (e >> 22) + 1;
-                a = (u32)((long long)t * TT_TILE_BYTES + (e & 2047u) - P.shift); slot = t * TT_TILE_BYTES + ((e >> 11) & 2047u);
+    // Measured crossover (1 M to 8 M chars of Unicode-heavy prose, 15 K to 120 K unsettled pieces): a warp per piece
+    // wins up to about 17 pieces per warp of the grid.
+    const bool tickets = NS + NT > TT_SHORT_WARP_FACTOR * W;         // short pieces 32 at a time by tickets, or job by job
+    const u32 J = tickets ? NW : NW + NT + NS;                       // with tickets only the warp-class pieces go job by job
+    // Job by job in order (warp-class pieces, closing pieces, short pieces); where some CTAs first had a long piece to merge, by
+    // tickets of `step` jobs, the next one drawn in advance.
+    const u32 step = longs ? max(1u, J / (2 * W)) : 1u;
+    u32 jt = gw, jn = gw + W;
+    if (longs) { jt = warp_take(&P.hdr->t_short, lane); jn = warp_take(&P.hdr->t_short, lane); }
+    for (u32 j = jt * step, left = step; j < J;) {                   // bounded by the number of jobs
+        const u32 job = j;
+        if (--left) j++;
+        else { j = jn * step; left = step; jn = longs ? (j < J ? warp_take(&P.hdr->t_short, lane) : jn) : jn + W; }
+        u32 a, n, slot;
+        if (job >= NW && job < NW + NT) {                            // the closing piece of tile job - NW
+            const int t = (int)(job - NW);
+            const u32 np = P.tile_cnt[t], last = P.tile_last[t], next = t + 1 < P.ntiles ? P.tile_first[t + 1] : TT_NONE;
+            if (np == 0) continue;
+            const u32 st = (u32)t * TT_TILE_BYTES + last;
+            n = (next != TT_NONE ? (u32)(t + 1) * TT_TILE_BYTES + next : closing_piece_end(P, t)) - st;
+            if (n > (u32)TT_WARP_PIECE_MAX) continue;                // a long piece
+            a = (u32)((long long)st - P.shift); slot = (u32)t * TT_TILE_BYTES + np - 1;
+            u32 v;
+            if (piece_settled_without_merge(P, text, a, n, v)) {     // every lane computes the same
+                if (lane == 0) { P.piece_cnt[slot] = v; atomicAdd(&P.tile_tok[t], 1u); }
+                continue;
             }
-            warp_merge_piece(P, text, a, n, slot, wbuf, lane);
-        }
-        if (!tickets) {
-            // the request's long pieces, once every warp of the CTA is through with its short ones
-            if (__syncthreads_or(a_nl != 0 || closing_long))
-                cta_long_pieces(P, text, t_lo, t_hi, a_nl, a_np, a_last, c_end, closing_long, s_buf, sc, s_long, &s_nlong);
-            return;
-        }
-    }
-    for (int t0 = t_lo; t0 < t_hi; t0 += MERGE_THREADS) {            // block-uniform; shares beyond MERGE_THREADS tiles reload their records
-        if (t0 != t_lo) {
-            const int t = t0 + tid;
-            a_nl = 0; a_np = 0; a_last = 0; c_end = 0; closing_long = false;
-            if (t < t_hi) {
-                a_nl = (P.tile_q[t] >> TQ_NL_SHIFT) & TQ_NL_MASK; a_np = P.tile_cnt[t]; a_last = P.tile_last[t];
-                if (a_np) { c_end = closing_piece_end(P, t); closing_long = c_end - ((u32)t * TT_TILE_BYTES + a_last) > (u32)TT_WARP_PIECE_MAX; }
+        } else {
+            // the k-th queued piece of its class
+            const bool wclass = job < NW;
+            const u32 k = wclass ? job : job - NW - NT;
+            const u32* const pre = wclass ? X.pre_w : X.pre_s;
+            const u32 en = merge_find(pre, (u32)entries, k);
+            u32 r = k - pre[en], t = en * (u32)unit;
+            for (int u = 0; u + 1 < unit; u++) {
+                const u32 q = P.tile_q[t], c = wclass ? (q >> TQ_NW_SHIFT) & TQ_NW_MASK : q & TQ_NS_MASK;
+                if (r < c) break;
+                r -= c; t++;
             }
+            const u32 e = P.q[(size_t)t * TT_TILE_QCAP + (wclass ? (u32)TT_TILE_QCAP - 1 - r : r)];
+            n = (e >> 22) + 1;
+            a = (u32)((long long)t * TT_TILE_BYTES + (e & 2047u) - P.shift); slot = t * TT_TILE_BYTES + ((e >> 11) & 2047u);
         }
-        if (__syncthreads_or(a_nl != 0 || closing_long))
-            cta_long_pieces(P, text, t0, t_hi, a_nl, a_np, a_last, c_end, closing_long, s_buf, sc, s_long, &s_nlong);
+        warp_merge_piece(P, text, a, n, slot, wbuf, lane);
     }
+    if (tickets) {
     // ---- tickets: a tile each; its short pieces (queued ones, then its closing piece if that is short) wait in the
     // lanes until 32 of them are together, so that every step of the thread-per-piece merge is full
-    {
         u32* const tok = reinterpret_cast<u32*>(wbuf);
         const u32 ntick = (u32)P.ntiles;
         u32 pa = 0, pn = 0, pslot = 0, pend = 0;                      // lanes below `pend` hold a short piece that waits for a full step
@@ -1238,6 +1600,7 @@ k_merge(const __grid_constant__ PieceParams P) {
             if (last_round) break;
         }
     }
+    if (longs == 2) long_phase(P, text, long_find_tasks(P), s_buf, sc, LS);
 }
 
 // ---- K5: coalesced scatter of the staged ids, one text tile per CTA iteration ---------------------------------

@@ -56,11 +56,12 @@ struct TTHeader {
     u32 nwq;                 // bulk text: lengths of the global lists of warp-class, short and long pieces and the ticket
     u32 nq_short, nq_long;   //            counter of the short list (all cleared by a memset before the chain)
     u32 t_short;
+    u32 long_take[6], long_done[6];   // long pieces: tickets and finished tasks of each step (see long_phase); zeroed by the first kernel
     u32 nq_short_x[3];       // bulk text: the short pieces have a list per length class; lengths of the other lists (cleared likewise)
     u32 dbg[8];              // first failed self-check of a kernel: site, then up to seven values (diagnostics only)
-    u32 pad[11];
+    u32 pad[31];
 };
-static_assert(sizeof(TTHeader) == 128, "header layout");
+static_assert(sizeof(TTHeader) == 256, "header layout");
 
 // The status word carries the epoch of the call that wrote it (a process-wide counter, never zero), so a
 // value left by an earlier call -- or whatever an unused workspace holds -- reads as TT_OK and a single
@@ -97,7 +98,8 @@ __device__ __forceinline__ void hdr_set_status(TTHeader* h, unsigned long long e
 //   tile_first[t]  offset in the tile of its first piece start, TT_NONE if it has none
 //   tile_last[t]   offset in the tile of its last piece start (that piece ends in a later tile, or with the text)
 //   tile_tok[t]    tokens of the tile's pieces (the first kernel stores the settled ones, k_merge adds the rest)
-//   tile_q[t]      unsettled pieces: short (<= 32 B) count | warp-class (33..256 B) count << 11 | long count << 18
+//   tile_q[t]      unsettled pieces: short (<= 32 B) count | warp-class (33..256 B) count << 11 | long count << 18; bit 31: a piece
+//                  of more than 256 bytes may begin or end here
 //   piece_off16    [t * TT_TILE_BYTES + i]  offset in the tile of piece i
 //   piece_cnt      [t * TT_TILE_BYTES + i]  the id of piece i if it is one token found without merging (>= 0),
 //                                           else minus the number of ids staged at the piece's text offset

@@ -291,7 +291,11 @@ k_pretok(const __grid_constant__ PretokParams P, const __grid_constant__ FrontPa
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     cudaTriggerProgrammaticLaunchCompletion();               // the next kernel may be placed; it waits for this grid's memory itself
     if (FUSED) {
-        if (blockIdx.x == 0 && tid == 0) { P.hdr->t_tiles = 0; P.hdr->merge_done = 0; }   // k_merge's counters (k_merge touches them only after this grid)
+        if (blockIdx.x == 0 && tid == 0) {                    // k_merge's counters (k_merge touches them only after this grid)
+            P.hdr->t_tiles = 0; P.hdr->merge_done = 0;
+            for (int s = 0; s < 6; s++) { P.hdr->long_take[s] = 0; P.hdr->long_done[s] = 0; }
+            if (F.wq == nullptr) { P.hdr->t_short = 0; P.hdr->nq_long = 0; }
+        }
         // the whole-piece table is probed at random a few microseconds from now: ask for it to be brought into L2
         if (F.toktab.slots != nullptr) grid_prefetch_l2(F.toktab.slots, ((size_t)F.toktab.mask + 1) * sizeof(TokSlot));
     }
@@ -410,11 +414,15 @@ k_pretok(const __grid_constant__ PretokParams P, const __grid_constant__ FrontPa
         for (u32 m = S; m; m &= m - 1) s_off[r++] = (u16)(tid * TT_WORD + tt_lobit(m));
         __syncthreads();
         const size_t p0 = (size_t)tile * TT_TILE_BYTES;              // pieces are indexed per tile
+        u32 may_long = 0;
         for (u32 i = tid; i < np; i += NT) F.piece_off16[p0 + i] = s_off[i];
         if (tid == 0) {
             P.tile_cnt[tile] = np;
             P.tile_first[tile] = np ? (u32)s_off[0] : TT_NONE;
             F.tile_last[tile] = np ? (u32)s_off[np - 1] : TT_NONE;
+            // a piece of more than 256 bytes that crosses a tile boundary leaves 129 bytes before it or 128 behind it
+            const u32 used = (u32)min((long long)TT_TILE_BYTES, P.hi - w_first * TT_WORD);
+            may_long = np == 0 || s_off[0] >= 128 || used - s_off[np - 1] > 128 ? TQ_MAY_LONG : 0u;
         }
         // ---- K4, first half: whole-piece lookups, a thread per piece, LW pieces per thread and step, their table slots
         // fetched side by side.  Pieces of at most 8 bytes -- most of them -- take a path of their own: two key words, one
@@ -482,7 +490,7 @@ k_pretok(const __grid_constant__ PretokParams P, const __grid_constant__ FrontPa
         __syncthreads();
         if (tid == 0) {
             F.tile_tok[tile] = s_total;
-            F.tile_q[tile] = s_ns | ((F.wq != nullptr ? 0u : s_nw) << TQ_NW_SHIFT) | (s_nl << TQ_NL_SHIFT);
+            F.tile_q[tile] = may_long | (s_nl ? TQ_MAY_LONG : 0u) | s_ns | ((F.wq != nullptr ? 0u : s_nw) << TQ_NW_SHIFT) | (s_nl << TQ_NL_SHIFT);
             if (F.wq != nullptr && s_nw) s_wbase = atomicAdd(&P.hdr->nwq, s_nw);
         }
         if (F.wq != nullptr && s_nw) {                                // block-uniform
