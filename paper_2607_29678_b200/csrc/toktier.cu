@@ -496,14 +496,29 @@ extern "C" size_t tt_workspace_bytes(const tt_vocab* v, size_t max_len, size_t m
 
 #define CK(x) do { if ((x) != cudaSuccess) { cudaGetLastError(); return TT_ERR_CUDA; } } while (0)
 
+// Launches `kernel` so that it may begin while the kernel before it on the stream is still draining
+// (programmatic dependent launch): its CTAs are placed as soon as every CTA of the predecessor has
+// signalled, and wait inside the kernel (cudaGridDependencySynchronize) until the predecessor's memory
+// is complete.  Only the launch latency is hidden; the data dependence is unchanged.
+template <typename... KernelParams, typename... Params>
+static cudaError_t launch_after(void (*kernel)(KernelParams...), int grid, int block, cudaStream_t st, size_t smem, bool early, const Params&... p) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3((unsigned)block); cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = early ? 1 : 0;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, p...);
+}
+
 // One instance of the first kernel per pattern (the pattern's rules are compiled in), chosen here.
 template <bool FUSED, int NT, int MINB>
-static void launch_pretok(int grid, cudaStream_t st, const PretokParams& P, const FrontParams& F) {
+static cudaError_t launch_pretok(int grid, cudaStream_t st, bool early, const PretokParams& P, const FrontParams& F) {
     switch (P.pattern) {
-    case TT_PATTERN_O200K:     k_pretok<FUSED, NT, MINB, TT_PATTERN_O200K><<<grid, NT, 0, st>>>(P, F); break;
-    case TT_PATTERN_CL100K_N1: k_pretok<FUSED, NT, MINB, TT_PATTERN_CL100K_N1><<<grid, NT, 0, st>>>(P, F); break;
-    case TT_PATTERN_CUTS:      if constexpr (!FUSED) k_pretok<false, NT, MINB, TT_PATTERN_CUTS><<<grid, NT, 0, st>>>(P, F); break;
-    default:                   k_pretok<FUSED, NT, MINB, TT_PATTERN_CL100K><<<grid, NT, 0, st>>>(P, F); break;
+    case TT_PATTERN_O200K:     return launch_after(k_pretok<FUSED, NT, MINB, TT_PATTERN_O200K>, grid, NT, st, 0, early, P, F);
+    case TT_PATTERN_CL100K_N1: return launch_after(k_pretok<FUSED, NT, MINB, TT_PATTERN_CL100K_N1>, grid, NT, st, 0, early, P, F);
+    case TT_PATTERN_CUTS:      if constexpr (!FUSED) return launch_after(k_pretok<false, NT, MINB, TT_PATTERN_CUTS>, grid, NT, st, 0, early, P, F); else return cudaErrorInvalidValue;
+    default:                   return launch_after(k_pretok<FUSED, NT, MINB, TT_PATTERN_CL100K>, grid, NT, st, 0, early, P, F);
     }
 }
 
@@ -511,7 +526,7 @@ static void launch_pretok(int grid, cudaStream_t st, const PretokParams& P, cons
 // the encode chain derives them per tile from the start flags).
 static int run_pretok(const tt_vocab* v, const uint8_t* text, size_t len, const int64_t* doc_off, size_t n_docs,
                       cudaStream_t st, TTWorkspace& w, u32* piece_off_dst, PretokParams& P, bool literals = false, bool fused = false,
-                      const uint8_t* host_src = nullptr) {
+                      const uint8_t* host_src = nullptr, bool early = true) {
     const uintptr_t addr = (uintptr_t)text;
     const long long shift = (long long)(addr & 15);
     P.base = (const u8*)(addr - shift);
@@ -558,7 +573,7 @@ static int run_pretok(const tt_vocab* v, const uint8_t* text, size_t len, const 
         PretokParams C1 = P;
         C1.pattern = TT_PATTERN_CUTS; C1.startmask = w.cutmask;
         C1.want_prefix = 0; C1.litstart = nullptr; C1.litin = nullptr;
-        launch_pretok<false, PRETOK_THREADS_REQUEST, PRETOK_CTAS_REQUEST>(grid, st, C1, FrontParams{});
+        CK((launch_pretok<false, PRETOK_THREADS_REQUEST, PRETOK_CTAS_REQUEST>(grid, st, early, C1, FrontParams{})));
         P.pattern = TT_PATTERN_CL100K; P.docmask = w.cutmask;
     }
     if (fused) {
@@ -566,9 +581,9 @@ static int run_pretok(const tt_vocab* v, const uint8_t* text, size_t len, const 
         F.tile_last = w.tile_last; F.tile_tok = w.tile_tok; F.tile_q = w.tile_q; F.tile_long = w.tile_long; F.piece_off16 = w.piece_off16;
         F.piece_cnt = w.piece_cnt; F.q = w.q; F.toktab = v->toktab; F.longtab = v->longtab; F.ext_id = v->d_ext_id;
         F.wq = P.ntiles > MERGE_SR_MAX_TILES ? w.wq : nullptr;
-        if (bulk) launch_pretok<true, PRETOK_THREADS_BULK, PRETOK_CTAS_BULK>(grid, st, P, F);
-        else launch_pretok<true, PRETOK_THREADS_REQUEST, PRETOK_CTAS_REQUEST>(grid, st, P, F);
-    } else launch_pretok<false, PRETOK_THREADS_REQUEST, PRETOK_CTAS_REQUEST>(grid, st, P, FrontParams{});
+        if (bulk) CK((launch_pretok<true, PRETOK_THREADS_BULK, PRETOK_CTAS_BULK>(grid, st, early, P, F)));
+        else CK((launch_pretok<true, PRETOK_THREADS_REQUEST, PRETOK_CTAS_REQUEST>(grid, st, early, P, F)));
+    } else CK((launch_pretok<false, PRETOK_THREADS_REQUEST, PRETOK_CTAS_REQUEST>(grid, st, early, P, FrontParams{})));
     if (piece_off_dst)
         k_compact<<<grid, TT_TILE_WORDS, 0, st>>>(w.startmask, w.tile_cnt, P.nwords, P.ntiles, shift, (long long)len,
                                                    piece_off_dst, w.hdr, P.epoch);
@@ -583,21 +598,6 @@ static int check_common(const tt_vocab* v, const void* text, size_t len, void* w
     if (((uintptr_t)workspace & 255) != 0) return TT_ERR_ARG;
     if (workspace_bytes < tt_workspace_bytes(v, len, n_docs)) return TT_ERR_ARG;
     return TT_OK;
-}
-
-// Launches `kernel` so that it may begin while the kernel before it on the stream is still draining
-// (programmatic dependent launch): its CTAs are placed as soon as every CTA of the predecessor has
-// signalled, and wait inside the kernel (cudaGridDependencySynchronize) until the predecessor's memory
-// is complete.  Only the launch latency is hidden; the data dependence is unchanged.
-template <typename Params>
-static cudaError_t launch_after(void (*kernel)(const Params), int grid, int block, cudaStream_t st, const Params& p, size_t smem = 0, bool early = true) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3((unsigned)block); cfg.dynamicSmemBytes = smem; cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = early ? 1 : 0;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, p);
 }
 
 static int encode_impl(const tt_vocab* v, const uint8_t* text, size_t len, const int64_t* doc_off, size_t n_docs,
@@ -624,7 +624,7 @@ static int encode_impl(const tt_vocab* v, const uint8_t* text, size_t len, const
     if (doc_off || literals || big || cap != cudaStreamCaptureStatusNone) CK(cudaMemsetAsync(w.hdr, 0, sizeof(TTHeader), st));
     MARK(0);
     PretokParams PP;
-    int rc = run_pretok(v, text, len, doc_off, n_docs, st, w, nullptr, PP, literals, true, host_src);
+    int rc = run_pretok(v, text, len, doc_off, n_docs, st, w, nullptr, PP, literals, true, host_src, ev == nullptr);
     if (rc != TT_OK) return rc;
     MARK(1);
     const int tile_grid = PP.ntiles < v->sm_count * 8 ? PP.ntiles : v->sm_count * 8;
@@ -641,10 +641,9 @@ static int encode_impl(const tt_vocab* v, const uint8_t* text, size_t len, const
     Q.lq = w.lq; Q.tok_len = v->d_tok_len;
     if (big) {                                                               // bulk text: closing pieces and the global lists first
         const int cgrid = (PP.ntiles + CLOSING_THREADS - 1) / CLOSING_THREADS;
-        if (ev) k_closing<<<cgrid, CLOSING_THREADS, 0, st>>>(Q);
-        else CK(launch_after(k_closing, cgrid, CLOSING_THREADS, st, Q));
+        CK(launch_after(k_closing, cgrid, CLOSING_THREADS, st, 0, ev == nullptr, Q));
     }
-    CK(launch_after(big ? k_merge_bulk : k_merge, merge_grid, MERGE_THREADS, st, Q, big ? MERGE_SMEM_BYTES : MERGE_SMEM_REQUEST, ev == nullptr));
+    CK(launch_after(big ? k_merge_bulk : k_merge, merge_grid, MERGE_THREADS, st, big ? MERGE_SMEM_BYTES : MERGE_SMEM_REQUEST, ev == nullptr, Q));
     MARK(2);
     ScatterParams S;
     S.shift = PP.lo; S.hi = PP.hi; S.ntiles = PP.ntiles; S.tile_cnt = w.tile_cnt; S.tile_tok = w.tile_tok; S.grp_tok = Q.grp_tok; S.piece_off16 = w.piece_off16;
@@ -652,8 +651,7 @@ static int encode_impl(const tt_vocab* v, const uint8_t* text, size_t len, const
     S.ids_out = ids_out; S.count_out = (long long*)count_out; S.status_out = status_out;
     S.docmask = doc_off ? w.docmask : nullptr; S.doc_off = (const long long*)doc_off; S.n_docs = (int)n_docs;
     S.ids_off_out = (long long*)ids_off_out;
-    if (ev) { if (big) k_scatter_bulk<<<tile_grid, BPE_THREADS, 0, st>>>(S); else k_scatter<<<tile_grid, BPE_THREADS, 0, st>>>(S); }
-    else CK(launch_after(big ? k_scatter_bulk : k_scatter, tile_grid, BPE_THREADS, st, S));
+    CK(launch_after(big ? k_scatter_bulk : k_scatter, tile_grid, BPE_THREADS, st, 0, ev == nullptr, S));
     MARK(3);
 #undef MARK
     CK(cudaGetLastError());

@@ -827,7 +827,7 @@ __device__ __forceinline__ int short_class(u32 n) {
 }
 
 __global__ void __launch_bounds__(CLOSING_THREADS)
-k_closing(const PieceParams P) {
+k_closing(const __grid_constant__ PieceParams P) {
     const int lane = threadIdx.x & 31;
     const u32 FULL = 0xFFFFFFFFu;
     cudaTriggerProgrammaticLaunchCompletion();

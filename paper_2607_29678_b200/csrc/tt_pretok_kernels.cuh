@@ -290,14 +290,15 @@ k_pretok(const __grid_constant__ PretokParams P, const __grid_constant__ FrontPa
 
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     cudaTriggerProgrammaticLaunchCompletion();               // the next kernel may be placed; it waits for this grid's memory itself
+    // the whole-piece table is probed at random a few microseconds from now: ask for it to be brought into L2
+    if (FUSED && F.toktab.slots != nullptr) grid_prefetch_l2(F.toktab.slots, ((size_t)F.toktab.mask + 1) * sizeof(TokSlot));
+    cudaGridDependencySynchronize();                         // what was enqueued before this call is complete: its text, its use of the workspace
     if (FUSED) {
         if (blockIdx.x == 0 && tid == 0) {                    // k_merge's counters (k_merge touches them only after this grid)
             P.hdr->t_tiles = 0; P.hdr->merge_done = 0;
             for (int s = 0; s < 6; s++) { P.hdr->long_take[s] = 0; P.hdr->long_done[s] = 0; }
             if (F.wq == nullptr) { P.hdr->t_short = 0; P.hdr->nq_long = 0; }
         }
-        // the whole-piece table is probed at random a few microseconds from now: ask for it to be brought into L2
-        if (F.toktab.slots != nullptr) grid_prefetch_l2(F.toktab.slots, ((size_t)F.toktab.mask + 1) * sizeof(TokSlot));
     }
     // The class tables stay in global memory (21 KB, read through L1): ASCII characters -- nearly all of a
     // transcript -- are classified without any table, so shared memory is left to the masks and more CTAs fit an SM.
