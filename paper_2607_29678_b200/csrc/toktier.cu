@@ -57,6 +57,7 @@ struct tt_vocab {
     uint4* d_slots = nullptr;
     u64* d_bytepair = nullptr;
     int32_t* d_ext_id = nullptr;
+    int32_t ext_delta = 0; bool ext_plain = false;      // every caller id is the internal one plus ext_delta
     u16* d_tok_len = nullptr;            // bytes of every internal token, 65,535 = at least that many
     u8* d_cls = nullptr;
     int cls_bytes = 0;
@@ -80,6 +81,7 @@ struct tt_vocab {
     cudaEvent_t slice_ev[8] = {};
 };
 
+static inline ExtMap ext_map(const tt_vocab* v) { ExtMap m; m.id = v->d_ext_id; m.delta = v->ext_delta; m.plain = v->ext_plain; return m; }
 static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // Epoch of a call: tags the status word of the workspace header (see TTHeader).  Never zero, never repeated.
@@ -220,7 +222,7 @@ static int build_token_table(tt_vocab* v, const tt_merge* merges, size_t n_merge
         Q.hdr = d_hdr; Q.epoch = next_epoch(); Q.tab = v->tab;
         Q.toktab.slots = nullptr; Q.toktab.mask = 0; Q.toktab.shift = 0;      // no table yet: every piece is merged
         Q.longtab = LongTable{}; Q.litstart = nullptr;
-        Q.ext_id = v->d_ext_id; Q.piece_cnt = d_cnt; Q.stage = d_stage; Q.pairbuf = nullptr; Q.tile_tok = d_tt; Q.grp_tok = nullptr; Q.wq = nullptr; Q.gq = nullptr; Q.gq_x[0] = Q.gq_x[1] = Q.gq_x[2] = nullptr; Q.lq = nullptr; Q.tok_len = nullptr;
+        Q.ext_id = ext_map(v); Q.piece_cnt = d_cnt; Q.stage = d_stage; Q.pairbuf = nullptr; Q.tile_tok = d_tt; Q.grp_tok = nullptr; Q.wq = nullptr; Q.gq = nullptr; Q.gq_x[0] = Q.gq_x[1] = Q.gq_x[2] = nullptr; Q.lq = nullptr; Q.tok_len = nullptr;
         k_merge<<<v->sm_count * MERGE_CTAS_PER_SM, MERGE_THREADS, MERGE_SMEM_REQUEST>>>(Q);
         ok = cudaGetLastError() == cudaSuccess && cudaDeviceSynchronize() == cudaSuccess;
     }
@@ -394,6 +396,8 @@ extern "C" int tt_vocab_load_ex(const tt_merge* merges, size_t n_merges, const i
     tt_vocab* v = new (std::nothrow) tt_vocab();
     if (!v) return TT_ERR_CUDA;
     v->pattern = pattern_id; v->n_merges = n_merges; v->ignore_merges = (flags & TT_VOCAB_IGNORE_MERGES) != 0;
+    v->ext_delta = ext_id[0]; v->ext_plain = true;
+    for (size_t i = 0; i < ext_id.size(); i++) if ((long long)ext_id[i] != (long long)i + v->ext_delta) { v->ext_plain = false; break; }
     // class tables: stage1 | stage2 | ascii
     const int stage2_bytes = TT_CLS_NBLOCKS * 128;
     v->cls_bytes = (int)align_up(0x1100 + stage2_bytes, 16) + 128;
@@ -634,7 +638,7 @@ static int encode_impl(const tt_vocab* v, const uint8_t* text, size_t len, const
     Q.tile_cnt = w.tile_cnt; Q.tile_first = w.tile_first; Q.tile_last = w.tile_last; Q.tile_q = w.tile_q; Q.tile_long = w.tile_long;
     Q.piece_off16 = w.piece_off16; Q.q = w.q;
     Q.hdr = w.hdr; Q.tab = v->tab; Q.toktab = v->toktab; Q.longtab = v->longtab; Q.litstart = literals ? w.litstart : nullptr; Q.epoch = PP.epoch;
-    Q.ext_id = v->d_ext_id; Q.piece_cnt = w.piece_cnt; Q.stage = w.stage; Q.pairbuf = w.pairbuf; Q.tile_tok = w.tile_tok;
+    Q.ext_id = ext_map(v); Q.piece_cnt = w.piece_cnt; Q.stage = w.stage; Q.pairbuf = w.pairbuf; Q.tile_tok = w.tile_tok;
     Q.grp_tok = PP.ntiles > MERGE_SR_MAX_TILES ? w.grp_tok : nullptr;   // group totals only where k_scatter's CTAs would otherwise sum thousands of tiles each
     Q.wq = big ? w.wq : nullptr; Q.gq = big ? w.gq : nullptr;
     for (int c = 0; c < TT_SHORT_CLASSES - 1; c++) Q.gq_x[c] = big ? w.gq_x[c] : nullptr;

@@ -185,69 +185,61 @@ __device__ __forceinline__ bool longtab_lookup(const LongTable& tab, const u8* _
     return false;
 }
 
+// Internal token -> the caller's id.  Where the ids are the internal ones plus a constant (bytes first, results in order of
+// rank, as trainers number them) no table is read.
+struct ExtMap {
+    const int32_t* id; int32_t delta; bool plain;
+    __device__ __forceinline__ int32_t operator[](u32 t) const { return plain ? (int32_t)t + delta : id[t]; }
+};
 constexpr u32 RK_STALE = 0xFFFFFFFEu;                 // rank must be probed again
 constexpr int BPE_WARPS = 8;                          // warps per CTA of the piece kernels
 constexpr int BPE_THREADS = BPE_WARPS * 32;           // = pieces per CTA iteration
 constexpr int WCH = TT_WARP_PIECE_MAX / 32;           // 32-token chunks per piece
 
-// Position of the (j + 1)-th set bit of mask (a value >= 32 where there is none): five halving steps.
-__device__ __forceinline__ u32 select_bit(u32 mask, u32 j) {
-    u32 pos = 0, c;
-    c = __popc(mask & 0xFFFFu);          if (j >= c) { pos = 16; j -= c; }
-    c = __popc((mask >> pos) & 0xFFu);   if (j >= c) { pos += 8; j -= c; }
-    c = __popc((mask >> pos) & 0xFu);    if (j >= c) { pos += 4; j -= c; }
-    c = __popc((mask >> pos) & 0x3u);    if (j >= c) { pos += 2; j -= c; }
-    c = (mask >> pos) & 1u;              if (j >= c) { pos += 1; j -= c; }
-    return ((mask >> (pos & 31)) & 1u) && j == 0 && pos < 32 ? pos : 32u;
-}
-
 // ---- warp merge rounds with at most 32 tokens: one token per lane, no shared memory -----------------------
 // t = token of position `lane`, p = (rank, cl, cr) of the pair (lane, lane + 1) or none, m = token count.
+// The tokens stay in their lanes: a mask says which lanes still hold one, and neighbours are found by bit searches.  (Moving
+// the survivors together after every round -- a bit selection and four shuffles between the selection and the next
+// probe -- made a round 1,200 cycles, two thirds of them the probe's.)
 // Runs rounds to the fixpoint, hands token j of the result to out(j, token) and returns their count.
 // A round: Q marks a pair identical to the pair on its left (t t t); a pair that is not Q heads a run; a head
 // may go if its left guard holds or it has the round's minimum rank; a pair goes if its run's head may go, it
 // lies an even number of places behind the head and its right guard holds (or it has the minimum rank).
 template <class Out>
 __device__ __forceinline__ u32 warp_merge_reg_rounds(u32 t, PairInfo p, u32 m, const PairTable& tab, int lane, Out out) {
-    const u32 FULL = 0xFFFFFFFFu, lt = (1u << lane) - 1, le = lt | (1u << lane);
+    const u32 FULL = 0xFFFFFFFFu, lt = (1u << lane) - 1, le = lt | (1u << lane), gt = ~le;
     u32 r = p.r, cl = p.cl, cr = p.cr;
-    if ((u32)lane + 1 >= m) r = cl = cr = TT_RANK_INF;      // the last token has no pair
-    const u32 max_rounds = m;                           // every round merges at least one pair
+    u32 al = m >= 32 ? FULL : (1u << m) - 1;                // lanes that hold a token; lane 0 always does
+    u32 up = al & gt, dn = al & lt;                         // ... of them above and below this one
+    int nx = __ffs(up) - 1, pv = 31 - __clz(dn);            // neighbours (-1: none)
+    u32 tl = __shfl_sync(FULL, t, pv & 31), tn = __shfl_sync(FULL, t, nx & 31);
+    if (!up || !((al >> lane) & 1)) r = cl = cr = TT_RANK_INF;      // the last token has no pair
+    const u32 max_rounds = m;                               // every round merges at least one pair
     for (u32 round = 0; round < max_rounds; round++) {
         const u32 mn = __reduce_min_sync(FULL, r);
         if (mn == TT_RANK_INF) break;
-        const u32 tl = __shfl_up_sync(FULL, t, 1), tn0 = __shfl_down_sync(FULL, t, 1);
-        u32 cll = __shfl_up_sync(FULL, cl, 1), crr = __shfl_down_sync(FULL, cr, 1);
-        if (lane == 0) cll = TT_RANK_INF;
-        if (lane == 31) crr = TT_RANK_INF;
+        u32 cll = __shfl_sync(FULL, cl, pv & 31), crr = __shfl_sync(FULL, cr, nx & 31);
+        if (!dn) cll = TT_RANK_INF;
+        if (!up) crr = TT_RANK_INF;
         const bool R = r != TT_RANK_INF, Mn = r == mn;
-        const bool Q = R && lane >= 1 && tl == t && t == tn0;
+        const bool Q = R && dn && tl == t && t == tn;
         const u32 qm = __ballot_sync(FULL, Q), hm = __ballot_sync(FULL, !Q && R && (r < cll || Mn));
-        const u32 h = 31u - (u32)__clz(~qm & le);       // bit 0 of qm is never set
-        const u32 sel = __ballot_sync(FULL, R && ((hm >> h) & 1) && !(((u32)lane - h) & 1) && (r <= crr || Mn));
+        const u32 h = 31u - (u32)__clz(~qm & al & le);      // the head of the run (lane 0 is never Q)
+        const u32 sel = __ballot_sync(FULL, R && ((hm >> h) & 1) && (__popc(al & le & (FULL << h)) & 1) && (r <= crr || Mn));
         const bool me = (sel >> lane) & 1;
-        const bool nxt = lane < 31 ? ((sel >> (lane + 1)) & 1) : false;
-        const u32 nt = me ? 256u + r : t;
-        const u32 nr = (me || nxt) ? RK_STALE : r;
-        // survivors move down: new lane j takes the j-th surviving old lane
-        u32 src;
-        if ((sel & (sel - 1)) == 0) {                   // one merge: everything above it moves down by one
-            src = (u32)lane + ((u32)lane > (u32)(__ffs(sel) - 1) ? 1u : 0u);
-        } else {
-            const u32 surv = ~(sel << 1) & (m >= 32 ? FULL : ((1u << m) - 1));
-            src = select_bit(surv, (u32)lane);
-        }
-        t = __shfl_sync(FULL, nt, src & 31);
-        r = __shfl_sync(FULL, nr, src & 31);
-        cl = __shfl_sync(FULL, cl, src & 31);
-        cr = __shfl_sync(FULL, cr, src & 31);
-        m -= __popc(sel);
-        const u32 tn = __shfl_down_sync(FULL, t, 1);
-        if ((u32)lane + 1 >= m) r = cl = cr = TT_RANK_INF;
-        else if (r == RK_STALE) { const PairInfo q = pair_probe(tab, t, tn); r = q.r; cl = q.cl; cr = q.cr; }
+        // a merge gives its lane the new token; the lane of its right token is empty from here on
+        const u32 gone = __ballot_sync(FULL, dn && ((al & sel) >> (pv & 31)) & 1);
+        al &= ~gone;
+        up = al & gt; dn = al & lt;
+        nx = __ffs(up) - 1; pv = 31 - __clz(dn);
+        if (me) t = 256u + r;
+        tl = __shfl_sync(FULL, t, pv & 31); tn = __shfl_sync(FULL, t, nx & 31);
+        const bool have = ((al >> lane) & 1) && up;
+        if (!have) r = cl = cr = TT_RANK_INF;
+        else if (me || ((sel >> (nx & 31)) & 1)) { const PairInfo q = pair_probe(tab, t, tn); r = q.r; cl = q.cl; cr = q.cr; }
     }
-    if ((u32)lane < m) out((u32)lane, t);
-    return m;
+    if ((al >> lane) & 1) out((u32)__popc(al & lt), t);
+    return (u32)__popc(al);
 }
 
 // A piece of up to 32 bytes.
@@ -394,7 +386,7 @@ __device__ __forceinline__ void pair_probe2(const PairTable& t, u32 a0, u32 b0, 
 // token, and the rank of a pair is kept at its left position, so a merge moves nothing: it rewrites the
 // left token, clears the partner's bit and marks the two pairs that changed for a new probe.
 __device__ __forceinline__ u32 lane_merge(u32* __restrict__ tok, u32* __restrict__ rk, int s, const u8* __restrict__ text, u32 a, u32 n,
-                                          const PairTable& tab, const int32_t* __restrict__ ext_id, int32_t* __restrict__ stage) {
+                                          const PairTable& tab, const ExtMap& ext_id, int32_t* __restrict__ stage) {
 #define TK(k) tok[(k) * LANE_SLOTS + s]
 #define RK(k) rk[(k) * LANE_SLOTS + s]
     u32 prev = text[a];
@@ -665,7 +657,7 @@ constexpr int LONG_SMEM_SLOTS = LONG_SMEM_TOKENS + LONG_SMEM_TOKENS / 16 + 8;   
 // Encodes one piece of n > TT_WARP_PIECE_MAX bytes with the whole CTA.  gbuf: n entries of global scratch; the
 // piece's own n words of the staging array serve as the second global array until the ids are staged there.
 // sbuf: LONG_SMEM_SLOTS u64 followed by LONG_SMEM_SLOTS u32.
-__device__ u32 cta_merge_long(const u8* __restrict__ text, u32 a, u32 n, const PairTable& tab, const int32_t* __restrict__ ext_id,
+__device__ u32 cta_merge_long(const u8* __restrict__ text, u32 a, u32 n, const PairTable& tab, const ExtMap& ext_id,
                               int32_t* __restrict__ stage, u64* gbuf, u64* sbuf, u32* s_scr) {
     const int tid = threadIdx.x, T = blockDim.x;
     u32* const scr = reinterpret_cast<u32*>(sbuf + LONG_SMEM_SLOTS);
@@ -725,7 +717,7 @@ struct PieceParams {
     TokTable toktab;           // slots == nullptr: no whole-piece table (while the table itself is being built)
     const u32* litstart;       // literal pass: a piece that begins at such a bit is an added token whose id is staged, or null
     LongTable longtab;         // ignore_merges: entries longer than the whole-piece table holds (else slots == nullptr)
-    const int32_t* ext_id;
+    ExtMap ext_id;
     u32* piece_cnt;
     int32_t* stage;            // ids staged at the text offset of their piece
     u64* pairbuf;              // global scratch of the long-piece path, indexed like the text
