@@ -62,7 +62,7 @@ struct tt_vocab {
     u8* d_cls = nullptr;
     int cls_bytes = 0;
     PairTable tab{};
-    TokSlot* d_tokslots = nullptr;
+    uint4* d_toktab = nullptr;
     TokTable toktab{};
     bool ignore_merges = false;
     LongSlot* d_longslots = nullptr; u8* d_longblob = nullptr;
@@ -115,7 +115,7 @@ extern "C" size_t tt_class_table(uint8_t* out, size_t cap) {
 extern "C" void tt_vocab_free(tt_vocab* v) {
     if (!v) return;
     v->sessions->close();
-    cudaFree(v->d_slots); cudaFree(v->d_bytepair); cudaFree(v->d_ext_id); cudaFree(v->d_tok_len); cudaFree(v->d_cls); cudaFree(v->d_lit_entries); cudaFree(v->d_lit_blob); cudaFree(v->d_tokslots); cudaFree(v->d_longslots); cudaFree(v->d_longblob); cudaFree(v->d_meta);
+    cudaFree(v->d_slots); cudaFree(v->d_bytepair); cudaFree(v->d_ext_id); cudaFree(v->d_tok_len); cudaFree(v->d_cls); cudaFree(v->d_lit_entries); cudaFree(v->d_lit_blob); cudaFree(v->d_toktab); cudaFree(v->d_longslots); cudaFree(v->d_longblob); cudaFree(v->d_meta);
     cudaFree(v->d_text); cudaFree(v->d_ids); cudaFree(v->d_count); cudaFree(v->d_status); cudaFree(v->d_ws);
     if (v->h_text) cudaFreeHost(v->h_text);
     if (v->h_ids) cudaFreeHost(v->h_ids);
@@ -220,7 +220,7 @@ static int build_token_table(tt_vocab* v, const tt_merge* merges, size_t n_merge
         Q.base = d_text; Q.shift = 0; Q.hi = (long long)nb; Q.ntiles = (int)ntiles;
         Q.tile_cnt = d_tc; Q.tile_first = d_tf; Q.tile_last = d_tl; Q.tile_q = d_tq; Q.tile_long = d_lg; Q.piece_off16 = d_o16; Q.q = d_q;
         Q.hdr = d_hdr; Q.epoch = next_epoch(); Q.tab = v->tab;
-        Q.toktab.slots = nullptr; Q.toktab.mask = 0; Q.toktab.shift = 0;      // no table yet: every piece is merged
+        Q.toktab = TokTable{};                                                // no table yet: every piece is merged
         Q.longtab = LongTable{}; Q.litstart = nullptr;
         Q.ext_id = ext_map(v); Q.piece_cnt = d_cnt; Q.stage = d_stage; Q.pairbuf = nullptr; Q.tile_tok = d_tt; Q.grp_tok = nullptr; Q.wq = nullptr; Q.gq = nullptr; Q.gq_x[0] = Q.gq_x[1] = Q.gq_x[2] = nullptr; Q.lq = nullptr; Q.tok_len = nullptr;
         k_merge<<<v->sm_count * MERGE_CTAS_PER_SM, MERGE_THREADS, MERGE_SMEM_REQUEST>>>(Q);
@@ -235,28 +235,68 @@ static int build_token_table(tt_vocab* v, const tt_merge* merges, size_t n_merge
         if ((int32_t)cnt[slot] == -1 && stage[off[i]] == ext_id[cand[i]]) keep.push_back((u32)i);           // minus the staged count
     }
     }
-    u32 cap = 1024;
-    while (cap < 2 * keep.size() + 2) cap <<= 1;
-    u32 log2cap = 0;
-    while ((1u << log2cap) < cap) log2cap++;
-    const u32 mask = cap - 1, shift = 32 - log2cap;
-    std::vector<TokSlot> slots(cap);
-    memset(slots.data(), 0, cap * sizeof(TokSlot));
+    // Two-choice placement (see TokTable), a bucket of the short table for every one to two entries and one of the other for every
+    // three to six, so that few buckets overflow; another seed where a placement fails.
+    struct Key { u32 n; int32_t id; u32 k[6], h; };
+    std::vector<Key> keys[2];
+    for (u32 b = 0; b < 256; b++) { Key e{}; e.n = 1; e.id = ext_id[b]; e.k[0] = b; keys[0].push_back(e); }
     for (u32 i : keep) {
-        const u32 n = off[i + 1] - off[i];
-        u8 key[24] = {0};
-        memcpy(key, cat.data() + off[i], n);
-        u32 k[6]; memcpy(k, key, 24);
-        u32 hh = toktab_hash_final(toktab_hash_rest(toktab_hash_short(k[0], k[1], n), k[2], k[3], k[4], k[5]), shift);
-        while (slots[hh].len != 0) hh = (hh + 1) & mask;
-        slots[hh].len = n; slots[hh].id = ext_id[cand[i]];
-        for (int j = 0; j < 6; j++) slots[hh].k[j] = k[j];
+        Key e{};
+        e.n = off[i + 1] - off[i]; e.id = ext_id[cand[i]];
+        u8 raw[24] = {0};
+        memcpy(raw, cat.data() + off[i], e.n);
+        memcpy(e.k, raw, 24);
+        keys[e.n <= TT_TOKTAB_SHORT ? 0 : 1].push_back(e);
     }
-    if (cudaMalloc(&v->d_tokslots, (size_t)cap * sizeof(TokSlot)) != cudaSuccess ||
-        cudaMemcpy(v->d_tokslots, slots.data(), (size_t)cap * sizeof(TokSlot), cudaMemcpyHostToDevice) != cudaSuccess) {
+    u32 log2n[2];
+    for (int c = 0; c < 2; c++) { log2n[c] = 8; while (((size_t)1 << log2n[c]) < (c ? 3 : 2) * keys[c].size()) log2n[c]++; }
+    const size_t short_slots = (size_t)2 << log2n[0], long_slots = (size_t)1 << log2n[1];
+    std::vector<uint4> table(short_slots + 2 * long_slots);
+    u32 seed = 0;
+    bool placed_all = false;
+    for (int attempt = 0; attempt < 64 && !placed_all; attempt++, seed += 0x6D2B79F5u) {
+        std::fill(table.begin(), table.end(), make_uint4(0, 0, 0, 0));
+        placed_all = true;
+        for (int c = 0; c < 2 && placed_all; c++) {
+            const u32 shift = 32 - log2n[c], width = c ? 1 : 2;           // slots of a bucket
+            std::vector<int> owner((size_t)width << log2n[c], -1);
+            u64 rng = 0x9E3779B97F4A7C15ull;
+            for (size_t i = 0; i < keys[c].size() && placed_all; i++) {
+                Key& e = keys[c][i];
+                const u32 s = toktab_hash_short(e.k[0], e.k[1], e.n, seed);
+                e.h = toktab_hash_final(c ? toktab_hash_rest(s, e.k[2], e.k[3], e.k[4], e.k[5]) : s);
+                int cur = (int)i;
+                for (int iter = 0; cur >= 0; iter++) {
+                    if (iter == 2000) { placed_all = false; break; }
+                    const u32 b[2] = {toktab_bucket(keys[c][cur].h, shift), toktab_bucket_alt(keys[c][cur].h, shift)};
+                    for (u32 q = 0; q < 2 * width && cur >= 0; q++) { int& o = owner[(size_t)b[q / width] * width + q % width]; if (o < 0) { o = cur; cur = -1; } }
+                    if (cur < 0) break;
+                    rng = rng * 6364136223846793005ull + 1442695040888963407ull;
+                    std::swap(cur, owner[(size_t)b[(rng >> 33) & 1] * width + ((rng >> 40) & (width - 1))]);
+                }
+            }
+            if (!placed_all) break;
+            uint4* const base = table.data() + (c ? short_slots : 0);
+            for (size_t o = 0; o < owner.size(); o++) {
+                if (owner[o] < 0) continue;
+                const Key& e = keys[c][owner[o]];
+                const size_t first = toktab_bucket(e.h, shift);
+                uint4& t = base[c ? 2 * o : o];
+                t.x |= e.n; t.y = (u32)e.id; t.z = e.k[0]; t.w = e.k[1];
+                if (c) base[2 * o + 1] = make_uint4(e.k[2], e.k[3], e.k[4], e.k[5]);
+                if (o / width != first) base[2 * first].x |= TOK_OVERFLOW;        // (a bucket is two uint4 in either table)
+            }
+        }
+        if (placed_all) break;
+    }
+    if (!placed_all) return TT_ERR_BAD_VOCAB;
+    const size_t table_bytes = table.size() * sizeof(uint4);
+    if (cudaMalloc(&v->d_toktab, table_bytes) != cudaSuccess ||
+        cudaMemcpy(v->d_toktab, table.data(), table_bytes, cudaMemcpyHostToDevice) != cudaSuccess) {
         cudaGetLastError(); return TT_ERR_CUDA;
     }
-    v->toktab.slots = v->d_tokslots; v->toktab.mask = mask; v->toktab.shift = shift;
+    v->toktab.shorts = v->d_toktab; v->toktab.slots = reinterpret_cast<const TokSlot*>(v->d_toktab + short_slots);
+    v->toktab.short_shift = 32 - log2n[0]; v->toktab.shift = 32 - log2n[1]; v->toktab.seed = seed; v->toktab.bytes = table_bytes;
     v->n_table_tokens = keep.size();
     return TT_OK;
 }

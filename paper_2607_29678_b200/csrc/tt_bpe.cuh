@@ -97,23 +97,34 @@ __device__ __forceinline__ void grid_prefetch_l2(const void* p, size_t bytes) {
 }
 
 // ---- whole-piece table: byte string of a vocabulary entry -> its id ------------------------------------
-// Holds every token of at most TT_TOKTAB_MAXLEN bytes whose own byte string encodes to exactly that
+// Holds the single bytes and every token of at most TT_TOKTAB_MAXLEN bytes whose own byte string encodes to exactly that
 // token (checked at load time by running the merge kernel below on every token string), so a hit
-// returns what the merge loop would return.  Slots are 32 bytes (one sector): length (0 = empty), the
-// caller's id and six key words (the bytes, little endian, zero padded); open addressing, linear probing,
-// load factor <= 0.5.  The first 16 bytes of a slot (length, id, key words 0 and 1) decide every piece of at
-// most 8 bytes -- most pieces of ordinary text -- with one vector load.
+// returns what the merge loop would return.  Two tables, both two-choice (cuckoo) hashed over 32-byte buckets (one
+// sector): entries of 1..8 bytes -- most pieces of ordinary text -- two 16-byte slots (length, the caller's id, two key words,
+// little endian, zero padded) to a bucket; entries of 9..24 bytes one slot with six key words.  A key is in its first
+// bucket, or, where that bucket's overflow bit is set, perhaps in its second one, so a look-up is one sector load and at
+// times another.  (Linear probing in one table of 32-byte slots: a miss walked to the next empty slot, the longest walk of
+// a warp's 32 was 5 to 8 dependent loads, and the first kernel spent 2 to 7 us of a request's 12 to 16 there.)
 constexpr int TT_TOKTAB_MAXLEN = 24;
+constexpr u32 TT_TOKTAB_SHORT = 8;
+constexpr u32 TOK_OVERFLOW = 0x80000000u, TOK_LEN = 0xFFu;        // word 0 of a bucket's first slot
 struct TokSlot { u32 len; int32_t id; u32 k[6]; };
 static_assert(sizeof(TokSlot) == 32, "slot layout");
-struct TokTable { const TokSlot* slots; u32 mask; u32 shift; };   // shift = 32 - log2(capacity)
+struct TokTable {
+    const uint4* shorts;      // 2 << (32 - short_shift) slots, then the longer entries; nullptr: no table
+    const TokSlot* slots;     // 1 << (32 - shift) of them
+    u32 short_shift, shift, seed;
+    size_t bytes;             // of both, from `shorts` on
+};
 
 // Key words beyond the piece are zero, so they add nothing: a piece of at most 8 bytes is hashed from two words.
-TT_HD u32 toktab_hash_short(u32 k0, u32 k1, u32 n) { return n * 0x9E3779B1u + k0 * 0x85EBCA6Bu + k1 * 0xC2B2AE35u; }
+TT_HD u32 toktab_hash_short(u32 k0, u32 k1, u32 n, u32 seed) { return seed + n * 0x9E3779B1u + k0 * 0x85EBCA6Bu + k1 * 0xC2B2AE35u; }
 TT_HD u32 toktab_hash_rest(u32 h, u32 k2, u32 k3, u32 k4, u32 k5) { return h + k2 * 0x27D4EB2Fu + k3 * 0x165667B1u + k4 * 0xD3A2646Du + k5 * 0xFD7046C5u; }
-TT_HD u32 toktab_hash_final(u32 h, u32 shift) {
-    h ^= h >> 15; h *= 0x2C1B3C6Du; h ^= h >> 12; h *= 0x297A2D39u; h ^= h >> 15;
-    return h >> shift;
+TT_HD u32 toktab_hash_final(u32 h) { h ^= h >> 15; h *= 0x2C1B3C6Du; h ^= h >> 12; h *= 0x297A2D39u; return h ^ (h >> 15); }
+TT_HD u32 toktab_bucket(u32 h, u32 shift) { return h >> shift; }
+TT_HD u32 toktab_bucket_alt(u32 h, u32 shift) {                   // the key's other bucket, never the first one
+    const u32 b = (h * 0x9E3779B1u) >> shift, a = h >> shift;
+    return b == a ? (a ^ 1u) : b;
 }
 TT_HD u32 toktab_mask_word(u32 w, u32 n, u32 j) {      // key word j of a piece of n bytes: bytes beyond the piece are zero
     const u32 have = n > 4 * j ? n - 4 * j : 0u;
@@ -128,7 +139,20 @@ __device__ __forceinline__ void toktab_key01(u32 x0, u32 x1, u32 x2, u32 sb, u32
     k0 = toktab_mask_word(__funnelshift_r(x0, x1, sh), n, 0);
     k1 = toktab_mask_word(__funnelshift_r(x1, x2, sh), n, 1);
 }
-// Looks a piece of 2..24 bytes up; returns true and the id on a hit.  (The first kernel has its own copy of the
+// A piece of 1..8 bytes, the two slots of its first bucket at hand; h: its hash.
+__device__ __forceinline__ bool toktab_short_match(const uint4 s, u32 n, u32 k0, u32 k1, u32& val) {
+    if ((((s.x ^ n) & TOK_LEN) | (s.z ^ k0) | (s.w ^ k1)) != 0) return false;
+    val = s.y;
+    return true;
+}
+__device__ __forceinline__ bool toktab_short(const TokTable& tab, const uint4 e0, const uint4 e1, u32 h, u32 n, u32 k0, u32 k1, u32& val) {
+    if (toktab_short_match(e0, n, k0, k1, val) || toktab_short_match(e1, n, k0, k1, val)) return true;
+    if (!(e0.x & TOK_OVERFLOW)) return false;
+    const uint4* const b = tab.shorts + 2 * (size_t)toktab_bucket_alt(h, tab.short_shift);
+    const uint4 f0 = __ldg(b), f1 = __ldg(b + 1);
+    return toktab_short_match(f0, n, k0, k1, val) || toktab_short_match(f1, n, k0, k1, val);
+}
+// Looks a piece of 1..24 bytes up; returns true and the id on a hit.  (The first kernel has its own copy of the
 // first steps for pieces of at most 8 bytes, four pieces in flight per thread.)
 __device__ __forceinline__ bool toktab_lookup(const TokTable& tab, const u8* __restrict__ text, u32 a, u32 n, int32_t& id) {
     const uintptr_t addr = (uintptr_t)(text + a);
@@ -140,17 +164,24 @@ __device__ __forceinline__ bool toktab_lookup(const TokTable& tab, const u8* __r
     u32 k[6];
 #pragma unroll
     for (int j = 0; j < 6; j++) k[j] = toktab_mask_word(__funnelshift_r(x[j], x[j + 1], sh), n, j);
-    u32 h = toktab_hash_final(toktab_hash_rest(toktab_hash_short(k[0], k[1], n), k[2], k[3], k[4], k[5]), tab.shift);
-    for (u32 probe = 0; probe <= tab.mask; probe++) {           // bounded by the capacity
-        const uint4* sp = reinterpret_cast<const uint4*>(tab.slots + h);
-        const uint4 lo = __ldg(sp);
-        if (lo.x == 0) return false;
-        if (lo.x == n && lo.z == k[0] && lo.w == k[1]) {
-            bool same = true;
-            if (n > 8) { const uint4 hi = __ldg(sp + 1); same = hi.x == k[2] && hi.y == k[3] && hi.z == k[4] && hi.w == k[5]; }
-            if (same) { id = (int32_t)lo.y; return true; }
-        }
-        h = (h + 1) & tab.mask;
+    const u32 s = toktab_hash_short(k[0], k[1], n, tab.seed);
+    if (n <= TT_TOKTAB_SHORT) {
+        const u32 h = toktab_hash_final(s);
+        const uint4* const b = tab.shorts + 2 * (size_t)toktab_bucket(h, tab.short_shift);
+        u32 val = 0;
+        const bool hit = toktab_short(tab, __ldg(b), __ldg(b + 1), h, n, k[0], k[1], val);
+        id = (int32_t)val;
+        return hit;
+    }
+    const u32 h = toktab_hash_final(toktab_hash_rest(s, k[2], k[3], k[4], k[5]));
+    u32 at = toktab_bucket(h, tab.shift);
+#pragma unroll 1
+    for (int probe = 0; probe < 2; probe++) {
+        const uint4* const sp = reinterpret_cast<const uint4*>(tab.slots + at);
+        const uint4 lo = __ldg(sp), hi = __ldg(sp + 1);
+        if ((((lo.x ^ n) & TOK_LEN) | (lo.z ^ k[0]) | (lo.w ^ k[1]) | (hi.x ^ k[2]) | (hi.y ^ k[3]) | (hi.z ^ k[4]) | (hi.w ^ k[5])) == 0) { id = (int32_t)lo.y; return true; }
+        if (!(lo.x & TOK_OVERFLOW)) return false;
+        at = toktab_bucket_alt(h, tab.shift);
     }
     return false;
 }
@@ -714,7 +745,7 @@ struct PieceParams {
     TTHeader* hdr;
     unsigned long long epoch;
     PairTable tab;
-    TokTable toktab;           // slots == nullptr: no whole-piece table (while the table itself is being built)
+    TokTable toktab;           // shorts == nullptr: no whole-piece table (while the table itself is being built)
     const u32* litstart;       // literal pass: a piece that begins at such a bit is an added token whose id is staged, or null
     LongTable longtab;         // ignore_merges: entries longer than the whole-piece table holds (else slots == nullptr)
     ExtMap ext_id;
@@ -779,7 +810,7 @@ __device__ __forceinline__ bool piece_settled_without_merge(const PieceParams& P
     int32_t id;
     if (n == 1) { value = (u32)P.ext_id[text[a]]; return true; }
     if (n <= TT_TOKTAB_MAXLEN) {
-        if (P.toktab.slots != nullptr && toktab_lookup(P.toktab, text, a, n, id)) { value = (u32)id; return true; }
+        if (P.toktab.shorts != nullptr && toktab_lookup(P.toktab, text, a, n, id)) { value = (u32)id; return true; }
     } else if (P.longtab.slots != nullptr && n <= P.longtab.maxlen && longtab_lookup(P.longtab, text, a, n, id)) { value = (u32)id; return true; }
     return false;
 }

@@ -224,20 +224,19 @@ struct FrontParams {
     u32* tile_last; u32* tile_tok; u32* tile_q; u16* tile_long; u16* piece_off16; u32* piece_cnt; u32* q;
     u64* wq;                   // bulk text (more tiles than a request's job search covers): the warp-class pieces of all tiles go
                                // to this one list, appended tile by tile (hdr->nwq, cleared before the chain); else null
-    TokTable toktab;           // slots == nullptr: none
+    TokTable toktab;           // shorts == nullptr: none
     LongTable longtab;         // ignore_merges: entries longer than the whole-piece table holds (else slots == nullptr)
     const int32_t* ext_id;
 };
 
-// A piece on the general path of the fused kernel: an extracted literal, a single byte, a vocabulary entry of up to
-// 24 bytes, or (ignore_merges) a longer entry.  Returns true and the value for piece_cnt if it needs no merging.
-// g: position of the piece in the aligned frame; tb + o: its n bytes in shared memory.
-__device__ __forceinline__ bool front_piece_general(const PretokParams& P, const FrontParams& F, long long g, const u8* tb, u32 o, u32 n, u32& val) {
+// A piece on the general path of the fused kernel: a single byte, a vocabulary entry of up to 24 bytes, or
+// (ignore_merges) a longer entry.  Returns true and the value for piece_cnt if it needs no merging.
+// tb + o: its n bytes in shared memory.
+__device__ __forceinline__ bool front_piece_general(const FrontParams& F, const u8* tb, u32 o, u32 n, u32& val) {
     int32_t id;
-    if (P.litstart != nullptr && ((P.litstart[g >> 5] >> (g & 31)) & 1)) { val = 0u - 1u; return true; }    // one staged id (written by the literal pass)
     if (n == 1) { val = (u32)F.ext_id[tb[o]]; return true; }
     if (n <= (u32)TT_TOKTAB_MAXLEN) {
-        if (F.toktab.slots != nullptr && toktab_lookup(F.toktab, tb, o, n, id)) { val = (u32)id; return true; }
+        if (F.toktab.shorts != nullptr && toktab_lookup(F.toktab, tb, o, n, id)) { val = (u32)id; return true; }
     } else if (F.longtab.slots != nullptr && n <= F.longtab.maxlen && longtab_lookup(F.longtab, tb, o, n, id)) { val = (u32)id; return true; }
     return false;
 }
@@ -291,7 +290,7 @@ k_pretok(const __grid_constant__ PretokParams P, const __grid_constant__ FrontPa
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     cudaTriggerProgrammaticLaunchCompletion();               // the next kernel may be placed; it waits for this grid's memory itself
     // the whole-piece table is probed at random a few microseconds from now: ask for it to be brought into L2
-    if (FUSED && F.toktab.slots != nullptr) grid_prefetch_l2(F.toktab.slots, ((size_t)F.toktab.mask + 1) * sizeof(TokSlot));
+    if (FUSED && F.toktab.shorts != nullptr) grid_prefetch_l2(F.toktab.shorts, F.toktab.bytes);
     cudaGridDependencySynchronize();                         // what was enqueued before this call is complete: its text, its use of the workspace
     if (FUSED) {
         if (blockIdx.x == 0 && tid == 0) {                    // k_merge's counters (k_merge touches them only after this grid)
@@ -425,32 +424,32 @@ k_pretok(const __grid_constant__ PretokParams P, const __grid_constant__ FrontPa
             const u32 used = (u32)min((long long)TT_TILE_BYTES, P.hi - w_first * TT_WORD);
             may_long = np == 0 || s_off[0] >= 128 || used - s_off[np - 1] > 128 ? TQ_MAY_LONG : 0u;
         }
-        // ---- K4, first half: whole-piece lookups, a thread per piece, LW pieces per thread and step, their table slots
-        // fetched side by side.  Pieces of at most 8 bytes -- most of them -- take a path of their own: two key words, one
-        // 16-byte half of the slot.  The text comes from shared memory.  The tile's last piece is left to k_merge.
+        // ---- K4, first half: whole-piece lookups, a thread per piece, LW pieces per thread and step, their buckets
+        // fetched side by side.  Pieces of at most 8 bytes -- most of them -- take a path of their own: two key words, a
+        // table of 16-byte slots.  The text comes from shared memory.  The tile's last piece is left to k_merge.
         const long long gt = w_first * TT_WORD;                       // the tile's first byte, aligned frame
         const u32 nlook = np ? np - 1 : 0;
-        const bool quick = P.litstart == nullptr && F.toktab.slots != nullptr;     // block-uniform
+        const bool quick = F.toktab.shorts != nullptr;               // block-uniform
         const u32* const tw = reinterpret_cast<const u32*>(tb);
         u32 wsum = 0;
         constexpr int LW = NT == PRETOK_THREADS_BULK ? 1 : 4;        // look-ups in flight per thread
         for (u32 ib = tid; ib < nlook; ib += LW * NT) {
             u32 o[LW], n[LW], k0[LW], k1[LW], h[LW];
-            uint4 sl[LW];
+            uint4 sl[LW], sm2[LW];
+            bool lit[LW];
 #pragma unroll
             for (int j = 0; j < LW; j++) {
                 const u32 i = ib + j * NT;
                 o[j] = 0; n[j] = 0;
                 if (i < nlook) { o[j] = s_off[i]; n[j] = (u32)s_off[i + 1] - o[j]; }
-                k0[j] = 0; k1[j] = 0; h[j] = 0; sl[j] = make_uint4(0, 0, 0, 0);
-                if (quick && n[j] != 0 && n[j] <= 8) {
+                k0[j] = 0; k1[j] = 0; h[j] = 0; sl[j] = make_uint4(0, 0, 0, 0); sm2[j] = sl[j]; lit[j] = false;
+                if (P.litstart != nullptr && n[j] != 0) lit[j] = (P.litstart[(gt + o[j]) >> 5] >> ((gt + o[j]) & 31)) & 1;
+                if (quick && n[j] != 0 && n[j] <= TT_TOKTAB_SHORT) {
                     const u32* const w = tw + (o[j] >> 2);
                     toktab_key01(w[0], w[1], w[2], o[j] & 3, n[j], k0[j], k1[j]);
-                    if (n[j] == 1) sl[j].y = (u32)F.ext_id[k0[j]];
-                    else {
-                        h[j] = toktab_hash_final(toktab_hash_short(k0[j], k1[j], n[j]), F.toktab.shift);
-                        sl[j] = __ldg(reinterpret_cast<const uint4*>(F.toktab.slots + h[j]));
-                    }
+                    h[j] = toktab_hash_final(toktab_hash_short(k0[j], k1[j], n[j], F.toktab.seed));
+                    const uint4* const b = F.toktab.shorts + 2 * (size_t)toktab_bucket(h[j], F.toktab.short_shift);
+                    sl[j] = __ldg(b); sm2[j] = __ldg(b + 1);
                 }
             }
 #pragma unroll
@@ -459,18 +458,10 @@ k_pretok(const __grid_constant__ PretokParams P, const __grid_constant__ FrontPa
                 if (n[j] == 0) continue;
                 bool settled = false;
                 u32 val = 0;
-                if (quick && n[j] == 1) { val = sl[j].y; settled = true; }
-                else if (quick && n[j] <= 8) {
-                    uint4 c = sl[j];
-                    u32 hh = h[j];
-                    for (u32 probe = 0; probe <= F.toktab.mask; probe++) {       // bounded by the capacity
-                        if (c.x == 0) break;
-                        if (c.x == n[j] && c.z == k0[j] && c.w == k1[j]) { val = c.y; settled = true; break; }
-                        hh = (hh + 1) & F.toktab.mask;
-                        c = __ldg(reinterpret_cast<const uint4*>(F.toktab.slots + hh));
-                    }
-                } else if (quick) { s_slow[atomicAdd(&s_nslow, 1u)] = (u16)i; continue; }     // longer pieces: together, below
-                else settled = front_piece_general(P, F, gt + o[j], tb, o[j], n[j], val);
+                if (lit[j]) { val = 0u - 1u; settled = true; }         // one staged id (written by the literal pass)
+                else if (quick && n[j] <= TT_TOKTAB_SHORT) settled = toktab_short(F.toktab, sl[j], sm2[j], h[j], n[j], k0[j], k1[j], val);
+                else if (quick) { s_slow[atomicAdd(&s_nslow, 1u)] = (u16)i; continue; }     // longer pieces: together, below
+                else settled = front_piece_general(F, tb, o[j], n[j], val);
                 if (settled) { F.piece_cnt[p0 + i] = val; wsum++; }
                 else front_piece_queue(F, tile, o[j], i, n[j], &s_ns, &s_nw, &s_nl, s_wlist);
             }
@@ -481,7 +472,7 @@ k_pretok(const __grid_constant__ PretokParams P, const __grid_constant__ FrontPa
             for (u32 e = tid; e < nslow; e += NT) {
                 const u32 i = s_slow[e], o = s_off[i], n = (u32)s_off[i + 1] - o;
                 u32 val = 0;
-                if (front_piece_general(P, F, gt + o, tb, o, n, val)) { F.piece_cnt[p0 + i] = val; wsum++; }
+                if (front_piece_general(F, tb, o, n, val)) { F.piece_cnt[p0 + i] = val; wsum++; }
                 else front_piece_queue(F, tile, o, i, n, &s_ns, &s_nw, &s_nl, s_wlist);
             }
         }
