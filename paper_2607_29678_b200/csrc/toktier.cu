@@ -444,6 +444,12 @@ extern "C" int tt_vocab_load_ex(const tt_merge* merges, size_t n_merges, const i
     std::vector<u8> cls(v->cls_bytes, 0);
     memcpy(cls.data(), tt_cls_stage1_host, 0x1100);
     memcpy(cls.data() + 0x1100, tt_cls_stage2_host, stage2_bytes);
+    static_assert(TT_CLS_NBLOCKS <= CLS_UNIFORM, "block numbers and uniform classes share a byte");
+    for (size_t i = 0; i < 0x1100; i++) {
+        const u8* const blk = tt_cls_stage2_host + 128 * (size_t)tt_cls_stage1_host[i];
+        const u8 c = blk[0] & 15;
+        if (blk[0] == (c | (c << 4)) && memcmp(blk, blk + 1, 127) == 0) cls[i] = (u8)(CLS_UNIFORM | c);
+    }
     tt_fill_ascii_table(cls.data() + v->cls_bytes - 128);
     bool ok = cudaGetDevice(&v->device) == cudaSuccess;
     ok = ok && cudaDeviceGetAttribute(&v->sm_count, cudaDevAttrMultiProcessorCount, v->device) == cudaSuccess;
@@ -671,7 +677,6 @@ static int encode_impl(const tt_vocab* v, const uint8_t* text, size_t len, const
     int rc = run_pretok(v, text, len, doc_off, n_docs, st, w, nullptr, PP, literals, true, host_src, ev == nullptr);
     if (rc != TT_OK) return rc;
     MARK(1);
-    const int tile_grid = PP.ntiles < v->sm_count * 8 ? PP.ntiles : v->sm_count * 8;
     const int merge_grid = v->sm_count * MERGE_CTAS_PER_SM;                  // all resident CTA slots: a request's unsettled pieces get a warp each
     PieceParams Q;
     Q.base = PP.base; Q.shift = PP.lo; Q.hi = PP.hi; Q.ntiles = PP.ntiles;
@@ -695,7 +700,10 @@ static int encode_impl(const tt_vocab* v, const uint8_t* text, size_t len, const
     S.ids_out = ids_out; S.count_out = (long long*)count_out; S.status_out = status_out;
     S.docmask = doc_off ? w.docmask : nullptr; S.doc_off = (const long long*)doc_off; S.n_docs = (int)n_docs;
     S.ids_off_out = (long long*)ids_off_out;
-    CK(launch_after(big ? k_scatter_bulk : k_scatter, tile_grid, BPE_THREADS, st, 0, ev == nullptr, S));
+    const bool many = PP.ntiles > v->sm_count * SCATTER_CTAS;
+    const int scatter_ctas = v->sm_count * 8;
+    CK(launch_after(big ? k_scatter_bulk : many ? k_scatter<SCATTER_CTAS_MANY> : k_scatter<SCATTER_CTAS>, PP.ntiles < scatter_ctas ? PP.ntiles : scatter_ctas,
+                    BPE_THREADS, st, 0, ev == nullptr, S));
     MARK(3);
 #undef MARK
     CK(cudaGetLastError());

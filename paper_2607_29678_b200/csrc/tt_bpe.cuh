@@ -1650,12 +1650,18 @@ struct ScatterParams {
 };
 
 constexpr int SCATTER_STAGE_IDS = 2048;                   // ids of one work item that are put together in shared memory
+// CTAs per SM the kernel is compiled for.  A text of at most 4 tiles per SM gets all 64 registers, its loads are what counts; with
+// more tiles than that five CTAs of 48 registers (Thai-like text of 2.9 MB 97 -> 89 us per call; eight of 32 registers
+// spill: 1M chars 32 -> 37 us).
+constexpr int SCATTER_CTAS = 4, SCATTER_CTAS_MANY = 5;
+constexpr u32 SCATTER_WARP_MAX = 512;                     // tokens of a piece that one warp copies; longer ones the whole CTA
 // Work items: (tile, block of 512 of its pieces), two neighbouring pieces per thread.  A request has a tile per CTA and most
 // tiles one item, so what counts is the chain of dependent steps: everything that does not depend on anything else -- the
 // tiles' token counts, the first item's values and offsets, read before its length is known -- is asked for at once, the sums
 // over the tiles and the scan over the item's pieces share one barrier, and a staged piece's ids are fetched side by
 // side.  (Step by step, with a barrier after each, the kernel took 7.5 us behind k_merge on a 1M-char request.)
-__global__ void __launch_bounds__(BPE_THREADS)
+template <int MINB>
+__global__ void __launch_bounds__(BPE_THREADS, MINB)
 k_scatter(const __grid_constant__ ScatterParams P) {
     __shared__ u32 s_scan[2][BPE_WARPS], s_before[BPE_WARPS], s_total[BPE_WARPS];
     __shared__ u32 s_big[TT_TILE_BYTES / 8][3];
@@ -1767,12 +1773,23 @@ k_scatter(const __grid_constant__ ScatterParams P) {
         if (staged) {                                             // block-uniform
             __syncthreads();
             for (u32 kk = tid; kk < tot; kk += BPE_THREADS) P.ids_out[carry + kk] = s_out[kk];
-        } else if (some_big) {                                    // block-uniform: pieces of more than 8 tokens, copied by the whole CTA
+        } else if (some_big) {                                    // block-uniform: pieces of more than 8 tokens
+            // a warp each, four loads in flight per lane (one after the other by the whole CTA they took 45 us where most pieces
+            // of 3 MB of text have 50 to 100 tokens); the few very long ones by the whole CTA
             __syncthreads();
             const u32 nbig = min(s_nbig, (u32)(TT_TILE_BYTES / 8));
             for (u32 e = 0; e < nbig; e++) {
-                const u32 src = s_big[e][0], d2 = s_big[e][1], cc = s_big[e][2];
-                for (u32 kk = tid; kk < cc; kk += BPE_THREADS) P.ids_out[d2 + kk] = P.stage[src + kk];
+                const u32 cc = s_big[e][2];
+                const bool whole = cc > SCATTER_WARP_MAX;         // block-uniform
+                if (!whole && (int)(e % BPE_WARPS) != wid) continue;
+                const u32 src = s_big[e][0], d2 = s_big[e][1], step = whole ? (u32)BPE_THREADS : 32u;
+                for (u32 k0 = whole ? (u32)tid : (u32)lane; k0 < cc; k0 += 4 * step) {
+                    int32_t id[4];
+#pragma unroll
+                    for (int u = 0; u < 4; u++) id[u] = k0 + u * step < cc ? P.stage[src + k0 + u * step] : 0;
+#pragma unroll
+                    for (int u = 0; u < 4; u++) if (k0 + u * step < cc) P.ids_out[d2 + k0 + u * step] = id[u];
+                }
             }
             __syncthreads();
             if (tid == 0) s_nbig = 0;                             // (the next item's barrier comes before anyone adds)

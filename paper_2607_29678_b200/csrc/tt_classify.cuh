@@ -25,9 +25,12 @@ struct WordMasks {
     u32 bad;                  // byte takes part in a UTF-8 violation
 };
 
+// Stage 1 names a block of stage 2, or (from CLS_UNIFORM on) the one class of all 256 code points: CJK and Hangul take one load.
+constexpr u32 CLS_UNIFORM = 0xF8;
 TT_HD u32 tt_class_of(u32 cp, const ClassTables& T) {
-    u32 blk = T.stage1[cp >> 8];
-    u32 v = T.stage2[blk * 128 + ((cp & 0xFF) >> 1)];
+    const u32 blk = T.stage1[cp >> 8];
+    if (blk >= CLS_UNIFORM) return blk & 7u;
+    const u32 v = T.stage2[blk * 128 + ((cp & 0xFF) >> 1)];
     return (cp & 1) ? (v >> 4) : (v & 15);
 }
 
