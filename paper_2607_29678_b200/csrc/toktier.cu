@@ -594,24 +594,20 @@ static int run_pretok(const tt_vocab* v, const uint8_t* text, size_t len, const 
     P.startmask = w.startmask; P.tile_cnt = w.tile_cnt; P.tile_first = w.tile_first; P.want_prefix = piece_off_dst != nullptr; P.hdr = w.hdr;
     P.cls_tables = v->d_cls; P.cls_bytes = v->cls_bytes;
     if (doc_off) {
-        CK(cudaMemsetAsync(w.docmask, 0, ((size_t)P.hi / 32 + 4) * sizeof(u32), st));
-        const int threads = 256, blocks = (int)((n_docs + 1 + threads - 1) / threads);
-        k_docmask<<<blocks, threads, 0, st>>>((const long long*)doc_off, (int)n_docs, shift, (long long)len, w.docmask, w.hdr, P.epoch);
+        const long long mask_words = P.hi / 32 + 4;
+        CK(launch_after(k_docmask, (int)((mask_words + DOCMASK_WORDS - 1) / DOCMASK_WORDS), DOCMASK_THREADS, st, 0, early, (const long long*)doc_off,
+                        (int)n_docs, shift, (long long)len, mask_words, w.docmask, w.hdr, P.epoch));
         P.docmask = w.docmask;
     }
     if (literals && !doc_off) {
         // added-token literal pass: extracted literals become documents of their own and single pieces
-        const size_t words = ((size_t)P.hi / 32 + 4) * sizeof(u32);
-        CK(cudaMemsetAsync(w.docmask, 0, words, st));
-        CK(cudaMemsetAsync(w.litstart, 0, words, st));
-        CK(cudaMemsetAsync(w.litin, 0, words, st));
         LitParams L;
         L.base = P.base; L.lo = P.lo; L.hi = P.hi; L.tab = v->lit; L.cand = w.cand; L.stage = w.stage;
         L.docmask = w.docmask; L.litstart = w.litstart; L.litin = w.litin;
-        const size_t want = (len + 255) / 256;
+        const size_t want = (size_t)(P.nchunks + LIT_THREADS - 1) / LIT_THREADS;
         const int lgrid = (int)(want < (size_t)v->sm_count * 8 ? want : (size_t)v->sm_count * 8);
-        k_lit_scan<<<lgrid, 256, 0, st>>>(L);
-        k_lit_select<<<lgrid, 256, 0, st>>>(L);
+        CK(launch_after(k_lit_scan, lgrid, LIT_THREADS, st, 0, early, L));
+        CK(launch_after(k_lit_select, lgrid, LIT_THREADS, st, 0, early, L));
         P.docmask = w.docmask; P.litstart = w.litstart; P.litin = w.litin;
     }
     const bool bulk = P.ntiles > MERGE_SR_MAX_TILES;
@@ -669,9 +665,10 @@ static int encode_impl(const tt_vocab* v, const uint8_t* text, size_t len, const
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) { cudaGetLastError(); cap = cudaStreamCaptureStatusActive; }
     // Bulk text (more tiles than a request's job search covers) uses one counter in the first kernel itself, the length
-    // of the global list of warp-class pieces: there the header is cleared too.
+    // of the global list of warp-class pieces: there the header is cleared too.  (The kernels in front of the first one
+    // touch only the status word.)
     const bool big = (((uintptr_t)text & 15) + len + TT_TILE_BYTES - 1) / TT_TILE_BYTES > (size_t)MERGE_SR_MAX_TILES;
-    if (doc_off || literals || big || cap != cudaStreamCaptureStatusNone) CK(cudaMemsetAsync(w.hdr, 0, sizeof(TTHeader), st));
+    if (big || cap != cudaStreamCaptureStatusNone) CK(cudaMemsetAsync(w.hdr, 0, sizeof(TTHeader), st));
     MARK(0);
     PretokParams PP;
     int rc = run_pretok(v, text, len, doc_off, n_docs, st, w, nullptr, PP, literals, true, host_src, ev == nullptr);

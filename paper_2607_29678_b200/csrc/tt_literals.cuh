@@ -1,7 +1,7 @@
 // Added-token literal pass (paper Sec. 4.3 / 4.4): added and special tokens are literal strings that map to one
 // reserved id each; a leftmost-longest pass extracts them before the tokenizer family handles the segments in
 // between.  Two kernels prepare what the ordinary chain then consumes:
-//   k_lit_scan    one thread per byte: the longest literal that matches at that byte (its length goes to
+//   k_lit_scan    for every byte the longest literal that matches there (its length goes to
 //                 cand[], its id to stage[] at the byte's text offset);
 //   k_lit_select  leftmost-longest selection.  A candidate that no other candidate overlaps from the left is
 //                 selected on its own; a chain of overlapping candidates is walked by the thread of its first
@@ -12,7 +12,7 @@
 // k_pretok then forces exactly one piece per literal (start bit at its first byte, none inside) and, in its look-up
 // half, takes the staged id for a piece that begins at a litstart bit.
 #pragma once
-#include "tt_common.cuh"
+#include "tt_classify.cuh"
 
 struct LitEntry { u32 first4; u32 off; u32 len; int32_t id; };       // first4: the first min(len, 4) bytes, low byte first
 struct LitTable {
@@ -29,29 +29,46 @@ struct LitParams {
     LitTable tab;
     u8* cand;                    // [hi + 1] aligned frame: length of the longest literal starting at the byte, 0 = none
     int32_t* stage;              // text offsets: id of that literal
-    u32* docmask; u32* litstart; u32* litin;     // bit per byte, aligned frame (zero on entry)
+    u32* docmask; u32* litstart; u32* litin;     // bit per byte, aligned frame (cleared by k_lit_scan)
 };
 
-__global__ void __launch_bounds__(256)
-k_lit_scan(const LitParams P) {
-    for (long long g = P.lo + (long long)blockIdx.x * blockDim.x + threadIdx.x; g < P.hi; g += (long long)gridDim.x * blockDim.x) {
-        const u32 b = P.base[g];
-        u32 found = 0;
-        if ((P.tab.first_byte[b >> 5] >> (b & 31)) & 1) {
+// A thread takes 16 bytes: nearly none of them begins a literal, so what counts is one load and one store for all of them.  (A
+// thread per byte took 8.9 us for 300 KB, and clearing the three masks three memsets more in front of it.)
+constexpr int LIT_THREADS = 128;
+__global__ void __launch_bounds__(LIT_THREADS)
+k_lit_scan(const __grid_constant__ LitParams P) {
+    __shared__ u32 s_first[8];
+    cudaTriggerProgrammaticLaunchCompletion();
+    if (threadIdx.x < 8) s_first[threadIdx.x] = P.tab.first_byte[threadIdx.x];
+    __syncthreads();
+    cudaGridDependencySynchronize();                         // the work before this call: its text, its use of the masks
+    const long long nchunks = (P.hi + TT_CHUNK - 1) / TT_CHUNK, nwords = P.hi / 32 + 4;
+    const long long step = (long long)gridDim.x * LIT_THREADS, first = (long long)blockIdx.x * LIT_THREADS + threadIdx.x;
+    for (long long w = first; w < nwords; w += step) { P.docmask[w] = 0; P.litstart[w] = 0; P.litin[w] = 0; }
+    for (long long c = first; c < nchunks; c += step) {
+        const long long g0 = c * TT_CHUNK;
+        const uint4 v = *reinterpret_cast<const uint4*>(P.base + g0);
+        const u32 x[4] = {v.x, v.y, v.z, v.w};
+        u32 hits = 0;                                        // bytes that may begin a literal
+#pragma unroll
+        for (int i = 0; i < TT_CHUNK; i++) { const u32 b = (x[i >> 2] >> (8 * (i & 3))) & 0xFFu; hits |= ((s_first[b >> 5] >> (b & 31)) & 1u) << i; }
+        hits &= tt_valid_bytes(g0, P.lo, P.hi);
+        *reinterpret_cast<uint4*>(P.cand + g0) = make_uint4(0, 0, 0, 0);
+        for (; hits; hits &= hits - 1) {
+            const long long g = g0 + __ffs(hits) - 1;
             const u32 avail = (u32)min((long long)P.tab.maxlen, P.hi - g);
-            u32 w = b;
+            u32 w = P.base[g];
             for (u32 k = 1; k < 4 && k < avail; k++) w |= (u32)P.base[g + k] << (8 * k);
-            for (u32 e = 0; e < P.tab.n && !found; e++) {          // longest first: the first match is the longest
+            for (u32 e = 0; e < P.tab.n; e++) {              // longest first: the first match is the longest
                 const LitEntry L = P.tab.entries[e];
                 if (L.len > avail) continue;
                 const u32 m = L.len >= 4 ? 0xFFFFFFFFu : (1u << (8 * L.len)) - 1;
                 if ((w & m) != L.first4) continue;
                 u32 k = 4;
                 while (k < L.len && P.tab.blob[L.off + k] == P.base[g + k]) k++;
-                if (k >= L.len) { found = L.len; P.stage[g - P.lo] = L.id; }
+                if (k >= L.len) { P.cand[g] = (u8)L.len; P.stage[g - P.lo] = L.id; break; }
             }
         }
-        P.cand[g] = (u8)found;
     }
 }
 
@@ -74,11 +91,19 @@ __device__ __forceinline__ bool lit_covered(const LitParams& P, long long g) {
     return false;
 }
 
-__global__ void __launch_bounds__(256)
-k_lit_select(const LitParams P) {
+// The text's literals one by one, by the thread of their chunk.
+__global__ void __launch_bounds__(LIT_THREADS)
+k_lit_select(const __grid_constant__ LitParams P) {
+    cudaTriggerProgrammaticLaunchCompletion();
+    cudaGridDependencySynchronize();                         // the candidates are complete from here on
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&P.docmask[P.lo >> 5], 1u << (P.lo & 31));      // the text itself starts a document
-    for (long long g0 = P.lo + (long long)blockIdx.x * blockDim.x + threadIdx.x; g0 < P.hi; g0 += (long long)gridDim.x * blockDim.x) {
-        if (!P.cand[g0] || lit_covered(P, g0)) continue;           // only the first member of a chain works
+    const long long nchunks = (P.hi + TT_CHUNK - 1) / TT_CHUNK;
+    for (long long c = (long long)blockIdx.x * LIT_THREADS + threadIdx.x; c < nchunks; c += (long long)gridDim.x * LIT_THREADS) {
+      const uint4 v = *reinterpret_cast<const uint4*>(P.cand + c * TT_CHUNK);
+      if ((v.x | v.y | v.z | v.w) == 0) continue;
+      for (int i = 0; i < TT_CHUNK; i++) {
+        const long long g0 = c * TT_CHUNK + i;
+        if (g0 < P.lo || g0 >= P.hi || !P.cand[g0] || lit_covered(P, g0)) continue;           // only the first member of a chain works
         long long g = g0;
         for (;;) {                                                 // bounded by the text length: g strictly grows
             const long long end = g + P.cand[g];
@@ -93,5 +118,6 @@ k_lit_select(const LitParams P) {
             if (r >= stop || !lit_covered(P, r)) break;            // none near, or it heads a chain of its own
             g = r;
         }
+      }
     }
 }

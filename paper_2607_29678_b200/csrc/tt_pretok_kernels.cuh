@@ -44,19 +44,47 @@ __device__ __forceinline__ u32 cta_exscan_u32(u32 v, u32* scratch /* >= 33 */, u
 }
 
 // ---- document mask ---------------------------------------------------------------------------
-// Sets the bit of every document's first byte (aligned frame).  Offsets must be ascending, start at
-// 0 and end at the total length; a violation is reported as TT_ERR_ARG in the status word.
-__global__ void k_docmask(const long long* __restrict__ doc_off, int n_docs, long long shift, long long len,
-                          u32* __restrict__ docmask, TTHeader* hdr, unsigned long long epoch) {
-    int d = blockIdx.x * blockDim.x + threadIdx.x;
-    if (d > n_docs) return;
-    long long o = doc_off[d];
-    bool ok = o >= 0 && o <= len && (d == 0 ? o == 0 : o >= doc_off[d - 1]) && (d < n_docs || o == len);
-    if (!ok) { hdr_set_status(hdr, epoch, 1 /* TT_ERR_ARG */); return; }
-    if (d < n_docs && o < len) {
-        long long g = o + shift;
-        atomicOr(&docmask[g >> 5], 1u << (g & 31));
+// Writes the mask with the bit of every document's first byte (aligned frame), and checks the offsets: they must be ascending,
+// start at 0 and end at the total length; a violation is reported as TT_ERR_ARG in the status word.  A CTA writes
+// DOCMASK_WORDS words: it finds the first document of its stretch by a search in 32 steps at a time.  (Clearing the mask and
+// setting bits in it with atomics were two launches, and two gaps, in front of the chain.)
+constexpr int DOCMASK_WORDS = 2048, DOCMASK_THREADS = 256;
+__global__ void __launch_bounds__(DOCMASK_THREADS)
+k_docmask(const long long* __restrict__ doc_off, int n_docs, long long shift, long long len, long long nwords,
+          u32* __restrict__ docmask, TTHeader* hdr, unsigned long long epoch) {
+    __shared__ __align__(16) u32 s_mask[DOCMASK_WORDS];
+    __shared__ int s_first;
+    const int tid = threadIdx.x, lane = tid & 31;
+    // (No early trigger: bulk text fills every place of the GPU with CTAs that stay, and what was placed beside this grid stayed
+    // unevenly spread: 535 -> 558 us for 12 MB.)
+    cudaGridDependencySynchronize();                         // the work before this call reads the mask, or writes the offsets
+    for (int i = tid; i < DOCMASK_WORDS; i += DOCMASK_THREADS) s_mask[i] = 0;
+    const long long w0 = (long long)blockIdx.x * DOCMASK_WORDS;
+    const long long from = w0 * 32 - shift, to = min((w0 + DOCMASK_WORDS) * 32 - shift, len);      // text bytes of the stretch
+    if (tid < 32) {                                           // first document that starts at `from` or behind it
+        int lo = 0, hi = n_docs;                              // (the answer is in [lo, hi])
+        while (hi > lo) {
+            const int step = (hi - lo + 31) / 32, at = lo + lane * step;
+            const bool less = at < hi && doc_off[at] < from;
+            const int c = __popc(__ballot_sync(0xFFFFFFFFu, less));                                // ascending: the first c probes are below
+            if (c == 0) hi = lo;
+            else { const int l2 = lo + (c - 1) * step + 1; hi = min(hi, lo + c * step); lo = l2; }
+        }
+        if (lane == 0) s_first = lo;
     }
+    __syncthreads();
+    for (int d = s_first + tid; d < n_docs; d += DOCMASK_THREADS) {
+        const long long o = doc_off[d];
+        if (o >= to) break;
+        if (o >= from && o >= 0) { const long long g = o + shift - w0 * 32; atomicOr(&s_mask[g >> 5], 1u << (g & 31)); }
+    }
+    for (long long d = (long long)blockIdx.x * DOCMASK_THREADS + tid; d <= n_docs; d += (long long)gridDim.x * DOCMASK_THREADS) {
+        const long long o = doc_off[d];
+        const bool ok = o >= 0 && o <= len && (d == 0 ? o == 0 : o >= doc_off[d - 1]) && (d < n_docs || o == len);
+        if (!ok) hdr_set_status(hdr, epoch, 1 /* TT_ERR_ARG */);
+    }
+    __syncthreads();
+    for (int i = tid; i < DOCMASK_WORDS && w0 + i < nwords; i += DOCMASK_THREADS) docmask[w0 + i] = s_mask[i];
 }
 
 __device__ __forceinline__ u32 doc_bits(const PretokParams& P, long long word) {
