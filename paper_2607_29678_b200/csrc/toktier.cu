@@ -838,7 +838,7 @@ extern "C" int tt_pretokenize(const tt_vocab* v, const uint8_t* text, size_t len
 
 extern "C" size_t tt_spans_workspace_bytes(const tt_vocab* v, size_t ids_cap) {
     (void)v;
-    return align_up(sizeof(SpanHeader), 256) + align_up((ids_cap / SPAN_THREADS + 3) * sizeof(uint2), 256);
+    return align_up((ids_cap / SPAN_BLOCK + 3) * sizeof(uint2), 256);
 }
 
 extern "C" int tt_spans(const tt_vocab* v, const int32_t* ids, const int64_t* count, size_t ids_cap, size_t text_len,
@@ -851,15 +851,13 @@ extern "C" int tt_spans(const tt_vocab* v, const int32_t* ids, const int64_t* co
     SpanParams P;
     P.ids = ids; P.count = (const long long*)count; P.ids_cap = ids_cap; P.text_len = text_len;
     P.meta = v->d_meta; P.meta_n = v->meta_n;
-    P.hdr = (SpanHeader*)workspace;
-    P.blk = (uint2*)((char*)workspace + align_up(sizeof(SpanHeader), 256));
+    P.blk = (uint2*)workspace;
     P.byte_off = byte_off_out; P.char_off = char_off_out; P.status_out = status_out;
-    CK(cudaMemsetAsync(P.hdr, 0, sizeof(SpanHeader), st));
-    size_t want = (ids_cap + SPAN_THREADS - 1) / SPAN_THREADS;
+    size_t want = (ids_cap + SPAN_BLOCK - 1) / SPAN_BLOCK;
     if (want < 1) want = 1;
-    const int grid = (int)(want > (size_t)v->sm_count * 2 ? (size_t)v->sm_count * 2 : want);
-    k_span_sums<<<grid, SPAN_THREADS, 0, st>>>(P);
-    k_span_write<<<grid, SPAN_THREADS, 0, st>>>(P);
+    const int grid = (int)(want > (size_t)v->sm_count * 4 ? (size_t)v->sm_count * 4 : want);
+    CK(launch_after(k_span_sums, grid, SPAN_THREADS, st, 0, true, P));
+    CK(launch_after(k_span_write, grid, SPAN_THREADS, st, 0, true, P));
     CK(cudaGetLastError());
     return TT_OK;
 }
