@@ -213,10 +213,11 @@ int tt_encode_added(const tt_vocab* v, const uint8_t* text, size_t len, void* st
  *   tt_session_view     DEVICE pointers to the IDs, to the byte offset of every token (count + 1 entries, the last
  *                       one the text length) and to the token count, plus the stored length in bytes; valid until
  *                       the next append or tt_session_free.
+ *   tt_session_tokens   the number of tokens stored, on the host.
  *   tt_session_copy     copies the records into caller-owned DEVICE buffers, asynchronously on `stream`:
  *                       ids_out int32[ids_cap] (may be NULL), off_out int32[ids_cap + 1] (may be NULL), count_out
- *                       int64.  min(stored bytes, ids_cap) entries are copied (a token has at least one byte);
- *                       entries beyond the count are unspecified.
+ *                       int64.  min(tokens, ids_cap) ids are copied, and one offset more; entries beyond are left
+ *                       as they are.
  * One session must not be used from two threads at once.
  */
 typedef struct tt_session tt_session;
@@ -235,6 +236,7 @@ int tt_session_set_window(tt_session* s, uint32_t window_chars);
 int tt_session_append(tt_session* s, const uint8_t* text, size_t len, void* stream, tt_append_info* info);
 int tt_session_view(const tt_session* s, const int32_t** ids_dev, const int32_t** off_dev, const int64_t** count_dev,
                     size_t* len_bytes);
+size_t tt_session_tokens(const tt_session* s);
 int tt_session_copy(const tt_session* s, int32_t* ids_out, size_t ids_cap, int32_t* off_out, int64_t* count_out,
                     void* stream);
 

@@ -105,6 +105,8 @@ def lib() -> ctypes.CDLL:
         L.tt_verifier_quarantined.argtypes = [c.c_void_p, c.c_size_t, c.POINTER(c.c_uint64), c.POINTER(c.c_uint64), c.POINTER(c.c_int64)]
         L.tt_verifier_free.restype = None
         L.tt_verifier_free.argtypes = [c.c_void_p]
+        L.tt_session_tokens.restype = c.c_size_t
+        L.tt_session_tokens.argtypes = [c.c_void_p]
         L.tt_session_copy.restype = c.c_int
         L.tt_session_copy.argtypes = [c.c_void_p, c.c_void_p, c.c_size_t, c.c_void_p, c.c_void_p, c.c_void_p]
         _lib = L
@@ -335,14 +337,14 @@ class Session:
         import torch
         n = ctypes.c_size_t()
         _check(lib().tt_session_view(self._h, None, None, None, ctypes.byref(n)), "tt_session_view")
-        ids = torch.empty(max(n.value, 1), dtype=torch.int32, device="cuda")
-        off = torch.empty(n.value + 1, dtype=torch.int32, device="cuda")
-        count = torch.zeros(1, dtype=torch.int64, device="cuda")
-        _check(lib().tt_session_copy(self._h, ids.data_ptr(), n.value, off.data_ptr(), count.data_ptr(), _stream_ptr(stream)),
+        k = int(lib().tt_session_tokens(self._h))
+        ids = torch.empty(max(k, 1), dtype=torch.int32, device="cuda")
+        off = torch.empty(k + 1, dtype=torch.int32, device="cuda")
+        count = torch.empty(1, dtype=torch.int64, device="cuda")
+        _check(lib().tt_session_copy(self._h, ids.data_ptr(), k, off.data_ptr(), count.data_ptr(), _stream_ptr(stream)),
                "tt_session_copy")
         torch.cuda.synchronize()
-        k = int(count.item())
-        return ids[:k], off[:k + 1], n.value
+        return ids[:k], off, n.value
 
 
 class VerifierStats(ctypes.Structure):

@@ -31,14 +31,14 @@
 // tt_vocab_free): fifteen cudaMalloc and cudaFree calls per session took 2 to 15 ms, more than the 17 tokenizations of
 // a conversation.  Sessions share ownership, so that one that outlives its vocabulary still frees what it holds.
 struct SessionHost;
-struct SessionArena { char* dev = nullptr; size_t bytes = 0; int device = 0; SessionHost* host = nullptr; };
+struct SessionArena { char* dev = nullptr; size_t bytes = 0; int device = 0; SessionHost* host = nullptr; size_t host_text = 0; };
 struct SessionPool {
     static constexpr size_t POOL_ARENAS = 8, POOL_BYTES = (size_t)512 << 20;
     std::mutex mu;
     std::vector<SessionArena> kept;
     bool closed = false;
     static void destroy(SessionArena& a) { cudaFree(a.dev); if (a.host) cudaFreeHost(a.host); a = SessionArena{}; }
-    bool get(size_t bytes, SessionArena& out);
+    bool get(size_t bytes, size_t host_text, SessionArena& out);
     void put(SessionArena a);
     void close() {
         std::lock_guard<std::mutex> lk(mu);
@@ -464,7 +464,8 @@ extern "C" int tt_vocab_load_ex(const tt_merge* merges, size_t n_merges, const i
     if (!ok) { cudaGetLastError(); tt_vocab_free(v); return TT_ERR_CUDA; }
     v->tab.slots = v->d_slots; v->tab.bytepair = v->d_bytepair; v->tab.mask = mask; v->tab.shift = shift;
     if (cudaFuncSetAttribute(k_merge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MERGE_SMEM_REQUEST) != cudaSuccess ||
-        cudaFuncSetAttribute(k_merge_bulk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MERGE_SMEM_BYTES) != cudaSuccess) { cudaGetLastError(); tt_vocab_free(v); return TT_ERR_CUDA; }
+        cudaFuncSetAttribute(k_merge_bulk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MERGE_SMEM_BYTES) != cudaSuccess ||
+        cudaFuncSetAttribute(k_repair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RepairSmem)) != cudaSuccess) { cudaGetLastError(); tt_vocab_free(v); return TT_ERR_CUDA; }
     { const int rc = build_token_table(v, merges, n_merges, ext_id); if (rc != TT_OK) { tt_vocab_free(v); return rc; } }
     {   // byte length and number of non-continuation bytes of every token, indexed by the caller's id
         std::vector<uint2> in(256 + n_merges);
@@ -996,21 +997,24 @@ extern "C" int tt_encode_static(const tt_vocab* v, const uint8_t* text, size_t l
 // ---- sessions: incremental repair on append (paper Sec. 3.3) ------------------------------------------
 // What one copy brings back to the host: scalars of the session in device memory, and their image in pinned memory.
 struct SessionScalars { RepairDecision dec; long long ntok, fcount; int32_t fstatus, sstatus; };
-struct SessionHost { SessionScalars s; };
+// (text: the end of the stored text and what is appended, on their way to the first kernel, which reads them from here)
+struct SessionHost { SessionScalars s; alignas(16) u8 text[16]; };
+constexpr size_t SESSION_HOST_TEXT = (size_t)256 << 10;       // most of it that a session holds
+static size_t session_host_text(size_t max_bytes) { return (max_bytes < SESSION_HOST_TEXT ? max_bytes : SESSION_HOST_TEXT) + 48; }
 
-bool SessionPool::get(size_t bytes, SessionArena& out) {
+bool SessionPool::get(size_t bytes, size_t host_text, SessionArena& out) {
     int device = 0;
     if (cudaGetDevice(&device) != cudaSuccess) { cudaGetLastError(); return false; }
     {
         std::lock_guard<std::mutex> lk(mu);
         size_t best = kept.size();
         for (size_t i = 0; i < kept.size(); i++)                 // the smallest one that is large enough, not wastefully so
-            if (kept[i].device == device && kept[i].bytes >= bytes && kept[i].bytes / 4 <= bytes && (best == kept.size() || kept[i].bytes < kept[best].bytes)) best = i;
+            if (kept[i].device == device && kept[i].bytes >= bytes && kept[i].host_text >= host_text && kept[i].bytes / 4 <= bytes && (best == kept.size() || kept[i].bytes < kept[best].bytes)) best = i;
         if (best < kept.size()) { out = kept[best]; kept.erase(kept.begin() + (ptrdiff_t)best); return true; }
     }
-    out.bytes = bytes; out.device = device;
+    out.bytes = bytes; out.device = device; out.host_text = host_text;
     if (cudaMalloc(&out.dev, bytes) != cudaSuccess) { cudaGetLastError(); out.dev = nullptr; return false; }
-    if (cudaMallocHost(&out.host, sizeof(SessionHost)) != cudaSuccess) { cudaGetLastError(); cudaFree(out.dev); out = SessionArena{}; return false; }
+    if (cudaMallocHost(&out.host, sizeof(SessionHost) + host_text) != cudaSuccess) { cudaGetLastError(); cudaFree(out.dev); out = SessionArena{}; return false; }
     return true;
 }
 void SessionPool::put(SessionArena a) {
@@ -1038,6 +1042,10 @@ struct tt_session {
     u8* d_eq = nullptr;
     SessionScalars* d_sc = nullptr;
     SessionScalars* h = nullptr;                                        // pinned
+    u8* h_stage = nullptr;                                              // pinned, h_stage_cap bytes
+    size_t h_stage_cap = 0;
+    bool records = false;                                               // the device's records are set (an empty session's: not yet)
+    size_t ntok = 0;
     void *d_ws = nullptr, *d_sws = nullptr;
     size_t ws_bytes = 0, sws_bytes = 0;
 };
@@ -1079,14 +1087,10 @@ extern "C" int tt_session_create(const tt_vocab* v, size_t max_bytes, tt_session
         s->d_ws = take(s->ws_bytes); s->d_sws = take(s->sws_bytes);
     };
     carve_all();
-    if (!s->pool->get(off, s->arena)) { delete s; return TT_ERR_CUDA; }
+    if (!s->pool->get(off, session_host_text(max_bytes), s->arena)) { delete s; return TT_ERR_CUDA; }
     base = s->arena.dev;
     carve_all();
-    s->h = &s->arena.host->s;
-    // no record yet: count 0, off[0] = 0.  (Waited for: the session may be used from any stream.)
-    const bool ok = cudaMemset(s->d_sc, 0, sizeof(SessionScalars)) == cudaSuccess && cudaMemset(s->d_off, 0, 4) == cudaSuccess &&
-                    cudaStreamSynchronize(nullptr) == cudaSuccess;
-    if (!ok) { cudaGetLastError(); tt_session_free(s); return TT_ERR_CUDA; }
+    s->h = &s->arena.host->s; s->h_stage = s->arena.host->text; s->h_stage_cap = s->arena.host_text;
     *out = s;
     return TT_OK;
 }
@@ -1097,9 +1101,23 @@ extern "C" int tt_session_set_window(tt_session* s, uint32_t window_chars) {
     return TT_OK;
 }
 
+// The records of a session without text: count 0, off[0] = 0, written when somebody looks for the first time.  (Waited for: the
+// session may be used from any stream.)
+static int session_empty_records(tt_session* s) {
+    if (s->records) return TT_OK;
+    CK(cudaMemset(s->d_sc, 0, sizeof(SessionScalars)));
+    CK(cudaMemset(s->d_off, 0, 4));
+    CK(cudaStreamSynchronize(nullptr));
+    s->records = true;
+    return TT_OK;
+}
+
+extern "C" size_t tt_session_tokens(const tt_session* s) { return s ? s->ntok : 0; }
+
 extern "C" int tt_session_view(const tt_session* s, const int32_t** ids_dev, const int32_t** off_dev,
                                const int64_t** count_dev, size_t* len_bytes) {
     if (!s) return TT_ERR_ARG;
+    if (ids_dev || off_dev || count_dev) { const int rc = session_empty_records(const_cast<tt_session*>(s)); if (rc != TT_OK) return rc; }
     if (ids_dev) *ids_dev = s->d_ids;
     if (off_dev) *off_dev = s->d_off;
     if (count_dev) *count_dev = (const int64_t*)&s->d_sc->ntok;
@@ -1107,11 +1125,12 @@ extern "C" int tt_session_view(const tt_session* s, const int32_t** ids_dev, con
     return TT_OK;
 }
 
-// Tokenizes text[from, new_len) into (ids, off, count) with offsets relative to `from`.
-static int session_tokenize(tt_session* s, size_t from, size_t new_len, cudaStream_t st, int32_t* ids, int32_t* off, long long* count) {
+// Tokenizes text[from, new_len) into (ids, count), and (off, with offsets relative to `from`) where off is given.  host_src: where
+// the first kernel reads that text, or null: it stands in d_text already.
+static int session_tokenize(tt_session* s, size_t from, size_t new_len, cudaStream_t st, int32_t* ids, int32_t* off, long long* count, const u8* host_src) {
     const size_t n = new_len - from;
-    int rc = encode_impl(s->v, s->d_text + from, n, nullptr, 1, st, ids, s->cap, (int64_t*)count, nullptr, &s->d_sc->fstatus, s->d_ws);
-    if (rc != TT_OK) return rc;
+    int rc = encode_impl(s->v, s->d_text + from, n, nullptr, 1, st, ids, s->cap, (int64_t*)count, nullptr, &s->d_sc->fstatus, s->d_ws, nullptr, false, host_src);
+    if (rc != TT_OK || !off) return rc;
     // (n bytes hold at most n tokens: the span kernels' grid follows the window, not the session's capacity)
     return tt_spans(s->v, ids, (const int64_t*)count, n, n, st, off, s->d_fchar, &s->d_sc->sstatus, s->d_sws, s->sws_bytes);
 }
@@ -1137,9 +1156,27 @@ extern "C" int tt_session_append(tt_session* s, const uint8_t* text, size_t len,
     const size_t old_len = s->len, new_len = old_len + len;
     // (an error return waits for the stream first: the copy from the caller's buffer may still be in flight)
     auto fail = [&](int code) { cudaStreamSynchronize(st); cudaGetLastError(); if (info) { local.status = code; *info = local; } return code; };
-    if (len) { if (cudaMemcpyAsync(s->d_text + old_len, text, len, cudaMemcpyHostToDevice, st) != cudaSuccess) { cudaGetLastError(); return fail(TT_ERR_CUDA); } }
     if (new_len == 0) { if (info) *info = local; return TT_OK; }
     const u8* ht = s->h_tail.data() - s->tail_base;          // ht[i] = byte i of the stored text, for i >= tail_base
+    // The appended text goes to the device with the first kernel that needs it: the window (its old part comes from the host's
+    // tail) is put together in pinned memory in the 16-byte frame of d_text, and that kernel reads it there and leaves it
+    // in d_text.  Text that does not fit is copied in front.
+    bool on_device = len == 0;
+    auto stage = [&](size_t from, const u8*& src) -> bool {  // src: text[from ..] in pinned memory, or null: read d_text
+        src = nullptr;
+        const size_t frame = from & ~(size_t)15;
+        if (on_device) return true;
+        if (frame >= s->tail_base && new_len - frame <= s->h_stage_cap - 32) {
+            if (old_len > frame) memcpy(s->h_stage, ht + frame, old_len - frame);
+            memcpy(s->h_stage + (old_len - frame), text, len);
+            src = s->h_stage + (from - frame);
+            on_device = true;                                // once that kernel has run
+            return true;
+        }
+        if (cudaMemcpyAsync(s->d_text + old_len, text, len, cudaMemcpyHostToDevice, st) != cudaSuccess) { cudaGetLastError(); return false; }
+        on_device = true;
+        return true;
+    };
     uint64_t w = s->window_chars;
     for (int attempt = 0; attempt <= 5 && old_len > 0; attempt++, w *= 2) {
         // byte offset of the character that lies w characters before the end of the stored text
@@ -1148,8 +1185,21 @@ extern "C" int tt_session_append(tt_session* s, const uint8_t* text, size_t len,
         if (left > 0 || ws == s->tail_base) ws = 0;           // the window reaches the start of the text (or beyond what the host kept: more work, same ids)
         local.attempts = attempt + 1;
         if (ws == 0) break;                                   // the window is the whole text
-        int rc = session_tokenize(s, ws, new_len, st, s->d_fids, s->d_foff, &s->d_sc->fcount);
+        const u8* src;
+        if (!stage(ws, src)) return fail(TT_ERR_CUDA);
+        const bool small = new_len - ws <= (size_t)REPAIR_MAX;
+        int rc = session_tokenize(s, ws, new_len, st, s->d_fids, small ? nullptr : s->d_foff, &s->d_sc->fcount, src);
         if (rc != TT_OK) return fail(rc);
+        if (small) {
+            RepairFused P;
+            P.ids = s->d_ids; P.off = s->d_off; P.ntok = &s->d_sc->ntok;
+            P.fids = s->d_fids; P.fcount = &s->d_sc->fcount; P.fstatus = &s->d_sc->fstatus;
+            P.meta = s->v->d_meta; P.meta_n = s->v->meta_n; P.text = s->d_text;
+            P.ws = (long long)ws; P.old_len = (long long)old_len; P.new_len = (long long)new_len;
+            P.cls = s->v->d_cls; P.cls_bytes = s->v->cls_bytes; P.max_tok_chars = (int)s->v->max_token_chars;
+            P.dec = &s->h->dec;
+            if (launch_after(k_repair, 1, REPAIR_THREADS, st, sizeof(RepairSmem), true, P) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) { cudaGetLastError(); return fail(TT_ERR_CUDA); }
+        } else {
         RepairParams P;
         P.ids = s->d_ids; P.off = s->d_off; P.ntok = &s->d_sc->ntok;
         P.fids = s->d_fids; P.foff = s->d_foff; P.fchar = s->d_fchar; P.fcount = &s->d_sc->fcount;
@@ -1163,10 +1213,11 @@ extern "C" int tt_session_append(tt_session* s, const uint8_t* text, size_t len,
         k_repair_apply<<<grid, 256, 0, st>>>(P);
         if (cudaMemcpyAsync(&s->h->dec, &s->d_sc->dec, sizeof(RepairDecision), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
             cudaStreamSynchronize(st) != cudaSuccess) { cudaGetLastError(); return fail(TT_ERR_CUDA); }
+        }
         const RepairDecision d = s->h->dec;
         if (d.status != TT_OK) return fail(d.status);          // e.g. the appended text is not valid UTF-8: nothing changed
         if (d.accept) {
-            s->len = new_len; session_keep_tail(s, text, len);
+            s->len = new_len; s->ntok = (size_t)d.new_ntok; session_keep_tail(s, text, len);
             local.window_chars = (int64_t)w; local.window_start = (int64_t)ws; local.run_tokens = d.j1 - d.j0;
             local.splice_byte = d.splice_byte; local.n_tokens = d.new_ntok; local.status = TT_OK;
             if (info) *info = local;
@@ -1178,21 +1229,21 @@ extern "C" int tt_session_append(tt_session* s, const uint8_t* text, size_t len,
     // fresh buffers first, so that an error leaves the session as it was
     const bool direct = old_len == 0;
     long long* const count = direct ? &s->d_sc->ntok : &s->d_sc->fcount;
-    int rc = session_tokenize(s, 0, new_len, st, direct ? s->d_ids : s->d_fids, direct ? s->d_off : s->d_foff, count);
+    const u8* src;
+    if (!stage(0, src)) return fail(TT_ERR_CUDA);
+    if (direct) s->records = false;                          // (an error leaves them to be written again)
+    int rc = session_tokenize(s, 0, new_len, st, direct ? s->d_ids : s->d_fids, direct ? s->d_off : s->d_foff, count, src);
     if (rc != TT_OK) return fail(rc);
     if (cudaMemcpyAsync(s->h, s->d_sc, sizeof(SessionScalars), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess) { cudaGetLastError(); return fail(TT_ERR_CUDA); }
     const int bad = s->h->fstatus != TT_OK ? s->h->fstatus : s->h->sstatus;
-    if (bad != TT_OK) {
-        if (direct) cudaMemsetAsync(&s->d_sc->ntok, 0, 8, st);
-        return fail(bad);
-    }
+    if (bad != TT_OK) return fail(bad);
     const size_t nt = (size_t)(direct ? s->h->ntok : s->h->fcount);
     if (!direct && (cudaMemcpyAsync(s->d_ids, s->d_fids, nt * 4, cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
         cudaMemcpyAsync(s->d_off, s->d_foff, (nt + 1) * 4, cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
         cudaMemcpyAsync(&s->d_sc->ntok, &s->d_sc->fcount, 8, cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)) { cudaGetLastError(); return fail(TT_ERR_CUDA); }
-    s->len = new_len; session_keep_tail(s, text, len);
+    s->len = new_len; s->ntok = nt; s->records = true; session_keep_tail(s, text, len);
     local.window_chars = 0; local.window_start = 0; local.run_tokens = 0; local.splice_byte = 0;
     local.n_tokens = (int64_t)nt; local.status = TT_OK;
     if (info) *info = local;
@@ -1203,11 +1254,10 @@ extern "C" int tt_session_copy(const tt_session* s, int32_t* ids_out, size_t ids
                                int64_t* count_out, void* stream) {
     if (!s || !count_out) return TT_ERR_ARG;
     cudaStream_t st = (cudaStream_t)stream;
-    // the count is known on the host only as an upper bound (one token per byte); copy by that bound
-    const size_t n = s->len < ids_cap ? s->len : ids_cap;
-    if (ids_out && n) CK(cudaMemcpyAsync(ids_out, s->d_ids, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
-    if (off_out) CK(cudaMemcpyAsync(off_out, s->d_off, (n + 1) * sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
-    CK(cudaMemcpyAsync(count_out, &s->d_sc->ntok, sizeof(int64_t), cudaMemcpyDeviceToDevice, st));
+    { const int rc = session_empty_records(const_cast<tt_session*>(s)); if (rc != TT_OK) return rc; }
+    const size_t n = s->ntok < ids_cap ? s->ntok : ids_cap, want = (n + 1 + 1023) / 1024, most = (size_t)s->v->sm_count * 4;
+    CK(launch_after(k_session_copy, (int)(want < most ? want : most), 256, st, 0, true, (const int32_t*)s->d_ids, (const int32_t*)s->d_off,
+                    (const long long*)&s->d_sc->ntok, (long long)n, (long long)n + 1, ids_out, off_out, (long long*)count_out));
     return TT_OK;
 }
 

@@ -93,15 +93,17 @@ __device__ __forceinline__ u32 doc_bits(const PretokParams& P, long long word) {
     return word == 0 ? (1u << P.lo) : 0u;                            // (0 <= lo < 16)
 }
 // Eight words of text of the mask word `word` (zero outside the text).
-__device__ __forceinline__ uint4 load_chunk(const PretokParams& P, const u8* rd, long long chunk) {
-    if (chunk < 0 || chunk >= P.nchunks) return make_uint4(0, 0, 0, 0);
-    uint4 v = *reinterpret_cast<const uint4*>(rd + chunk * TT_CHUNK);
+__device__ __forceinline__ uint4 load_chunk_raw(const PretokParams& P, const u8* rd, long long chunk) {
+    return chunk < 0 || chunk >= P.nchunks ? make_uint4(0, 0, 0, 0) : *reinterpret_cast<const uint4*>(rd + chunk * TT_CHUNK);
+}
+__device__ __forceinline__ uint4 text_of_chunk(const PretokParams& P, uint4 v, long long chunk) {
     if (chunk == 0 || chunk == P.nchunks - 1) {                      // the ends of the text
         const u32 valid = tt_valid_bytes((chunk >> 1) * TT_WORD, P.lo, P.hi);
         v = tt_zero_invalid(v, (chunk & 1) ? valid >> 16 : valid & 0xFFFFu);
     }
     return v;
 }
+__device__ __forceinline__ uint4 load_chunk(const PretokParams& P, const u8* rd, long long chunk) { return text_of_chunk(P, load_chunk_raw(P, rd, chunk), chunk); }
 
 // ---- bounded CTA-cooperative walks over the text (runs that leave the shared-memory window) ----
 // Every loop below advances by a word per thread and iteration and stops at the ends of the text.  All
@@ -348,8 +350,8 @@ k_pretok(const __grid_constant__ PretokParams P, const __grid_constant__ FrontPa
         {
             const long long c0 = 2 * (w_first - TT_LOW_HALO);
             for (int c = tid; c < 2 * TT_SLOTS; c += NT) {
-                const uint4 v = load_chunk(P, rd, c0 + c);
-                *reinterpret_cast<uint4*>(s_text + 4 + 4 * c) = v;
+                const uint4 v = load_chunk_raw(P, rd, c0 + c);
+                *reinterpret_cast<uint4*>(s_text + 4 + 4 * c) = text_of_chunk(P, v, c0 + c);
                 if (P.src && c >= 2 * TT_LOW_HALO && c < 2 * (TT_LOW_HALO + TT_TILE_WORDS) && c0 + c < P.nchunks) *reinterpret_cast<uint4*>(P.copy + (c0 + c) * TT_CHUNK) = v;
             }
             if (tid == NT - 1) s_text[3] = load_chunk(P, rd, c0 - 1).w;
