@@ -399,6 +399,109 @@ TT_HD u32 tt_walk_back_slash(MaskRows sm, int s, int top, bool& open_s, bool& op
     return 0;
 }
 
+// ---- the sequential matcher on the tile's masks -------------------------------------------------------
+// The same matches as tt_seq_match_p1, found on the class masks of the tile's window (positions: slot * 32 + bit): a run of a class
+// ends at the first zero of a mask, whatever its length, where the matcher over the text decodes and classifies character
+// by character, up to four times each (300K chars of words with combining marks: 108 us for the worst tile, now 25).
+// Marks inside words count as caseless letters in these masks, which changes no match: a match that has taken their letter goes
+// on over them.
+enum { WK_UP, WK_LW, WK_PUNCT, WK_SPACE, WK_TAIL, WK_LEAD, WK_NL };
+template <int K> TT_HD u32 tt_win_word(MaskRows sm, int s) {
+    return K == WK_UP ? sm[F_UPP][s] | sm[F_CLESS][s] | sm[F_MARK][s] : K == WK_LW ? sm[F_LOW][s] | sm[F_CLESS][s] | sm[F_MARK][s]
+         : K == WK_PUNCT ? sm[F_OTH][s] | sm[F_MARK][s] : K == WK_SPACE ? sm[F_SPC][s] : K == WK_TAIL ? sm[F_NL][s] | sm[F_SL][s]
+         : K == WK_LEAD ? sm[F_LEAD][s] : sm[F_NL][s];
+}
+template <int K> TT_HD bool tt_win_is(MaskRows sm, int q) { return (tt_win_word<K>(sm, q >> 5) >> (q & 31)) & 1; }
+// First position in [q, end) that is (ONE) / is not (!ONE) of the kind, or end.
+template <int K, bool ONE> TT_HD int tt_win_find(MaskRows sm, int q, int end) {
+    u32 keep = 0xFFFFFFFFu << (q & 31);
+    for (int s = q >> 5; s * TT_WORD < end; s++, keep = 0xFFFFFFFFu) {
+        const u32 x = (ONE ? tt_win_word<K>(sm, s) : ~tt_win_word<K>(sm, s)) & keep;
+        if (x) { const int at = s * TT_WORD + tt_lobit(x); return at < end ? at : end; }
+    }
+    return end;
+}
+// Last position in [p, t) of the kind, or -1.
+template <int K> TT_HD int tt_win_last(MaskRows sm, int p, int t) {
+    if (t <= p) return -1;
+    u32 keep = 0xFFFFFFFFu >> (31 - ((t - 1) & 31));
+    for (int s = (t - 1) >> 5; s * TT_WORD + TT_WORD > p; s--, keep = 0xFFFFFFFFu) {
+        const u32 x = tt_win_word<K>(sm, s) & keep;
+        if (x) { const int at = s * TT_WORD + tt_hibit(x); return at >= p ? at : -1; }
+    }
+    return -1;
+}
+// U* Lw+ (lower) / U+ Lw* from q; returns the end, or q.  (Where a run ends at `end`, the caller looks whether that is real.)
+TT_HD int tt_win_body(MaskRows sm, bool lower, int q, int end) {
+    const int t = tt_win_find<WK_UP, false>(sm, q, end);
+    if (!lower) return t == q ? q : tt_win_find<WK_LW, false>(sm, t, end);
+    if (t < end && tt_win_is<WK_LW>(sm, t)) return tt_win_find<WK_LW, false>(sm, t, end);
+    const int last = tt_win_last<WK_LW>(sm, q, t);           // the stretch is given back up to its last caseless letter or mark
+    return last >= 0 ? last + 1 : q;
+}
+// One match at p < end; the end of the piece, or -1 where it looks at `end` and that is only the end of the window.
+TT_HD int tt_win_match_p1(MaskRows sm, const u8* wtx, int p, int end, bool exact) {
+#define AT(f, q) ((sm[f][(q) >> 5] >> ((q) & 31)) & 1u)
+    const int next = tt_win_find<WK_LEAD, true>(sm, p + 1, end);         // the character behind the first one
+    if (next >= end && !exact) return -1;
+    const bool letter = (AT(F_LOW, p) | AT(F_UPP, p) | AT(F_CLESS, p)) != 0, number = AT(F_NUM, p) != 0;
+    const bool prefix_ok = !AT(F_NL, p) && !letter && !number;
+    const bool word = letter || AT(F_MARK, p);
+    int e = -1;
+    for (int alt = 0; alt < 2 && e < 0; alt++) {
+        if (prefix_ok && next < end) { const int v = tt_win_body(sm, alt == 0, next, end); if (v > next) { e = v; break; } }
+        if (word) { const int v = tt_win_body(sm, alt == 0, p, end); if (v > p) e = v; }
+    }
+    if (e >= 0) {
+        if (e + 3 > end && !exact) return -1;
+        // (a body given back may end before a run that went to the end of the window)
+        if (!exact && tt_win_find<WK_UP, false>(sm, p, end) >= end) return -1;
+        if (!exact && next < end && tt_win_find<WK_UP, false>(sm, next, end) >= end) return -1;
+        if (e < end && AT(F_AP, e)) e += tt_contraction_len(e + 1 < end ? wtx[e + 1] : 0u, e + 2 < end ? wtx[e + 2] : 0u);
+        return e;
+    }
+    int t = p;
+    if (number) { for (int k = 0; k < 3 && t < end && AT(F_NUM, t); k++) t = tt_win_find<WK_LEAD, true>(sm, t + 1, end); }
+    else {
+        const int q = AT(F_SP, p) && p + 1 < end && tt_win_is<WK_PUNCT>(sm, p + 1) ? p + 1 : tt_win_is<WK_PUNCT>(sm, p) ? p : -1;
+        if (q >= 0) { t = tt_win_find<WK_PUNCT, false>(sm, q, end); t = tt_win_find<WK_TAIL, false>(sm, t, end); }
+        else {                                               // whitespace: \s*[\r\n]+ | \s+(?!\S) | \s+
+            t = tt_win_find<WK_SPACE, false>(sm, p, end);
+            if (t >= end && !exact) return -1;
+            const int nl = tt_win_last<WK_NL>(sm, p, t);
+            if (nl >= 0) return nl + 1;
+            if (t >= end) return t;
+            if (next < t) return tt_win_last<WK_LEAD>(sm, p, t);
+            return t > p ? t : next;
+        }
+    }
+    return t >= end && !exact ? -1 : t;
+#undef AT
+}
+// Piece starts in the word `slot` by matching from the piece start `from` (window positions), as tt_seq_starts_p1; hi: end of the text.
+// false: some match leaves the window.  doc_end is exact whenever it lies before the end of the word.
+TT_HD_COLD bool tt_win_starts_p1(MaskRows sm, const u8* wtx, int from, int slot, long long hi, u32& bits, int& doc_end) {
+    constexpr int WIN = TT_SLOTS * TT_WORD;
+    int end = hi < WIN ? (int)hi : WIN;
+    bool exact = hi <= WIN;
+    {   // the end of the document
+        u32 keep = (from & 31) == 31 ? 0u : 0xFFFFFFFEu << (from & 31);
+        for (int s = from >> 5; s * TT_WORD < end; s++, keep = 0xFFFFFFFFu) {
+            const u32 d = sm[F_DOC][s] & keep;
+            if (d) { const int at = s * TT_WORD + tt_lobit(d); if (at < end) { end = at; exact = true; } break; }
+        }
+    }
+    const int w0 = slot * TT_WORD, stop = w0 + TT_WORD < end ? w0 + TT_WORD : end;
+    bits = 0; doc_end = end;
+    for (int p = from; p < stop;) {
+        const int e = tt_win_match_p1(sm, wtx, p, end, exact);
+        if (e < 0) return false;
+        if (p >= w0) bits |= 1u << (p - w0);
+        p = e > p ? e : p + 1;
+    }
+    return true;
+}
+
 // A 64-bit window over the masks of field f: bits 0..15 = the last sixteen bytes of the word before, bits 16..47 = the
 // word in `slot`, bits 48..63 = the first sixteen bytes of the word after it.
 TT_HD u64 tt_win64(MaskRows sm, int f, int slot) {
@@ -540,7 +643,11 @@ TT_HD u32 tt_eval_word_p1(MaskRows sm, int slot, const u8* tx, const SeqCtx& C, 
         }
         if (from < 0) break;
         long long doc_end;
-        const u32 seq = tt_seq_starts_p1(C, from, g0, doc_end);
+        u32 seq;
+        const long long gs0 = g0 - (long long)slot * TT_WORD;         // byte 0 of slot 0
+        int wdoc;
+        if (from >= gs0 && tt_win_starts_p1(sm, tx - slot * TT_WORD, (int)(from - gs0), slot, C.hi - gs0, seq, wdoc)) doc_end = gs0 + wdoc;
+        else seq = tt_seq_starts_p1(C, from, g0, doc_end);
         const int fb = from > g0 ? (int)(from - g0) : 0;
         u32 take = 0xFFFFFFFFu << fb;
         if (doc_end - g0 < 32) take &= (1u << (int)(doc_end - g0)) - 1u;      // (doc_end > from, and from >= g0 or doc_end > g0 + first)
