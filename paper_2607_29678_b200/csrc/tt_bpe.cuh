@@ -1482,8 +1482,8 @@ __device__ __forceinline__ bool merge_index(const PieceParams& P, int unit, int 
     for (int o = 1; o < 32; o <<= 1) { const u64 t = __shfl_up_sync(0xFFFFFFFFu, x, o); if (lane >= o) x += t; }
     if (lane == 31) X.wtot[wid] = x;
     __syncthreads();
-    u64 before = x - mine;
-    for (int w = 0; w < wid; w++) before += X.wtot[w];
+    const u64 wt = lane < wid ? X.wtot[lane] : 0ull;             // (a warp's counts fit 32 bits each)
+    const u64 before = x - mine + __reduce_add_sync(0xFFFFFFFFu, (u32)wt) + ((u64)__reduce_add_sync(0xFFFFFFFFu, (u32)(wt >> 32)) << 32);
     if (4 * tid < entries) {
         u32 s = (u32)before, w = (u32)(before >> 32);
 #pragma unroll
@@ -1737,10 +1737,10 @@ k_scatter(const __grid_constant__ ScatterParams P) {
         u32 d0 = carry + inc - c[0] - c[1], tot = 0;
 #pragma unroll
         for (int w = 0; w < BPE_WARPS; w++) { const u32 y = s_scan[item & 1][w]; tot += y; if (w < wid) d0 += y; }
-        // An item without pieces of more than eight tokens (nearly all) is put together in shared memory and leaves in
-        // whole lines, every thread writing consecutive words: the output may be mapped host memory, where a warp that
-        // writes every other word costs a bus transaction per word.
-        const bool staged = !some_big && tot <= (u32)SCATTER_STAGE_IDS;
+        // An item of at most SCATTER_STAGE_IDS tokens (nearly all) is put together in shared memory and leaves in whole lines, every
+        // thread writing consecutive words: the output may be mapped host memory, where a warp that writes every other word
+        // costs a bus transaction per word (100 KB of Unicode-heavy text, written piece by piece: 27 us instead of 9).
+        const bool staged = tot <= (u32)SCATTER_STAGE_IDS;
         int32_t* const out = staged ? s_out - carry : P.ids_out;             // same index either way
 #pragma unroll
         for (int h = 0; h < 2; h++) {
@@ -1770,13 +1770,10 @@ k_scatter(const __grid_constant__ ScatterParams P) {
                 }
             }
         }
-        if (staged) {                                             // block-uniform
-            __syncthreads();
-            for (u32 kk = tid; kk < tot; kk += BPE_THREADS) P.ids_out[carry + kk] = s_out[kk];
-        } else if (some_big) {                                    // block-uniform: pieces of more than 8 tokens
+        if (staged || some_big) __syncthreads();                  // (both block-uniform)
+        if (some_big) {                                           // pieces of more than 8 tokens
             // a warp each, four loads in flight per lane (one after the other by the whole CTA they took 45 us where most pieces
             // of 3 MB of text have 50 to 100 tokens); the few very long ones by the whole CTA
-            __syncthreads();
             const u32 nbig = min(s_nbig, (u32)(TT_TILE_BYTES / 8));
             for (u32 e = 0; e < nbig; e++) {
                 const u32 cc = s_big[e][2];
@@ -1788,12 +1785,13 @@ k_scatter(const __grid_constant__ ScatterParams P) {
 #pragma unroll
                     for (int u = 0; u < 4; u++) id[u] = k0 + u * step < cc ? P.stage[src + k0 + u * step] : 0;
 #pragma unroll
-                    for (int u = 0; u < 4; u++) if (k0 + u * step < cc) P.ids_out[d2 + k0 + u * step] = id[u];
+                    for (int u = 0; u < 4; u++) if (k0 + u * step < cc) out[d2 + k0 + u * step] = id[u];
                 }
             }
             __syncthreads();
             if (tid == 0) s_nbig = 0;                             // (the next item's barrier comes before anyone adds)
         }
+        if (staged) for (u32 kk = tid; kk < tot; kk += BPE_THREADS) P.ids_out[carry + kk] = s_out[kk];
         carry += tot;
         if (tile2 >= tile_hi) break;
         tile = tile2; b = b2; np = np2; v = vn; o2 = on;
