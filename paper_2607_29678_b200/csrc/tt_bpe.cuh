@@ -128,6 +128,11 @@ TT_HD u32 toktab_bucket_alt(u32 h, u32 shift) {                   // the key's o
 }
 TT_HD u32 toktab_mask_word(u32 w, u32 n, u32 j) {      // key word j of a piece of n bytes: bytes beyond the piece are zero
     const u32 have = n > 4 * j ? n - 4 * j : 0u;
+#if defined(__CUDA_ARCH__)
+    u32 m;
+    asm("bmsk.clamp.b32 %0, 0, %1;" : "=r"(m) : "r"(8 * have));       // the low 8 * have bits, at most all 32
+    return w & m;
+#endif
     return have >= 4 ? w : have == 0 ? 0u : w & ((1u << (8 * have)) - 1u);
 }
 
@@ -1346,32 +1351,31 @@ __device__ __noinline__ u32 cta_find_long(const PieceParams& P, const u8* __rest
     return 2;
 }
 
-// Bulk text: the last CTA of k_merge to finish sums the token counts of every group of 256 tiles for k_scatter (a
-// counter cleared before the chain tells which CTA that is; nobody waits for anybody).  Called by every warp.
-__device__ __forceinline__ void merge_group_totals(const PieceParams& P, u32* s_warps_done) {
-    const int lane = threadIdx.x & 31;
+// Bulk text: the last CTA of k_merge_bulk to finish sums the token counts of every group of 256 tiles for k_scatter_bulk (a
+// counter cleared before the chain tells which CTA that is; nobody waits for anybody), a warp a group.  (One warp for all the
+// groups took 100 us behind the merges of a 132 MB batch.)
+__device__ __forceinline__ void merge_group_totals(const PieceParams& P, u32* s_last) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const u32 FULL = 0xFFFFFFFFu;
-    if (P.grp_tok == nullptr) return;
     __threadfence();
-    __syncwarp();
-    u32 fin = 0;
-    if (lane == 0 && atomicAdd(s_warps_done, 1u) == MERGE_WARPS - 1) fin = atomicAdd(&P.hdr->merge_done, 1u) == gridDim.x - 1;
-    if (!__shfl_sync(FULL, fin, 0)) return;
+    __syncthreads();
+    if (threadIdx.x == 0) *s_last = atomicAdd(&P.hdr->merge_done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!*s_last) return;
     __threadfence();
     const int ngroups = (P.ntiles + TT_GROUP_TILES - 1) / TT_GROUP_TILES;
-    for (int g = 0; g < ngroups; g++) {                               // one warp: eight loads per lane and group
+    for (int g = wid; g < ngroups; g += MERGE_WARPS) {                // eight loads per lane and group
         u32 sum = 0;
 #pragma unroll
         for (int u = 0; u < TT_GROUP_TILES / 32; u++) { const int t = g * TT_GROUP_TILES + u * 32 + lane; if (t < P.ntiles) sum += __ldcg(&P.tile_tok[t]); }
-#pragma unroll
-        for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(FULL, sum, o);
+        sum = __reduce_add_sync(FULL, sum);
         if (lane == 0) P.grp_tok[g] = sum;
     }
 }
 
 // Bulk text (k_closing has gathered the lists): long pieces a CTA each where that is quick, else window by window with the
 // whole grid, warp-class pieces a warp each by index, short pieces 32 of one length class at a time by ticket, a thread each.
-__device__ void merge_bulk_lists(const PieceParams& P, const u8* __restrict__ text, u64* s_buf, u32* sc, LongShared& LS, u32* s_warps_done) {
+__device__ void merge_bulk_lists(const PieceParams& P, const u8* __restrict__ text, u64* s_buf, u32* sc, LongShared& LS, u32* s_last) {
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const u32 FULL = 0xFFFFFFFFu;
     const u32 nl = P.hdr->nq_long, nw = P.hdr->nwq, ns = P.hdr->nq_short;
@@ -1427,7 +1431,7 @@ __device__ void merge_bulk_lists(const PieceParams& P, const u8* __restrict__ te
         __syncwarp();
     }
     if (nl) long_phase(P, text, nl, s_buf, sc, LS);
-    merge_group_totals(P, s_warps_done);
+    merge_group_totals(P, s_last);
 }
 
 // The merge kernel of bulk text (more tiles than a request's job search covers): works off the lists k_closing built.
@@ -1435,16 +1439,14 @@ __global__ void __launch_bounds__(MERGE_THREADS, MERGE_CTAS_PER_SM)
 k_merge_bulk(const __grid_constant__ PieceParams P) {
     extern __shared__ __align__(16) u64 s_buf[];              // MERGE_SMEM_BYTES
     __shared__ u32 sc[SCR_WORDS];
-    __shared__ u32 s_warps_done;
+    __shared__ u32 s_last;
     __shared__ LongShared LS;
     cudaTriggerProgrammaticLaunchCompletion();               // k_scatter may be placed; it waits for this grid's memory itself
     grid_prefetch_l2(P.tab.slots, ((size_t)P.tab.mask + 1) * 2 * sizeof(uint4));
     grid_prefetch_l2(P.tab.bytepair, 65536 * sizeof(u64));
-    if (threadIdx.x == 0) s_warps_done = 0;
     cudaGridDependencySynchronize();                         // k_closing's lists are complete from here on
-    __syncthreads();
     if (hdr_status(P.hdr, P.epoch) != 0) return;
-    merge_bulk_lists(P, P.base + P.shift, s_buf, sc, LS, &s_warps_done);
+    merge_bulk_lists(P, P.base + P.shift, s_buf, sc, LS, &s_last);
 }
 
 // Where a request's unsettled pieces stand, for the job search of k_merge: exclusive prefixes of the tiles' counts of short
