@@ -700,7 +700,7 @@ static int encode_impl(const tt_vocab* v, const uint8_t* text, size_t len, const
     S.docmask = doc_off ? w.docmask : nullptr; S.doc_off = (const long long*)doc_off; S.n_docs = (int)n_docs;
     S.ids_off_out = (long long*)ids_off_out;
     const bool many = PP.ntiles > v->sm_count * SCATTER_CTAS;
-    const int scatter_ctas = v->sm_count * 8;
+    const int scatter_ctas = v->sm_count * (big ? SCATTER_BULK_CTAS : 8);
     CK(launch_after(big ? k_scatter_bulk : many ? k_scatter<SCATTER_CTAS_MANY> : k_scatter<SCATTER_CTAS>, PP.ntiles < scatter_ctas ? PP.ntiles : scatter_ctas,
                     BPE_THREADS, st, 0, ev == nullptr, S));
     MARK(3);

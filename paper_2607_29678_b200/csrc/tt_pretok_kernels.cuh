@@ -327,10 +327,11 @@ __device__ __forceinline__ void front_piece_queue(const FrontParams& F, int tile
 // NT = threads per CTA, MINB = CTAs per SM the kernel is compiled for.  A request (at most a few tiles per CTA) is a latency
 // chain: 128 threads, so that classification (72 words with the halo) is one step and the look-ups are short, and
 // four table look-ups in flight per thread.  Bulk text is bound by instruction issue: 64 threads, as many as a tile has
-// words, so that no warp waits idle for the predicate, and one look-up at a time per thread.
+// words, so that no warp waits idle for the predicate, and one look-up at a time per thread; 20 CTAs per SM leave 48 registers
+// (24 with 40: 20 MB of Unicode-heavy text 500 -> 477 us per call, the 132 MB batch 921 -> 905; 16 and 18 are slower for it).
 // PAT = the pattern the kernel is compiled for (P.pattern says the same): each pattern's rules are a lot of code, and a
 // kernel that carries all of them keeps missing the instruction caches on its way through the one it runs.
-constexpr int PRETOK_THREADS_REQUEST = 128, PRETOK_CTAS_REQUEST = 6, PRETOK_THREADS_BULK = 64, PRETOK_CTAS_BULK = 24;
+constexpr int PRETOK_THREADS_REQUEST = 128, PRETOK_CTAS_REQUEST = 6, PRETOK_THREADS_BULK = 64, PRETOK_CTAS_BULK = 20;
 template <int PAT> struct PretokSmem {
     static constexpr int ROWS = PAT == 1 ? F_COUNT : F_P0_COUNT;
     // the piece offsets take the place of the masks once the predicate has been evaluated
