@@ -848,7 +848,7 @@ __device__ __forceinline__ void warp_merge_piece(const PieceParams& P, const u8*
 // per warp), so that k_merge's warps take 32 short pieces at a time whatever tile they come from; warp-class
 // closing pieces join the first kernel's list, long pieces get a list of their own.  The counters were cleared
 // by the memset in front of the chain.
-constexpr int CLOSING_THREADS = 256;
+constexpr int CLOSING_THREADS = 64;
 // Length class of a short piece (2..32 bytes).
 __device__ __forceinline__ int short_class(u32 n) {
     return n <= (u32)tt_short_class_max(0) ? 0 : n <= (u32)tt_short_class_max(1) ? 1 : n <= (u32)tt_short_class_max(2) ? 2 : 3;
@@ -868,6 +868,12 @@ k_closing(const __grid_constant__ PieceParams P) {
         const u32 q = P.tile_q[t];
         ns = q & TQ_NS_MASK; nl = (q >> TQ_NL_SHIFT) & TQ_NL_MASK; np = P.tile_cnt[t];
     }
+    // the tile's first queue entries, on their way while the closing piece is looked up (one at a time in the two loops below, the
+    // kernel took 19 us whatever the text's length)
+    constexpr u32 AHEAD = 8;
+    u32 ahead[AHEAD];
+#pragma unroll
+    for (u32 e = 0; e < AHEAD; e++) ahead[e] = e < ns ? P.q[(size_t)t * TT_TILE_QCAP + e] : 0u;
     u32 cn = 0, ca = 0, cslot = 0, clast = 0;
     if (np) {
         clast = P.tile_last[t];
@@ -893,7 +899,9 @@ k_closing(const __grid_constant__ PieceParams P) {
     // short pieces: three lists by length (a warp later merges 32 pieces of one list at a time, a thread each, and
     // waits for the longest), one reservation per warp and list
     u64 mine = 0;                                             // four counts of 16 bits (a warp's 32 tiles hold fewer than 2^16 pieces)
-    for (u32 e = 0; e < ns; e++) mine += 1ull << (16 * short_class((P.q[(size_t)t * TT_TILE_QCAP + e] >> 22) + 1));
+#pragma unroll
+    for (u32 e = 0; e < AHEAD; e++) if (e < ns) mine += 1ull << (16 * short_class((ahead[e] >> 22) + 1));
+    for (u32 e = AHEAD; e < ns; e++) mine += 1ull << (16 * short_class((P.q[(size_t)t * TT_TILE_QCAP + e] >> 22) + 1));
     if (centry) mine += 1ull << (16 * short_class(cn));
     u64 pre = mine;
 #pragma unroll
@@ -909,16 +917,18 @@ k_closing(const __grid_constant__ PieceParams P) {
     pre -= mine;
 #pragma unroll
     for (int c = 0; c < TT_SHORT_CLASSES; c++) base[c] = __shfl_sync(FULL, base[c], 31) + ((u32)(pre >> (16 * c)) & 0xFFFFu);
-    for (u32 e = 0; e <= ns; e++) {
-        if (e == ns && !centry) break;
-        const u32 entry = e < ns ? P.q[(size_t)t * TT_TILE_QCAP + e] : centry;
+    const auto list = [&](u32 entry) {
         const int c = short_class((entry >> 22) + 1);
         const u64 x = ((u64)(u32)t << 32) | entry;
         if (c == 0) P.gq[base[0]++] = x;
         else if (c == 1) P.gq_x[0][base[1]++] = x;
         else if (c == 2) P.gq_x[1][base[2]++] = x;
         else P.gq_x[2][base[3]++] = x;
-    }
+    };
+#pragma unroll
+    for (u32 e = 0; e < AHEAD; e++) if (e < ns) list(ahead[e]);
+    for (u32 e = AHEAD; e < ns; e++) list(P.q[(size_t)t * TT_TILE_QCAP + e]);
+    if (centry) list(centry);
 }
 
 // ---- long pieces --------------------------------------------------------------------------------------------------
