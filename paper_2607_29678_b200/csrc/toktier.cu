@@ -31,13 +31,13 @@
 // tt_vocab_free): fifteen cudaMalloc and cudaFree calls per session took 2 to 15 ms, more than the 17 tokenizations of
 // a conversation.  Sessions share ownership, so that one that outlives its vocabulary still frees what it holds.
 struct SessionHost;
-struct SessionArena { char* dev = nullptr; size_t bytes = 0; int device = 0; SessionHost* host = nullptr; size_t host_text = 0; };
+struct SessionArena { char* dev = nullptr; size_t bytes = 0; int device = 0; SessionHost* host = nullptr; size_t host_text = 0; cudaEvent_t copied = nullptr; };
 struct SessionPool {
     static constexpr size_t POOL_ARENAS = 8, POOL_BYTES = (size_t)512 << 20;
     std::mutex mu;
     std::vector<SessionArena> kept;
     bool closed = false;
-    static void destroy(SessionArena& a) { cudaFree(a.dev); if (a.host) cudaFreeHost(a.host); a = SessionArena{}; }
+    static void destroy(SessionArena& a) { cudaFree(a.dev); if (a.host) cudaFreeHost(a.host); if (a.copied) cudaEventDestroy(a.copied); a = SessionArena{}; }
     bool get(size_t bytes, size_t host_text, SessionArena& out);
     void put(SessionArena a);
     void close() {
@@ -1023,7 +1023,8 @@ bool SessionPool::get(size_t bytes, size_t host_text, SessionArena& out) {
     }
     out.bytes = bytes; out.device = device; out.host_text = host_text;
     if (cudaMalloc(&out.dev, bytes) != cudaSuccess) { cudaGetLastError(); out.dev = nullptr; return false; }
-    if (cudaMallocHost(&out.host, sizeof(SessionHost) + host_text) != cudaSuccess) { cudaGetLastError(); cudaFree(out.dev); out = SessionArena{}; return false; }
+    if (cudaMallocHost(&out.host, sizeof(SessionHost) + host_text) != cudaSuccess) { cudaGetLastError(); out.host = nullptr; destroy(out); return false; }
+    if (cudaEventCreateWithFlags(&out.copied, cudaEventDisableTiming) != cudaSuccess) { cudaGetLastError(); out.copied = nullptr; destroy(out); return false; }
     return true;
 }
 void SessionPool::put(SessionArena a) {
@@ -1055,21 +1056,22 @@ struct tt_session {
     size_t h_stage_cap = 0;
     bool records = false;                                               // the device's records are set (an empty session's: not yet)
     size_t ntok = 0;
+    bool shared = false;                                                // somebody else may be reading the device memory: see tt_session_free
+    bool copied = false;                                                // arena.copied marks the end of the copies so far
     void *d_ws = nullptr, *d_sws = nullptr;
     size_t ws_bytes = 0, sws_bytes = 0;
 };
 
 extern "C" void tt_session_free(tt_session* s) {
     if (!s) return;
+    // The memory is handed on to the next session only when nothing reads it any more.  An append waits for its stream, and copies are
+    // marked by an event; where the caller was given pointers (tt_session_view), or captured a copy into a graph, readers are
+    // not known, and the memory is returned to the driver, which waits for them.  (Waiting for the device instead would break
+    // a stream capture that another thread has under way.)
     if (s->arena.dev) {
-        // copies out of the session, or kernels of the caller that read its view, may still be running on some stream; the
-        // memory is handed on only when they are through (as cudaFree would wait for them)
-        int dev = s->arena.device;
-        cudaGetDevice(&dev);
-        if (dev != s->arena.device) cudaSetDevice(s->arena.device);
-        if (cudaDeviceSynchronize() == cudaSuccess) s->pool->put(s->arena);
-        else { cudaGetLastError(); SessionPool::destroy(s->arena); cudaGetLastError(); }
-        if (dev != s->arena.device) cudaSetDevice(dev);
+        if (!s->shared && s->copied && cudaEventSynchronize(s->arena.copied) != cudaSuccess) { cudaGetLastError(); s->shared = true; }
+        if (!s->shared) s->pool->put(s->arena);
+        else SessionPool::destroy(s->arena);
     }
     delete s;
 }
@@ -1126,7 +1128,7 @@ extern "C" size_t tt_session_tokens(const tt_session* s) { return s ? s->ntok : 
 extern "C" int tt_session_view(const tt_session* s, const int32_t** ids_dev, const int32_t** off_dev,
                                const int64_t** count_dev, size_t* len_bytes) {
     if (!s) return TT_ERR_ARG;
-    if (ids_dev || off_dev || count_dev) { const int rc = session_empty_records(const_cast<tt_session*>(s)); if (rc != TT_OK) return rc; }
+    if (ids_dev || off_dev || count_dev) { const int rc = session_empty_records(const_cast<tt_session*>(s)); if (rc != TT_OK) return rc; const_cast<tt_session*>(s)->shared = true; }
     if (ids_dev) *ids_dev = s->d_ids;
     if (off_dev) *off_dev = s->d_off;
     if (count_dev) *count_dev = (const int64_t*)&s->d_sc->ntok;
@@ -1263,10 +1265,19 @@ extern "C" int tt_session_copy(const tt_session* s, int32_t* ids_out, size_t ids
                                int64_t* count_out, void* stream) {
     if (!s || !count_out) return TT_ERR_ARG;
     cudaStream_t st = (cudaStream_t)stream;
+    tt_session* const own = const_cast<tt_session*>(s);      // (only what tt_session_free has to know is written)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) { cudaGetLastError(); cap = cudaStreamCaptureStatusActive; }
+    const bool captured = cap != cudaStreamCaptureStatusNone;
+    if (captured) own->shared = true;                        // (the graph can be launched at any time)
+    else if (s->copied) CK(cudaStreamWaitEvent(st, s->arena.copied, 0));     // so that one event stands for all copies
     { const int rc = session_empty_records(const_cast<tt_session*>(s)); if (rc != TT_OK) return rc; }
     const size_t n = s->ntok < ids_cap ? s->ntok : ids_cap, want = (n + 1 + 1023) / 1024, most = (size_t)s->v->sm_count * 4;
     CK(launch_after(k_session_copy, (int)(want < most ? want : most), 256, st, 0, true, (const int32_t*)s->d_ids, (const int32_t*)s->d_off,
                     (const long long*)&s->d_sc->ntok, (long long)n, (long long)n + 1, ids_out, off_out, (long long*)count_out));
+    if (captured) return TT_OK;
+    if (cudaEventRecord(s->arena.copied, st) == cudaSuccess) own->copied = true;
+    else { cudaGetLastError(); own->shared = true; }
     return TT_OK;
 }
 

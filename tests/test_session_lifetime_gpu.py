@@ -1,0 +1,81 @@
+"""Sessions beside other work on the device: what their creation, copies and end do to other streams, captures and memory."""
+import ctypes
+import threading
+
+import numpy as np
+import pytest
+
+import workloads as wl
+from gpu_util import cpu_vocab, gpu_vocab, same
+
+pytestmark = pytest.mark.gpu
+
+
+def _during_a_capture_of_another_thread(action):
+    """Runs action() while a capture (thread-local mode) is under way here; the graph has to come out whole."""
+    import torch
+    x = torch.zeros(1024, device="cuda")
+    torch.cuda.synchronize()
+    go, done, errors = threading.Event(), threading.Event(), []
+
+    def other():
+        go.wait()
+        try:
+            action()
+        except Exception as e:
+            errors.append(e)
+        done.set()
+
+    t = threading.Thread(target=other)
+    t.start()
+    graph = torch.cuda.CUDAGraph()
+    try:
+        with torch.cuda.graph(graph, stream=torch.cuda.Stream(), capture_error_mode="thread_local"):
+            x.add_(1)
+            go.set()
+            done.wait(60)
+            x.add_(1)
+    finally:
+        go.set()
+        t.join()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert not errors and bool((x == 2).all())
+
+
+@pytest.mark.parametrize("copied", [False, True])
+def test_the_end_of_a_session_leaves_other_captures_alone(copied):
+    import paper_2607_29678_b200 as tt
+    sess = tt.Session(gpu_vocab("C1"), 50_000)
+    sess.append(wl.generate(0, 1, 5_000))
+    if copied:
+        sess.records()
+    _during_a_capture_of_another_thread(sess.close)
+
+
+def test_a_copy_on_its_way_survives_the_session():
+    """The memory of a freed session goes to the next one, but not before the copies out of it are through."""
+    import torch
+    import paper_2607_29678_b200 as tt
+    gv, cv = gpu_vocab("C1"), cpu_vocab("C1")
+    text = wl.generate(0, 2, 20_000)
+    want = cv.encode(text, 0)[0]
+    sess = tt.Session(gv, 30_000)
+    sess.append(text)
+    outs = []
+    for stream in (torch.cuda.Stream(), torch.cuda.Stream()):
+        ids = torch.zeros(want.size, dtype=torch.int32, device="cuda")
+        off = torch.zeros(want.size + 1, dtype=torch.int32, device="cuda")
+        count = torch.zeros(1, dtype=torch.int64, device="cuda")
+        torch.cuda.current_stream().synchronize()
+        with torch.cuda.stream(stream):
+            torch.cuda._sleep(40_000_000)
+            tt._check(tt.lib().tt_session_copy(sess._h, ids.data_ptr(), want.size, off.data_ptr(), count.data_ptr(), stream.cuda_stream), "tt_session_copy")
+        outs.append((ids, off, count))
+    sess.close()
+    other = tt.Session(gv, 30_000)
+    other.append(wl.generate(1, 3, 25_000))
+    torch.cuda.synchronize()
+    for ids, off, count in outs:
+        assert int(count) == want.size and same(ids.cpu().numpy(), want) and same(off.cpu().numpy(), cv.spans(text, want)[0])
+    other.close()
