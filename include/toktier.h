@@ -218,6 +218,8 @@ int tt_encode_added(const tt_vocab* v, const uint8_t* text, size_t len, void* st
  *                       ids_out int32[ids_cap] (may be NULL), off_out int32[ids_cap + 1] (may be NULL), count_out
  *                       int64.  min(tokens, ids_cap) ids are copied, and one offset more; entries beyond are left
  *                       as they are.
+ *   tt_session_free     waits for the copies under way; where tt_session_view gave out device pointers, or a copy was
+ *                       captured into a graph, it returns the memory with cudaFree, which waits for the device.
  * One session must not be used from two threads at once.
  */
 typedef struct tt_session tt_session;

@@ -2,8 +2,8 @@
 // tables, workspace layout and the kernel chain  k_pretok<fused> (K1+K2, K3 per tile in shared memory, whole-piece
 // lookups) -> k_merge (K4's merges, from the per-tile queues) -> k_scatter (K5); sessions
 // (incremental repair), the added-token literal pass and the shadow verifier (host only) sit on top of it.
-// Nothing here synchronises with the device except tt_vocab_load, tt_encode_host, tt_encode_timed and
-// tt_session_append.
+// Nothing here synchronises with the device except tt_vocab_load, tt_vocab_add_literals, tt_encode_host, tt_encode_timed,
+// tt_session_append and tt_session_free (for the copies out of its session).
 #include "../../include/toktier.h"
 #include "tt_common.cuh"
 #include "tt_pretok_kernels.cuh"
@@ -70,6 +70,7 @@ struct tt_vocab {
     size_t n_table_tokens = 0;
     uint2* d_meta = nullptr;             // per caller id: (byte length, non-continuation bytes) for tt_spans
     u32 meta_n = 0;
+    u8* d_zero = nullptr;                // 16 zero bytes: the records of a session without text
     LitEntry* d_lit_entries = nullptr; u8* d_lit_blob = nullptr;
     LitTable lit{};                      // added-token literals (tt_vocab_add_literals), n == 0: none
     u32 max_token_chars = 1;             // characters of the longest entry (stable boundary check of the sessions)
@@ -115,7 +116,7 @@ extern "C" size_t tt_class_table(uint8_t* out, size_t cap) {
 extern "C" void tt_vocab_free(tt_vocab* v) {
     if (!v) return;
     v->sessions->close();
-    cudaFree(v->d_slots); cudaFree(v->d_bytepair); cudaFree(v->d_ext_id); cudaFree(v->d_tok_len); cudaFree(v->d_cls); cudaFree(v->d_lit_entries); cudaFree(v->d_lit_blob); cudaFree(v->d_toktab); cudaFree(v->d_longslots); cudaFree(v->d_longblob); cudaFree(v->d_meta);
+    cudaFree(v->d_slots); cudaFree(v->d_bytepair); cudaFree(v->d_ext_id); cudaFree(v->d_tok_len); cudaFree(v->d_cls); cudaFree(v->d_lit_entries); cudaFree(v->d_lit_blob); cudaFree(v->d_toktab); cudaFree(v->d_longslots); cudaFree(v->d_longblob); cudaFree(v->d_meta); cudaFree(v->d_zero);
     cudaFree(v->d_text); cudaFree(v->d_ids); cudaFree(v->d_count); cudaFree(v->d_status); cudaFree(v->d_ws);
     if (v->h_text) cudaFreeHost(v->h_text);
     if (v->h_ids) cudaFreeHost(v->h_ids);
@@ -493,6 +494,7 @@ extern "C" int tt_vocab_load_ex(const tt_merge* merges, size_t n_merges, const i
             v->meta_n = (u32)meta.size();
         }
     }
+    if (cudaMalloc(&v->d_zero, 16) != cudaSuccess || cudaMemset(v->d_zero, 0, 16) != cudaSuccess || cudaStreamSynchronize(nullptr) != cudaSuccess) { cudaGetLastError(); tt_vocab_free(v); return TT_ERR_CUDA; }
     *out = v;
     return TT_OK;
 }
@@ -1054,7 +1056,6 @@ struct tt_session {
     SessionScalars* h = nullptr;                                        // pinned
     u8* h_stage = nullptr;                                              // pinned, h_stage_cap bytes
     size_t h_stage_cap = 0;
-    bool records = false;                                               // the device's records are set (an empty session's: not yet)
     size_t ntok = 0;
     bool shared = false;                                                // somebody else may be reading the device memory: see tt_session_free
     bool copied = false;                                                // arena.copied marks the end of the copies so far
@@ -1112,26 +1113,20 @@ extern "C" int tt_session_set_window(tt_session* s, uint32_t window_chars) {
     return TT_OK;
 }
 
-// The records of a session without text: count 0, off[0] = 0, written when somebody looks for the first time.  (Waited for: the
-// session may be used from any stream.)
-static int session_empty_records(tt_session* s) {
-    if (s->records) return TT_OK;
-    CK(cudaMemset(s->d_sc, 0, sizeof(SessionScalars)));
-    CK(cudaMemset(s->d_off, 0, 4));
-    CK(cudaStreamSynchronize(nullptr));
-    s->records = true;
-    return TT_OK;
-}
+// The records of a session without text -- count 0, off[0] = 0 -- are zeros that the vocabulary holds: nothing has to be written
+// for them, on no stream.
+static const int32_t* session_off(const tt_session* s) { return s->len ? s->d_off : (const int32_t*)s->v->d_zero; }
+static const long long* session_count(const tt_session* s) { return s->len ? &s->d_sc->ntok : (const long long*)s->v->d_zero; }
 
 extern "C" size_t tt_session_tokens(const tt_session* s) { return s ? s->ntok : 0; }
 
 extern "C" int tt_session_view(const tt_session* s, const int32_t** ids_dev, const int32_t** off_dev,
                                const int64_t** count_dev, size_t* len_bytes) {
     if (!s) return TT_ERR_ARG;
-    if (ids_dev || off_dev || count_dev) { const int rc = session_empty_records(const_cast<tt_session*>(s)); if (rc != TT_OK) return rc; const_cast<tt_session*>(s)->shared = true; }
+    if (ids_dev || off_dev || count_dev) const_cast<tt_session*>(s)->shared = true;
     if (ids_dev) *ids_dev = s->d_ids;
-    if (off_dev) *off_dev = s->d_off;
-    if (count_dev) *count_dev = (const int64_t*)&s->d_sc->ntok;
+    if (off_dev) *off_dev = session_off(s);
+    if (count_dev) *count_dev = (const int64_t*)session_count(s);
     if (len_bytes) *len_bytes = s->len;
     return TT_OK;
 }
@@ -1242,7 +1237,6 @@ extern "C" int tt_session_append(tt_session* s, const uint8_t* text, size_t len,
     long long* const count = direct ? &s->d_sc->ntok : &s->d_sc->fcount;
     const u8* src;
     if (!stage(0, src)) return fail(TT_ERR_CUDA);
-    if (direct) s->records = false;                          // (an error leaves them to be written again)
     int rc = session_tokenize(s, 0, new_len, st, direct ? s->d_ids : s->d_fids, direct ? s->d_off : s->d_foff, count, src);
     if (rc != TT_OK) return fail(rc);
     if (cudaMemcpyAsync(s->h, s->d_sc, sizeof(SessionScalars), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
@@ -1254,7 +1248,7 @@ extern "C" int tt_session_append(tt_session* s, const uint8_t* text, size_t len,
         cudaMemcpyAsync(s->d_off, s->d_foff, (nt + 1) * 4, cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
         cudaMemcpyAsync(&s->d_sc->ntok, &s->d_sc->fcount, 8, cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)) { cudaGetLastError(); return fail(TT_ERR_CUDA); }
-    s->len = new_len; s->ntok = nt; s->records = true; session_keep_tail(s, text, len);
+    s->len = new_len; s->ntok = nt; session_keep_tail(s, text, len);
     local.window_chars = 0; local.window_start = 0; local.run_tokens = 0; local.splice_byte = 0;
     local.n_tokens = (int64_t)nt; local.status = TT_OK;
     if (info) *info = local;
@@ -1271,10 +1265,9 @@ extern "C" int tt_session_copy(const tt_session* s, int32_t* ids_out, size_t ids
     const bool captured = cap != cudaStreamCaptureStatusNone;
     if (captured) own->shared = true;                        // (the graph can be launched at any time)
     else if (s->copied) CK(cudaStreamWaitEvent(st, s->arena.copied, 0));     // so that one event stands for all copies
-    { const int rc = session_empty_records(const_cast<tt_session*>(s)); if (rc != TT_OK) return rc; }
     const size_t n = s->ntok < ids_cap ? s->ntok : ids_cap, want = (n + 1 + 1023) / 1024, most = (size_t)s->v->sm_count * 4;
-    CK(launch_after(k_session_copy, (int)(want < most ? want : most), 256, st, 0, true, (const int32_t*)s->d_ids, (const int32_t*)s->d_off,
-                    (const long long*)&s->d_sc->ntok, (long long)n, (long long)n + 1, ids_out, off_out, (long long*)count_out));
+    CK(launch_after(k_session_copy, (int)(want < most ? want : most), 256, st, 0, true, (const int32_t*)s->d_ids, session_off(s), session_count(s),
+                    (long long)n, (long long)n + 1, ids_out, off_out, (long long*)count_out));
     if (captured) return TT_OK;
     if (cudaEventRecord(s->arena.copied, st) == cudaSuccess) own->copied = true;
     else { cudaGetLastError(); own->shared = true; }

@@ -79,3 +79,35 @@ def test_a_copy_on_its_way_survives_the_session():
     for ids, off, count in outs:
         assert int(count) == want.size and same(ids.cpu().numpy(), want) and same(off.cpu().numpy(), cv.spans(text, want)[0])
     other.close()
+
+
+def test_the_view_of_an_empty_session_leaves_other_captures_alone():
+    import paper_2607_29678_b200 as tt
+    sess = tt.Session(gpu_vocab("C1"), 50_000)
+    pointers = [ctypes.c_void_p() for _ in range(3)]
+    size = ctypes.c_size_t(7)
+    _during_a_capture_of_another_thread(lambda: tt._check(tt.lib().tt_session_view(sess._h, *map(ctypes.byref, pointers), ctypes.byref(size)), "tt_session_view"))
+    assert size.value == 0 and all(p.value for p in pointers)
+    sess.close()
+
+
+@pytest.mark.parametrize("failed", [False, True])
+def test_a_copy_of_an_empty_session_can_be_captured(failed):
+    """Also after an append that failed and left the session empty."""
+    import torch
+    import paper_2607_29678_b200 as tt
+    sess = tt.Session(gpu_vocab("C1"), 50_000)
+    if failed:
+        with pytest.raises(tt.TokTierError):
+            sess.append(np.frombuffer(b"abc \xff def", dtype=np.uint8))
+    off = torch.full((4,), 7, dtype=torch.int32, device="cuda")
+    count = torch.full((1,), 7, dtype=torch.int64, device="cuda")
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, capture_error_mode="thread_local"):
+        tt._check(tt.lib().tt_session_copy(sess._h, None, 3, off.data_ptr(), count.data_ptr(), torch.cuda.current_stream().cuda_stream), "tt_session_copy")
+    graph.replay()
+    torch.cuda.synchronize()
+    assert int(count) == 0 and off.tolist() == [0, 7, 7, 7]
+    ids, offsets, size = sess.records()
+    assert ids.numel() == 0 and offsets.tolist() == [0] and size == 0
+    sess.close()
