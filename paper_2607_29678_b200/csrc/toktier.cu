@@ -1265,9 +1265,9 @@ extern "C" int tt_session_copy(const tt_session* s, int32_t* ids_out, size_t ids
     const bool captured = cap != cudaStreamCaptureStatusNone;
     if (captured) own->shared = true;                        // (the graph can be launched at any time)
     else if (s->copied) CK(cudaStreamWaitEvent(st, s->arena.copied, 0));     // so that one event stands for all copies
-    const size_t n = s->ntok < ids_cap ? s->ntok : ids_cap, want = (n + 1 + 1023) / 1024, most = (size_t)s->v->sm_count * 4;
+    const size_t cap_ids = ids_cap < (size_t)INT32_MAX ? ids_cap : (size_t)INT32_MAX, n = s->ntok < cap_ids ? s->ntok : cap_ids, want = (n + 1 + 1023) / 1024, most = (size_t)s->v->sm_count * 4;
     CK(launch_after(k_session_copy, (int)(want < most ? want : most), 256, st, 0, true, (const int32_t*)s->d_ids, session_off(s), session_count(s),
-                    (long long)n, (long long)n + 1, ids_out, off_out, (long long*)count_out));
+                    (long long)cap_ids, ids_out, off_out, (long long*)count_out));
     if (captured) return TT_OK;
     if (cudaEventRecord(s->arena.copied, st) == cudaSuccess) own->copied = true;
     else { cudaGetLastError(); own->shared = true; }

@@ -253,13 +253,15 @@ k_repair(const __grid_constant__ RepairFused P) {
     }
 }
 
-// ids, offsets and count of a session into the caller's buffers.
+// ids, offsets and count of a session into the caller's buffers: as many as the session has when the kernel runs (a captured copy
+// may be replayed after more appends), at most ids_cap and one offset more.
 __global__ void __launch_bounds__(256)
-k_session_copy(const int32_t* __restrict__ ids, const int32_t* __restrict__ off, const long long* __restrict__ ntok, long long n_ids, long long n_off,
+k_session_copy(const int32_t* __restrict__ ids, const int32_t* __restrict__ off, const long long* __restrict__ ntok, long long ids_cap,
                int32_t* ids_out, int32_t* off_out, long long* count_out) {
     cudaGridDependencySynchronize();
     const long long first = (long long)blockIdx.x * blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
-    if (ids_out) for (long long i = first; i < n_ids; i += step) ids_out[i] = ids[i];
-    if (off_out) for (long long i = first; i < n_off; i += step) off_out[i] = off[i];
-    if (first == 0) *count_out = *ntok;
+    const long long count = *ntok, n = min(count, ids_cap);
+    if (ids_out) for (long long i = first; i < n; i += step) ids_out[i] = ids[i];
+    if (off_out) for (long long i = first; i <= n; i += step) off_out[i] = off[i];
+    if (first == 0) *count_out = count;
 }

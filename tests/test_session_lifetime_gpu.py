@@ -111,3 +111,31 @@ def test_a_copy_of_an_empty_session_can_be_captured(failed):
     ids, offsets, size = sess.records()
     assert ids.numel() == 0 and offsets.tolist() == [0] and size == 0
     sess.close()
+
+
+def test_a_captured_copy_takes_what_the_session_has_when_it_runs():
+    import torch
+    import paper_2607_29678_b200 as tt
+    gv, cv = gpu_vocab("C1"), cpu_vocab("C1")
+    parts = [wl.generate(0, 4, 500), wl.generate(0, 5, 4_000)]
+    sess = tt.Session(gv, 10_000)
+    sess.append(parts[0])
+    cap = 1_000
+    ids = torch.zeros(cap, dtype=torch.int32, device="cuda")
+    off = torch.zeros(cap + 1, dtype=torch.int32, device="cuda")
+    count = torch.zeros(1, dtype=torch.int64, device="cuda")
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, capture_error_mode="thread_local"):
+        tt._check(tt.lib().tt_session_copy(sess._h, ids.data_ptr(), cap, off.data_ptr(), count.data_ptr(), torch.cuda.current_stream().cuda_stream), "tt_session_copy")
+    text = np.zeros(0, np.uint8)
+    for part in [None] + parts[1:]:
+        if part is not None:
+            sess.append(part)
+        text = np.r_[text, parts[0] if part is None else part]
+        graph.replay()
+        torch.cuda.synchronize()
+        want, n = cv.encode(text, 0)[0], int(count)
+        k = min(n, cap)
+        assert n == want.size and same(ids[:k].cpu().numpy(), want[:k]) and same(off[:k + 1].cpu().numpy(), cv.spans(text, want)[0][:k + 1])
+    assert n > cap
+    sess.close()
