@@ -236,8 +236,8 @@ static int build_token_table(tt_vocab* v, const tt_merge* merges, size_t n_merge
         if ((int32_t)cnt[slot] == -1 && stage[off[i]] == ext_id[cand[i]]) keep.push_back((u32)i);           // minus the staged count
     }
     }
-    // Two-choice placement (see TokTable), a bucket of the short table for every one to two entries and one of the other for every
-    // three to six, so that few buckets overflow; another seed where a placement fails.
+    // Two-choice placement (see TokTable), two to four buckets of the short table for every entry and three to six of the other, so
+    // that few buckets overflow.  Where an entry finds no place, other multipliers are tried, and from time to time a larger table.
     struct Key { u32 n; int32_t id; u32 k[6], h; };
     std::vector<Key> keys[2];
     for (u32 b = 0; b < 256; b++) { Key e{}; e.n = 1; e.id = ext_id[b]; e.k[0] = b; keys[0].push_back(e); }
@@ -251,12 +251,21 @@ static int build_token_table(tt_vocab* v, const tt_merge* merges, size_t n_merge
     }
     u32 log2n[2];
     for (int c = 0; c < 2; c++) { log2n[c] = 8; while (((size_t)1 << log2n[c]) < (c ? 3 : 2) * keys[c].size()) log2n[c]++; }
-    const size_t short_slots = (size_t)2 << log2n[0], long_slots = (size_t)1 << log2n[1];
-    std::vector<uint4> table(short_slots + 2 * long_slots);
-    u32 seed = 0;
+    size_t short_slots = 0, long_slots = 0;
+    std::vector<uint4> table;
+    TokTable& T = v->toktab;
+    const u32 first_mul[6] = {0x85EBCA6Bu, 0xC2B2AE35u, 0x27D4EB2Fu, 0x165667B1u, 0xD3A2646Du, 0xFD7046C5u};
+    memcpy(T.mul, first_mul, sizeof(first_mul));
+    u64 mrng = 0x2545F4914F6CDD1Dull;
     bool placed_all = false;
-    for (int attempt = 0; attempt < 64 && !placed_all; attempt++, seed += 0x6D2B79F5u) {
-        std::fill(table.begin(), table.end(), make_uint4(0, 0, 0, 0));
+    int failed = 0;
+    for (int attempt = 0; attempt < 64; attempt++) {
+        if (attempt > 0) {
+            for (int j = 0; j < 6; j++) { mrng = mrng * 6364136223846793005ull + 1442695040888963407ull; T.mul[j] = (u32)(mrng >> 32) | 1u; }
+            if (attempt % 8 == 0 && log2n[failed] < 24) log2n[failed]++;
+        }
+        short_slots = (size_t)2 << log2n[0]; long_slots = (size_t)1 << log2n[1];
+        table.assign(short_slots + 2 * long_slots, make_uint4(0, 0, 0, 0));
         placed_all = true;
         for (int c = 0; c < 2 && placed_all; c++) {
             const u32 shift = 32 - log2n[c], width = c ? 1 : 2;           // slots of a bucket
@@ -264,8 +273,8 @@ static int build_token_table(tt_vocab* v, const tt_merge* merges, size_t n_merge
             u64 rng = 0x9E3779B97F4A7C15ull;
             for (size_t i = 0; i < keys[c].size() && placed_all; i++) {
                 Key& e = keys[c][i];
-                const u32 s = toktab_hash_short(e.k[0], e.k[1], e.n, seed);
-                e.h = toktab_hash_final(c ? toktab_hash_rest(s, e.k[2], e.k[3], e.k[4], e.k[5]) : s);
+                const u32 s = toktab_hash_short(T, e.k[0], e.k[1], e.n);
+                e.h = toktab_hash_final(c ? toktab_hash_rest(T, s, e.k[2], e.k[3], e.k[4], e.k[5]) : s);
                 int cur = (int)i;
                 for (int iter = 0; cur >= 0; iter++) {
                     if (iter == 2000) { placed_all = false; break; }
@@ -276,7 +285,7 @@ static int build_token_table(tt_vocab* v, const tt_merge* merges, size_t n_merge
                     std::swap(cur, owner[(size_t)b[(rng >> 33) & 1] * width + ((rng >> 40) & (width - 1))]);
                 }
             }
-            if (!placed_all) break;
+            if (!placed_all) { failed = c; break; }
             uint4* const base = table.data() + (c ? short_slots : 0);
             for (size_t o = 0; o < owner.size(); o++) {
                 if (owner[o] < 0) continue;
@@ -297,7 +306,7 @@ static int build_token_table(tt_vocab* v, const tt_merge* merges, size_t n_merge
         cudaGetLastError(); return TT_ERR_CUDA;
     }
     v->toktab.shorts = v->d_toktab; v->toktab.slots = reinterpret_cast<const TokSlot*>(v->d_toktab + short_slots);
-    v->toktab.short_shift = 32 - log2n[0]; v->toktab.shift = 32 - log2n[1]; v->toktab.seed = seed; v->toktab.bytes = table_bytes;
+    v->toktab.short_shift = 32 - log2n[0]; v->toktab.shift = 32 - log2n[1]; v->toktab.bytes = table_bytes;
     v->n_table_tokens = keep.size();
     return TT_OK;
 }

@@ -113,13 +113,15 @@ static_assert(sizeof(TokSlot) == 32, "slot layout");
 struct TokTable {
     const uint4* shorts;      // 2 << (32 - short_shift) slots, then the longer entries; nullptr: no table
     const TokSlot* slots;     // 1 << (32 - shift) of them
-    u32 short_shift, shift, seed;
+    u32 short_shift, shift;
+    u32 mul[6];               // multipliers of the key words (odd)
     size_t bytes;             // of both, from `shorts` on
 };
 
 // Key words beyond the piece are zero, so they add nothing: a piece of at most 8 bytes is hashed from two words.
-TT_HD u32 toktab_hash_short(u32 k0, u32 k1, u32 n, u32 seed) { return seed + n * 0x9E3779B1u + k0 * 0x85EBCA6Bu + k1 * 0xC2B2AE35u; }
-TT_HD u32 toktab_hash_rest(u32 h, u32 k2, u32 k3, u32 k4, u32 k5) { return h + k2 * 0x27D4EB2Fu + k3 * 0x165667B1u + k4 * 0xD3A2646Du + k5 * 0xFD7046C5u; }
+// The multipliers belong to the table: entries that collide under some (equal sums share both buckets) part under others.
+TT_HD u32 toktab_hash_short(const TokTable& tab, u32 k0, u32 k1, u32 n) { return n * 0x9E3779B1u + k0 * tab.mul[0] + k1 * tab.mul[1]; }
+TT_HD u32 toktab_hash_rest(const TokTable& tab, u32 h, u32 k2, u32 k3, u32 k4, u32 k5) { return h + k2 * tab.mul[2] + k3 * tab.mul[3] + k4 * tab.mul[4] + k5 * tab.mul[5]; }
 TT_HD u32 toktab_hash_final(u32 h) { h ^= h >> 15; h *= 0x2C1B3C6Du; h ^= h >> 12; h *= 0x297A2D39u; return h ^ (h >> 15); }
 TT_HD u32 toktab_bucket(u32 h, u32 shift) { return h >> shift; }
 TT_HD u32 toktab_bucket_alt(u32 h, u32 shift) {                   // the key's other bucket, never the first one
@@ -169,7 +171,7 @@ __device__ __forceinline__ bool toktab_lookup(const TokTable& tab, const u8* __r
     u32 k[6];
 #pragma unroll
     for (int j = 0; j < 6; j++) k[j] = toktab_mask_word(__funnelshift_r(x[j], x[j + 1], sh), n, j);
-    const u32 s = toktab_hash_short(k[0], k[1], n, tab.seed);
+    const u32 s = toktab_hash_short(tab, k[0], k[1], n);
     if (n <= TT_TOKTAB_SHORT) {
         const u32 h = toktab_hash_final(s);
         const uint4* const b = tab.shorts + 2 * (size_t)toktab_bucket(h, tab.short_shift);
@@ -178,7 +180,7 @@ __device__ __forceinline__ bool toktab_lookup(const TokTable& tab, const u8* __r
         id = (int32_t)val;
         return hit;
     }
-    const u32 h = toktab_hash_final(toktab_hash_rest(s, k[2], k[3], k[4], k[5]));
+    const u32 h = toktab_hash_final(toktab_hash_rest(tab, s, k[2], k[3], k[4], k[5]));
     u32 at = toktab_bucket(h, tab.shift);
 #pragma unroll 1
     for (int probe = 0; probe < 2; probe++) {
