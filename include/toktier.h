@@ -220,6 +220,9 @@ int tt_encode_added(const tt_vocab* v, const uint8_t* text, size_t len, void* st
  *                       as they are.
  *   tt_session_free     waits for the copies under way; where tt_session_view gave out device pointers, or a copy was
  *                       captured into a graph, it returns the memory with cudaFree, which waits for the device.
+ *                       Otherwise the vocabulary keeps the memory for its next session: the last eight freed
+ *                       sessions' at most, 512 MB of device memory (and 256 KB of pinned memory each), until
+ *                       tt_vocab_free or until an allocation of this vocabulary finds no memory.
  * One session must not be used from two threads at once.
  */
 typedef struct tt_session tt_session;

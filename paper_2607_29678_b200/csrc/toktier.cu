@@ -27,9 +27,10 @@
 #include <algorithm>
 
 // Device and pinned memory of the sessions of one vocabulary.  A session's arrays are one allocation, and the memory of a
-// freed session is kept for the next one (at most POOL_ARENAS of them, POOL_BYTES in all; given back by
-// tt_vocab_free): fifteen cudaMalloc and cudaFree calls per session took 2 to 15 ms, more than the 17 tokenizations of
-// a conversation.  Sessions share ownership, so that one that outlives its vocabulary still frees what it holds.
+// freed session is kept for the next one: fifteen cudaMalloc and cudaFree calls per session took 2 to 15 ms, more than the 17
+// tokenizations of a conversation.  At most POOL_ARENAS of them, POOL_BYTES in all, the most recently freed; given back by
+// tt_vocab_free, and as soon as an allocation for this vocabulary finds no memory.  Sessions share ownership, so that one
+// that outlives its vocabulary still frees what it holds.
 struct SessionHost;
 struct SessionArena { char* dev = nullptr; size_t bytes = 0; int device = 0; SessionHost* host = nullptr; size_t host_text = 0; cudaEvent_t copied = nullptr; };
 struct SessionPool {
@@ -39,13 +40,15 @@ struct SessionPool {
     bool closed = false;
     static void destroy(SessionArena& a) { cudaFree(a.dev); if (a.host) cudaFreeHost(a.host); if (a.copied) cudaEventDestroy(a.copied); a = SessionArena{}; }
     bool get(size_t bytes, size_t host_text, SessionArena& out);
+    static bool create(size_t bytes, size_t host_text, int device, SessionArena& out);
     void put(SessionArena a);
-    void close() {
-        std::lock_guard<std::mutex> lk(mu);
-        closed = true;
-        for (SessionArena& a : kept) destroy(a);
-        kept.clear();
+    bool trim() {                                            // gives back all that is kept; was there anything?
+        std::vector<SessionArena> all;
+        { std::lock_guard<std::mutex> lk(mu); all.swap(kept); }
+        for (SessionArena& a : all) destroy(a);
+        return !all.empty();
     }
+    void close() { { std::lock_guard<std::mutex> lk(mu); closed = true; } trim(); }
 };
 
 struct tt_vocab {
@@ -898,9 +901,14 @@ extern "C" int tt_encode_host(tt_vocab* v, const uint8_t* text, size_t len, int3
         v->d_text = nullptr; v->d_ids = nullptr; v->d_ws = nullptr; v->h_text = nullptr; v->h_ids = nullptr; v->host_cap = 0;
         const size_t cap = align_up(len + 1 + len / 4, 4096);
         v->ws_cap = tt_workspace_bytes(v, cap, 1);
-        CK(cudaMalloc(&v->d_text, cap + 64));
-        CK(cudaMalloc(&v->d_ids, cap * sizeof(int32_t)));
-        CK(cudaMalloc(&v->d_ws, v->ws_cap));
+        const auto get = [&](auto** p, size_t bytes) {         // (memory that freed sessions left is released first)
+            if (cudaMalloc(p, bytes) == cudaSuccess) return cudaSuccess;
+            cudaGetLastError();
+            return v->sessions->trim() ? cudaMalloc(p, bytes) : cudaErrorMemoryAllocation;
+        };
+        CK(get(&v->d_text, cap + 64));
+        CK(get(&v->d_ids, cap * sizeof(int32_t)));
+        CK(get(&v->d_ws, v->ws_cap));
         CK(cudaMallocHost(&v->h_text, cap + 64));
         CK(cudaMallocHost(&v->h_ids, cap * sizeof(int32_t)));
         if (!v->d_count) CK(cudaMalloc(&v->d_count, sizeof(long long)));
@@ -1032,20 +1040,32 @@ bool SessionPool::get(size_t bytes, size_t host_text, SessionArena& out) {
             if (kept[i].device == device && kept[i].bytes >= bytes && kept[i].host_text >= host_text && kept[i].bytes / 4 <= bytes && (best == kept.size() || kept[i].bytes < kept[best].bytes)) best = i;
         if (best < kept.size()) { out = kept[best]; kept.erase(kept.begin() + (ptrdiff_t)best); return true; }
     }
-    out.bytes = bytes; out.device = device; out.host_text = host_text;
-    if (cudaMalloc(&out.dev, bytes) != cudaSuccess) { cudaGetLastError(); out.dev = nullptr; return false; }
-    if (cudaMallocHost(&out.host, sizeof(SessionHost) + host_text) != cudaSuccess) { cudaGetLastError(); out.host = nullptr; destroy(out); return false; }
-    if (cudaEventCreateWithFlags(&out.copied, cudaEventDisableTiming) != cudaSuccess) { cudaGetLastError(); out.copied = nullptr; destroy(out); return false; }
+    // (what is kept and did not fit may be what is missing: released, and tried once more)
+    if (!create(bytes, host_text, device, out) && !(trim() && create(bytes, host_text, device, out))) return false;
     return true;
 }
+bool SessionPool::create(size_t bytes, size_t host_text, int device, SessionArena& out) {
+    out = SessionArena{};
+    out.bytes = bytes; out.device = device; out.host_text = host_text;
+    const bool ok = cudaMalloc(&out.dev, bytes) == cudaSuccess && cudaMallocHost(&out.host, sizeof(SessionHost) + host_text) == cudaSuccess &&
+                    cudaEventCreateWithFlags(&out.copied, cudaEventDisableTiming) == cudaSuccess;
+    if (!ok) { cudaGetLastError(); destroy(out); }
+    return ok;
+}
 void SessionPool::put(SessionArena a) {
+    std::vector<SessionArena> out;                           // to be destroyed: outside the lock, it may wait for the device
     {
         std::lock_guard<std::mutex> lk(mu);
-        size_t total = a.bytes;
-        for (const SessionArena& k : kept) total += k.bytes;
-        if (!closed && kept.size() < POOL_ARENAS && total <= POOL_BYTES) { kept.push_back(a); return; }
+        if (closed || a.bytes > POOL_BYTES) out.push_back(a);
+        else {
+            size_t total = a.bytes, first = kept.size();     // the most recent ones that fit beside it stay
+            while (first > 0 && kept.size() - first + 2 <= POOL_ARENAS && total + kept[first - 1].bytes <= POOL_BYTES) total += kept[--first].bytes;
+            out.assign(kept.begin(), kept.begin() + (ptrdiff_t)first);
+            kept.erase(kept.begin(), kept.begin() + (ptrdiff_t)first);
+            kept.push_back(a);
+        }
     }
-    destroy(a);
+    for (SessionArena& o : out) destroy(o);
 }
 
 struct tt_session {

@@ -139,3 +139,57 @@ def test_a_captured_copy_takes_what_the_session_has_when_it_runs():
         assert n == want.size and same(ids[:k].cpu().numpy(), want[:k]) and same(off[:k + 1].cpu().numpy(), cv.spans(text, want)[0][:k + 1])
     assert n > cap
     sess.close()
+
+
+def _free():
+    import torch
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    return torch.cuda.mem_get_info()[0]
+
+
+def _own_vocab():
+    import paper_2607_29678_b200 as tt
+    return tt.Vocab(*wl.load_vocab(wl.CONFIGS["C1"]), 0)
+
+
+def test_a_larger_session_finds_a_place_among_the_kept_ones():
+    """Eight small sessions have ended; a larger one leaves its memory to the next one of its size all the same."""
+    import paper_2607_29678_b200 as tt
+    v = _own_vocab()
+    small = [tt.Session(v, 1_000_000) for _ in range(8)]
+    for s in small:
+        s.close()
+    tt.Session(v, 6_000_000).close()                         # (about 45 bytes of device memory per byte: more than 4 times a small one's)
+    before = _free()
+    large = tt.Session(v, 6_000_000)
+    assert _free() == before                                  # nothing was allocated for it
+    large.append(wl.generate(0, 1, 3_000))
+    large.close()
+    assert _free() == before
+    v.close()
+    assert _free() > before + (200 << 20)
+
+
+@pytest.mark.parametrize("what", ["session", "host call"])
+def test_kept_memory_gives_way_when_none_is_left(what):
+    import torch
+    import paper_2607_29678_b200 as tt
+    v, cv = _own_vocab(), cpu_vocab("C1")
+    text = wl.generate(0, 1, 8_000_000 if what == "host call" else 3_000)
+    want = cv.encode(text, 0, nthreads=8)[0]
+    kept = [tt.Session(v, 1_300_000) for _ in range(8)]       # about 60 MB each
+    for s in kept:
+        s.close()
+    hold = torch.empty(_free() - (150 << 20), dtype=torch.uint8, device="cuda")      # 150 MB are left, and what the vocabulary keeps
+    try:
+        if what == "session":
+            sess = tt.Session(v, 8_000_000)                   # about 380 MB
+            assert sess.append(text)["n_tokens"] == want.size
+            sess.close()
+        else:
+            assert same(v.encode_host(text), want)            # about 360 MB of device memory
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+        v.close()
