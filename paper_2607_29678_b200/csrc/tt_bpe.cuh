@@ -1805,7 +1805,9 @@ k_scatter(const __grid_constant__ ScatterParams P) {
             __syncthreads();
             if (tid == 0) s_nbig = 0;                             // (the next item's barrier comes before anyone adds)
         }
-        if (staged) for (u32 kk = tid; kk < tot; kk += BPE_THREADS) P.ids_out[carry + kk] = s_out[kk];
+        // (not beyond the total that was checked against the capacity, whatever the pieces of the item add up to)
+        const u32 leave = carry < total ? min(tot, total - carry) : 0u;
+        if (staged) for (u32 kk = tid; kk < leave; kk += BPE_THREADS) P.ids_out[carry + kk] = s_out[kk];
         carry += tot;
         if (tile2 >= tile_hi) break;
         tile = tile2; b = b2; np = np2; v = vn; o2 = on;
