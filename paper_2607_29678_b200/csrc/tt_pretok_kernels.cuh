@@ -352,7 +352,7 @@ k_pretok(const __grid_constant__ PretokParams P, const __grid_constant__ FrontPa
     __shared__ u16 s_wlist[TT_TILE_BYTES / (LANE_MAX + 1) + 2];       // bulk text: the tile's warp-class pieces
     __shared__ u16 s_slow[TT_TILE_BYTES / 9 + 4];                     // pieces of more than 8 bytes (looked up together)
     __shared__ u32 s_nslow;
-    static_assert(NT >= TT_TILE_WORDS && NT % 32 == 0, "a thread per word of the tile");
+    static_assert(NT >= TT_TILE_WORDS && NT % 32 == 0 && TT_TILE_WORDS % 32 == 0, "a thread per word of the tile, whole warps of them (tt_eval_word_p1 asks the warp)");
 
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     cudaTriggerProgrammaticLaunchCompletion();               // the next kernel may be placed; it waits for this grid's memory itself
