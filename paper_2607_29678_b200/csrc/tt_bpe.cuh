@@ -1683,8 +1683,12 @@ k_scatter(const __grid_constant__ ScatterParams P) {
     __shared__ int32_t s_out[SCATTER_STAGE_IDS];              // the ids of one item on their way out
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const u32 FULL = 0xFFFFFFFFu;
-    cudaTriggerProgrammaticLaunchCompletion();               // the next call's first kernel may be placed; it waits for this grid itself
     cudaGridDependencySynchronize();                         // k_merge's (and with it the first kernel's) results are complete from here on
+    // The next call's first kernel may be placed from here on; it waits for this grid itself.  (Allowed earlier, while this grid still waits
+    // for k_merge, its CTAs -- and those of the call's other kernels -- gathered on the SMs whose k_merge CTA was through first:
+    // 150,000 pieces of two bytes, call after call, 177 us instead of 108, 300 KB of short accented words 815 instead of 651;
+    // 300 KB of Unicode-heavy text 38.8 instead of 35.5.)
+    cudaTriggerProgrammaticLaunchCompletion();
     // Each CTA takes a contiguous range of tiles and sums the token counts before it, and all of them (the count, and the
     // capacity check, which every CTA makes for itself).
     const int per = (P.ntiles + (int)gridDim.x - 1) / (int)gridDim.x;
@@ -1827,8 +1831,8 @@ k_scatter_bulk(const __grid_constant__ ScatterParams P) {
     __shared__ unsigned long long s_sum[66];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const u32 FULL = 0xFFFFFFFFu;
-    cudaTriggerProgrammaticLaunchCompletion();               // the next call's first kernel may be placed; it waits for this grid itself
     cudaGridDependencySynchronize();                         // k_merge_bulk's (and with it the kernels' before it) results are complete
+    cudaTriggerProgrammaticLaunchCompletion();               // the next call's first kernel may be placed (see k_scatter)
     const int per = (P.ntiles + (int)gridDim.x - 1) / (int)gridDim.x;
     const int tile_lo = (int)blockIdx.x * per, tile_hi = min(P.ntiles, tile_lo + per);
     unsigned long long before = 0, total = 0;
