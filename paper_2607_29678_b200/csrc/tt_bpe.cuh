@@ -1513,6 +1513,53 @@ __device__ __forceinline__ u32 merge_find(const u32* pre, u32 entries, u32 k) {
     return lo;
 }
 
+constexpr u32 SHORT_PER_WARP = 12;                    // more short pieces than that per warp of the grid: see k_merge
+// The k-th queued piece of its class (warp-class or short).
+__device__ __forceinline__ void merge_queued(const PieceParams& P, const MergeIndex& X, int unit, int entries, bool wclass, u32 k, u32& a, u32& n, u32& slot) {
+    const u32* const pre = wclass ? X.pre_w : X.pre_s;
+    const u32 en = merge_find(pre, (u32)entries, k);
+    u32 r = k - pre[en], t = en * (u32)unit;
+    for (int u = 0; u + 1 < unit; u++) {
+        const u32 q = P.tile_q[t], c = wclass ? (q >> TQ_NW_SHIFT) & TQ_NW_MASK : q & TQ_NS_MASK;
+        if (r < c) break;
+        r -= c; t++;
+    }
+    const u32 e = P.q[(size_t)t * TT_TILE_QCAP + (wclass ? (u32)TT_TILE_QCAP - 1 - r : r)];
+    n = (e >> 22) + 1;
+    a = (u32)((long long)t * TT_TILE_BYTES + (e & 2047u) - P.shift); slot = t * TT_TILE_BYTES + ((e >> 11) & 2047u);
+}
+// The closing piece of tile t, where it has at most 256 bytes and needs merging (every lane computes the same).
+__device__ __forceinline__ bool merge_closing(const PieceParams& P, const u8* __restrict__ text, u32 t, int lane, u32& a, u32& n, u32& slot) {
+    const u32 np = P.tile_cnt[t], last = P.tile_last[t], next = t + 1 < (u32)P.ntiles ? P.tile_first[t + 1] : TT_NONE;
+    if (np == 0) return false;
+    const u32 st = t * TT_TILE_BYTES + last;
+    n = (next != TT_NONE ? (t + 1) * TT_TILE_BYTES + next : closing_piece_end(P, (int)t)) - st;
+    if (n > (u32)TT_WARP_PIECE_MAX) return false;                    // a long piece
+    a = (u32)((long long)st - P.shift); slot = t * TT_TILE_BYTES + np - 1;
+    u32 v;
+    if (!piece_settled_without_merge(P, text, a, n, v)) return true;
+    if (lane == 0) { P.piece_cnt[slot] = v; atomicAdd(&P.tile_tok[t], 1u); }
+    return false;
+}
+// The queued short pieces 32 by 32 in their order, whatever tiles they stand in, a thread each; the batches are spread over the
+// grid, by tickets where some CTAs first had a long piece.  (With a ticket per tile 147 warps took the 150,000 two-byte pieces of
+// 300 KB, most of them on the few SMs that came first: 78 to 118 us, now 54 to 66.)
+__device__ __forceinline__ void merge_short_batches(const PieceParams& P, const u8* __restrict__ text, const MergeIndex& X, int unit, int entries, bool by_ticket, u32* tok) {
+    const u32 lane = threadIdx.x & 31, NS = X.pre_s[entries], nb = (NS + 31) / 32;
+    u32 b = by_ticket ? warp_take(&P.hdr->t_tiles, (int)lane) : (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    while (b < nb) {
+        const u32 k = 32 * b + lane;
+        if (k < NS) {
+            u32 a, n, slot;
+            merge_queued(P, X, unit, entries, false, k, a, n, slot);
+            if (!piece_in_range(P, a, n, slot, 4u) || n < 2 || n > (u32)LANE_MAX) hdr_selfcheck_failed(P.hdr, P.epoch, 5u, a, n, slot, k);
+            else piece_done(P, slot, lane_merge(tok, tok + LANE_SLOTS * LANE_MAX, (int)lane, text, a, n, P.tab, P.ext_id, P.stage));
+        }
+        __syncwarp();
+        b = by_ticket ? warp_take(&P.hdr->t_tiles, (int)lane) : b + gridDim.x * MERGE_WARPS;
+    }
+}
+
 __global__ void __launch_bounds__(MERGE_THREADS, MERGE_CTAS_PER_SM)
 k_merge(const __grid_constant__ PieceParams P) {
     extern __shared__ __align__(16) u64 s_buf[];              // MERGE_SMEM_REQUEST
@@ -1520,7 +1567,6 @@ k_merge(const __grid_constant__ PieceParams P) {
     __shared__ LongShared LS;
     MergeIndex& X = *reinterpret_cast<MergeIndex*>(s_buf + MERGE_WARPS * WARP_SMEM_WORDS);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const u32 FULL = 0xFFFFFFFFu;
     cudaTriggerProgrammaticLaunchCompletion();               // k_scatter may be placed; it waits for this grid's memory itself
     grid_prefetch_l2(P.tab.slots, ((size_t)P.tab.mask + 1) * 2 * sizeof(uint4));
     grid_prefetch_l2(P.tab.bytepair, 65536 * sizeof(u64));
@@ -1534,13 +1580,12 @@ k_merge(const __grid_constant__ PieceParams P) {
     u64* wbuf = s_buf + wid * WARP_SMEM_WORDS;
     const u32 W = gridDim.x * MERGE_WARPS, gw = (u32)wid * gridDim.x + blockIdx.x;   // numbered across the CTAs first
     const u32 NS = X.pre_s[entries], NW = X.pre_w[entries], NT = (u32)P.ntiles;
-#ifndef TT_SHORT_WARP_FACTOR
-#define TT_SHORT_WARP_FACTOR 12u
-#endif
-    // Measured crossover (1 M to 8 M chars of Unicode-heavy prose, 15 K to 120 K unsettled pieces): a warp per piece
-    // wins up to about 17 pieces per warp of the grid.
-    const bool tickets = NS + NT > TT_SHORT_WARP_FACTOR * W;         // short pieces 32 at a time by tickets, or job by job
-    const u32 J = tickets ? NW : NW + NT + NS;                       // with tickets only the warp-class pieces go job by job
+    // A warp per piece, or a thread per piece and a warp for 32 of them?  A batch takes as long as its slowest piece: 25 us for words of nine
+    // letters, 50 to 60 for the mixed lengths of prose, however few batches there are.  Measured, short pieces per warp of the
+    // grid -> k_merge with a warp / a thread per piece: Unicode-heavy prose 4.3 -> 36 / 50 us, 13.2 -> 76 / 59, 13.5 -> 70 / 66, 16 ->
+    // 75 / 75; transcripts 10 -> 60 / 73; nine-letter words 3 -> 19 / 23, 4.3 -> 25 / 25, 8.6 -> 40 / 29, 17 -> 66 / 38.
+    const bool many = NS + NT > SHORT_PER_WARP * W;
+    const u32 J = many ? NW : NW + NT + NS;                          // jobs of a warp: all pieces, or the warp-class ones
     // Job by job in order (warp-class pieces, closing pieces, short pieces); where some CTAs first had a long piece to merge, by
     // tickets of `step` jobs, the next one drawn in advance.
     const u32 step = longs ? max(1u, J / (2 * W)) : 1u;
@@ -1552,90 +1597,18 @@ k_merge(const __grid_constant__ PieceParams P) {
         else { j = jn * step; left = step; jn = longs ? (j < J ? warp_take(&P.hdr->t_short, lane) : jn) : jn + W; }
         u32 a, n, slot;
         if (job >= NW && job < NW + NT) {                            // the closing piece of tile job - NW
-            const int t = (int)(job - NW);
-            const u32 np = P.tile_cnt[t], last = P.tile_last[t], next = t + 1 < P.ntiles ? P.tile_first[t + 1] : TT_NONE;
-            if (np == 0) continue;
-            const u32 st = (u32)t * TT_TILE_BYTES + last;
-            n = (next != TT_NONE ? (u32)(t + 1) * TT_TILE_BYTES + next : closing_piece_end(P, t)) - st;
-            if (n > (u32)TT_WARP_PIECE_MAX) continue;                // a long piece
-            a = (u32)((long long)st - P.shift); slot = (u32)t * TT_TILE_BYTES + np - 1;
-            u32 v;
-            if (piece_settled_without_merge(P, text, a, n, v)) {     // every lane computes the same
-                if (lane == 0) { P.piece_cnt[slot] = v; atomicAdd(&P.tile_tok[t], 1u); }
-                continue;
-            }
-        } else {
-            // the k-th queued piece of its class
-            const bool wclass = job < NW;
-            const u32 k = wclass ? job : job - NW - NT;
-            const u32* const pre = wclass ? X.pre_w : X.pre_s;
-            const u32 en = merge_find(pre, (u32)entries, k);
-            u32 r = k - pre[en], t = en * (u32)unit;
-            for (int u = 0; u + 1 < unit; u++) {
-                const u32 q = P.tile_q[t], c = wclass ? (q >> TQ_NW_SHIFT) & TQ_NW_MASK : q & TQ_NS_MASK;
-                if (r < c) break;
-                r -= c; t++;
-            }
-            const u32 e = P.q[(size_t)t * TT_TILE_QCAP + (wclass ? (u32)TT_TILE_QCAP - 1 - r : r)];
-            n = (e >> 22) + 1;
-            a = (u32)((long long)t * TT_TILE_BYTES + (e & 2047u) - P.shift); slot = t * TT_TILE_BYTES + ((e >> 11) & 2047u);
-        }
+            if (!merge_closing(P, text, job - NW, lane, a, n, slot)) continue;
+        } else merge_queued(P, X, unit, entries, job < NW, job < NW ? job : job - NW - NT, a, n, slot);
         warp_merge_piece(P, text, a, n, slot, wbuf, lane);
     }
-    if (tickets) {
-    // ---- tickets: a tile each; its short pieces (queued ones, then its closing piece if that is short) wait in the
-    // lanes until 32 of them are together, so that every step of the thread-per-piece merge is full
-        u32* const tok = reinterpret_cast<u32*>(wbuf);
-        const u32 ntick = (u32)P.ntiles;
-        u32 pa = 0, pn = 0, pslot = 0, pend = 0;                      // lanes below `pend` hold a short piece that waits for a full step
-        for (;;) {                                                    // bounded by the number of tickets
-            u32 t = 0;
-            if (lane == 0) t = atomicAdd(&P.hdr->t_tiles, 1u);
-            t = __shfl_sync(FULL, t, 0);
-            const bool last_round = t >= ntick;
-            u32 ns = 0, ca = 0, cn = 0, cslot = 0;                    // cn == 0: no closing piece left to merge
-            if (!last_round) {                                        // warp-uniform; every lane computes the same
-                const u32 q = P.tile_q[t], np = P.tile_cnt[t], last = P.tile_last[t];
-                const u32 nf = t + 1 < ntick ? P.tile_first[t + 1] : TT_NONE;
-                ns = q & TQ_NS_MASK;
-                if (np) {
-                    const u32 st = t * TT_TILE_BYTES + last;
-                    cn = (t + 1 >= ntick ? (u32)P.hi : nf != TT_NONE ? (t + 1) * TT_TILE_BYTES + nf : closing_piece_end(P, (int)t)) - st;
-                    ca = (u32)((long long)st - P.shift); cslot = t * TT_TILE_BYTES + np - 1;
-                    u32 v;
-                    if (cn > (u32)TT_WARP_PIECE_MAX) cn = 0;          // settled by a CTA above
-                    else if (piece_settled_without_merge(P, text, ca, cn, v)) { if (lane == 0) { P.piece_cnt[cslot] = v; atomicAdd(&P.tile_tok[t], 1u); } cn = 0; }
-                    else if (cn > (u32)LANE_MAX) { warp_merge_piece(P, text, ca, cn, cslot, wbuf, lane); cn = 0; }
-                }
-            }
-            const u32 nj = ns + (cn ? 1u : 0u);
-            u32 e0 = 0;                                               // new pieces handed to lanes so far
-            for (;;) {                                                // warp-uniform; bounded by nj / 32 + 2
-                const u32 left = nj - e0;
-                const bool run = pend + left >= 32u || (last_round && pend != 0);
-                const u32 take = min(32u - pend, left);               // lanes pend .. pend + take - 1 take new pieces
-                const u32 e = e0 + ((u32)lane - pend);
-                if ((u32)lane >= pend && (u32)lane - pend < take) {
-                    if (e < ns) {
-                        const u32 qe = P.q[(size_t)t * TT_TILE_QCAP + e];
-                        pn = (qe >> 22) + 1;
-                        pa = (u32)((long long)t * TT_TILE_BYTES + (qe & 2047u) - P.shift); pslot = t * TT_TILE_BYTES + ((qe >> 11) & 2047u);
-                    } else { pa = ca; pn = cn; pslot = cslot; }
-                }
-                e0 += take; pend += take;
-                if (!run) break;
-                if ((u32)lane < pend) {
-                    if (!piece_in_range(P, pa, pn, pslot, 4u) || pn < 2 || pn > (u32)LANE_MAX) hdr_selfcheck_failed(P.hdr, P.epoch, 5u, pa, pn, pslot, e);
-                    else {
-                        const u32 m = lane_merge(tok, tok + LANE_SLOTS * LANE_MAX, lane, text, pa, pn, P.tab, P.ext_id, P.stage);
-                        piece_done(P, pslot, m);
-                    }
-                }
-                __syncwarp();
-                pend = 0;
-            }
-            if (last_round) break;
+    if (many) {
+        // (a place of their own for the closing pieces: with the merges in one place for both ways, the way without batches took 3 %
+        // longer on transcripts and long runs)
+        for (u32 t = gw; t < NT; t += W) {
+            u32 a, n, slot;
+            if (merge_closing(P, text, t, lane, a, n, slot)) warp_merge_piece(P, text, a, n, slot, wbuf, lane);
         }
+        merge_short_batches(P, text, X, unit, entries, longs != 0, reinterpret_cast<u32*>(wbuf));
     }
     if (longs == 2) long_phase(P, text, long_find_tasks(P), s_buf, sc, LS);
 }

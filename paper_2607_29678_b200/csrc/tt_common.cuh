@@ -51,7 +51,7 @@ struct TTHeader {
     unsigned long long status_tag;   // (epoch of the call << 8) | device-side error code of that call
     u32 pretok_done;         // CTAs that finished the pre-tokenization pass (tt_pretokenize only; cleared by a memset)
     u32 n_pieces;            // number of pieces found (tt_pretokenize only)
-    u32 t_tiles;             // ticket counter of k_merge's bulk mode (groups of tiles handed out); zeroed by the kernel before it
+    u32 t_tiles;             // ticket counter of k_merge's batches of short pieces; zeroed by the kernel before it
     u32 merge_done;          // CTAs of k_merge that have finished (bulk text: the last one sums the groups); zeroed likewise
     u32 nwq;                 // bulk text: lengths of the global lists of warp-class, short and long pieces and the ticket
     u32 nq_short, nq_long;   //            counter of the short list (all cleared by a memset before the chain)
