@@ -28,3 +28,27 @@ def test_calls_back_to_back():
     assert int(bufs["status"]) == 0 and same(bufs["ids"][:int(bufs["count"])].cpu().numpy(), cv.encode(text, gv.pattern_id)[0])
     # 1.28 times where the first kernel of a call was placed before the merges of the one before it were through
     assert among < 1.18 * alone + 0.004, (alone, among)
+
+
+def test_kernels_of_bulk_text_in_a_row():
+    """A call of over 4 MB takes no longer than its kernels one by one."""
+    import torch
+    gv, cv = gpu_vocab("C3"), cpu_vocab("C3")
+    rng = np.random.default_rng(3)
+    words = (97 + rng.integers(0, 26, (1_200_000, 5))).astype(np.uint8)
+    words[:, 4] = 32
+    text = words.ravel()
+    d, bufs = to_dev(text), gv.alloc(text.size)
+    ms = []
+    for _ in range(9):
+        t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        torch.cuda._sleep(200_000)
+        t0.record()
+        gv.encode(d, bufs, length=text.size)
+        t1.record()
+        torch.cuda.synchronize()
+        ms.append(t0.elapsed_time(t1))
+    alone = np.median([sum(gv.encode_timed(d, bufs).values()) for _ in range(9)])
+    assert int(bufs["status"]) == 0 and same(bufs["ids"][:int(bufs["count"])].cpu().numpy(), cv.encode(text, 0, nthreads=8)[0])
+    # 1.25 times where the kernel behind the first one was placed early
+    assert np.median(ms) < 1.12 * alone, (np.median(ms), alone)
