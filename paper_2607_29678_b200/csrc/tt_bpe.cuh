@@ -1195,6 +1195,7 @@ __device__ __forceinline__ void long_write(const PieceParams& P, uint4 q, u32 k,
 
 // A piece of at most as many windows as the CTA has warps is the CTA's own: nobody waits for it.
 constexpr u32 LONG_CTA_MAX = (MERGE_WARPS - 1) * LSTEP + LWIN;
+constexpr u32 LONG_MANY = 8;
 __device__ __noinline__ void cta_window_piece(const PieceParams& P, const u8* __restrict__ text, uint4 q, u64* s_buf, u32* sc) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const u32 nw = long_windows(q.y), k = (u32)wid;
@@ -1215,10 +1216,10 @@ __device__ __noinline__ void cta_window_piece(const PieceParams& P, const u8* __
     if (threadIdx.x == 0) piece_done(P, q.z, total);
     __syncthreads();
 }
-// What a CTA does with a long piece that it comes upon; false: the piece is for the whole grid.
-__device__ __forceinline__ bool cta_long_piece(const PieceParams& P, const u8* __restrict__ text, uint4 q, u64* s_buf, u32* sc, LongShared& LS) {
+// What a CTA does with a long piece that it comes upon; false: the piece is for the whole grid.  many: so are all but runs of bytes.
+__device__ __forceinline__ bool cta_long_piece(const PieceParams& P, const u8* __restrict__ text, uint4 q, u64* s_buf, u32* sc, LongShared& LS, bool many = false) {
     if (cta_run_piece(P, text, q.x, q.y, q.z, LS)) return true;
-    if (q.y > LONG_CTA_MAX) return false;
+    if (many || q.y > LONG_CTA_MAX) return false;
     cta_window_piece(P, text, q, s_buf, sc);
     return true;
 }
@@ -1391,13 +1392,16 @@ __device__ void merge_bulk_lists(const PieceParams& P, const u8* __restrict__ te
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const u32 FULL = 0xFFFFFFFFu;
     const u32 nl = P.hdr->nq_long, nw = P.hdr->nwq, ns = P.hdr->nq_short;
+    // With more long pieces than LONG_MANY per CTA their windows go to the warps of the whole grid: a CTA that takes a piece of 300 bytes
+    // has work for two of its 24 warps (6 MB of words of 300 letters, 20,000 pieces, 4,096 merges: 6.3 ms a call so, now 4.3; with one CTA for a whole piece 5.6).
+    const bool many = nl > LONG_MANY * gridDim.x;
     if (nl) {
         u32 mine = 0;
         for (u32 e; (e = cta_take(&P.hdr->long_take[0], &LS.ticket)) < nl;) {     // block-uniform
             mine++;
             const uint4 q = P.lq[e];
             u32 state = LQ_DONE;
-            if (piece_in_range(P, q.x, q.y, q.z, 3u) && !cta_long_piece(P, text, q, s_buf, sc, LS)) state = LQ_WINDOWS;
+            if (piece_in_range(P, q.x, q.y, q.z, 3u) && !cta_long_piece(P, text, q, s_buf, sc, LS, many)) state = LQ_WINDOWS;
             if (tid == 0) P.lq[e].w = state;
         }
         __syncthreads();

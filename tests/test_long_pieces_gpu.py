@@ -70,3 +70,18 @@ def test_many_long_pieces_in_one_call():
     assert status == 0
     for d, doc in enumerate(docs):
         assert same(ids[ids_off[d]:ids_off[d + 1]], cv.encode(doc, 0, nthreads=8)[0]), d
+
+
+@pytest.mark.parametrize("size", [257, 300, 700, 4_672, 4_673])
+@pytest.mark.parametrize("name", ["C1", "C4"])
+def test_bulk_text_with_more_long_pieces_than_ctas_take(name, size):
+    """Beyond eight per CTA (1,184 on 148 SMs) the windows of the pieces go to the whole grid; runs of bytes stay with a CTA."""
+    rng = np.random.default_rng(size)
+    gv, cv = gpu_vocab(name), cpu_vocab(name)
+    n = max(1_200, 4_400_000 // size)
+    text = (97 + rng.integers(0, 26, (n, size + 1))).astype(np.uint8)
+    text[:, size] = 32
+    text[5::97, :size] = ord("=")
+    text[7::89, : size // 2] = 97
+    ids, status = gpu_encode(gv, text.ravel())
+    assert status == 0 and same(ids, cv.encode(text.ravel(), gv.pattern_id, nthreads=8)[0])
