@@ -610,8 +610,11 @@ static int run_pretok(const tt_vocab* v, const uint8_t* text, size_t len, const 
     P.cls_tables = v->d_cls; P.cls_bytes = v->cls_bytes;
     if (doc_off) {
         const long long mask_words = P.hi / 32 + 4;
-        CK(launch_after(k_docmask, (int)((mask_words + DOCMASK_WORDS - 1) / DOCMASK_WORDS), DOCMASK_THREADS, st, 0, early, (const long long*)doc_off,
-                        (int)n_docs, shift, (long long)len, mask_words, w.docmask, w.hdr, P.epoch));
+        const int stretch = docmask_stretch(mask_words, (long long)n_docs);
+        const long long mask_ctas = (mask_words + stretch - 1) / stretch, check = ((long long)n_docs + DOCMASK_THREADS * DOCMASK_AHEAD) / (DOCMASK_THREADS * DOCMASK_AHEAD);
+        const long long check_ctas = check < 4ll * v->sm_count ? check : 4ll * v->sm_count;
+        CK(launch_after(k_docmask, (int)(mask_ctas > check_ctas ? mask_ctas : check_ctas), DOCMASK_THREADS, st, 0, early, (const long long*)doc_off,
+                        (int)n_docs, shift, (long long)len, mask_words, stretch, w.docmask, w.hdr, P.epoch));
         P.docmask = w.docmask;
     }
     if (literals && !doc_off) {

@@ -45,46 +45,81 @@ __device__ __forceinline__ u32 cta_exscan_u32(u32 v, u32* scratch /* >= 33 */, u
 
 // ---- document mask ---------------------------------------------------------------------------
 // Writes the mask with the bit of every document's first byte (aligned frame), and checks the offsets: they must be ascending,
-// start at 0 and end at the total length; a violation is reported as TT_ERR_ARG in the status word.  A CTA writes
+// start at 0 and end at the total length; a violation is reported as TT_ERR_ARG in the status word.  A CTA writes a stretch of
 // DOCMASK_WORDS words: it finds the first document of its stretch by a search in 32 steps at a time.  (Clearing the mask and
-// setting bits in it with atomics were two launches, and two gaps, in front of the chain.)
-constexpr int DOCMASK_WORDS = 2048, DOCMASK_THREADS = 256;
+// setting bits in it with atomics were two launches, and two gaps, in front of the chain.)  Documents of a few bytes each, of
+// which a stretch holds thousands, get shorter stretches (docmask_stretch) and DOCMASK_AHEAD offsets in flight per thread, and
+// all CTAs share the check: 400 KB in documents of one byte 207 us a call, so 64.
+constexpr int DOCMASK_WORDS = 2048, DOCMASK_WORDS_DENSE = 256, DOCMASK_THREADS = 256, DOCMASK_AHEAD = 8;
+// More documents than one round of the loop takes per stretch?
+inline int docmask_stretch(long long mask_words, long long n_docs) {
+    return n_docs > (long long)DOCMASK_THREADS * DOCMASK_AHEAD * ((mask_words + DOCMASK_WORDS - 1) / DOCMASK_WORDS) ? DOCMASK_WORDS_DENSE : DOCMASK_WORDS;
+}
 __global__ void __launch_bounds__(DOCMASK_THREADS)
-k_docmask(const long long* __restrict__ doc_off, int n_docs, long long shift, long long len, long long nwords,
+k_docmask(const long long* __restrict__ doc_off, int n_docs, long long shift, long long len, long long nwords, int stretch,
           u32* __restrict__ docmask, TTHeader* hdr, unsigned long long epoch) {
     __shared__ __align__(16) u32 s_mask[DOCMASK_WORDS];
     __shared__ int s_first;
     const int tid = threadIdx.x, lane = tid & 31;
+    const u32 FULL = 0xFFFFFFFFu;
     // (No early trigger: bulk text fills every place of the GPU with CTAs that stay, and what was placed beside this grid stayed
     // unevenly spread: 535 -> 558 us for 12 MB.)
     cudaGridDependencySynchronize();                         // the work before this call reads the mask, or writes the offsets
-    for (int i = tid; i < DOCMASK_WORDS; i += DOCMASK_THREADS) s_mask[i] = 0;
-    const long long w0 = (long long)blockIdx.x * DOCMASK_WORDS;
-    const long long from = w0 * 32 - shift, to = min((w0 + DOCMASK_WORDS) * 32 - shift, len);      // text bytes of the stretch
-    if (tid < 32) {                                           // first document that starts at `from` or behind it
-        int lo = 0, hi = n_docs;                              // (the answer is in [lo, hi])
-        while (hi > lo) {
-            const int step = (hi - lo + 31) / 32, at = lo + lane * step;
-            const bool less = at < hi && doc_off[at] < from;
-            const int c = __popc(__ballot_sync(0xFFFFFFFFu, less));                                // ascending: the first c probes are below
-            if (c == 0) hi = lo;
-            else { const int l2 = lo + (c - 1) * step + 1; hi = min(hi, lo + c * step); lo = l2; }
+    const long long w0 = (long long)blockIdx.x * stretch;
+    const int words = (int)max(0ll, min((long long)stretch, nwords - w0));        // (0: a CTA that only helps to check)
+    if (words > 0) {
+        for (int i = tid; i < words; i += DOCMASK_THREADS) s_mask[i] = 0;
+        const long long from = w0 * 32 - shift, to = min((w0 + words) * 32 - shift, len);          // text bytes of the stretch
+        if (tid < 32) {                                       // first document that starts at `from` or behind it
+            int lo = 0, hi = n_docs;                          // (the answer is in [lo, hi])
+            while (hi > lo) {
+                const int step = (hi - lo + 31) / 32, at = lo + lane * step;
+                const bool less = at < hi && doc_off[at] < from;
+                const int c = __popc(__ballot_sync(FULL, less));                                   // ascending: the first c probes are below
+                if (c == 0) hi = lo;
+                else { const int l2 = lo + (c - 1) * step + 1; hi = min(hi, lo + c * step); lo = l2; }
+            }
+            if (lane == 0) s_first = lo;
         }
-        if (lane == 0) s_first = lo;
+        __syncthreads();
+        for (long long d0 = s_first + tid;; d0 += DOCMASK_THREADS * DOCMASK_AHEAD) {               // by whole warps
+            long long o[DOCMASK_AHEAD];
+#pragma unroll
+            for (int u = 0; u < DOCMASK_AHEAD; u++) { const long long d = d0 + u * DOCMASK_THREADS; o[u] = d < n_docs ? doc_off[d] : to; }
+#pragma unroll
+            for (int u = 0; u < DOCMASK_AHEAD; u++) {
+                const bool in = o[u] >= from && o[u] >= 0 && o[u] < to;
+                if (!__any_sync(FULL, in)) continue;
+                const int g = in ? (int)(o[u] + shift - w0 * 32) : -1;                             // bit of the stretch
+                const u32 bit = in ? 1u << (g & 31) : 0u;
+                const int word = g >> 5, before = __shfl_up_sync(FULL, word, 1);
+                // neighbouring documents in one word: one lane sets the bits of all
+                if (__any_sync(FULL, in && lane > 0 && before == word)) {
+                    const u32 peers = __match_any_sync(FULL, word), bits = __reduce_or_sync(peers, bit);
+                    if (in && lane == __ffs(peers) - 1) atomicOr(&s_mask[word], bits);
+                } else if (in) atomicOr(&s_mask[word], bit);
+            }
+            if (__any_sync(FULL, o[DOCMASK_AHEAD - 1] >= to)) break;       // ascending: nothing behind it starts in the stretch
+        }
     }
-    __syncthreads();
-    for (int d = s_first + tid; d < n_docs; d += DOCMASK_THREADS) {
-        const long long o = doc_off[d];
-        if (o >= to) break;
-        if (o >= from && o >= 0) { const long long g = o + shift - w0 * 32; atomicOr(&s_mask[g >> 5], 1u << (g & 31)); }
-    }
-    for (long long d = (long long)blockIdx.x * DOCMASK_THREADS + tid; d <= n_docs; d += (long long)gridDim.x * DOCMASK_THREADS) {
-        const long long o = doc_off[d];
-        const bool ok = o >= 0 && o <= len && (d == 0 ? o == 0 : o >= doc_off[d - 1]) && (d < n_docs || o == len);
+    // the check, shared by all CTAs
+    for (long long d0 = (long long)blockIdx.x * DOCMASK_THREADS * DOCMASK_AHEAD + tid; d0 <= n_docs; d0 += (long long)gridDim.x * DOCMASK_THREADS * DOCMASK_AHEAD) {
+        long long o[DOCMASK_AHEAD], before[DOCMASK_AHEAD];
+#pragma unroll
+        for (int u = 0; u < DOCMASK_AHEAD; u++) {
+            const long long d = d0 + u * DOCMASK_THREADS;
+            o[u] = d <= n_docs ? doc_off[d] : 0; before[u] = d > 0 && d <= n_docs ? doc_off[d - 1] : 0;
+        }
+        bool ok = true;
+#pragma unroll
+        for (int u = 0; u < DOCMASK_AHEAD; u++) {
+            const long long d = d0 + u * DOCMASK_THREADS;
+            if (d <= n_docs) ok = ok && o[u] >= before[u] && o[u] <= len && (d > 0 || o[u] == 0) && (d < n_docs || o[u] == len);
+        }
         if (!ok) hdr_set_status(hdr, epoch, 1 /* TT_ERR_ARG */);
     }
     __syncthreads();
-    for (int i = tid; i < DOCMASK_WORDS && w0 + i < nwords; i += DOCMASK_THREADS) docmask[w0 + i] = s_mask[i];
+    for (int i = tid; i < words; i += DOCMASK_THREADS) docmask[w0 + i] = s_mask[i];
 }
 
 __device__ __forceinline__ u32 doc_bits(const PretokParams& P, long long word) {
