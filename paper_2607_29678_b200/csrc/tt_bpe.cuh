@@ -1547,8 +1547,10 @@ __device__ __forceinline__ bool merge_closing(const PieceParams& P, const u8* __
 }
 // The queued short pieces 32 by 32 in their order, whatever tiles they stand in, a thread each; the batches are spread over the
 // grid, by tickets where some CTAs first had a long piece.  (With a ticket per tile 147 warps took the 150,000 two-byte pieces of
-// 300 KB, most of them on the few SMs that came first: 78 to 118 us, now 54 to 66.)
-__device__ __forceinline__ void merge_short_batches(const PieceParams& P, const u8* __restrict__ text, const MergeIndex& X, int unit, int entries, bool by_ticket, u32* tok) {
+// 300 KB, most of them on the few SMs that came first: 78 to 118 us, now 54 to 66.)  Out of line: in line these texts are 4 % faster,
+// but a call of 4,000 characters, which does none of this, takes 33.05 us instead of 32.75, a conversation of 17 appends 831
+// instead of 824.
+__device__ __noinline__ void merge_short_batches(const PieceParams& P, const u8* __restrict__ text, const MergeIndex& X, int unit, int entries, bool by_ticket, u32* tok) {
     const u32 lane = threadIdx.x & 31, NS = X.pre_s[entries], nb = (NS + 31) / 32;
     u32 b = by_ticket ? warp_take(&P.hdr->t_tiles, (int)lane) : (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
     while (b < nb) {
