@@ -4,13 +4,14 @@
 // GPU hash tables; a round's minimum rank identifies one pair value, merging all its leftmost
 // non-overlapping occurrences equals iterated single merges, and only pairs next to a completed
 // merge need to be probed again.  Work is dispatched by piece length and difficulty:
-//   * the first kernel (k_pretok, fused) has looked every piece up as a whole vocabulary entry (one 32-byte probe) and
+//   * the first kernel (k_pretok, fused) has looked every piece up as a whole vocabulary entry (one sector, at times two) and
 //     left the others in its tile's queue region by length class;
 //   * k_merge (a request) / k_closing + k_merge_bulk (bulk text): a warp per piece (<= 32 bytes: tokens in registers,
 //     candidates as ballot masks; <= 256 bytes: several tokens per lane, compaction through shared memory), or, where
-//     the call has many pieces of <= 32 bytes, 32 of them at once, a thread per piece (lane_merge); longer pieces
-//     are merged by a whole CTA of 768 threads (cta_merge_long: state in shared memory, or in global scratch while
-//     the piece still has more than 14,336 tokens).
+//     the call has many pieces of <= 32 bytes, 32 of them at once, a thread per piece (lane_merge); a longer piece is
+//     merged as runs of bytes if it has few, else cut into windows of 256 bytes, a warp each, that are joined at
+//     shared tokens (see "long pieces"); where windows do not meet, the piece is merged whole by a CTA of 768 threads
+//     (cta_merge_long: state in shared memory, or in global scratch while it still has more than 14,336 tokens).
 // Token ids inside the kernels are "internal": byte b -> b, result of the merge of rank r -> 256 + r;
 // the caller's ids are looked up when the tokens are staged.
 //
@@ -223,8 +224,10 @@ __device__ __forceinline__ bool longtab_lookup(const LongTable& tab, const u8* _
     return false;
 }
 
-// Internal token -> the caller's id.  Where the ids are the internal ones plus a constant (bytes first, results in order of
-// rank, as trainers number them) no table is read.
+// Internal token -> the caller's id.  Where the ids are the internal ones plus a constant (bytes in order first, results in order of
+// rank) no table is read: 1M chars of Thai-like text 84.0 us, with the table 85.6; 1M of transcripts 32.9 and 33.1.  Vocabularies
+// that permute the bytes, as GPT-2's do, take the table.  (The constant for the results and the table for the bytes only: no
+// faster than the table for those, and 1 to 3 % slower for the others.)
 struct ExtMap {
     const int32_t* id; int32_t delta; bool plain;
     __device__ __forceinline__ int32_t operator[](u32 t) const { return plain ? (int32_t)t + delta : id[t]; }
@@ -771,16 +774,15 @@ struct PieceParams {
 
 // ---- K4, second half: the merges ------------------------------------------------------------------------------
 // Work of this kernel: the unsettled pieces the first kernel queued per tile, and the last piece of every tile.
-//   (A) pieces of more than 256 bytes, a whole CTA each: every CTA looks through a contiguous share of the
-//       tiles (the in-tile long pieces the first kernel listed, and tile-closing pieces that turn out long).
-//   (B) everything else, warp by warp, without any barrier:
-//       - a request (few tiles, few unsettled pieces): job j belongs to warp j of the grid.  Jobs are numbered
-//         warp-class pieces first (the longest chains), then the tile-closing pieces, then the short pieces;
-//         a warp finds its job from the per-tile counts alone (every lane sums a stretch of tiles, one warp
-//         scan), so nothing is handed out through a counter.  One warp per piece, tokens in registers.
-//       - bulk text: the warp-class pieces stand in one global list (they come in clusters; a list lets every warp
-//         take its share), then warps draw tickets of one tile and settle its short pieces 32 at a time, a thread
-//         each (lane_merge); pieces wait in the lanes across tickets until 32 are together.
+// A request (k_merge): every CTA scans the tiles' counts once (merge_index), so that a warp finds any queued piece by bisection
+// and nothing is handed out through a list.  Then
+//   - pieces of more than 256 bytes, where a tile allows for one (cta_find_long): those of every gridDim.x-th tile by a CTA, or,
+//     if one is too long for that, by tickets, its windows later by the whole grid (long_phase);
+//   - everything else by warps, without a barrier: job j is warp j's, in the order warp-class pieces (the longest chains),
+//     closing pieces of the tiles, short pieces; by tickets where CTAs had long pieces first.  With many short pieces these go 32
+//     by 32, a thread each (merge_short_batches).
+// Bulk text (k_merge_bulk): k_closing has gathered global lists.  Long pieces by tickets of a CTA, warp-class pieces a warp each
+// by index, short pieces by tickets of 32 of one length class, a thread each, the longest class first.
 #ifndef TT_MERGE_WARPS
 #define TT_MERGE_WARPS 24
 #endif
@@ -789,14 +791,14 @@ constexpr int MERGE_THREADS = MERGE_WARPS * 32;
 constexpr int WARP_SMEM_WORDS = 1024;                 // u64 per warp: two lane-path arrays of 32 x 32 u32, or two copies of four 256-word merge arrays
 static_assert(MERGE_WARPS * WARP_SMEM_WORDS * sizeof(u64) >= LONG_SMEM_SLOTS * (sizeof(u64) + sizeof(u32)), "the CTA's buffer must hold a long piece");
 static_assert(LONG_SMEM_TOKENS >= MERGE_WARPS * 32 * LK, "the survivors of a chunk (threads x LK positions) must fit the shared buffer");
-constexpr size_t MERGE_SMEM_BYTES = (size_t)MERGE_WARPS * WARP_SMEM_WORDS * sizeof(u64);   // dynamic shared memory of k_merge (64 KiB)
+constexpr size_t MERGE_SMEM_BYTES = (size_t)MERGE_WARPS * WARP_SMEM_WORDS * sizeof(u64);   // dynamic shared memory of k_merge_bulk (192 KiB)
 static_assert(WARP_SMEM_WORDS * sizeof(u64) >= 2 * LANE_SLOTS * LANE_MAX * sizeof(u32) && WARP_SMEM_WORDS * sizeof(u64) >= 2 * 4 * TT_WARP_PIECE_MAX * sizeof(u32), "per-warp buffer");
 constexpr int MERGE_SR_MAX_TILES = 2048;              // the per-warp job search covers at most 32 lanes x 64 tiles
 
 #ifndef TT_MERGE_CTAS_PER_SM
 #define TT_MERGE_CTAS_PER_SM 1
 #endif
-constexpr int MERGE_CTAS_PER_SM = TT_MERGE_CTAS_PER_SM;   // resident CTAs per SM (registers and the 64 KiB of shared memory each)
+constexpr int MERGE_CTAS_PER_SM = TT_MERGE_CTAS_PER_SM;   // resident CTAs per SM (registers and the 192 KiB of shared memory each)
 
 // End (aligned frame) of the piece that starts last in `tile`: the first piece start of a later tile, or the text end.
 __device__ __forceinline__ u32 closing_piece_end(const PieceParams& P, int tile) {
@@ -898,7 +900,7 @@ k_closing(const __grid_constant__ PieceParams P) {
         }
         if (cn > (u32)TT_WARP_PIECE_MAX) P.lq[b] = make_uint4(ca, cn, cslot, 0u);
     }
-    // short pieces: three lists by length (a warp later merges 32 pieces of one list at a time, a thread each, and
+    // short pieces: four lists by length (a warp later merges 32 pieces of one list at a time, a thread each, and
     // waits for the longest), one reservation per warp and list
     u64 mine = 0;                                             // four counts of 16 bits (a warp's 32 tiles hold fewer than 2^16 pieces)
 #pragma unroll

@@ -40,7 +40,6 @@ enum : u32 { CC_OTHER = 0, CC_MARK = 1, CC_SPACE = 2, CC_NUMBER = 3, CC_LOWER = 
 constexpr u32 TT_ID_BITS = 18;                    // internal ids: byte b -> b, merge of rank r -> 256 + r
 constexpr u32 TT_MAX_INTERNAL = 1u << TT_ID_BITS;
 constexpr u32 TT_RANK_INF = 0xFFFFFFFFu;
-constexpr u64 TT_SLOT_EMPTY = ~0ull;              // pair-table slot: (left << 38) | (right << 20) | rank
 constexpr int TT_WARP_PIECE_MAX = 256;            // bytes; longer pieces take the block-cooperative path
 // Bulk text: length classes of the pieces of at most 32 bytes (largest length of each class).
 constexpr int TT_SHORT_CLASSES = 4;
@@ -53,9 +52,10 @@ struct TTHeader {
     u32 n_pieces;            // number of pieces found (tt_pretokenize only)
     u32 t_tiles;             // ticket counter of k_merge's batches of short pieces; zeroed by the kernel before it
     u32 merge_done;          // CTAs of k_merge that have finished (bulk text: the last one sums the groups); zeroed likewise
-    u32 nwq;                 // bulk text: lengths of the global lists of warp-class, short and long pieces and the ticket
-    u32 nq_short, nq_long;   //            counter of the short list (all cleared by a memset before the chain)
-    u32 t_short;
+    u32 nwq;                 // bulk text: lengths of the global lists of warp-class and of short pieces,
+    u32 nq_short, nq_long;   // (either) of the list of long ones,
+    u32 t_short;             // and the tickets of the short list, of a request's jobs where CTAs had long pieces first (bulk
+                             // text: all cleared by a memset before the chain; a request: zeroed by the first kernel)
     u32 long_take[6], long_done[6];   // long pieces: tickets and finished tasks of each step (see long_phase); zeroed by the first kernel
     u32 nq_short_x[3];       // bulk text: the short pieces have a list per length class; lengths of the other lists (cleared likewise)
     u32 dbg[8];              // first failed self-check of a kernel: site, then up to seven values (diagnostics only)
@@ -123,7 +123,7 @@ struct TTWorkspace {
     u64* wq;           // bulk text only: warp-class pieces of all tiles (len / 33 + 64 entries)
     u64* gq;           // bulk text only: short pieces of all tiles by length class (see tt_short_class_max): a warp merges 32
     u64* gq_x[3];      // pieces of one list at a time, a thread each, and is done when the longest of them is
-    uint4* lq;         // bulk text only: long pieces of all tiles (len / 257 + 16 entries)
+    uint4* lq;         // long pieces (len / 257 + 16 entries): all of bulk text, those for the whole grid of a request
     int32_t* stage;    // token ids staged at the byte offset of their piece (len)
     u64* pairbuf;      // (token, rank) pairs of the long-piece path, indexed like the text (len)
     u8* cand;          // literal pass: length of the longest added-token literal starting at each byte (aligned frame)
