@@ -741,6 +741,7 @@ extern "C" int tt_encode(const tt_vocab* v, const uint8_t* text, size_t len, voi
 
 extern "C" int tt_vocab_add_literals(tt_vocab* v, const uint8_t* bytes, const uint32_t* off, const int32_t* ids, size_t n) {
     if (!v || v->lit.n != 0 || n == 0 || n > 65535 || !bytes || !off || !ids) return TT_ERR_ARG;
+    static_assert(65535u * 255u < (1u << 24), "an offset and a length share a word");
     std::vector<LitEntry> e(n);
     std::unordered_set<std::string> seen;
     u32 maxlen = 0;
@@ -749,17 +750,19 @@ extern "C" int tt_vocab_add_literals(tt_vocab* v, const uint8_t* bytes, const ui
         if (off[i + 1] <= off[i] || off[i + 1] - off[i] > 255 || ids[i] < 0) return TT_ERR_ARG;
         const u32 len = off[i + 1] - off[i];
         if (!seen.insert(std::string((const char*)bytes + off[i], len)).second) return TT_ERR_ARG;     // the same literal twice
-        u32 f4 = 0;
-        for (u32 k = 0; k < 4 && k < len; k++) f4 |= (u32)bytes[off[i] + k] << (8 * k);
-        e[i].first4 = f4; e[i].off = off[i]; e[i].len = len; e[i].id = ids[i];
+        e[i] = LitEntry{0, 0, ((off[i] - off[0]) << 8) | len, ids[i]};
+        for (u32 k = 0; k < 4 && k < len; k++) e[i].first4 |= (u32)bytes[off[i] + k] << (8 * k);
+        for (u32 k = 4; k < 8 && k < len; k++) e[i].next4 |= (u32)bytes[off[i] + k] << (8 * (k - 4));
         maxlen = maxlen > len ? maxlen : len;
         T.first_byte[bytes[off[i]] >> 5] |= 1u << (bytes[off[i]] & 31);
+        if (len > 1) T.second_byte[bytes[off[i] + 1] >> 5] |= 1u << (bytes[off[i] + 1] & 31);
+        else for (u32& w : T.second_byte) w = 0xFFFFFFFFu;
     }
-    std::stable_sort(e.begin(), e.end(), [](const LitEntry& a, const LitEntry& b) { return a.len > b.len; });
-    const size_t blob = off[n];
+    std::stable_sort(e.begin(), e.end(), [](const LitEntry& a, const LitEntry& b) { return lit_len(a) > lit_len(b); });
+    const size_t blob = off[n] - off[0];                     // (at most 65,535 literals of 255 bytes: the offsets fit 24 bits)
     if (cudaMalloc(&v->d_lit_entries, n * sizeof(LitEntry)) != cudaSuccess || cudaMalloc(&v->d_lit_blob, blob + 16) != cudaSuccess ||
         cudaMemcpy(v->d_lit_entries, e.data(), n * sizeof(LitEntry), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemcpy(v->d_lit_blob, bytes, blob, cudaMemcpyHostToDevice) != cudaSuccess) {
+        cudaMemcpy(v->d_lit_blob, bytes + off[0], blob, cudaMemcpyHostToDevice) != cudaSuccess) {
         cudaGetLastError(); cudaFree(v->d_lit_entries); cudaFree(v->d_lit_blob); v->d_lit_entries = nullptr; v->d_lit_blob = nullptr;
         return TT_ERR_CUDA;
     }
