@@ -72,7 +72,8 @@ __device__ __forceinline__ PairInfo pair_probe(const PairTable& t, u32 a, u32 b)
     const u32 h0 = pair_bucket(key, t.shift), h1 = pair_bucket_alt(key, t.shift, h0);
     const uint4* b0 = t.slots + 2 * (size_t)h0;
     const uint4* b1 = t.slots + 2 * (size_t)h1;
-    const uint4 x0 = __ldg(b0), y0 = __ldg(b0 + 1), x1 = __ldg(b1), y1 = __ldg(b1 + 1);
+    uint4 x0, y0, x1, y1;
+    ldg_sector(b0, x0, y0); ldg_sector(b1, x1, y1);
     PairInfo out = pair_none();
     if (!pair_match(x0, key, out) && !pair_match(y0, key, out) && !pair_match(x1, key, out)) pair_match(y1, key, out);
     return out;
@@ -157,7 +158,8 @@ __device__ __forceinline__ bool toktab_short(const TokTable& tab, const uint4 e0
     if (toktab_short_match(e0, n, k0, k1, val) || toktab_short_match(e1, n, k0, k1, val)) return true;
     if (!(e0.x & TOK_OVERFLOW)) return false;
     const uint4* const b = tab.shorts + 2 * (size_t)toktab_bucket_alt(h, tab.short_shift);
-    const uint4 f0 = __ldg(b), f1 = __ldg(b + 1);
+    uint4 f0, f1;
+    ldg_sector(b, f0, f1);
     return toktab_short_match(f0, n, k0, k1, val) || toktab_short_match(f1, n, k0, k1, val);
 }
 // Looks a piece of 1..24 bytes up; returns true and the id on a hit.  (The first kernel has its own copy of the
@@ -177,7 +179,9 @@ __device__ __forceinline__ bool toktab_lookup(const TokTable& tab, const u8* __r
         const u32 h = toktab_hash_final(s);
         const uint4* const b = tab.shorts + 2 * (size_t)toktab_bucket(h, tab.short_shift);
         u32 val = 0;
-        const bool hit = toktab_short(tab, __ldg(b), __ldg(b + 1), h, n, k[0], k[1], val);
+        uint4 e0, e1;
+        ldg_sector(b, e0, e1);
+        const bool hit = toktab_short(tab, e0, e1, h, n, k[0], k[1], val);
         id = (int32_t)val;
         return hit;
     }
@@ -185,8 +189,8 @@ __device__ __forceinline__ bool toktab_lookup(const TokTable& tab, const u8* __r
     u32 at = toktab_bucket(h, tab.shift);
 #pragma unroll 1
     for (int probe = 0; probe < 2; probe++) {
-        const uint4* const sp = reinterpret_cast<const uint4*>(tab.slots + at);
-        const uint4 lo = __ldg(sp), hi = __ldg(sp + 1);
+        uint4 lo, hi;
+        ldg_sector(reinterpret_cast<const uint4*>(tab.slots + at), lo, hi);
         if ((((lo.x ^ n) & TOK_LEN) | (lo.z ^ k[0]) | (lo.w ^ k[1]) | (hi.x ^ k[2]) | (hi.y ^ k[3]) | (hi.z ^ k[4]) | (hi.w ^ k[5])) == 0) { id = (int32_t)lo.y; return true; }
         if (!(lo.x & TOK_OVERFLOW)) return false;
         at = toktab_bucket_alt(h, tab.shift);
@@ -415,8 +419,8 @@ __device__ __forceinline__ void pair_probe2(const PairTable& t, u32 a0, u32 b0, 
     const u32 h10 = pair_bucket(key1, t.shift), h11 = pair_bucket_alt(key1, t.shift, h10);
     const uint4* p00 = t.slots + 2 * (size_t)h00; const uint4* p01 = t.slots + 2 * (size_t)h01;
     const uint4* p10 = t.slots + 2 * (size_t)h10; const uint4* p11 = t.slots + 2 * (size_t)h11;
-    const uint4 a00 = __ldg(p00), a01 = __ldg(p00 + 1), a02 = __ldg(p01), a03 = __ldg(p01 + 1);
-    const uint4 a10 = __ldg(p10), a11 = __ldg(p10 + 1), a12 = __ldg(p11), a13 = __ldg(p11 + 1);
+    uint4 a00, a01, a02, a03, a10, a11, a12, a13;
+    ldg_sector(p00, a00, a01); ldg_sector(p01, a02, a03); ldg_sector(p10, a10, a11); ldg_sector(p11, a12, a13);
     PairInfo q0 = pair_none(), q1 = pair_none();
     if (!pair_match(a00, key0, q0) && !pair_match(a01, key0, q0) && !pair_match(a02, key0, q0)) pair_match(a03, key0, q0);
     if (!pair_match(a10, key1, q1) && !pair_match(a11, key1, q1) && !pair_match(a12, key1, q1)) pair_match(a13, key1, q1);

@@ -550,8 +550,7 @@ k_pretok(const __grid_constant__ PretokParams P, const __grid_constant__ FrontPa
                     const u32* const w = tw + (o[j] >> 2);
                     toktab_key01(w[0], w[1], w[2], o[j] & 3, n[j], k0[j], k1[j]);
                     h[j] = toktab_hash_final(toktab_hash_short(F.toktab, k0[j], k1[j], n[j]));
-                    const uint4* const b = F.toktab.shorts + 2 * (size_t)toktab_bucket(h[j], F.toktab.short_shift);
-                    sl[j] = __ldg(b); sm2[j] = __ldg(b + 1);
+                    ldg_sector(F.toktab.shorts + 2 * (size_t)toktab_bucket(h[j], F.toktab.short_shift), sl[j], sm2[j]);
                 }
             }
 #pragma unroll
