@@ -714,7 +714,7 @@ static int encode_impl(const tt_vocab* v, const uint8_t* text, size_t len, const
     CK(launch_after(big ? k_merge_bulk : k_merge, merge_grid, MERGE_THREADS, st, big ? MERGE_SMEM_BYTES : MERGE_SMEM_REQUEST, ev == nullptr, Q));
     MARK(2);
     ScatterParams S;
-    S.shift = PP.lo; S.hi = PP.hi; S.ntiles = PP.ntiles; S.tile_cnt = w.tile_cnt; S.tile_tok = w.tile_tok; S.grp_tok = Q.grp_tok; S.piece_off16 = w.piece_off16;
+    S.shift = PP.lo; S.hi = PP.hi; S.ntiles = PP.ntiles; S.tile_cnt = w.tile_cnt; S.tile_tok = w.tile_tok; S.grp_tok = Q.grp_tok; S.piece_off16 = w.piece_off16; S.tile_q = w.tile_q;
     S.ids_cap = (unsigned long long)ids_cap; S.piece_cnt = w.piece_cnt; S.stage = w.stage; S.hdr = w.hdr; S.epoch = PP.epoch;
     S.ids_out = ids_out; S.count_out = (long long*)count_out; S.status_out = status_out;
     S.docmask = doc_off ? w.docmask : nullptr; S.doc_off = (const long long*)doc_off; S.n_docs = (int)n_docs;

@@ -743,6 +743,7 @@ __device__ u32 cta_merge_long(const u8* __restrict__ text, u32 a, u32 n, const P
 // settles it, looking the end up in tile_first of the following tiles.
 __device__ __forceinline__ u32 tile_queue_entry(u32 off, u32 idx, u32 n) { return off | (idx << 11) | ((n - 1) << 22); }
 constexpr u32 TQ_MAY_LONG = 0x80000000u;              // tile_q: the tile allows for a piece of more than 256 bytes (see k_pretok)
+constexpr u32 TQ_HAS_DOC = 0x40000000u;               // tile_q, bulk text: a document starts in the tile
 constexpr u32 TQ_NS_MASK = 0x7FFu, TQ_NW_SHIFT = 11, TQ_NW_MASK = 0x7Fu, TQ_NL_SHIFT = 18, TQ_NL_MASK = 0xFu;
 
 struct PieceParams {
@@ -813,12 +814,19 @@ __device__ __forceinline__ u32 closing_piece_end(const PieceParams& P, int tile)
     return (u32)P.hi;
 }
 
+// Bulk text: what k_scatter_bulk needs of a merged piece in one word -- bit 31, its number of ids (20 bits), its offset in the tile -- so that
+// the pieces' offsets are neither written nor read (2 bytes a piece, both ways; see k_scatter_bulk).  PIECE_MANY: at least as many ids;
+// such a piece covers the whole tile behind the one it starts in, and the first word of that one's pieces holds the number.
+constexpr u32 PIECE_STAGED = 0x80000000u, PIECE_MANY = 0xFFFFFu;
+static_assert(PIECE_MANY >= 2 * TT_TILE_BYTES, "a piece of so many bytes covers the tile behind its own");
+TT_HD u32 piece_staged_word(u32 off, u32 m) { return PIECE_STAGED | (m << 11) | off; }
+
 // A piece that needs no merging: an extracted literal (its id is staged already), a single byte, or a whole
 // vocabulary entry.  Returns true and the value for piece_cnt.  One thread.
 __device__ __forceinline__ bool piece_settled_without_merge(const PieceParams& P, const u8* __restrict__ text, u32 a, u32 n, u32& value) {
     if (P.litstart != nullptr) {
         const long long g = (long long)a + P.shift;
-        if ((P.litstart[g >> 5] >> (g & 31)) & 1) { value = 0u - 1u; return true; }
+        if ((P.litstart[g >> 5] >> (g & 31)) & 1) { value = P.gq != nullptr ? piece_staged_word((u32)(g % TT_TILE_BYTES), 1u) : 0u - 1u; return true; }
     }
     int32_t id;
     if (n == 1) { value = (u32)P.ext_id[text[a]]; return true; }
@@ -828,8 +836,11 @@ __device__ __forceinline__ bool piece_settled_without_merge(const PieceParams& P
     return false;
 }
 
-__device__ __forceinline__ void piece_done(const PieceParams& P, u32 slot, u32 m) {
-    P.piece_cnt[slot] = 0u - m;
+__device__ __forceinline__ void piece_done(const PieceParams& P, u32 a, u32 slot, u32 m) {
+    if (P.gq != nullptr) {
+        P.piece_cnt[slot] = piece_staged_word((u32)(a + P.shift) % TT_TILE_BYTES, min(m, PIECE_MANY));
+        if (m >= PIECE_MANY) P.piece_cnt[(slot / TT_TILE_BYTES + 1) * TT_TILE_BYTES] = m;
+    } else P.piece_cnt[slot] = 0u - m;
     atomicAdd(&P.tile_tok[slot / TT_TILE_BYTES], m);
 }
 
@@ -847,7 +858,7 @@ __device__ __forceinline__ void warp_merge_piece(const PieceParams& P, const u8*
                 : n <= 64 ? warp_merge_perm<2>(pbuf, text, a, n, P.tab, lane, out)
                 : n <= 128 ? warp_merge_perm<4>(pbuf, text, a, n, P.tab, lane, out)
                            : warp_merge_perm<WCH>(pbuf, text, a, n, P.tab, lane, out);
-    if (lane == 0) piece_done(P, slot, m);
+    if (lane == 0) piece_done(P, a, slot, m);
 }
 
 // ---- bulk text only: the closing pieces, and one list per length class for the whole text ---------------------
@@ -1114,7 +1125,7 @@ __device__ __noinline__ bool cta_run_piece(const PieceParams& P, const u8* __res
         const int32_t id = P.ext_id[LS.rtok[r]];
         for (u32 j = (r ? LS.rcnt[r - 1] : 0u) + tid; j < LS.rcnt[r]; j += T) P.stage[a + j] = id;
     }
-    if (tid == 0) piece_done(P, slot, total);
+    if (tid == 0) piece_done(P, a, slot, total);
     __syncthreads();
     return true;
 }
@@ -1219,7 +1230,7 @@ __device__ __noinline__ void cta_window_piece(const PieceParams& P, const u8* __
         for (int w = 0; w < MERGE_WARPS; w++) { const u32 c = sc[w]; total += c; if (w < wid) at += c; }
         long_write(P, q, k, left, right, at, lane);
     } else total = cta_merge_long(text, q.x, q.y, P.tab, P.ext_id, P.stage, P.pairbuf + q.x, s_buf, sc);
-    if (threadIdx.x == 0) piece_done(P, q.z, total);
+    if (threadIdx.x == 0) piece_done(P, q.x, q.z, total);
     __syncthreads();
 }
 // What a CTA does with a long piece that it comes upon; false: the piece is for the whole grid.  many: so are all but runs of bytes.
@@ -1280,7 +1291,7 @@ __device__ __noinline__ void long_phase(const PieceParams& P, const u8* __restri
                 carry += total;
                 __syncthreads();
             }
-            if (tid == 0) piece_done(P, q.z, carry);
+            if (tid == 0) piece_done(P, q.x, q.z, carry);
         }
         __syncthreads();
         if (tid == 0 && mine) long_did(P, 3, mine);
@@ -1297,7 +1308,7 @@ __device__ __noinline__ void long_phase(const PieceParams& P, const u8* __restri
         const uint4 q = __ldcg(&P.lq[e]);
         if (q.w != LQ_FALLBACK) continue;
         const u32 m = cta_merge_long(text, q.x, q.y, P.tab, P.ext_id, P.stage, P.pairbuf + q.x, s_buf, sc);
-        if (tid == 0) piece_done(P, q.z, m);
+        if (tid == 0) piece_done(P, q.x, q.z, m);
     }
     __syncthreads();
 }
@@ -1447,7 +1458,7 @@ __device__ void merge_bulk_lists(const PieceParams& P, const u8* __restrict__ te
             if (!piece_in_range(P, a, n, slot, 4u) || n < 2 || n > (u32)LANE_MAX) hdr_selfcheck_failed(P.hdr, P.epoch, 5u, a, n, slot, e0);
             else {
                 const u32 m = lane_merge(tok, tok + LANE_SLOTS * LANE_MAX, lane, text, a, n, P.tab, P.ext_id, P.stage);
-                piece_done(P, slot, m);
+                piece_done(P, a, slot, m);
             }
         }
         __syncwarp();
@@ -1565,7 +1576,7 @@ __device__ __noinline__ void merge_short_batches(const PieceParams& P, const u8*
             u32 a, n, slot;
             merge_queued(P, X, unit, entries, false, k, a, n, slot);
             if (!piece_in_range(P, a, n, slot, 4u) || n < 2 || n > (u32)LANE_MAX) hdr_selfcheck_failed(P.hdr, P.epoch, 5u, a, n, slot, k);
-            else piece_done(P, slot, lane_merge(tok, tok + LANE_SLOTS * LANE_MAX, (int)lane, text, a, n, P.tab, P.ext_id, P.stage));
+            else piece_done(P, a, slot, lane_merge(tok, tok + LANE_SLOTS * LANE_MAX, (int)lane, text, a, n, P.tab, P.ext_id, P.stage));
         }
         __syncwarp();
         b = by_ticket ? warp_take(&P.hdr->t_tiles, (int)lane) : b + gridDim.x * MERGE_WARPS;
@@ -1634,6 +1645,7 @@ struct ScatterParams {
     const u32* tile_tok;       // tokens per tile
     const u32* grp_tok;        // bulk text: tokens per group of TT_GROUP_TILES tiles, else null
     const u16* piece_off16;
+    const u32* tile_q;         // bulk text: says where a document starts in the tile
     unsigned long long ids_cap;
     const u32* piece_cnt;
     const int32_t* stage;
@@ -1805,15 +1817,18 @@ k_scatter(const __grid_constant__ ScatterParams P) {
 
 // ---- K5 for bulk text: a warp per tile, no barrier after the prologue -----------------------------------------
 // Each CTA takes a contiguous range of tiles, its warps every eighth tile of it.  A warp knows where its tile's ids
-// go from the token counts of the tiles before it (group totals, then tile counts), scans the tile's pieces 128 at
-// a time (four neighbouring pieces per lane, one 16-byte load) with warp shuffles, and copies pieces of more than
-// eight tokens with all its lanes.
-// SCATTER_BULK_CTAS CTAs per SM: as many as are resident, so that the ranges are one wave (twice as many: 20 MB of Unicode-heavy
-// text 477 -> 453 us per call with one).
-constexpr int SCATTER_BULK_CTAS = 4;
+// go from the token counts of the tiles before it (group totals, then tile counts) and takes the tile's pieces 32 by 32, one per
+// lane, the loads of SCATTER_AHEAD such groups in flight: loads and stores are whole lines, a group without merged pieces (two
+// thirds of the transcripts' groups) needs no scan, and merged pieces are listed and copied many at a time.  What bounds it is
+// instruction issue.  (Four neighbouring pieces per lane, scanned in any case, with their offsets: 132 MB batch 897 us a call, so
+// 838; the loop kept short on purpose: unrolled eight times it waited for instructions, 871.)
+// SCATTER_BULK_CTAS CTAs per SM: as many as are resident, so that the ranges are one wave (132 MB batch: 5 CTAs 806 us, 6 796, 8 with
+// 32 registers 864).
+constexpr int SCATTER_BULK_CTAS = 6, SCATTER_AHEAD = 4, SCATTER_LIST = 64, SCATTER_NEXT = 14;
 __global__ void __launch_bounds__(BPE_THREADS, SCATTER_BULK_CTAS)
 k_scatter_bulk(const __grid_constant__ ScatterParams P) {
     __shared__ unsigned long long s_sum[66];
+    __shared__ uint3 s_list[BPE_WARPS][SCATTER_LIST];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const u32 FULL = 0xFFFFFFFFu;
     cudaGridDependencySynchronize();                         // k_merge_bulk's (and with it the kernels' before it) results are complete
@@ -1839,93 +1854,107 @@ k_scatter_bulk(const __grid_constant__ ScatterParams P) {
         return;
     }
     if (P.ids_off_out && blockIdx.x == 0) {
-        const long long len = P.hi - P.shift;
-        for (int d = P.n_docs - tid; d >= 0 && P.doc_off[d] >= len; d -= blockDim.x) P.ids_off_out[d] = (long long)total;
+        for (int d = P.n_docs - tid; d >= 0 && P.doc_off[d] >= P.hi - P.shift; d -= blockDim.x) P.ids_off_out[d] = (long long)total;
     }
     // tokens of the tiles of this CTA's range before the warp's first tile
     u32 carry = (u32)before;
     {
-        u32 x = (lane < wid && tile_lo + lane < tile_hi) ? P.tile_tok[tile_lo + lane] : 0u;
-#pragma unroll
-        for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(FULL, x, o);
-        carry += x;
+        const u32 x = (lane < wid && tile_lo + lane < tile_hi) ? P.tile_tok[tile_lo + lane] : 0u;
+        carry += __reduce_add_sync(FULL, x);
     }
+    const long long len = P.hi - P.shift;
+    const u32 total32 = (u32)total;                          // (a text has fewer than 2^31 bytes)
+    uint3* const list = s_list[wid];                         // merged pieces that are still to be copied: source, destination, ids
+    u32 listed = 0;
+    // a lane each, all loads side by side; pieces of more than eight ids by the whole warp, four loads in flight per lane
+    const auto copy_listed = [&]() {
+        __syncwarp();
+#pragma unroll 1
+        for (u32 e0 = 0; e0 < listed; e0 += 32) {
+            uint3 e = make_uint3(0, 0, 0);
+            if (e0 + lane < listed) e = list[e0 + lane];
+            const u32 few = e.z <= 8 ? e.z : 0u;
+            int32_t id[8];
+#pragma unroll
+            for (int k = 0; k < 8; k++) id[k] = (u32)k < few ? P.stage[e.x + k] : 0;
+#pragma unroll
+            for (int k = 0; k < 8; k++) if ((u32)k < few) P.ids_out[e.y + k] = id[k];
+#pragma unroll 1
+            for (u32 m = __ballot_sync(FULL, e.z > 8); m; m &= m - 1) {                   // warp-uniform
+                const int l = __ffs(m) - 1;
+                const u32 s2 = __shfl_sync(FULL, e.x, l), d2 = __shfl_sync(FULL, e.y, l), c2 = __shfl_sync(FULL, e.z, l);
+#pragma unroll 1
+                for (u32 k0 = lane; k0 < c2; k0 += 128) {
+                    int32_t x[4];
+#pragma unroll
+                    for (int u = 0; u < 4; u++) x[u] = k0 + 32 * u < c2 ? P.stage[s2 + k0 + 32 * u] : 0;
+#pragma unroll
+                    for (int u = 0; u < 4; u++) if (k0 + 32 * u < c2) P.ids_out[d2 + k0 + 32 * u] = x[u];
+                }
+            }
+        }
+        listed = 0;
+        __syncwarp();
+    };
+#pragma unroll 1
     for (int tile = tile_lo + wid; tile < tile_hi; tile += BPE_WARPS) {   // warp-uniform
+        const u32* const pc = P.piece_cnt + (size_t)tile * TT_TILE_BYTES;
+        // the tile's first pieces, asked for before their number is known (the array has a place for every byte)
+        u32 v[SCATTER_AHEAD];
+#pragma unroll
+        for (int g = 0; g < SCATTER_AHEAD; g++) v[g] = pc[32 * g + lane];
+        // ... and those of the warp's next tile brought into L2
+        if (lane < SCATTER_NEXT && tile + BPE_WARPS < tile_hi) asm volatile("prefetch.global.L2 [%0];" ::"l"(pc + BPE_WARPS * TT_TILE_BYTES + 32 * lane));
         const u32 np = P.tile_cnt[tile];
+        // does any document start in this tile?  (few tiles: the pieces of the others need not look)
+        const bool tile_has_doc = P.docmask != nullptr && (P.tile_q[tile] & TQ_HAS_DOC) != 0;
         // the seven tiles between this one and the warp's next
         u32 skip = (lane >= 1 && lane < BPE_WARPS && tile + lane < tile_hi) ? P.tile_tok[tile + lane] : 0u;
-        const size_t p0 = (size_t)tile * TT_TILE_BYTES;
         const long long t0 = (long long)tile * TT_TILE_BYTES - P.shift;      // text offset of the tile start
-        // does any document start in this tile?  (few tiles: the pieces of the others need not look)
-        bool tile_has_doc = false;
-        if (P.docmask) {
-            const size_t wi = (size_t)tile * (TT_TILE_BYTES / 32) + 2 * lane, nwords = (size_t)(P.hi >> 5) + 4;   // (the mask's cleared extent)
-            uint2 dm = make_uint2(0, 0);
-            if (wi + 1 < nwords) dm = *reinterpret_cast<const uint2*>(P.docmask + wi);
-            else if (wi < nwords) dm.x = P.docmask[wi];
-            tile_has_doc = __any_sync(FULL, (dm.x | dm.y) != 0);
-        }
         u32 run = carry;
-        uint4 v = make_uint4(0, 0, 0, 0);
-        uint2 o4 = make_uint2(0, 0);
-        if (4u * lane < np) { v = *reinterpret_cast<const uint4*>(P.piece_cnt + p0 + 4 * lane); o4 = *reinterpret_cast<const uint2*>(P.piece_off16 + p0 + 4 * lane); }
-        for (u32 b = 0; b < np; b += 128) {                               // warp-uniform
-            // the next 128 pieces
-            uint4 vn = make_uint4(0, 0, 0, 0);
-            uint2 on = make_uint2(0, 0);
-            const u32 j0 = b + 128 + 4 * lane;
-            if (j0 < np) { vn = *reinterpret_cast<const uint4*>(P.piece_cnt + p0 + j0); on = *reinterpret_cast<const uint2*>(P.piece_off16 + p0 + j0); }
-            const u32 i0 = b + 4 * lane;
-            const int32_t x[4] = {(int32_t)v.x, (int32_t)v.y, (int32_t)v.z, (int32_t)v.w};
-            const u32 off[4] = {o4.x & 0xFFFFu, o4.x >> 16, o4.y & 0xFFFFu, o4.y >> 16};
-            u32 c[4], mine = 0;
+#pragma unroll 1
+        for (u32 b = 0; b < np; b += 32) {                                // warp-uniform
+            const u32 i = b + lane, x = v[0];
 #pragma unroll
-            for (int h = 0; h < 4; h++) { c[h] = i0 + h < np ? (x[h] >= 0 ? 1u : (u32)(-x[h])) : 0u; mine += c[h]; }
-            u32 inc = mine;
+            for (int g = 0; g + 1 < SCATTER_AHEAD; g++) v[g] = v[g + 1];
+            if (i + 32 * SCATTER_AHEAD < np) v[SCATTER_AHEAD - 1] = pc[i + 32 * SCATTER_AHEAD];
+            const bool in = i < np, staged = in && (int32_t)x < 0;
+            const u32 m = __ballot_sync(FULL, staged);
+            u32 dst = run + lane;
+            run += min(32u, np - b);
+            if (m) {
+                u32 c = in ? 1u : 0u;
+                if (staged) { c = (x >> 11) & PIECE_MANY; if (c == PIECE_MANY) c = pc[TT_TILE_BYTES]; }
+                u32 inc = c;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) { const u32 y = __shfl_up_sync(FULL, inc, o); if (lane >= o) inc += y; }
-            const u32 tot = __shfl_sync(FULL, inc, 31);
-            u32 dst = run + inc - mine;
-            u32 bigmask = 0;                                              // which of my four pieces have more than eight tokens
-#pragma unroll
-            for (int h = 0; h < 4; h++) {
-                const u32 i = i0 + h;
-                if (i < np) {
-                    const u32 src = (u32)(t0 + off[h]);
-                    if ((unsigned long long)dst + c[h] > total || (x[h] < 0 && t0 + off[h] + c[h] > P.hi - P.shift)) hdr_selfcheck_failed(P.hdr, P.epoch, 7u, (u32)tile, i, (u32)x[h], dst);
-                    else if (x[h] >= 0) P.ids_out[dst] = x[h];
-                    else if (c[h] <= 8) { for (u32 kk = 0; kk < c[h]; kk++) P.ids_out[dst + kk] = P.stage[src + kk]; }
-                    else bigmask |= 1u << h;
-                    if (tile_has_doc) {
-                        const long long g = (long long)tile * TT_TILE_BYTES + off[h];
-                        if ((P.docmask[g >> 5] >> (g & 31)) & 1) {
-                            // every document that starts at this byte (empty ones included) gets this token offset
-                            const long long want = g - P.shift;
-                            int lo = 0, hi2 = P.n_docs;
-                            while (lo < hi2) { int mid = (lo + hi2) >> 1; if (P.doc_off[mid] < want) lo = mid + 1; else hi2 = mid; }
-                            for (int d = lo; d <= P.n_docs && P.doc_off[d] == want; d++) P.ids_off_out[d] = dst;
-                        }
-                    }
+                for (int o = 1; o < 32; o <<= 1) { const u32 y = __shfl_up_sync(FULL, inc, o); if (lane >= o) inc += y; }
+                dst += inc - c - lane; run = dst - (inc - c) + __shfl_sync(FULL, inc, 31);
+                if (staged) {
+                    const u32 src = (u32)(t0 + (x & (TT_TILE_BYTES - 1)));
+                    const bool fits = c <= total32 && dst <= total32 - c && (long long)src + c <= len;
+                    if (!fits) hdr_selfcheck_failed(P.hdr, P.epoch, 7u, (u32)tile, i, x, dst);
+                    list[listed + __popc(m & ((1u << lane) - 1))] = make_uint3(src, dst, fits ? c : 0u);
                 }
-                dst += c[h];
+                listed += __popc(m);
+                if (listed > SCATTER_LIST - 32) copy_listed();
             }
-            // pieces of more than eight tokens: copied by the whole warp, one after the other
-#pragma unroll
-            for (int h = 0; h < 4; h++) {
-                for (u32 m = __ballot_sync(FULL, (bigmask >> h) & 1); m; m &= m - 1) {     // warp-uniform
-                    const int l = __ffs(m) - 1;
-                    u32 d2 = run + inc - mine;
-#pragma unroll
-                    for (int g = 0; g < 4; g++) if (g < h) d2 += c[g];
-                    const u32 src = __shfl_sync(FULL, (u32)(t0 + off[h]), l), dd = __shfl_sync(FULL, d2, l), cc = __shfl_sync(FULL, c[h], l);
-                    for (u32 kk = lane; kk < cc; kk += 32) P.ids_out[dd + kk] = P.stage[src + kk];
+            if (in && !staged) {
+                if (dst < total32) P.ids_out[dst] = (int32_t)x;
+                else hdr_selfcheck_failed(P.hdr, P.epoch, 7u, (u32)tile, i, x, dst);
+            }
+            if (tile_has_doc && in) {
+                const long long gpos = (long long)tile * TT_TILE_BYTES + P.piece_off16[(size_t)tile * TT_TILE_BYTES + i];
+                if ((P.docmask[gpos >> 5] >> (gpos & 31)) & 1) {
+                    // every document that starts at this byte (empty ones included) gets this token offset
+                    const long long want = gpos - P.shift;
+                    int lo = 0, hi2 = P.n_docs;
+                    while (lo < hi2) { int mid = (lo + hi2) >> 1; if (P.doc_off[mid] < want) lo = mid + 1; else hi2 = mid; }
+                    for (int d = lo; d <= P.n_docs && P.doc_off[d] == want; d++) P.ids_off_out[d] = dst;
                 }
             }
-            run += tot;
-            v = vn; o4 = on;
         }
-#pragma unroll
-        for (int o = 16; o; o >>= 1) skip += __shfl_xor_sync(FULL, skip, o);
-        carry = run + skip;
+        if (listed > SCATTER_LIST / 4) copy_listed();
+        carry = run + __reduce_add_sync(FULL, skip);
     }
+    if (listed) copy_listed();
 }

@@ -343,7 +343,10 @@ __device__ __forceinline__ bool front_piece_general(const FrontParams& F, const 
 }
 // An unsettled piece (offset o in the tile, index i, n bytes) goes to the tile's queue of its length class.
 __device__ __forceinline__ void front_piece_queue(const FrontParams& F, int tile, u32 o, u32 i, u32 n, u32* s_ns, u32* s_nw, u32* s_nl, u16* s_wlist) {
-    if (n > (u32)TT_WARP_PIECE_MAX) F.tile_long[(size_t)tile * TT_TILE_LONGCAP + atomicAdd(s_nl, 1u)] = (u16)i;
+    if (n > (u32)TT_WARP_PIECE_MAX) {
+        F.tile_long[(size_t)tile * TT_TILE_LONGCAP + atomicAdd(s_nl, 1u)] = (u16)i;
+        if (F.wq != nullptr) { u16* const at = F.piece_off16 + (size_t)tile * TT_TILE_BYTES + i; at[0] = (u16)o; at[1] = (u16)(o + n); }   // (see k_pretok)
+    }
     else if (n > (u32)LANE_MAX) {
         const u32 k = atomicAdd(s_nw, 1u);
         if (F.wq != nullptr) s_wlist[k] = (u16)i;
@@ -389,6 +392,7 @@ k_pretok(const __grid_constant__ PretokParams P, const __grid_constant__ FrontPa
     __shared__ u32 s_nslow;
     static_assert(NT >= TT_TILE_WORDS && NT % 32 == 0 && TT_TILE_WORDS % 32 == 0, "a thread per word of the tile, whole warps of them (tt_eval_word_p1 asks the warp)");
 
+    constexpr bool BULK = FUSED && NT == PRETOK_THREADS_BULK;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     cudaTriggerProgrammaticLaunchCompletion();               // the next kernel may be placed; it waits for this grid's memory itself
     // the whole-piece table is probed at random a few microseconds from now: ask for it to be brought into L2
@@ -509,7 +513,9 @@ k_pretok(const __grid_constant__ PretokParams P, const __grid_constant__ FrontPa
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) { const u32 t = __shfl_up_sync(0xFFFFFFFFu, x, o); if (lane >= o) x += t; }
         if (has_word && lane == 31) s_wtot[wid] = x;
-        __syncthreads();                                              // (the masks have been read: their place is free)
+        bool has_doc = false;                                         // bulk text: a document starts in the tile
+        if (BULK) has_doc = __syncthreads_or(sm[F_DOC][slot] != 0);
+        else __syncthreads();                                         // (the masks have been read: their place is free)
         u32 np = 0, r = x - cnt;
 #pragma unroll
         for (int w = 0; w < TT_TILE_WORDS / 32; w++) { const u32 v = s_wtot[w]; np += v; if (w < wid) r += v; }
@@ -517,7 +523,8 @@ k_pretok(const __grid_constant__ PretokParams P, const __grid_constant__ FrontPa
         __syncthreads();
         const size_t p0 = (size_t)tile * TT_TILE_BYTES;              // pieces are indexed per tile
         u32 may_long = 0;
-        for (u32 i = tid; i < np; i += NT) F.piece_off16[p0 + i] = s_off[i];
+        // (bulk text: the offsets of a tile are asked for only where a document starts in it, and those of long pieces)
+        if (!BULK || has_doc) for (u32 i = tid; i < np; i += NT) F.piece_off16[p0 + i] = s_off[i];
         if (tid == 0) {
             P.tile_cnt[tile] = np;
             P.tile_first[tile] = np ? (u32)s_off[0] : TT_NONE;
@@ -559,7 +566,7 @@ k_pretok(const __grid_constant__ PretokParams P, const __grid_constant__ FrontPa
                 if (n[j] == 0) continue;
                 bool settled = false;
                 u32 val = 0;
-                if (lit[j]) { val = 0u - 1u; settled = true; }         // one staged id (written by the literal pass)
+                if (lit[j]) { val = BULK ? piece_staged_word(o[j], 1u) : 0u - 1u; settled = true; }         // one staged id (written by the literal pass)
                 else if (quick && n[j] <= TT_TOKTAB_SHORT) settled = toktab_short(F.toktab, sl[j], sm2[j], h[j], n[j], k0[j], k1[j], val);
                 else if (quick) { s_slow[atomicAdd(&s_nslow, 1u)] = (u16)i; continue; }     // longer pieces: together, below
                 else settled = front_piece_general(F, tb, o[j], n[j], val);
@@ -583,7 +590,7 @@ k_pretok(const __grid_constant__ PretokParams P, const __grid_constant__ FrontPa
         __syncthreads();
         if (tid == 0) {
             F.tile_tok[tile] = s_total;
-            F.tile_q[tile] = may_long | (s_nl ? TQ_MAY_LONG : 0u) | s_ns | ((F.wq != nullptr ? 0u : s_nw) << TQ_NW_SHIFT) | (s_nl << TQ_NL_SHIFT);
+            F.tile_q[tile] = may_long | (BULK && has_doc ? TQ_HAS_DOC : 0u) | (s_nl ? TQ_MAY_LONG : 0u) | s_ns | ((F.wq != nullptr ? 0u : s_nw) << TQ_NW_SHIFT) | (s_nl << TQ_NL_SHIFT);
             if (F.wq != nullptr && s_nw) s_wbase = atomicAdd(&P.hdr->nwq, s_nw);
         }
         if (F.wq != nullptr && s_nw) {                                // block-uniform

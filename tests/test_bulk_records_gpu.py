@@ -1,0 +1,34 @@
+"""What the first kernel, the merges and the scatter of bulk text hand each other, against the oracle."""
+import numpy as np
+import pytest
+
+import workloads as wl
+from gpu_util import cpu_vocab, gpu_encode, gpu_encode_batch, gpu_vocab, same
+
+pytestmark = pytest.mark.gpu
+
+
+# pieces of so many tokens that their number does not fit the record (2^20 - 1 and more), and fewer; starts all over the tile
+@pytest.mark.parametrize("tokens", [1_048_573, 1_048_574, 1_048_575, 2_200_000])
+@pytest.mark.parametrize("before", [0, 1, 2_040])
+def test_a_piece_of_more_tokens_than_the_record_holds(tokens, before):
+    gv, cv = gpu_vocab("C1"), cpu_vocab("C1")
+    # control characters: one punctuation piece with the line feed behind it; no merge knows them (checked below), so a token per byte
+    long = np.tile(np.uint8([1, 2, 3]), tokens // 3 + 1)[:tokens]
+    assert cv.encode(long[:3_000], 0)[0].size == 3_000
+    text = np.r_[np.full(before, 97, np.uint8), np.uint8([10]), long, np.frombuffer(b"\nand so on.\n", np.uint8), wl.generate(0, 3, 4_300_000)]
+    ids, status = gpu_encode(gv, text)
+    assert status == 0 and same(ids, cv.encode(text, 0, nthreads=8)[0])
+
+
+# groups of 32 pieces: none, one and all of them merged, of up to eight tokens and of more
+@pytest.mark.parametrize("every", [1, 2, 31, 32, 33, 200])
+@pytest.mark.parametrize("size", [9, 14, 90])
+def test_merged_pieces_among_settled_ones(every, size):
+    rng = np.random.default_rng(every * 100 + size)
+    gv, cv = gpu_vocab("C3"), cpu_vocab("C3")
+    settled = b" the" * (every - 1)
+    words = (97 + rng.integers(0, 26, (4_400_000 // (len(settled) + size + 1), size))).astype(np.uint8)
+    text = np.concatenate([np.r_[np.frombuffer(settled, np.uint8), np.uint8([32]), w] for w in words])
+    ids, status = gpu_encode(gv, text)
+    assert status == 0 and same(ids, cv.encode(text, 0, nthreads=8)[0])
