@@ -403,80 +403,99 @@ __device__ __forceinline__ u32 warp_merge_perm(u32* buf /* 2 * 4 * 32 E words of
 }
 
 // ---- a thread per piece, <= 32 bytes: tokens and pair ranks in shared memory ------------------------------
-// Paper Sec. 4.2 gives the shortest length class to single threads.  Here a warp per piece has the shorter
-// dependent chain (one probe latency per round for the whole piece), so it serves a request's few
-// unmatched pieces; a thread per piece keeps 32 independent chains per warp in flight and issues an order
-// of magnitude fewer instructions per piece, so it serves bulk text.  Same rounds as everywhere: the
-// minimum rank of the piece, all its leftmost non-overlapping occurrences, new probes only next to a merge.
-// Column s of tok[LANE_MAX][LANE_SLOTS] / rk[LANE_MAX][LANE_SLOTS] (one pair of arrays per warp): any two
-// threads of the warp hit different banks whatever rows they are at.
+// Paper Sec. 4.2 gives the shortest length class to single threads.  A warp per piece takes fewer rounds (it merges more than one pair
+// a round), a thread per piece keeps 32 independent chains per warp in flight and issues an order of magnitude fewer
+// instructions per piece.  A round is one merge: the leftmost pair of the lowest rank, as the definition has it.  What bounds a
+// batch is the chain of a round -- minimum, neighbours, two probes side by side -- times the merges of its slowest
+// piece, so the minimum is found without a dependent step per position: a pair's rank and position are one word, the words of
+// four positions one 16-byte load, and places without a pair hold all ones (walking the live positions one after the other
+// and merging all occurrences of the rank at once, a batch of 32 pieces took 50 to 110 us; 132 MB batch 851 -> 804, 3M chars of long
+// runs 236 -> 198, 1,000 messages 68.5 -> 61).
 constexpr int LANE_SLOTS = 32;                        // pieces a warp merges at once
 constexpr int LANE_MAX = 32;                          // bytes per piece on this path
-// Two independent probes (ranks only), all loads in flight together.
-__device__ __forceinline__ void pair_probe2(const PairTable& t, u32 a0, u32 b0, u32 a1, u32 b1, u32& r0, u32& r1) {
-    const u64 key0 = ((u64)a0 << TT_ID_BITS) | b0, key1 = ((u64)a1 << TT_ID_BITS) | b1;
-    const u32 h00 = pair_bucket(key0, t.shift), h01 = pair_bucket_alt(key0, t.shift, h00);
-    const u32 h10 = pair_bucket(key1, t.shift), h11 = pair_bucket_alt(key1, t.shift, h10);
-    const uint4* p00 = t.slots + 2 * (size_t)h00; const uint4* p01 = t.slots + 2 * (size_t)h01;
-    const uint4* p10 = t.slots + 2 * (size_t)h10; const uint4* p11 = t.slots + 2 * (size_t)h11;
+constexpr u32 LANE_NONE = 0xFFFFFFFFu;                // no pair begins here
+// Two independent probes, ranks only (TT_F20 or more: none).  A slot's first word holds the key's low 12 bits over the rank: where key and
+// slot agree, their difference is the rank.  ALL: all four buckets at once, the shorter chain, for a request; else a key's second
+// bucket only where the first has not got it, for bulk text, whose warps saturate the way to L2 (132 MB batch: all at once 773 us a
+// call, so 740; 15,000 pieces of 1,000 messages: the second bucket afterwards 60 us, all at once 55.6).
+__device__ __forceinline__ u32 pair_rank_of(const uint4 s, u32 hi, u32 lo) { return s.y == hi ? s.x ^ lo : TT_RANK_INF; }
+template <bool ALL>
+__device__ __forceinline__ void pair_probe2(const PairTable& t, u64 key0, u64 key1, u32& r0, u32& r1) {
+    const u32 h00 = pair_bucket(key0, t.shift), h10 = pair_bucket(key1, t.shift);
+    const uint4* const p01 = t.slots + 2 * (size_t)pair_bucket_alt(key0, t.shift, h00);
+    const uint4* const p11 = t.slots + 2 * (size_t)pair_bucket_alt(key1, t.shift, h10);
+    const u32 hi0 = (u32)(key0 >> 12), lo0 = (u32)key0 << 20, hi1 = (u32)(key1 >> 12), lo1 = (u32)key1 << 20;
     uint4 a00, a01, a02, a03, a10, a11, a12, a13;
-    ldg_sector(p00, a00, a01); ldg_sector(p01, a02, a03); ldg_sector(p10, a10, a11); ldg_sector(p11, a12, a13);
-    PairInfo q0 = pair_none(), q1 = pair_none();
-    if (!pair_match(a00, key0, q0) && !pair_match(a01, key0, q0) && !pair_match(a02, key0, q0)) pair_match(a03, key0, q0);
-    if (!pair_match(a10, key1, q1) && !pair_match(a11, key1, q1) && !pair_match(a12, key1, q1)) pair_match(a13, key1, q1);
-    r0 = q0.r; r1 = q1.r;
+    ldg_sector(t.slots + 2 * (size_t)h00, a00, a01); ldg_sector(t.slots + 2 * (size_t)h10, a10, a11);
+    if (ALL) { ldg_sector(p01, a02, a03); ldg_sector(p11, a12, a13); }
+    r0 = min(pair_rank_of(a00, hi0, lo0), pair_rank_of(a01, hi0, lo0));
+    r1 = min(pair_rank_of(a10, hi1, lo1), pair_rank_of(a11, hi1, lo1));
+    if (!ALL) {
+        a02 = a03 = a12 = a13 = make_uint4(0, 0xFFFFFFFFu, 0, 0);             // (no key's: a key has 36 bits, 24 of them here)
+        if (r0 > TT_F20) ldg_sector(p01, a02, a03);
+        if (r1 > TT_F20) ldg_sector(p11, a12, a13);
+    }
+    r0 = min(r0, min(pair_rank_of(a02, hi0, lo0), pair_rank_of(a03, hi0, lo0)));
+    r1 = min(r1, min(pair_rank_of(a12, hi1, lo1), pair_rank_of(a13, hi1, lo1)));
 }
 
-// Tokens stay at the byte position where they began; `al` has a bit per position that still holds a
-// token, and the rank of a pair is kept at its left position, so a merge moves nothing: it rewrites the
-// left token, clears the partner's bit and marks the two pairs that changed for a new probe.
-__device__ __forceinline__ u32 lane_merge(u32* __restrict__ tok, u32* __restrict__ rk, int s, const u8* __restrict__ text, u32 a, u32 n,
+// Tokens stay at the byte position where they began; `al` has a bit per position that still holds a token, and the word of a
+// pair is kept at its left position, so a merge moves nothing.  tok[LANE_MAX][LANE_SLOTS], a column per thread; the
+// words of positions 4j .. 4j + 3 are rk[j][thread]: any two threads of the warp find their tokens, and any eight
+// neighbouring threads their four words, in different banks.
+__device__ __forceinline__ u32 lane_word(u32 r20, u32 k) { return r20 >= TT_F20 ? LANE_NONE : (r20 << 5) | k; }
+template <bool ALL>
+__device__ __forceinline__ u32 lane_merge(u32* __restrict__ tok, int s, const u8* __restrict__ text, u32 a, u32 n,
                                           const PairTable& tab, const ExtMap& ext_id, int32_t* __restrict__ stage) {
+    u32* const rk = tok + LANE_MAX * LANE_SLOTS;
 #define TK(k) tok[(k) * LANE_SLOTS + s]
-#define RK(k) rk[(k) * LANE_SLOTS + s]
-    u32 prev = text[a];
-    TK(0) = prev;
-#pragma unroll 4
-    for (u32 k = 1; k < n; k++) {
-        const u32 t = text[a + k];
-        TK(k) = t;
-        RK(k - 1) = f20_decode((u32)__ldg(tab.bytepair + ((prev << 8) | t)) & TT_F20);
-        prev = t;
+#define RK(k) rk[(((k) >> 2) * LANE_SLOTS + s) * 4 + ((k) & 3)]
+    uint4* const rk4 = reinterpret_cast<uint4*>(rk) + s;
+    const bool wide = n > 16;
+    {
+        const uintptr_t addr = (uintptr_t)(text + a);
+        const u32* const w = reinterpret_cast<const u32*>(addr & ~(uintptr_t)3);
+        const u32 sh = (u32)(addr & 3) * 8, used = (u32)(addr & 3) + n;       // bytes of the aligned words that hold the piece
+        const u32* const bp = reinterpret_cast<const u32*>(tab.bytepair);     // (the rank is in the low half of an entry)
+        u32 x[9];
+#pragma unroll
+        for (int j = 0; j < 9; j++) x[j] = used > 4u * j ? w[j] : 0u;          // only words that hold a piece byte
+#pragma unroll
+        for (int j = 0; j < 8; j++) {
+            if (j >= 4 && !wide) break;
+            const u32 v = __funnelshift_r(x[j], x[j + 1], sh), vn = j < 7 ? __funnelshift_r(x[j + 1], x[j + 2 < 9 ? j + 2 : 8], sh) : 0u;
+            const u32 t0 = v & 0xFFu, t1 = (v >> 8) & 0xFFu, t2 = (v >> 16) & 0xFFu, t3 = v >> 24, t4 = vn & 0xFFu;
+            const u32 k = 4 * j;
+            uint4 r = make_uint4(TT_F20, TT_F20, TT_F20, TT_F20);
+            if (k + 1 < n) r.x = __ldg(bp + 2 * ((t0 << 8) | t1)) & TT_F20;
+            if (k + 2 < n) r.y = __ldg(bp + 2 * ((t1 << 8) | t2)) & TT_F20;
+            if (k + 3 < n) r.z = __ldg(bp + 2 * ((t2 << 8) | t3)) & TT_F20;
+            if (k + 4 < n) r.w = __ldg(bp + 2 * ((t3 << 8) | t4)) & TT_F20;
+            rk4[j * LANE_SLOTS] = make_uint4(lane_word(r.x, k), lane_word(r.y, k + 1), lane_word(r.z, k + 2), lane_word(r.w, k + 3));
+            TK(k) = t0; TK(k + 1) = t1; TK(k + 2) = t2; TK(k + 3) = t3;
+        }
     }
     u32 al = 0xFFFFFFFFu >> (32 - n);
-    u32 stale = 0;
-    for (u32 round = 0; round < n; round++) {
-        while (stale) {                                   // every thread of the warp walks its own list in step
-            const u32 k0 = __ffs(stale) - 1;
-            stale &= stale - 1;
-            const u32 k1 = stale ? __ffs(stale) - 1 : k0;
-            stale &= stale - 1;
-            const u32 up0 = al & (0xFFFFFFFEu << k0), up1 = al & (0xFFFFFFFEu << k1);
-            u32 r0 = TT_RANK_INF, r1 = TT_RANK_INF;         // (a position without a token above it has no pair)
-            pair_probe2(tab, TK(k0), up0 ? TK(__ffs(up0) - 1) : 0u, TK(k1), up1 ? TK(__ffs(up1) - 1) : 0u, r0, r1);
-            RK(k0) = up0 ? r0 : TT_RANK_INF;
-            RK(k1) = up1 ? r1 : TT_RANK_INF;
-        }
-        u32 mn = TT_RANK_INF, c = 0;
-        for (u32 x = al & ~(0x80000000u >> __clz(al)); x; x &= x - 1) {      // every position but the topmost
-            const u32 k = __ffs(x) - 1;
-            const u32 r = RK(k);
-            if (r < mn) { mn = r; c = 0; }
-            c |= (r == mn ? 1u : 0u) << k;
-        }
-        if (mn == TT_RANK_INF) break;
-        const u32 nt = 256u + mn;
-        u32 blocked = 32;
-        for (u32 x = c; x; x &= x - 1) {                  // leftmost non-overlapping occurrences, ascending
-            const u32 k = __ffs(x) - 1;
-            if (k == blocked) continue;                   // its token went into the merge before it
-            const u32 p = __ffs(al & (0xFFFFFFFEu << k)) - 1;
-            TK(k) = nt;
-            al &= ~(1u << p);
-            blocked = p;
-            const u32 below = al & ((1u << k) - 1);
-            stale |= (1u << k) | (below ? 0x80000000u >> __clz(below) : 0u);
-        }
+    for (u32 round = 1; round < n; round++) {             // at most n - 1 merges
+        const auto min8 = [&](int j) {
+            const uint4 x = rk4[j * LANE_SLOTS], y = rk4[(j + 1) * LANE_SLOTS];
+            return __vimin3_u32(__vimin3_u32(x.x, x.y, x.z), __vimin3_u32(x.w, y.x, y.y), min(y.z, y.w));
+        };
+        u32 mn = min(min8(0), min8(2));
+        if (wide) mn = __vimin3_u32(mn, min8(4), min8(6));
+        if (mn == LANE_NONE) break;
+        const u32 k = mn & 31u, t = 256u + (mn >> 5);
+        u32 up = al & (0xFFFFFFFEu << k);                 // the tokens above; the first of them goes into the merge
+        const u32 p = __ffs(up) - 1;
+        up &= up - 1; al &= ~(1u << p);
+        const u32 q = __ffs(up) - 1, dn = al & ((1u << k) - 1), l = 31 - __clz(dn);
+        TK(k) = t;
+        RK(p) = LANE_NONE;
+        const u64 right = ((u64)t << TT_ID_BITS) | (up ? TK(q) : 0u), left = dn ? ((u64)TK(l) << TT_ID_BITS) | t : right;
+        u32 rl, rr;
+        pair_probe2<ALL>(tab, left, right, rl, rr);
+        if (dn) RK(l) = lane_word(rl, l);
+        RK(k) = up ? lane_word(rr, k) : LANE_NONE;
     }
     u32 m = 0;
     for (u32 x = al; x; x &= x - 1) stage[a + m++] = ext_id[TK(__ffs(x) - 1)];
@@ -784,8 +803,8 @@ struct PieceParams {
 //   - pieces of more than 256 bytes, where a tile allows for one (cta_find_long): those of every gridDim.x-th tile by a CTA, or,
 //     if one is too long for that, by tickets, its windows later by the whole grid (long_phase);
 //   - everything else by warps, without a barrier: job j is warp j's, in the order warp-class pieces (the longest chains),
-//     closing pieces of the tiles, short pieces; by tickets where CTAs had long pieces first.  With many short pieces these go 32
-//     by 32, a thread each (merge_short_batches).
+//     closing pieces of the tiles, short pieces; by tickets where CTAs had long pieces first.  With many short pieces these go in
+//     batches, a thread each (merge_short_batches).
 // Bulk text (k_merge_bulk): k_closing has gathered global lists.  Long pieces by tickets of a CTA, warp-class pieces a warp each
 // by index, short pieces by tickets of 32 of one length class, a thread each, the longest class first.
 #ifndef TT_MERGE_WARPS
@@ -798,6 +817,11 @@ static_assert(MERGE_WARPS * WARP_SMEM_WORDS * sizeof(u64) >= LONG_SMEM_SLOTS * (
 static_assert(LONG_SMEM_TOKENS >= MERGE_WARPS * 32 * LK, "the survivors of a chunk (threads x LK positions) must fit the shared buffer");
 constexpr size_t MERGE_SMEM_BYTES = (size_t)MERGE_WARPS * WARP_SMEM_WORDS * sizeof(u64);   // dynamic shared memory of k_merge_bulk (192 KiB)
 static_assert(WARP_SMEM_WORDS * sizeof(u64) >= 2 * LANE_SLOTS * LANE_MAX * sizeof(u32) && WARP_SMEM_WORDS * sizeof(u64) >= 2 * 4 * TT_WARP_PIECE_MAX * sizeof(u32), "per-warp buffer");
+// Pieces of a batch of lane_merge: as few as give BATCH_WARPS of a CTA's warps one each, up to 32.  More warps with fewer pieces each
+// only issue the same instructions more often (1,000 messages: all 24 warps 60.4 us, 12 warps 55.6, 8 56.4, 5 57.0; 3M chars of long
+// runs 197, 190, 200, 204).
+constexpr u32 BATCH_WARPS = 12;
+__device__ __forceinline__ u32 short_batch(u32 pieces) { const u32 warps = gridDim.x * BATCH_WARPS; return min((u32)LANE_SLOTS, max(1u, (pieces + warps - 1) / warps)); }
 constexpr int MERGE_SR_MAX_TILES = 2048;              // the per-warp job search covers at most 32 lanes x 64 tiles
 
 #ifndef TT_MERGE_CTAS_PER_SM
@@ -1435,7 +1459,11 @@ __device__ void merge_bulk_lists(const PieceParams& P, const u8* __restrict__ te
     // tickets: 32 pieces of one list each, the list of the longest pieces first
     u32 cnts[TT_SHORT_CLASSES], nb[TT_SHORT_CLASSES], nball = 0;
 #pragma unroll
-    for (int c = 0; c < TT_SHORT_CLASSES; c++) { cnts[c] = c ? P.hdr->nq_short_x[c - 1] : ns; nb[c] = (cnts[c] + LANE_SLOTS - 1) / LANE_SLOTS; nball += nb[c]; }
+    for (int c = 0; c < TT_SHORT_CLASSES; c++) { cnts[c] = c ? P.hdr->nq_short_x[c - 1] : ns; nball += cnts[c]; }
+    const u32 per = short_batch(nball);
+    nball = 0;
+#pragma unroll
+    for (int c = 0; c < TT_SHORT_CLASSES; c++) { nb[c] = (cnts[c] + per - 1) / per; nball += nb[c]; }
     for (;;) {                                                        // bounded by the number of tickets
         u32 tk = 0;
         if (lane == 0) tk = atomicAdd(&P.hdr->t_short, 1u);
@@ -1447,17 +1475,17 @@ __device__ void merge_bulk_lists(const PieceParams& P, const u8* __restrict__ te
             bool found = false;
 #pragma unroll
             for (int c = TT_SHORT_CLASSES - 1; c >= 0; c--) {
-                if (!found && r < nb[c]) { list = c ? P.gq_x[c - 1] : P.gq; cnt = cnts[c]; e0 = r * LANE_SLOTS; found = true; }
+                if (!found && r < nb[c]) { list = c ? P.gq_x[c - 1] : P.gq; cnt = cnts[c]; e0 = r * per; found = true; }
                 if (!found) r -= nb[c];
             }
         }
-        if (e0 + lane < cnt) {
+        if ((u32)lane < per && e0 + lane < cnt) {
             const u64 x = list[e0 + lane];
             const u32 t = (u32)(x >> 32), e = (u32)x;
             const u32 a = (u32)((long long)t * TT_TILE_BYTES + (e & 2047u) - P.shift), n = (e >> 22) + 1, slot = t * TT_TILE_BYTES + ((e >> 11) & 2047u);
             if (!piece_in_range(P, a, n, slot, 4u) || n < 2 || n > (u32)LANE_MAX) hdr_selfcheck_failed(P.hdr, P.epoch, 5u, a, n, slot, e0);
             else {
-                const u32 m = lane_merge(tok, tok + LANE_SLOTS * LANE_MAX, lane, text, a, n, P.tab, P.ext_id, P.stage);
+                const u32 m = lane_merge<false>(tok, lane, text, a, n, P.tab, P.ext_id, P.stage);
                 piece_done(P, a, slot, m);
             }
         }
@@ -1534,7 +1562,7 @@ __device__ __forceinline__ u32 merge_find(const u32* pre, u32 entries, u32 k) {
     return lo;
 }
 
-constexpr u32 SHORT_PER_WARP = 12;                    // more short pieces than that per warp of the grid: see k_merge
+constexpr u32 SHORT_PER_WARP = 5;                    // more short pieces than that per warp of the grid: see k_merge
 // The k-th queued piece of its class (warp-class or short).
 __device__ __forceinline__ void merge_queued(const PieceParams& P, const MergeIndex& X, int unit, int entries, bool wclass, u32 k, u32& a, u32& n, u32& slot) {
     const u32* const pre = wclass ? X.pre_w : X.pre_s;
@@ -1562,24 +1590,24 @@ __device__ __forceinline__ bool merge_closing(const PieceParams& P, const u8* __
     if (lane == 0) { P.piece_cnt[slot] = v; atomicAdd(&P.tile_tok[t], 1u); }
     return false;
 }
-// The queued short pieces 32 by 32 in their order, whatever tiles they stand in, a thread each; the batches are spread over the
+// The queued short pieces in batches, in their order, whatever tiles they stand in, a thread each; the batches are spread over the
 // grid, by tickets where some CTAs first had a long piece.  (With a ticket per tile 147 warps took the 150,000 two-byte pieces of
 // 300 KB, most of them on the few SMs that came first: 78 to 118 us, now 54 to 66.)  Out of line: in line these texts are 4 % faster,
 // but a call of 4,000 characters, which does none of this, takes 33.05 us instead of 32.75, a conversation of 17 appends 831
 // instead of 824.
-__device__ __noinline__ void merge_short_batches(const PieceParams& P, const u8* __restrict__ text, const MergeIndex& X, int unit, int entries, bool by_ticket, u32* tok) {
-    const u32 lane = threadIdx.x & 31, NS = X.pre_s[entries], nb = (NS + 31) / 32;
+__device__ __noinline__ void merge_short_batches(const PieceParams& P, const u8* __restrict__ text, const MergeIndex& X, int unit, int entries, bool by_ticket, u32* buf) {
+    const u32 lane = threadIdx.x & 31, W = gridDim.x * MERGE_WARPS, NS = X.pre_s[entries], per = short_batch(NS), nb = (NS + per - 1) / per;
     u32 b = by_ticket ? warp_take(&P.hdr->t_tiles, (int)lane) : (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
     while (b < nb) {
-        const u32 k = 32 * b + lane;
-        if (k < NS) {
+        const u32 k = per * b + lane;
+        if (lane < per && k < NS) {
             u32 a, n, slot;
             merge_queued(P, X, unit, entries, false, k, a, n, slot);
             if (!piece_in_range(P, a, n, slot, 4u) || n < 2 || n > (u32)LANE_MAX) hdr_selfcheck_failed(P.hdr, P.epoch, 5u, a, n, slot, k);
-            else piece_done(P, a, slot, lane_merge(tok, tok + LANE_SLOTS * LANE_MAX, (int)lane, text, a, n, P.tab, P.ext_id, P.stage));
+            else piece_done(P, a, slot, lane_merge<true>(buf, (int)lane, text, a, n, P.tab, P.ext_id, P.stage));
         }
         __syncwarp();
-        b = by_ticket ? warp_take(&P.hdr->t_tiles, (int)lane) : b + gridDim.x * MERGE_WARPS;
+        b = by_ticket ? warp_take(&P.hdr->t_tiles, (int)lane) : b + W;
     }
 }
 
@@ -1603,10 +1631,10 @@ k_merge(const __grid_constant__ PieceParams P) {
     u64* wbuf = s_buf + wid * WARP_SMEM_WORDS;
     const u32 W = gridDim.x * MERGE_WARPS, gw = (u32)wid * gridDim.x + blockIdx.x;   // numbered across the CTAs first
     const u32 NS = X.pre_s[entries], NW = X.pre_w[entries], NT = (u32)P.ntiles;
-    // A warp per piece, or a thread per piece and a warp for 32 of them?  A batch takes as long as its slowest piece: 25 us for words of nine
-    // letters, 50 to 60 for the mixed lengths of prose, however few batches there are.  Measured, short pieces per warp of the
-    // grid -> k_merge with a warp / a thread per piece: Unicode-heavy prose 4.3 -> 36 / 50 us, 13.2 -> 76 / 59, 13.5 -> 70 / 66, 16 ->
-    // 75 / 75; transcripts 10 -> 60 / 73; nine-letter words 3 -> 19 / 23, 4.3 -> 25 / 25, 8.6 -> 40 / 29, 17 -> 66 / 38.
+    // A warp per piece, or a thread per piece?  A warp takes its pieces one after the other, 4 to 6 us each; a batch takes as long as its
+    // slowest piece, 20 to 25 us, however few pieces there are.  Measured, short pieces and tiles per warp of the grid -> us a call with
+    // a warp / a thread per piece: Unicode-heavy prose 2.5 -> 41.8 / 44.6, 5.0 -> 68.5 / 55.6, 8 -> 75.8 / 61.4; prose with 4,096
+    // merges 4 -> 41.0 / 47.6, 6 -> 50.4 / 46.0, 7.5 -> 56.1 / 48.8; transcripts 2.5 -> 57.0 / 66.
     const bool many = NS + NT > SHORT_PER_WARP * W;
     const u32 J = many ? NW : NW + NT + NS;                          // jobs of a warp: all pieces, or the warp-class ones
     // Job by job in order (warp-class pieces, closing pieces, short pieces); where some CTAs first had a long piece to merge, by
