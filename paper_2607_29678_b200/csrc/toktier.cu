@@ -631,6 +631,8 @@ static int run_pretok(const tt_vocab* v, const uint8_t* text, size_t len, const 
     const bool bulk = P.ntiles > MERGE_SR_MAX_TILES;
     const int per_sm = bulk && fused ? PRETOK_CTAS_BULK : PRETOK_CTAS_REQUEST;
     const int grid = P.ntiles < v->sm_count * per_sm ? P.ntiles : v->sm_count * per_sm;
+    P.run = 1;
+    if (bulk && fused && !host_src) while (P.run < PRETOK_RUN && P.ntiles >= 2 * P.run * grid) P.run *= 2;
     if (v->pattern == TT_PATTERN_SPLIT3) {
         // stages A and B: span starts into cutmask (with the caller's document starts); stage C: pattern 0 with
         // those cuts as its document boundaries

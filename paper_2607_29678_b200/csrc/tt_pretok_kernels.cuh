@@ -365,11 +365,11 @@ __device__ __forceinline__ void front_piece_queue(const FrontParams& F, int tile
 // NT = threads per CTA, MINB = CTAs per SM the kernel is compiled for.  A request (at most a few tiles per CTA) is a latency
 // chain: 128 threads, so that classification (72 words with the halo) is one step and the look-ups are short, and
 // four table look-ups in flight per thread.  Bulk text is bound by instruction issue: 64 threads, as many as a tile has
-// words, so that no warp waits idle for the predicate, and one look-up at a time per thread; 20 CTAs per SM leave 48 registers
-// (24 with 40: 20 MB of Unicode-heavy text 500 -> 477 us per call, the 132 MB batch 921 -> 905; 16 and 18 are slower for it).
+// words, so that no warp waits idle for the predicate, and one look-up at a time per thread; 18 CTAs per SM leave 56 registers
+// (132 MB batch: 16 CTAs 791 us a call, 17 765, 18 763, 19 794, 20 with 48 registers 788; two look-ups in flight 808 to 815).
 // PAT = the pattern the kernel is compiled for (P.pattern says the same): each pattern's rules are a lot of code, and a
 // kernel that carries all of them keeps missing the instruction caches on its way through the one it runs.
-constexpr int PRETOK_THREADS_REQUEST = 128, PRETOK_CTAS_REQUEST = 6, PRETOK_THREADS_BULK = 64, PRETOK_CTAS_BULK = 20;
+constexpr int PRETOK_THREADS_REQUEST = 128, PRETOK_CTAS_REQUEST = 6, PRETOK_THREADS_BULK = 64, PRETOK_CTAS_BULK = 18, PRETOK_RUN = 8;
 template <int PAT> struct PretokSmem {
     static constexpr int ROWS = PAT == 1 ? F_COUNT : F_P0_COUNT;
     // the piece offsets take the place of the masks once the predicate has been evaluated
@@ -393,6 +393,14 @@ k_pretok(const __grid_constant__ PretokParams P, const __grid_constant__ FrontPa
     static_assert(NT >= TT_TILE_WORDS && NT % 32 == 0 && TT_TILE_WORDS % 32 == 0, "a thread per word of the tile, whole warps of them (tt_eval_word_p1 asks the warp)");
 
     constexpr bool BULK = FUSED && NT == PRETOK_THREADS_BULK;
+    // Bulk text: a CTA takes runs of P.run neighbouring tiles and keeps the masks of the last eight slots (the next tile's low halo and
+    // first word) and the text of the very last, so that 64 threads load and classify 64 words; with the halo taken in anew, one
+    // warp went through both a second time for eight words while the other waited (132 MB batch 823 -> 809 us).  (Pattern 1 rewrites
+    // the masks of its window afterwards, and host text is copied tile by tile: P.run is 1 there.)
+    constexpr bool CARRY = BULK && PAT != 1;
+    constexpr int CARRY_ROWS = F_P0_COUNT;
+    static_assert(!CARRY || NT == TT_TILE_WORDS, "the words of a run's later tiles, one per thread");
+    __shared__ u32 s_carry[CARRY ? CARRY_ROWS * (TT_LOW_HALO + 1) : 1];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     cudaTriggerProgrammaticLaunchCompletion();               // the next kernel may be placed; it waits for this grid's memory itself
     // the whole-piece table is probed at random a few microseconds from now: ask for it to be brought into L2
@@ -418,24 +426,33 @@ k_pretok(const __grid_constant__ PretokParams P, const __grid_constant__ FrontPa
     u8* const stx = reinterpret_cast<u8*>(s_text + 4);                // byte 0 of slot 0
     const u8* const tb = stx + TT_LOW_HALO * TT_WORD;                 // byte 0 of the tile
 
-    for (int tile = blockIdx.x; tile < P.ntiles; tile += gridDim.x) {
+    const int run = CARRY ? P.run : 1;
+    for (int tile = (int)blockIdx.x * run; tile < P.ntiles; tile += CARRY && ((tile + 1) & (run - 1)) ? 1 : ((int)gridDim.x - 1) * run + 1) {
         __syncthreads();
+        const bool carried = CARRY && (tile & (run - 1)) != 0;        // the tile before was this CTA's: block-uniform
         if (tid == 0) { s_need = 0; s_first = 0xFFFFFFFFu; s_ns = 0; s_nw = 0; s_nl = 0; s_total = 0; s_nslow = 0; }
         const long long w_first = (long long)tile * TT_TILE_WORDS;    // mask word of the tile's first byte
         // phase A: the text of the tile and its halo into shared memory, a vector load per thread and step
         {
             const long long c0 = 2 * (w_first - TT_LOW_HALO);
-            for (int c = tid; c < 2 * TT_SLOTS; c += NT) {
+            if (carried) {
+                // (the threads that are about to replace the text of the high halo and of the word before it keep the one as the tile's
+                // first word and the other's last bytes, which a contraction may begin in)
+                if (tid == NT - 3) s_text[4 + 8 * TT_LOW_HALO - 1] = s_text[4 + 8 * (TT_SLOTS - 1) - 1];
+                if (tid >= NT - 2) *reinterpret_cast<uint4*>(s_text + 4 + 4 * (2 * TT_LOW_HALO + tid - (NT - 2))) = *reinterpret_cast<const uint4*>(s_text + 4 + 4 * (2 * (TT_SLOTS - 1) + tid - (NT - 2)));
+                for (int e = tid; e < CARRY_ROWS * (TT_LOW_HALO + 1); e += NT) sm[e / (TT_LOW_HALO + 1)][e % (TT_LOW_HALO + 1)] = s_carry[e];
+            }
+            for (int c = tid + (carried ? 2 * (TT_LOW_HALO + 1) : 0); c < 2 * TT_SLOTS; c += NT) {
                 const uint4 v = load_chunk_raw(P, rd, c0 + c);
                 *reinterpret_cast<uint4*>(s_text + 4 + 4 * c) = text_of_chunk(P, v, c0 + c);
                 if (P.src && c >= 2 * TT_LOW_HALO && c < 2 * (TT_LOW_HALO + TT_TILE_WORDS) && c0 + c < P.nchunks) *reinterpret_cast<uint4*>(P.copy + (c0 + c) * TT_CHUNK) = v;
             }
-            if (tid == NT - 1) s_text[3] = load_chunk(P, rd, c0 - 1).w;
+            if (tid == NT - 1 && !carried) s_text[3] = load_chunk(P, rd, c0 - 1).w;
             if (tid == NT - 2) s_text[4 + TT_SLOTS * 8] = load_chunk(P, rd, c0 + 2 * TT_SLOTS).x;
         }
         __syncthreads();
         // phase B: classify, a word per thread and step
-        for (int s = tid; s < TT_SLOTS; s += NT) {
+        for (int s = tid + (carried ? TT_LOW_HALO + 1 : 0); s < TT_SLOTS; s += NT) {
             const long long word = w_first - TT_LOW_HALO + s;
             const uint4 a = *reinterpret_cast<const uint4*>(s_text + 4 + 8 * s), b = *reinterpret_cast<const uint4*>(s_text + 8 + 8 * s);
             const u32 x[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
@@ -443,7 +460,7 @@ k_pretok(const __grid_constant__ PretokParams P, const __grid_constant__ FrontPa
             const WordMasks m = tt_classify_word(x, stx + s * TT_WORD, valid, T);
             const u32 d = doc_bits(P, word);
             store_slot<PAT>(sm, s, m, d);
-            if (s >= TT_LOW_HALO && s < TT_LOW_HALO + TT_TILE_WORDS) any_bad |= m.bad | (d & ~m.lead & valid & ~m.bad);
+            if (s >= TT_LOW_HALO && (CARRY || s < TT_LOW_HALO + TT_TILE_WORDS)) any_bad |= m.bad | (d & ~m.lead & valid & ~m.bad);
         }
         __syncthreads();
         if (PAT == 1) {                                          // marks inside words count as caseless letters from here on
@@ -514,6 +531,7 @@ k_pretok(const __grid_constant__ PretokParams P, const __grid_constant__ FrontPa
         for (int o = 1; o < 32; o <<= 1) { const u32 t = __shfl_up_sync(0xFFFFFFFFu, x, o); if (lane >= o) x += t; }
         if (has_word && lane == 31) s_wtot[wid] = x;
         bool has_doc = false;                                         // bulk text: a document starts in the tile
+        if (CARRY) for (int e = tid; e < CARRY_ROWS * (TT_LOW_HALO + 1); e += NT) s_carry[e] = sm[e / (TT_LOW_HALO + 1)][TT_TILE_WORDS + e % (TT_LOW_HALO + 1)];
         if (BULK) has_doc = __syncthreads_or(sm[F_DOC][slot] != 0);
         else __syncthreads();                                         // (the masks have been read: their place is free)
         u32 np = 0, r = x - cnt;

@@ -32,3 +32,33 @@ def test_merged_pieces_among_settled_ones(every, size):
     text = np.concatenate([np.r_[np.frombuffer(settled, np.uint8), np.uint8([32]), w] for w in words])
     ids, status = gpu_encode(gv, text)
     assert status == 0 and same(ids, cv.encode(text, 0, nthreads=8)[0])
+
+
+# runs of neighbouring tiles are one CTA's, which keeps the end of the tile before: constructs of every kind across every edge,
+# at every place, in one text and in documents
+SNIPPETS = [b"it's we'll they've I'd ", b" 1234567890123 ", b"   \n\n  \r\n   x", b"!!!\n\n??? \n", "é ñ日本語 x  y ".encode(), b"don't" * 3, b" '' 's 't 'll",
+            b"a" * 70, b" " * 300 + b"x", b"7" * 400]
+
+
+@pytest.mark.parametrize("pattern", [0, 1, 2, 3])
+@pytest.mark.parametrize("megabytes,docs", [(5, 0), (14, 0), (14, 3_000), (26, 0)])
+def test_constructs_across_the_edges_of_neighbouring_tiles(pattern, megabytes, docs):
+    rng = np.random.default_rng(megabytes + pattern)
+    gv, cv = gpu_vocab("C1", pattern=pattern), cpu_vocab("C1")
+    filler = wl.generate(0, 17, megabytes * 1_000_000)
+    at = 2_048
+    while at + 2_048 < filler.size:                                    # a construct across every edge, one byte further each time
+        s = np.frombuffer(SNIPPETS[int(rng.integers(len(SNIPPETS)))], np.uint8)
+        from_ = at - int(rng.integers(0, s.size + 1))
+        filler[from_:from_ + s.size] = s
+        at += 2_048
+    if not docs:
+        ids, status = gpu_encode(gv, filler)
+        assert status == 0 and same(ids, cv.encode(filler, pattern, nthreads=8)[0])
+        return
+    cuts = np.unique(rng.integers(1, filler.size, docs))
+    cuts = cuts[(filler[cuts] & 0xC0) != 0x80]
+    off = np.r_[0, cuts, filler.size].astype(np.int64)
+    ids, ioff, status = gpu_encode_batch(gv, filler, off)
+    want, woff = cv.encode_batch(filler, off, pattern, nthreads=8)
+    assert status == 0 and same(ids, want) and same(ioff, woff)
