@@ -624,8 +624,12 @@ static int run_pretok(const tt_vocab* v, const uint8_t* text, size_t len, const 
         L.docmask = w.docmask; L.litstart = w.litstart; L.litin = w.litin;
         const size_t want = (size_t)(P.nchunks + LIT_THREADS - 1) / LIT_THREADS;
         const int lgrid = (int)(want < (size_t)v->sm_count * 8 ? want : (size_t)v->sm_count * 8);
-        CK(launch_after(k_lit_scan, lgrid, LIT_THREADS, st, 0, early, L));
-        CK(launch_after(k_lit_select, lgrid, LIT_THREADS, st, 0, early, L));
+        const size_t stretches = (size_t)(P.hi / 32 + 4 + LIT_TILE_WORDS - 1) / LIT_TILE_WORDS;
+        if (v->lit.apart) CK(launch_after(k_lit_mark, (int)(stretches < (size_t)v->sm_count * 8 ? stretches : (size_t)v->sm_count * 8), LIT_MARK_THREADS, st, 0, early, L));
+        else {
+            CK(launch_after(k_lit_scan, lgrid, LIT_THREADS, st, 0, early, L));
+            CK(launch_after(k_lit_select, lgrid, LIT_THREADS, st, 0, early, L));
+        }
         P.docmask = w.docmask; P.litstart = w.litstart; P.litin = w.litin;
     }
     const bool bulk = P.ntiles > MERGE_SR_MAX_TILES;
@@ -769,6 +773,9 @@ extern "C" int tt_vocab_add_literals(tt_vocab* v, const uint8_t* bytes, const ui
         return TT_ERR_CUDA;
     }
     T.entries = v->d_lit_entries; T.blob = v->d_lit_blob; T.n = (u32)n; T.maxlen = maxlen;
+    T.apart = true;
+    for (size_t i = 0; i < n; i++)
+        for (u32 k = off[i] + 1; k < off[i + 1]; k++) if ((T.first_byte[bytes[k] >> 5] >> (bytes[k] & 31)) & 1u) T.apart = false;
     // the literals are registered (v->lit) only once every allocation and copy below has succeeded, so that a
     // failed call leaves the vocabulary as it was and may be repeated
     auto undo = [&]() { cudaFree(v->d_lit_entries); cudaFree(v->d_lit_blob); v->d_lit_entries = nullptr; v->d_lit_blob = nullptr; };
