@@ -462,7 +462,15 @@ extern "C" int tt_vocab_load_ex(const tt_merge* merges, size_t n_merges, const i
             }
             if (!placed) { ok_all = false; break; }
         }
-        if (ok_all) break;
+        if (!ok_all) continue;
+        for (size_t h = 0; h < nbuckets; h++) slots[2 * h].y &= ~PAIR_OVERFLOW;
+        for (size_t i = 0; i < cap; i++) {
+            if (is_free(uint4{slots[i].x, slots[i].y | PAIR_OVERFLOW, 0, 0})) continue;
+            const u64 key = ((((u64)(slots[i].y & PAIR_HI)) << 32) | slots[i].x) >> 20;
+            const u32 h0 = pair_bucket(key, shift);
+            if (h0 != i / 2) slots[2 * (size_t)h0].y |= PAIR_OVERFLOW;
+        }
+        break;
     }
     tt_vocab* v = new (std::nothrow) tt_vocab();
     if (!v) return TT_ERR_CUDA;

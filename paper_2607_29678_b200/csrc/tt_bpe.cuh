@@ -37,7 +37,8 @@
 // Two-choice (cuckoo) hashing over buckets of two 16-byte slots (one 32-byte sector): a key is in one of its
 // two buckets or nowhere, so a probe is two independent sector loads and no chain to walk, hit or miss.
 // slot = { (left << 38) | (right << 20) | rank20, cl, cr } with rank20 = 0xFFFFF for a pair that is no merge
-// itself (it is in the table for its guards); a free slot is all ones.
+// itself (it is in the table for its guards).  A free slot is all ones.  The top bit of a bucket's first slot's second word is zero
+// where no key with this first bucket had to go to its second one: who can wait for the first bucket need not look there.
 struct PairInfo { u32 r, cl, cr; };                   // TT_RANK_INF where there is none
 struct PairTable {
     const uint4* slots;   // 2 * (mask + 1) slots
@@ -60,10 +61,13 @@ TT_HD u32 pair_bucket_alt(u64 key, u32 shift, u32 first) {      // the key's oth
 }
 
 __device__ __forceinline__ PairInfo pair_none() { PairInfo p; p.r = p.cl = p.cr = TT_RANK_INF; return p; }
-__device__ __forceinline__ bool pair_match(const uint4 s, u64 key, PairInfo& out) {
-    const u64 kr = ((u64)s.y << 32) | s.x;
-    if ((kr >> 20) != key) return false;
-    out.r = f20_decode((u32)kr & TT_F20); out.cl = s.z; out.cr = s.w;
+constexpr u32 PAIR_HI = 0x00FFFFFFu, PAIR_OVERFLOW = 0x80000000u;      // second word of a slot: the key's upper 24 bits; of a bucket's first slot: see above
+// A slot's first word holds the key's low 12 bits over the rank: where key and slot agree, their difference is the rank.  (A free slot
+// reads as the pair of the two highest ids, which is no merge and has no guards.)
+__device__ __forceinline__ bool pair_match(const uint4 s, u32 hi, u32 lo, PairInfo& out) {
+    const u32 r = s.x ^ lo;
+    if (((s.y ^ hi) & PAIR_HI) != 0 || r > TT_F20) return false;
+    out.r = f20_decode(r); out.cl = s.z; out.cr = s.w;
     return true;
 }
 
@@ -75,7 +79,8 @@ __device__ __forceinline__ PairInfo pair_probe(const PairTable& t, u32 a, u32 b)
     uint4 x0, y0, x1, y1;
     ldg_sector(b0, x0, y0); ldg_sector(b1, x1, y1);
     PairInfo out = pair_none();
-    if (!pair_match(x0, key, out) && !pair_match(y0, key, out) && !pair_match(x1, key, out)) pair_match(y1, key, out);
+    const u32 hi = (u32)(key >> 12), lo = (u32)key << 20;
+    if (!pair_match(x0, hi, lo, out) && !pair_match(y0, hi, lo, out) && !pair_match(x1, hi, lo, out)) pair_match(y1, hi, lo, out);
     return out;
 }
 __device__ __forceinline__ PairInfo bytepair_info(const PairTable& t, u32 a, u32 b) {
@@ -416,9 +421,10 @@ constexpr int LANE_MAX = 32;                          // bytes per piece on this
 constexpr u32 LANE_NONE = 0xFFFFFFFFu;                // no pair begins here
 // Two independent probes, ranks only (TT_F20 or more: none).  A slot's first word holds the key's low 12 bits over the rank: where key and
 // slot agree, their difference is the rank.  ALL: all four buckets at once, the shorter chain, for a request; else a key's second
-// bucket only where the first has not got it, for bulk text, whose warps saturate the way to L2 (132 MB batch: all at once 773 us a
-// call, so 740; 15,000 pieces of 1,000 messages: the second bucket afterwards 60 us, all at once 55.6).
-__device__ __forceinline__ u32 pair_rank_of(const uint4 s, u32 hi, u32 lo) { return s.y == hi ? s.x ^ lo : TT_RANK_INF; }
+// bucket only where the first has not got it and says that it overflowed, for bulk text, whose warps saturate the way to L2 (132 MB batch:
+// all at once 773 us a call, the second afterwards 740, only of those that overflowed 731; 64 documents of 100,000 characters with
+// 4,096 merges 241, 225, 213.  15,000 pieces of 1,000 messages: the second bucket afterwards 60 us, all at once 55.6).
+__device__ __forceinline__ u32 pair_rank_of(const uint4 s, u32 hi, u32 lo) { return ((s.y ^ hi) & PAIR_HI) == 0 ? s.x ^ lo : TT_RANK_INF; }
 template <bool ALL>
 __device__ __forceinline__ void pair_probe2(const PairTable& t, u64 key0, u64 key1, u32& r0, u32& r1) {
     const u32 h00 = pair_bucket(key0, t.shift), h10 = pair_bucket(key1, t.shift);
@@ -431,9 +437,9 @@ __device__ __forceinline__ void pair_probe2(const PairTable& t, u64 key0, u64 ke
     r0 = min(pair_rank_of(a00, hi0, lo0), pair_rank_of(a01, hi0, lo0));
     r1 = min(pair_rank_of(a10, hi1, lo1), pair_rank_of(a11, hi1, lo1));
     if (!ALL) {
-        a02 = a03 = a12 = a13 = make_uint4(0, 0xFFFFFFFFu, 0, 0);             // (no key's: a key has 36 bits, 24 of them here)
-        if (r0 > TT_F20) ldg_sector(p01, a02, a03);
-        if (r1 > TT_F20) ldg_sector(p11, a12, a13);
+        a02 = a03 = make_uint4(~lo0, hi0, 0, 0); a12 = a13 = make_uint4(~lo1, hi1, 0, 0);             // (not this key's)
+        if (r0 > TT_F20 && (a00.y & PAIR_OVERFLOW)) ldg_sector(p01, a02, a03);
+        if (r1 > TT_F20 && (a10.y & PAIR_OVERFLOW)) ldg_sector(p11, a12, a13);
     }
     r0 = min(r0, min(pair_rank_of(a02, hi0, lo0), pair_rank_of(a03, hi0, lo0)));
     r1 = min(r1, min(pair_rank_of(a12, hi1, lo1), pair_rank_of(a13, hi1, lo1)));

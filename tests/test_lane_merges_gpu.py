@@ -32,10 +32,11 @@ def test_words_of_every_length(name, alphabet, lo, hi, per_warp):
 
 
 # more than 4 MB: the lists of bulk text, with few and with many pieces of a class
+@pytest.mark.parametrize("name", ["C1", "C4"])
 @pytest.mark.parametrize("lo,hi,size", [(2, 32, 5_000_000), (30, 66, 5_000_000), (33, 64, 6_000_000), (100, 250, 5_000_000)])
-def test_bulk_words_of_every_length(lo, hi, size):
+def test_bulk_words_of_every_length(name, lo, hi, size):
     rng = np.random.default_rng(lo + hi)
-    gv, cv = gpu_vocab("C1"), cpu_vocab("C1")
+    gv, cv = gpu_vocab(name), cpu_vocab(name)
     text = _words(rng, rng.integers(lo, hi + 1, 2 * size // (lo + hi)), b"etaoinshr")
     ids, status = gpu_encode(gv, text)
     assert status == 0 and same(ids, cv.encode(text, gv.pattern_id, nthreads=8)[0])
