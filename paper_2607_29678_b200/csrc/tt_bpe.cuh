@@ -8,7 +8,7 @@
 //     left the others in its tile's queue region by length class;
 //   * k_merge (a request) / k_closing + k_merge_bulk (bulk text): a warp per piece (<= 32 bytes: tokens in registers,
 //     candidates as ballot masks; <= 256 bytes: several tokens per lane, compaction through shared memory), or, where
-//     the call has many pieces of <= 32 bytes, 32 of them at once, a thread per piece (lane_merge); a longer piece is
+//     the call has many pieces of <= 32 bytes, up to 32 of them at once, a thread per piece (lane_merge); a longer piece is
 //     merged as runs of bytes if it has few, else cut into windows of 256 bytes, a warp each, that are joined at
 //     shared tokens (see "long pieces"); where windows do not meet, the piece is merged whole by a CTA of 768 threads
 //     (cta_merge_long: state in shared memory, or in global scratch while it still has more than 14,336 tokens).
@@ -812,7 +812,7 @@ struct PieceParams {
 //     closing pieces of the tiles, short pieces; by tickets where CTAs had long pieces first.  With many short pieces these go in
 //     batches, a thread each (merge_short_batches).
 // Bulk text (k_merge_bulk): k_closing has gathered global lists.  Long pieces by tickets of a CTA, warp-class pieces a warp each
-// by index, short pieces by tickets of 32 of one length class, a thread each, the longest class first.
+// by index, short pieces by tickets of up to 32 of one length class, a thread each, the longest class first.
 #ifndef TT_MERGE_WARPS
 #define TT_MERGE_WARPS 24
 #endif
@@ -1434,7 +1434,7 @@ __device__ __forceinline__ void merge_group_totals(const PieceParams& P, u32* s_
 }
 
 // Bulk text (k_closing has gathered the lists): long pieces a CTA each where that is quick, else window by window with the
-// whole grid, warp-class pieces a warp each by index, short pieces 32 of one length class at a time by ticket, a thread each.
+// whole grid, warp-class pieces a warp each by index, short pieces in batches of one length class by ticket, a thread each.
 __device__ void merge_bulk_lists(const PieceParams& P, const u8* __restrict__ text, u64* s_buf, u32* sc, LongShared& LS, u32* s_last) {
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const u32 FULL = 0xFFFFFFFFu;
@@ -1462,7 +1462,7 @@ __device__ void merge_bulk_lists(const PieceParams& P, const u8* __restrict__ te
         warp_merge_piece(P, text, (u32)((long long)t * TT_TILE_BYTES + (e & 2047u) - P.shift), (e >> 22) + 1, t * TT_TILE_BYTES + ((e >> 11) & 2047u), wbuf, lane);
     }
     u32* const tok = reinterpret_cast<u32*>(wbuf);
-    // tickets: 32 pieces of one list each, the list of the longest pieces first
+    // tickets: a batch of one list each, the list of the longest pieces first
     u32 cnts[TT_SHORT_CLASSES], nb[TT_SHORT_CLASSES], nball = 0;
 #pragma unroll
     for (int c = 0; c < TT_SHORT_CLASSES; c++) { cnts[c] = c ? P.hdr->nq_short_x[c - 1] : ns; nball += cnts[c]; }

@@ -107,10 +107,10 @@ __device__ __forceinline__ void hdr_set_status(TTHeader* h, unsigned long long e
 //   tile_last[t]   offset in the tile of its last piece start (that piece ends in a later tile, or with the text)
 //   tile_tok[t]    tokens of the tile's pieces (the first kernel stores the settled ones, k_merge adds the rest)
 //   tile_q[t]      unsettled pieces: short (<= 32 B) count | warp-class (33..256 B) count << 11 | long count << 18; bit 31: a piece
-//                  of more than 256 bytes may begin or end here
-//   piece_off16    [t * TT_TILE_BYTES + i]  offset in the tile of piece i
+//                  of more than 256 bytes may begin or end here; bit 30 (bulk text): a document starts here
+//   piece_off16    [t * TT_TILE_BYTES + i]  offset in the tile of piece i (bulk text: only in tiles with a document start, and of long pieces)
 //   piece_cnt      [t * TT_TILE_BYTES + i]  the id of piece i if it is one token found without merging (>= 0),
-//                                           else minus the number of ids staged at the piece's text offset
+//                                           else minus the number of ids staged at the piece's text offset (bulk text: see PIECE_STAGED)
 //   q              [t * TT_TILE_QCAP ...]   queue entries of the tile: short pieces from the front, warp-class
 //                                           pieces from the back; entry = offset in tile | index << 11 | (bytes-1) << 22
 //   tile_long      [t * TT_TILE_LONGCAP + k] index of the k-th piece of > 256 bytes that lies inside the tile
