@@ -629,12 +629,12 @@ def csrc_hash() -> str:
 # captures.  They belong to the source state whose hash is recorded with them; with other sources they are not
 # printed as measurements (the keys are null and "capture_stale" is true).
 NCU_CAPTURE = {
-    "csrc": "1b43ad580abf1f9b",
+    "csrc": "7fea48fa5fb435cd",
     # kernel -> dram__bytes_read.sum + dram__bytes_write.sum per launch, one cold C3 request (ncu --set full)
-    "c3_dram_bytes": {"front": 13650432, "merge": 9395200, "scatter": 2049536},
+    "c3_dram_bytes": {"front": 13650688, "merge": 9397248, "scatter": 2048512},
     # kernel -> smsp__inst_executed.sum per launch of the 256-request batch: captured on the first 32 documents of the same
     # batch (16,315,836 bytes) and scaled by text bytes to the full 132,689,913 (all work is per tile or per piece)
-    "batch_warp_inst": {"front": 296646000, "closing": 2482000, "merge_bulk": 108434000, "scatter_bulk": 78840000},
+    "batch_warp_inst": {"front": 279323000, "closing": 2480000, "merge_bulk": 89060000, "scatter_bulk": 83813000},
 }
 
 
