@@ -1775,8 +1775,9 @@ __device__ __forceinline__ void scatter_tiles(const ScatterParams& P, ScatterSha
                 if (P.count_out) *P.count_out = status ? 0 : (long long)total;
             }
             if (status != 0) {
-                if (P.ids_off_out)
-                    for (long long d = (long long)blockIdx.x * blockDim.x + tid; d <= P.n_docs; d += (long long)gridDim.x * blockDim.x) P.ids_off_out[d] = 0;
+                // (by the CTAs that are here: those without a tile have left)
+                const long long step = (long long)((P.ntiles + per - 1) / per) * blockDim.x;
+                if (P.ids_off_out) for (long long d = (long long)blockIdx.x * blockDim.x + tid; d <= P.n_docs; d += step) P.ids_off_out[d] = 0;
                 return;
             }
             if (P.ids_off_out && blockIdx.x == 0) {

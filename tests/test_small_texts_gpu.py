@@ -87,3 +87,34 @@ def test_replayed_from_a_graph_and_beside_other_streams():
         g.replay()
     torch.cuda.synchronize()
     assert same(bufs[0]["ids"][:int(bufs[0]["count"])].cpu().numpy(), cv.encode(other.cpu().numpy(), gv.pattern_id)[0])
+
+
+# Entries of ids_off are cleared by the CTAs that have a tile: texts of which some CTAs have none (a few tiles in the one launch; more tiles than
+# CTAs, two to a CTA, in the scatter of a request), with more documents than one such CTA has threads.
+@pytest.mark.parametrize("size", [100, 2_000, 4_000, 8_000, 9_000, 1_300 * TILE])
+@pytest.mark.parametrize("n_docs", [1_000, 5_000, 13_000, 400_000])
+def test_every_offset_is_zero_on_an_error(size, n_docs):
+    import torch
+    gv, cv = gpu_vocab("C1"), cpu_vocab("C1")
+    text = wl.generate(0, size, size)
+    off = np.sort(np.random.default_rng(n_docs).integers(0, size + 1, n_docs + 1))
+    off[0], off[-1] = 0, size
+    bad, crossed = text.copy(), off.copy()
+    bad[size // 2] = 0xFF
+    crossed[1] = size + 1
+    n = cv.encode_batch(text, off, 0)[0].size
+    for t, o, cap, want in ((bad, off, size, 4), (text, off, n - 1, 5), (text, crossed, size, 1), (text, off, n, 0)):
+        bufs = gv.alloc(size, max_docs=n_docs)
+        bufs["ids"] = bufs["ids"][:cap]
+        bufs["ids_off"].fill_(77)
+        try:
+            gv.encode_batch(torch.from_numpy(t).cuda(), torch.from_numpy(o).cuda(), bufs)
+        except Exception as e:
+            pytest.fail(str(e))
+        torch.cuda.synchronize()
+        assert int(bufs["status"]) == want, want
+        got = bufs["ids_off"].cpu().numpy()
+        if want:
+            assert np.flatnonzero(got).size == 0, (want, np.flatnonzero(got).size)
+        else:
+            assert same(got, cv.encode_batch(text, off, 0)[1])
