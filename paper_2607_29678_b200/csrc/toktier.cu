@@ -7,7 +7,6 @@
 #include "../../include/toktier.h"
 #include "tt_common.cuh"
 #include "tt_pretok_kernels.cuh"
-#include "tt_small.cuh"
 #include "tt_bpe.cuh"
 #include "tt_spans.cuh"
 #include "tt_session.cuh"
@@ -57,7 +56,6 @@ struct tt_vocab {
     int pattern = 0;
     int device = 0;
     int sm_count = 148;
-    bool one_launch = false;             // small texts take k_small (the device can place its cluster)
     size_t n_merges = 0;
     uint4* d_slots = nullptr;
     u64* d_bytepair = nullptr;
@@ -86,22 +84,6 @@ struct tt_vocab {
     cudaStream_t host_stream = nullptr;
     cudaEvent_t slice_ev[8] = {};
 };
-
-// Can the device place such a cluster?
-template <class K> static bool small_fits(K kernel) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(SMALL_CTAS); cfg.blockDim = dim3(MERGE_THREADS); cfg.dynamicSmemBytes = SMALL_SMEM_BYTES;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = SMALL_CTAS; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    int n = 0;
-    const bool ok = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMALL_SMEM_BYTES) == cudaSuccess &&
-                    cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-                    cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n > 0;
-    if (!ok) cudaGetLastError();
-    return ok;
-}
 
 static inline ExtMap ext_map(const tt_vocab* v) { ExtMap m; m.id = v->d_ext_id; m.delta = v->ext_delta; m.plain = v->ext_plain; return m; }
 static inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -505,7 +487,6 @@ extern "C" int tt_vocab_load_ex(const tt_merge* merges, size_t n_merges, const i
     if (cudaFuncSetAttribute(k_merge, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MERGE_SMEM_REQUEST) != cudaSuccess ||
         cudaFuncSetAttribute(k_merge_bulk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MERGE_SMEM_BYTES) != cudaSuccess ||
         cudaFuncSetAttribute(k_repair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RepairSmem)) != cudaSuccess) { cudaGetLastError(); tt_vocab_free(v); return TT_ERR_CUDA; }
-    v->one_launch = small_fits(k_small<TT_PATTERN_CL100K>) && small_fits(k_small<TT_PATTERN_O200K>) && small_fits(k_small<TT_PATTERN_CL100K_N1>);
     { const int rc = build_token_table(v, merges, n_merges, ext_id); if (rc != TT_OK) { tt_vocab_free(v); return rc; } }
     {   // byte length and number of non-continuation bytes of every token, indexed by the caller's id
         std::vector<uint2> in(256 + n_merges);
@@ -614,26 +595,11 @@ static cudaError_t launch_pretok(int grid, cudaStream_t st, bool early, const Pr
     }
 }
 
-static cudaError_t launch_small(cudaStream_t st, const PretokParams& P, const FrontParams& F, const PieceParams& Q, const ScatterParams& S) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(SMALL_CTAS); cfg.blockDim = dim3(MERGE_THREADS); cfg.dynamicSmemBytes = SMALL_SMEM_BYTES; cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = SMALL_CTAS; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
-    cfg.attrs = attr; cfg.numAttrs = 2;
-    switch (P.pattern) {
-    case TT_PATTERN_O200K:     return cudaLaunchKernelEx(&cfg, k_small<TT_PATTERN_O200K>, P, F, Q, S);
-    case TT_PATTERN_CL100K_N1: return cudaLaunchKernelEx(&cfg, k_small<TT_PATTERN_CL100K_N1>, P, F, Q, S);
-    default:                   return cudaLaunchKernelEx(&cfg, k_small<TT_PATTERN_CL100K>, P, F, Q, S);
-    }
-}
 // Enqueues K1+K2 (and K3 when piece_off_dst is given: only tt_pretokenize materialises the offsets;
-// the encode chain derives them per tile from the start flags).  front: the fused kernel is not launched, its parameters are left there.
+// the encode chain derives them per tile from the start flags).
 static int run_pretok(const tt_vocab* v, const uint8_t* text, size_t len, const int64_t* doc_off, size_t n_docs,
                       cudaStream_t st, TTWorkspace& w, u32* piece_off_dst, PretokParams& P, bool literals = false, bool fused = false,
-                      const uint8_t* host_src = nullptr, bool early = true, FrontParams* front = nullptr) {
+                      const uint8_t* host_src = nullptr, bool early = true) {
     const uintptr_t addr = (uintptr_t)text;
     const long long shift = (long long)(addr & 15);
     P.base = (const u8*)(addr - shift);
@@ -694,8 +660,7 @@ static int run_pretok(const tt_vocab* v, const uint8_t* text, size_t len, const 
         F.tile_last = w.tile_last; F.tile_tok = w.tile_tok; F.tile_q = w.tile_q; F.tile_long = w.tile_long; F.piece_off16 = w.piece_off16;
         F.piece_cnt = w.piece_cnt; F.q = w.q; F.toktab = v->toktab; F.longtab = v->longtab; F.ext_id = v->d_ext_id;
         F.wq = P.ntiles > MERGE_SR_MAX_TILES ? w.wq : nullptr;
-        if (front) *front = F;
-        else if (bulk) CK((launch_pretok<true, PRETOK_THREADS_BULK, PRETOK_CTAS_BULK>(grid, st, early, P, F)));
+        if (bulk) CK((launch_pretok<true, PRETOK_THREADS_BULK, PRETOK_CTAS_BULK>(grid, st, early, P, F)));
         else CK((launch_pretok<true, PRETOK_THREADS_REQUEST, PRETOK_CTAS_REQUEST>(grid, st, early, P, F)));
     } else CK((launch_pretok<false, PRETOK_THREADS_REQUEST, PRETOK_CTAS_REQUEST>(grid, st, early, P, FrontParams{})));
     if (piece_off_dst)
@@ -738,11 +703,8 @@ static int encode_impl(const tt_vocab* v, const uint8_t* text, size_t len, const
     const bool big = (((uintptr_t)text & 15) + len + TT_TILE_BYTES - 1) / TT_TILE_BYTES > (size_t)MERGE_SR_MAX_TILES;
     if (big || cap != cudaStreamCaptureStatusNone) CK(cudaMemsetAsync(w.hdr, 0, sizeof(TTHeader), st));
     MARK(0);
-    // A text of at most SMALL_TILES tiles is one launch (tt_encode_timed, which times the kernels one by one, has three).
-    const bool small = v->one_launch && ev == nullptr && (((uintptr_t)text & 15) + len + TT_TILE_BYTES - 1) / TT_TILE_BYTES <= (size_t)SMALL_TILES;
     PretokParams PP;
-    FrontParams front;
-    int rc = run_pretok(v, text, len, doc_off, n_docs, st, w, nullptr, PP, literals, true, host_src, ev == nullptr, small ? &front : nullptr);
+    int rc = run_pretok(v, text, len, doc_off, n_docs, st, w, nullptr, PP, literals, true, host_src, ev == nullptr);
     if (rc != TT_OK) return rc;
     MARK(1);
     const int merge_grid = v->sm_count * MERGE_CTAS_PER_SM;                  // all resident CTA slots: a request's unsettled pieces get a warp each
@@ -756,17 +718,6 @@ static int encode_impl(const tt_vocab* v, const uint8_t* text, size_t len, const
     Q.wq = big ? w.wq : nullptr; Q.gq = big ? w.gq : nullptr;
     for (int c = 0; c < TT_SHORT_CLASSES - 1; c++) Q.gq_x[c] = big ? w.gq_x[c] : nullptr;
     Q.lq = w.lq; Q.tok_len = v->d_tok_len;
-    ScatterParams S;
-    S.shift = PP.lo; S.hi = PP.hi; S.ntiles = PP.ntiles; S.tile_cnt = w.tile_cnt; S.tile_tok = w.tile_tok; S.grp_tok = Q.grp_tok; S.piece_off16 = w.piece_off16; S.tile_q = w.tile_q;
-    S.ids_cap = (unsigned long long)ids_cap; S.piece_cnt = w.piece_cnt; S.stage = w.stage; S.hdr = w.hdr; S.epoch = PP.epoch;
-    S.ids_out = ids_out; S.count_out = (long long*)count_out; S.status_out = status_out;
-    S.docmask = doc_off ? w.docmask : nullptr; S.doc_off = (const long long*)doc_off; S.n_docs = (int)n_docs;
-    S.ids_off_out = (long long*)ids_off_out;
-    if (small) {
-        CK(launch_small(st, PP, front, Q, S));
-        CK(cudaGetLastError());
-        return TT_OK;
-    }
     if (big) {                                                               // bulk text: closing pieces and the global lists first
         const int cgrid = (PP.ntiles + CLOSING_THREADS - 1) / CLOSING_THREADS;
         // (placed only when the first kernel is through: placed early, together with k_merge_bulk, the merges took up to a third longer --
@@ -776,6 +727,12 @@ static int encode_impl(const tt_vocab* v, const uint8_t* text, size_t len, const
     }
     CK(launch_after(big ? k_merge_bulk : k_merge, merge_grid, MERGE_THREADS, st, big ? MERGE_SMEM_BYTES : MERGE_SMEM_REQUEST, ev == nullptr, Q));
     MARK(2);
+    ScatterParams S;
+    S.shift = PP.lo; S.hi = PP.hi; S.ntiles = PP.ntiles; S.tile_cnt = w.tile_cnt; S.tile_tok = w.tile_tok; S.grp_tok = Q.grp_tok; S.piece_off16 = w.piece_off16; S.tile_q = w.tile_q;
+    S.ids_cap = (unsigned long long)ids_cap; S.piece_cnt = w.piece_cnt; S.stage = w.stage; S.hdr = w.hdr; S.epoch = PP.epoch;
+    S.ids_out = ids_out; S.count_out = (long long*)count_out; S.status_out = status_out;
+    S.docmask = doc_off ? w.docmask : nullptr; S.doc_off = (const long long*)doc_off; S.n_docs = (int)n_docs;
+    S.ids_off_out = (long long*)ids_off_out;
     const bool many = PP.ntiles > v->sm_count * SCATTER_CTAS;
     const int scatter_ctas = v->sm_count * (big ? SCATTER_BULK_CTAS : 8);
     CK(launch_after(big ? k_scatter_bulk : many ? k_scatter<SCATTER_CTAS_MANY> : k_scatter<SCATTER_CTAS>, PP.ntiles < scatter_ctas ? PP.ntiles : scatter_ctas,

@@ -1617,10 +1617,17 @@ __device__ __noinline__ void merge_short_batches(const PieceParams& P, const u8*
     }
 }
 
-// The kernel's work once the first kernel's records are complete.  s_buf: MERGE_SMEM_REQUEST bytes.
-__device__ __forceinline__ void merge_request(const PieceParams& P, u64* s_buf, u32* sc, LongShared& LS) {
+__global__ void __launch_bounds__(MERGE_THREADS, MERGE_CTAS_PER_SM)
+k_merge(const __grid_constant__ PieceParams P) {
+    extern __shared__ __align__(16) u64 s_buf[];              // MERGE_SMEM_REQUEST
+    __shared__ u32 sc[SCR_WORDS];
+    __shared__ LongShared LS;
     MergeIndex& X = *reinterpret_cast<MergeIndex*>(s_buf + MERGE_WARPS * WARP_SMEM_WORDS);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    cudaTriggerProgrammaticLaunchCompletion();               // k_scatter may be placed; it waits for this grid's memory itself
+    grid_prefetch_l2(P.tab.slots, ((size_t)P.tab.mask + 1) * 2 * sizeof(uint4));
+    grid_prefetch_l2(P.tab.bytepair, 65536 * sizeof(u64));
+    cudaGridDependencySynchronize();                         // the first kernel's per-tile records are complete from here on
     const int status = hdr_status(P.hdr, P.epoch);
     const int unit = (P.ntiles + MERGE_ENTRIES - 1) / MERGE_ENTRIES, entries = (P.ntiles + unit - 1) / unit;   // tiles per entry: 1 for a request
     const bool may_long = merge_index(P, unit, entries, X);
@@ -1662,17 +1669,6 @@ __device__ __forceinline__ void merge_request(const PieceParams& P, u64* s_buf, 
     }
     if (longs == 2) long_phase(P, text, long_find_tasks(P), s_buf, sc, LS);
 }
-__global__ void __launch_bounds__(MERGE_THREADS, MERGE_CTAS_PER_SM)
-k_merge(const __grid_constant__ PieceParams P) {
-    extern __shared__ __align__(16) u64 s_buf[];              // MERGE_SMEM_REQUEST
-    __shared__ u32 sc[SCR_WORDS];
-    __shared__ LongShared LS;
-    cudaTriggerProgrammaticLaunchCompletion();               // k_scatter may be placed; it waits for this grid's memory itself
-    grid_prefetch_l2(P.tab.slots, ((size_t)P.tab.mask + 1) * 2 * sizeof(uint4));
-    grid_prefetch_l2(P.tab.bytepair, 65536 * sizeof(u64));
-    cudaGridDependencySynchronize();                         // the first kernel's per-tile records are complete from here on
-    merge_request(P, s_buf, sc, LS);
-}
 
 // ---- K5: coalesced scatter of the staged ids, one text tile per CTA iteration ---------------------------------
 // Also writes the token offset of every document that starts in the tile (batch calls).
@@ -1709,19 +1705,21 @@ constexpr u32 SCATTER_WARP_MAX = 512;                     // tokens of a piece t
 // tiles' token counts, the first item's values and offsets, read before its length is known -- is asked for at once, the sums
 // over the tiles and the scan over the item's pieces share one barrier, and a staged piece's ids are fetched side by
 // side.  (Step by step, with a barrier after each, the kernel took 7.5 us behind k_merge on a 1M-char request.)
-template <int NT> struct ScatterShared {
-    u32 scan[2][NT / 32], before[NT / 32], total[NT / 32];
-    u32 big[TT_TILE_BYTES / 8][3];
-    u32 nbig;
-    int32_t out[SCATTER_STAGE_IDS];                          // the ids of one item on their way out
-};
-// The kernel's work once the merges are complete.
-template <int NT>
-__device__ __forceinline__ void scatter_tiles(const ScatterParams& P, ScatterShared<NT>& SH) {
-    auto& s_scan = SH.scan; auto& s_before = SH.before; auto& s_total = SH.total; auto& s_big = SH.big; auto& s_out = SH.out;
-    u32& s_nbig = SH.nbig;
+template <int MINB>
+__global__ void __launch_bounds__(BPE_THREADS, MINB)
+k_scatter(const __grid_constant__ ScatterParams P) {
+    __shared__ u32 s_scan[2][BPE_WARPS], s_before[BPE_WARPS], s_total[BPE_WARPS];
+    __shared__ u32 s_big[TT_TILE_BYTES / 8][3];
+    __shared__ u32 s_nbig;
+    __shared__ int32_t s_out[SCATTER_STAGE_IDS];              // the ids of one item on their way out
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const u32 FULL = 0xFFFFFFFFu;
+    cudaGridDependencySynchronize();                         // k_merge's (and with it the first kernel's) results are complete from here on
+    // The next call's first kernel may be placed from here on; it waits for this grid itself.  (Allowed earlier, while this grid still waits
+    // for k_merge, its CTAs -- and those of the call's other kernels -- gathered on the SMs whose k_merge CTA was through first:
+    // 150,000 pieces of two bytes, call after call, 177 us instead of 108, 300 KB of short accented words 815 instead of 651;
+    // 300 KB of Unicode-heavy text 38.8 instead of 35.5.)
+    cudaTriggerProgrammaticLaunchCompletion();
     // Each CTA takes a contiguous range of tiles and sums the token counts before it, and all of them (the count, and the
     // capacity check, which every CTA makes for itself).
     const int per = (P.ntiles + (int)gridDim.x - 1) / (int)gridDim.x;
@@ -1734,12 +1732,12 @@ __device__ __forceinline__ void scatter_tiles(const ScatterParams& P, ScatterSha
     u32 o2 = *reinterpret_cast<const u32*>(P.piece_off16 + (size_t)tile * TT_TILE_BYTES + 2 * tid);
     int status = hdr_status(P.hdr, P.epoch);
     u32 before = 0, total = 0;                                // (a text has fewer than 2^31 bytes)
-    for (int t0 = 0; t0 < P.ntiles; t0 += NT * 4) {
+    for (int t0 = 0; t0 < P.ntiles; t0 += BPE_THREADS * 4) {
         u32 x[4];
 #pragma unroll
-        for (int u = 0; u < 4; u++) { const int t = t0 + u * NT + tid; x[u] = t < P.ntiles ? P.tile_tok[t] : 0u; }
+        for (int u = 0; u < 4; u++) { const int t = t0 + u * BPE_THREADS + tid; x[u] = t < P.ntiles ? P.tile_tok[t] : 0u; }
 #pragma unroll
-        for (int u = 0; u < 4; u++) { total += x[u]; if (t0 + u * NT + tid < tile_lo) before += x[u]; }
+        for (int u = 0; u < 4; u++) { total += x[u]; if (t0 + u * BPE_THREADS + tid < tile_lo) before += x[u]; }
     }
     before = __reduce_add_sync(FULL, before); total = __reduce_add_sync(FULL, total);
     if (lane == 0) { s_before[wid] = before; s_total[wid] = total; }
@@ -1747,7 +1745,7 @@ __device__ __forceinline__ void scatter_tiles(const ScatterParams& P, ScatterSha
     for (int item = 0;; item++) {                             // block-uniform
         // the item after this one
         int tile2 = tile;
-        u32 b2 = b + 2 * NT, np2 = np;
+        u32 b2 = b + 2 * BPE_THREADS, np2 = np;
         if (b2 >= np) { b2 = 0; tile2++; np2 = tile2 < tile_hi ? P.tile_cnt[tile2] : 0u; }
         uint2 vn = make_uint2(0, 0);
         u32 on = 0;
@@ -1768,7 +1766,7 @@ __device__ __forceinline__ void scatter_tiles(const ScatterParams& P, ScatterSha
         if (item == 0) {
             total = 0;
 #pragma unroll
-            for (int w = 0; w < (NT / 32); w++) { carry += s_before[w]; total += s_total[w]; }
+            for (int w = 0; w < BPE_WARPS; w++) { carry += s_before[w]; total += s_total[w]; }
             if (status == 0 && total > P.ids_cap) status = 5;         // TT_ERR_CAPACITY
             if (blockIdx.x == 0 && tid == 0) {
                 if (P.status_out) *P.status_out = status;
@@ -1788,7 +1786,7 @@ __device__ __forceinline__ void scatter_tiles(const ScatterParams& P, ScatterSha
         }
         u32 d0 = carry + inc - c[0] - c[1], tot = 0;
 #pragma unroll
-        for (int w = 0; w < (NT / 32); w++) { const u32 y = s_scan[item & 1][w]; tot += y; if (w < wid) d0 += y; }
+        for (int w = 0; w < BPE_WARPS; w++) { const u32 y = s_scan[item & 1][w]; tot += y; if (w < wid) d0 += y; }
         // An item of at most SCATTER_STAGE_IDS tokens (nearly all) is put together in shared memory and leaves in whole lines, every
         // thread writing consecutive words: the output may be mapped host memory, where a warp that writes every other word
         // costs a bus transaction per word (100 KB of Unicode-heavy text, written piece by piece: 27 us instead of 9).
@@ -1830,8 +1828,8 @@ __device__ __forceinline__ void scatter_tiles(const ScatterParams& P, ScatterSha
             for (u32 e = 0; e < nbig; e++) {
                 const u32 cc = s_big[e][2];
                 const bool whole = cc > SCATTER_WARP_MAX;         // block-uniform
-                if (!whole && (int)(e % (NT / 32)) != wid) continue;
-                const u32 src = s_big[e][0], d2 = s_big[e][1], step = whole ? (u32)NT : 32u;
+                if (!whole && (int)(e % BPE_WARPS) != wid) continue;
+                const u32 src = s_big[e][0], d2 = s_big[e][1], step = whole ? (u32)BPE_THREADS : 32u;
                 for (u32 k0 = whole ? (u32)tid : (u32)lane; k0 < cc; k0 += 4 * step) {
                     int32_t id[4];
 #pragma unroll
@@ -1845,23 +1843,11 @@ __device__ __forceinline__ void scatter_tiles(const ScatterParams& P, ScatterSha
         }
         // (not beyond the total that was checked against the capacity, whatever the pieces of the item add up to)
         const u32 leave = carry < total ? min(tot, total - carry) : 0u;
-        if (staged) for (u32 kk = tid; kk < leave; kk += NT) P.ids_out[carry + kk] = s_out[kk];
+        if (staged) for (u32 kk = tid; kk < leave; kk += BPE_THREADS) P.ids_out[carry + kk] = s_out[kk];
         carry += tot;
         if (tile2 >= tile_hi) break;
         tile = tile2; b = b2; np = np2; v = vn; o2 = on;
     }
-}
-template <int MINB>
-__global__ void __launch_bounds__(BPE_THREADS, MINB)
-k_scatter(const __grid_constant__ ScatterParams P) {
-    __shared__ ScatterShared<BPE_THREADS> SH;
-    cudaGridDependencySynchronize();                         // k_merge's (and with it the first kernel's) results are complete from here on
-    // The next call's first kernel may be placed from here on; it waits for this grid itself.  (Allowed earlier, while this grid still waits
-    // for k_merge, its CTAs -- and those of the call's other kernels -- gathered on the SMs whose k_merge CTA was through first:
-    // 150,000 pieces of two bytes, call after call, 177 us instead of 108, 300 KB of short accented words 815 instead of 651;
-    // 300 KB of Unicode-heavy text 38.8 instead of 35.5.)
-    cudaTriggerProgrammaticLaunchCompletion();
-    scatter_tiles<BPE_THREADS>(P, SH);
 }
 
 // ---- K5 for bulk text: a warp per tile, no barrier after the prologue -----------------------------------------

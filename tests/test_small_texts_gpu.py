@@ -1,4 +1,4 @@
-"""Texts of a few tiles, which one launch takes, at the edges of its range and with everything a text can hold, against the oracle."""
+"""Texts of a few tiles, at the tiles' edges and with everything a text can hold, against the oracle."""
 import numpy as np
 import pytest
 
@@ -32,7 +32,7 @@ def test_every_kind_of_text_and_pattern(pattern, kind):
         assert status == 0 and same(ids, cv.encode(text, pattern)[0]), chars
 
 
-# pieces of a CTA's size and of the whole cluster's, many short pieces, runs that leave the window
+# pieces of a CTA's size and longer ones, many short pieces, runs that leave the window
 @pytest.mark.parametrize("name", ["C1", "C4"])
 def test_long_pieces_many_pieces_and_runs(name):
     rng = np.random.default_rng(3)
@@ -89,8 +89,8 @@ def test_replayed_from_a_graph_and_beside_other_streams():
     assert same(bufs[0]["ids"][:int(bufs[0]["count"])].cpu().numpy(), cv.encode(other.cpu().numpy(), gv.pattern_id)[0])
 
 
-# Entries of ids_off are cleared by the CTAs that have a tile: texts of which some CTAs have none (a few tiles in the one launch; more tiles than
-# CTAs, two to a CTA, in the scatter of a request), with more documents than one such CTA has threads.
+# Entries of ids_off are cleared by the CTAs that have a tile: texts of a few tiles, and one of which some CTAs have none (more tiles than CTAs, two
+# to a CTA), with more documents than the CTAs with a tile have threads.
 @pytest.mark.parametrize("size", [100, 2_000, 4_000, 8_000, 9_000, 1_300 * TILE])
 @pytest.mark.parametrize("n_docs", [1_000, 5_000, 13_000, 400_000])
 def test_every_offset_is_zero_on_an_error(size, n_docs):
