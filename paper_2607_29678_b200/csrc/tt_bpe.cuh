@@ -1617,17 +1617,10 @@ __device__ __noinline__ void merge_short_batches(const PieceParams& P, const u8*
     }
 }
 
-__global__ void __launch_bounds__(MERGE_THREADS, MERGE_CTAS_PER_SM)
-k_merge(const __grid_constant__ PieceParams P) {
-    extern __shared__ __align__(16) u64 s_buf[];              // MERGE_SMEM_REQUEST
-    __shared__ u32 sc[SCR_WORDS];
-    __shared__ LongShared LS;
+// The kernel's work once the first kernel's records are complete.  s_buf: MERGE_SMEM_REQUEST bytes.
+__device__ __forceinline__ void merge_request(const PieceParams& P, u64* s_buf, u32* sc, LongShared& LS) {
     MergeIndex& X = *reinterpret_cast<MergeIndex*>(s_buf + MERGE_WARPS * WARP_SMEM_WORDS);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    cudaTriggerProgrammaticLaunchCompletion();               // k_scatter may be placed; it waits for this grid's memory itself
-    grid_prefetch_l2(P.tab.slots, ((size_t)P.tab.mask + 1) * 2 * sizeof(uint4));
-    grid_prefetch_l2(P.tab.bytepair, 65536 * sizeof(u64));
-    cudaGridDependencySynchronize();                         // the first kernel's per-tile records are complete from here on
     const int status = hdr_status(P.hdr, P.epoch);
     const int unit = (P.ntiles + MERGE_ENTRIES - 1) / MERGE_ENTRIES, entries = (P.ntiles + unit - 1) / unit;   // tiles per entry: 1 for a request
     const bool may_long = merge_index(P, unit, entries, X);
@@ -1669,6 +1662,17 @@ k_merge(const __grid_constant__ PieceParams P) {
     }
     if (longs == 2) long_phase(P, text, long_find_tasks(P), s_buf, sc, LS);
 }
+__global__ void __launch_bounds__(MERGE_THREADS, MERGE_CTAS_PER_SM)
+k_merge(const __grid_constant__ PieceParams P) {
+    extern __shared__ __align__(16) u64 s_buf[];              // MERGE_SMEM_REQUEST
+    __shared__ u32 sc[SCR_WORDS];
+    __shared__ LongShared LS;
+    cudaTriggerProgrammaticLaunchCompletion();               // k_scatter may be placed; it waits for this grid's memory itself
+    grid_prefetch_l2(P.tab.slots, ((size_t)P.tab.mask + 1) * 2 * sizeof(uint4));
+    grid_prefetch_l2(P.tab.bytepair, 65536 * sizeof(u64));
+    cudaGridDependencySynchronize();                         // the first kernel's per-tile records are complete from here on
+    merge_request(P, s_buf, sc, LS);
+}
 
 // ---- K5: coalesced scatter of the staged ids, one text tile per CTA iteration ---------------------------------
 // Also writes the token offset of every document that starts in the tile (batch calls).
@@ -1705,21 +1709,19 @@ constexpr u32 SCATTER_WARP_MAX = 512;                     // tokens of a piece t
 // tiles' token counts, the first item's values and offsets, read before its length is known -- is asked for at once, the sums
 // over the tiles and the scan over the item's pieces share one barrier, and a staged piece's ids are fetched side by
 // side.  (Step by step, with a barrier after each, the kernel took 7.5 us behind k_merge on a 1M-char request.)
-template <int MINB>
-__global__ void __launch_bounds__(BPE_THREADS, MINB)
-k_scatter(const __grid_constant__ ScatterParams P) {
-    __shared__ u32 s_scan[2][BPE_WARPS], s_before[BPE_WARPS], s_total[BPE_WARPS];
-    __shared__ u32 s_big[TT_TILE_BYTES / 8][3];
-    __shared__ u32 s_nbig;
-    __shared__ int32_t s_out[SCATTER_STAGE_IDS];              // the ids of one item on their way out
+struct ScatterShared {
+    u32 scan[2][BPE_WARPS], before[BPE_WARPS], total[BPE_WARPS];
+    u32 big[TT_TILE_BYTES / 8][3];
+    u32 nbig;
+    int32_t out[SCATTER_STAGE_IDS];                          // the ids of one item on their way out
+};
+// The kernel's work once the merges are complete.  (A function of its own with its shared memory in one structure: written out in the kernel, the
+// five-CTA instance took 20.5 us instead of 18.4 for 2.9 MB of Thai-like text.)
+__device__ __forceinline__ void scatter_tiles(const ScatterParams& P, ScatterShared& SH) {
+    auto& s_scan = SH.scan; auto& s_before = SH.before; auto& s_total = SH.total; auto& s_big = SH.big; auto& s_out = SH.out;
+    u32& s_nbig = SH.nbig;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const u32 FULL = 0xFFFFFFFFu;
-    cudaGridDependencySynchronize();                         // k_merge's (and with it the first kernel's) results are complete from here on
-    // The next call's first kernel may be placed from here on; it waits for this grid itself.  (Allowed earlier, while this grid still waits
-    // for k_merge, its CTAs -- and those of the call's other kernels -- gathered on the SMs whose k_merge CTA was through first:
-    // 150,000 pieces of two bytes, call after call, 177 us instead of 108, 300 KB of short accented words 815 instead of 651;
-    // 300 KB of Unicode-heavy text 38.8 instead of 35.5.)
-    cudaTriggerProgrammaticLaunchCompletion();
     // Each CTA takes a contiguous range of tiles and sums the token counts before it, and all of them (the count, and the
     // capacity check, which every CTA makes for itself).
     const int per = (P.ntiles + (int)gridDim.x - 1) / (int)gridDim.x;
@@ -1848,6 +1850,18 @@ k_scatter(const __grid_constant__ ScatterParams P) {
         if (tile2 >= tile_hi) break;
         tile = tile2; b = b2; np = np2; v = vn; o2 = on;
     }
+}
+template <int MINB>
+__global__ void __launch_bounds__(BPE_THREADS, MINB)
+k_scatter(const __grid_constant__ ScatterParams P) {
+    __shared__ ScatterShared SH;
+    cudaGridDependencySynchronize();                         // k_merge's (and with it the first kernel's) results are complete from here on
+    // The next call's first kernel may be placed from here on; it waits for this grid itself.  (Allowed earlier, while this grid still waits
+    // for k_merge, its CTAs -- and those of the call's other kernels -- gathered on the SMs whose k_merge CTA was through first:
+    // 150,000 pieces of two bytes, call after call, 177 us instead of 108, 300 KB of short accented words 815 instead of 651;
+    // 300 KB of Unicode-heavy text 38.8 instead of 35.5.)
+    cudaTriggerProgrammaticLaunchCompletion();
+    scatter_tiles(P, SH);
 }
 
 // ---- K5 for bulk text: a warp per tile, no barrier after the prologue -----------------------------------------

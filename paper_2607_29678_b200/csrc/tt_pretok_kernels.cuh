@@ -376,36 +376,35 @@ template <int PAT> struct PretokSmem {
     static constexpr size_t MASK_BYTES = (size_t)ROWS * TT_SLOTS * sizeof(u32), OFF_BYTES = (TT_TILE_BYTES + 2) * sizeof(u16);
     static constexpr size_t BYTES = ((MASK_BYTES > OFF_BYTES ? MASK_BYTES : OFF_BYTES) + 15) / 16 * 16;
 };
-template <bool FUSED, int NT, int MINB, int PAT>
-__global__ void __launch_bounds__(NT, MINB)
-k_pretok(const __grid_constant__ PretokParams P, const __grid_constant__ FrontParams F) {
-    __shared__ __align__(16) u8 smem_raw[PretokSmem<PAT>::BYTES];
-    u32 (*const sm)[TT_SLOTS] = reinterpret_cast<u32 (*)[TT_SLOTS]>(smem_raw);      // class masks of the tile and its halo
-    u16* const s_off = reinterpret_cast<u16*>(smem_raw);                             // later: piece offsets of the tile
-    __shared__ __align__(16) u32 s_text[4 + TT_SLOTS * 8 + 4];                       // the text of the slots, four bytes more on either side
-    __shared__ long long scratch[40];
-    __shared__ u32 s_need, s_first;
-    __shared__ u32 s_islast;
-    __shared__ u32 s_wtot[TT_TILE_WORDS / 32], s_ns, s_nw, s_nl, s_total, s_wbase;
-    __shared__ u16 s_wlist[TT_TILE_BYTES / (LANE_MAX + 1) + 2];       // bulk text: the tile's warp-class pieces
-    __shared__ u16 s_slow[TT_TILE_BYTES / 9 + 4];                     // pieces of more than 8 bytes (looked up together)
-    __shared__ u32 s_nslow;
+// Bulk text: a CTA takes runs of P.run neighbouring tiles and keeps the masks of the last eight slots (the next tile's low halo and
+// first word) and the text of the very last, so that 64 threads load and classify 64 words; with the halo taken in anew, one
+// warp went through both a second time for eight words while the other waited (132 MB batch 823 -> 809 us).  (Pattern 1 rewrites
+// the masks of its window afterwards, and host text is copied tile by tile: P.run is 1 there.)
+template <bool FUSED, int NT, int PAT> struct PretokShared {
+    static constexpr bool BULK = FUSED && NT == PRETOK_THREADS_BULK, CARRY = BULK && PAT != 1;
+    static constexpr int CARRY_ROWS = F_P0_COUNT;
+    alignas(16) u8 raw[PretokSmem<PAT>::BYTES];              // class masks of the tile and its halo; later: piece offsets of the tile
+    alignas(16) u32 text[4 + TT_SLOTS * 8 + 4];              // the text of the slots, four bytes more on either side
+    long long scratch[40];
+    u32 need, first, islast, wtot[TT_TILE_WORDS / 32], ns, nw, nl, total, wbase, nslow;
+    u16 wlist[TT_TILE_BYTES / (LANE_MAX + 1) + 2];           // bulk text: the tile's warp-class pieces
+    u16 slow[TT_TILE_BYTES / 9 + 4];                         // pieces of more than 8 bytes (looked up together)
+    u32 carry[CARRY ? CARRY_ROWS * (TT_LOW_HALO + 1) : 1];
+};
+// The kernel's work once what it reads is complete.
+template <bool FUSED, int NT, int PAT>
+__device__ __forceinline__ void pretok_tiles(const PretokParams& P, const FrontParams& F, PretokShared<FUSED, NT, PAT>& SH) {
     static_assert(NT >= TT_TILE_WORDS && NT % 32 == 0 && TT_TILE_WORDS % 32 == 0, "a thread per word of the tile, whole warps of them (tt_eval_word_p1 asks the warp)");
-
-    constexpr bool BULK = FUSED && NT == PRETOK_THREADS_BULK;
-    // Bulk text: a CTA takes runs of P.run neighbouring tiles and keeps the masks of the last eight slots (the next tile's low halo and
-    // first word) and the text of the very last, so that 64 threads load and classify 64 words; with the halo taken in anew, one
-    // warp went through both a second time for eight words while the other waited (132 MB batch 823 -> 809 us).  (Pattern 1 rewrites
-    // the masks of its window afterwards, and host text is copied tile by tile: P.run is 1 there.)
-    constexpr bool CARRY = BULK && PAT != 1;
-    constexpr int CARRY_ROWS = F_P0_COUNT;
+    constexpr bool BULK = SH.BULK, CARRY = SH.CARRY;
+    constexpr int CARRY_ROWS = SH.CARRY_ROWS;
     static_assert(!CARRY || NT == TT_TILE_WORDS, "the words of a run's later tiles, one per thread");
-    __shared__ u32 s_carry[CARRY ? CARRY_ROWS * (TT_LOW_HALO + 1) : 1];
+    u32 (*const sm)[TT_SLOTS] = reinterpret_cast<u32 (*)[TT_SLOTS]>(SH.raw);
+    u16* const s_off = reinterpret_cast<u16*>(SH.raw);
+    u32 (&s_text)[4 + TT_SLOTS * 8 + 4] = SH.text;
+    long long (&scratch)[40] = SH.scratch;
+    u32 &s_need = SH.need, &s_first = SH.first, &s_islast = SH.islast, &s_ns = SH.ns, &s_nw = SH.nw, &s_nl = SH.nl, &s_total = SH.total, &s_wbase = SH.wbase, &s_nslow = SH.nslow;
+    auto& s_wtot = SH.wtot; auto& s_wlist = SH.wlist; auto& s_slow = SH.slow; auto& s_carry = SH.carry;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    cudaTriggerProgrammaticLaunchCompletion();               // the next kernel may be placed; it waits for this grid's memory itself
-    // the whole-piece table is probed at random a few microseconds from now: ask for it to be brought into L2
-    if (FUSED && F.toktab.shorts != nullptr) grid_prefetch_l2(F.toktab.shorts, F.toktab.bytes);
-    cudaGridDependencySynchronize();                         // what was enqueued before this call is complete: its text, its use of the workspace
     if (FUSED) {
         if (blockIdx.x == 0 && tid == 0) {                    // k_merge's counters (k_merge touches them only after this grid)
             P.hdr->t_tiles = 0; P.hdr->merge_done = 0;
@@ -559,7 +558,7 @@ k_pretok(const __grid_constant__ PretokParams P, const __grid_constant__ FrontPa
         const bool quick = F.toktab.shorts != nullptr;               // block-uniform
         const u32* const tw = reinterpret_cast<const u32*>(tb);
         u32 wsum = 0;
-        constexpr int LW = NT == PRETOK_THREADS_BULK ? 1 : 4;        // look-ups in flight per thread
+        constexpr int LW = NT == PRETOK_THREADS_REQUEST ? 4 : 1;        // look-ups in flight per thread
         for (u32 ib = tid; ib < nlook; ib += LW * NT) {
             u32 o[LW], n[LW], k0[LW], k1[LW], h[LW];
             uint4 sl[LW], sm2[LW];
@@ -642,6 +641,16 @@ k_pretok(const __grid_constant__ PretokParams P, const __grid_constant__ FrontPa
         }
         if (tid == 0) { P.tile_cnt[P.ntiles] = carry; P.hdr->n_pieces = carry; }
     }
+}
+template <bool FUSED, int NT, int MINB, int PAT>
+__global__ void __launch_bounds__(NT, MINB)
+k_pretok(const __grid_constant__ PretokParams P, const __grid_constant__ FrontParams F) {
+    __shared__ PretokShared<FUSED, NT, PAT> SH;
+    cudaTriggerProgrammaticLaunchCompletion();               // the next kernel may be placed; it waits for this grid's memory itself
+    // the whole-piece table is probed at random a few microseconds from now: ask for it to be brought into L2
+    if (FUSED && F.toktab.shorts != nullptr) grid_prefetch_l2(F.toktab.shorts, F.toktab.bytes);
+    cudaGridDependencySynchronize();                         // what was enqueued before this call is complete: its text, its use of the workspace
+    pretok_tiles<FUSED, NT, PAT>(P, F, SH);
 }
 
 // ---- K3: compaction of the start flags into piece offsets (tt_pretokenize) --------------------------
