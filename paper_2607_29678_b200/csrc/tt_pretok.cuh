@@ -33,7 +33,7 @@ struct PretokParams {
     long long nchunks;       // ceil(hi / 16): vector loads
     long long nwords;        // ceil(hi / 32): mask words
     int ntiles;
-    int run;                 // neighbouring tiles that a CTA takes one after the other (a power of two; see CARRY in k_pretok)
+    int run;                 // neighbouring tiles that a CTA takes one after the other (see CARRY in k_pretok)
     int pattern;
     const u32* docmask;      // bit per byte (aligned frame) marking document starts, or null (one document)
     const u32* litstart;     // literal pass: first bytes of extracted literals (each becomes exactly one piece), or null

@@ -426,9 +426,10 @@ __device__ __forceinline__ void pretok_tiles(const PretokParams& P, const FrontP
     const u8* const tb = stx + TT_LOW_HALO * TT_WORD;                 // byte 0 of the tile
 
     const int run = CARRY ? P.run : 1;
-    for (int tile = (int)blockIdx.x * run; tile < P.ntiles; tile += CARRY && ((tile + 1) & (run - 1)) ? 1 : ((int)gridDim.x - 1) * run + 1) {
+    int left = run;                                               // tiles of the run from this one on
+    for (int tile = (int)blockIdx.x * run; tile < P.ntiles; tile += CARRY && --left ? 1 : (left = run, ((int)gridDim.x - 1) * run + 1)) {
         __syncthreads();
-        const bool carried = CARRY && (tile & (run - 1)) != 0;        // the tile before was this CTA's: block-uniform
+        const bool carried = CARRY && left != run;        // the tile before was this CTA's: block-uniform
         if (tid == 0) { s_need = 0; s_first = 0xFFFFFFFFu; s_ns = 0; s_nw = 0; s_nl = 0; s_total = 0; s_nslow = 0; }
         const long long w_first = (long long)tile * TT_TILE_WORDS;    // mask word of the tile's first byte
         // phase A: the text of the tile and its halo into shared memory, a vector load per thread and step

@@ -40,8 +40,9 @@ SNIPPETS = [b"it's we'll they've I'd ", b" 1234567890123 ", b"   \n\n  \r\n   x"
             b"a" * 70, b" " * 300 + b"x", b"7" * 400]
 
 
-@pytest.mark.parametrize("pattern", [0, 1, 2, 3])
-@pytest.mark.parametrize("megabytes,docs", [(5, 0), (14, 0), (14, 3_000), (26, 0)])
+# (on 148 SMs the CTAs take runs of 1, 2, 2, 3, 5 and 8 tiles)
+@pytest.mark.parametrize("pattern,megabytes,docs", [(p, m, d) for p in (0, 1, 2, 3) for m, d in ((5, 0), (14, 0), (14, 3_000), (26, 0))] +
+                         [(0, 44, 0), (2, 44, 5_000), (3, 44, 0), (2, 62, 0), (0, 103, 0), (0, 103, 9_000)])
 def test_constructs_across_the_edges_of_neighbouring_tiles(pattern, megabytes, docs):
     rng = np.random.default_rng(megabytes + pattern)
     gv, cv = gpu_vocab("C1", pattern=pattern), cpu_vocab("C1")
