@@ -93,3 +93,50 @@ def gpu_pretok(v, text: np.ndarray, doc_off: np.ndarray | None = None, offset: i
     v.pretokenize(d, po, npc, bufs, doc_off=off)
     torch.cuda.synchronize()
     return po[:int(npc.item())].cpu().numpy().astype(np.int64), int(bufs["status"].item())
+
+
+def merge_rule():
+    """(short pieces and tiles per warp up to which k_merge gives a warp to each short piece, warps per CTA, bytes of a tile), as the sources have them."""
+    import os
+    import re
+    src = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2607_29678_b200", "csrc")
+    with open(os.path.join(src, "tt_bpe.cuh")) as f:
+        bpe = f.read()
+    return int(re.search(r"constexpr u32 SHORT_PER_WARP = (\d+);", bpe).group(1)), int(re.search(r"#define TT_MERGE_WARPS (\d+)", bpe).group(1)), 2_048
+
+
+def short_pieces(cv, text: np.ndarray, pattern: int, offset: int = 0):
+    """What k_merge counts when it chooses between a warp and a thread per short piece, after every piece: (ends, counts), where
+    text[:ends[i]] has counts[i] pieces of 2 to 32 bytes that the first kernel leaves it, but for the last one of each tile, and tiles."""
+    import oracle
+    tile = merge_rule()[2]
+    start = oracle.pretokenize(text, pattern)
+    end = np.r_[start[1:], text.size]
+    n = end - start
+    one = {}                                                           # a vocabulary entry of at most 24 bytes as a whole: settled
+    raw = text.tobytes()
+    whole = np.zeros(n.size, bool)
+    for i, (a, k) in enumerate(zip(start.tolist(), n.tolist())):
+        if k == 1:
+            whole[i] = True
+        elif k <= 24:
+            b = raw[a:a + k]
+            if b not in one:
+                one[b] = cv.bpe(b).size == 1
+            whole[i] = one[b]
+    at = (start + offset) // tile
+    queued = ~whole & (n <= 32)
+    inner = queued & (at == np.r_[at[1:], -1])                         # not the last piece of its tile
+    before = np.r_[0, np.cumsum(inner)][:-1]                           # the text ends behind piece i: i itself is its tile's last
+    return end, before + (end - 1 + offset) // tile + 1
+
+
+def at_the_merge_rule(cv, text: np.ndarray, pattern: int, offset: int = 0):
+    """(longest beginning of the text that k_merge merges a warp per piece, shortest one that it merges a thread per piece)."""
+    import torch
+    per_warp, warps, tile = merge_rule()
+    limit = per_warp * warps * torch.cuda.get_device_properties(0).multi_processor_count
+    end, count = short_pieces(cv, text, pattern, offset)
+    k = int(np.argmax(count > limit))
+    assert 0 < k and limit - 2 <= count[k - 1] <= limit < count[k] <= limit + 2 and end[k] + offset <= 2_048 * tile, (k, count[-1], limit)
+    return text[:end[k - 1]], text[:end[k]]
