@@ -415,7 +415,7 @@ __device__ __forceinline__ u32 warp_merge_perm(u32* buf /* 2 * 4 * 32 E words of
 // piece, so the minimum is found without a dependent step per position: a pair's rank and position are one word, the words of
 // four positions one 16-byte load, and places without a pair hold all ones (walking the live positions one after the other
 // and merging all occurrences of the rank at once, a batch of 32 pieces took 50 to 110 us; 132 MB batch 851 -> 804, 3M chars of long
-// runs 236 -> 198, 1,000 messages 68.5 -> 61).
+// runs 1.1 to 1.2 times as fast by text, 1,000 messages 68.5 -> 61).
 constexpr int LANE_SLOTS = 32;                        // pieces a warp merges at once
 constexpr int LANE_MAX = 32;                          // bytes per piece on this path
 constexpr u32 LANE_NONE = 0xFFFFFFFFu;                // no pair begins here
@@ -945,7 +945,7 @@ k_closing(const __grid_constant__ PieceParams P) {
         }
         if (cn > (u32)TT_WARP_PIECE_MAX) P.lq[b] = make_uint4(ca, cn, cslot, 0u);
     }
-    // short pieces: four lists by length (a warp later merges 32 pieces of one list at a time, a thread each, and
+    // short pieces: four lists by length (a warp later merges up to 32 pieces of one list at a time, a thread each, and
     // waits for the longest), one reservation per warp and list
     u64 mine = 0;                                             // four counts of 16 bits (a warp's 32 tiles hold fewer than 2^16 pieces)
 #pragma unroll
@@ -1598,9 +1598,9 @@ __device__ __forceinline__ bool merge_closing(const PieceParams& P, const u8* __
 }
 // The queued short pieces in batches, in their order, whatever tiles they stand in, a thread each; the batches are spread over the
 // grid, by tickets where some CTAs first had a long piece.  (With a ticket per tile 147 warps took the 150,000 two-byte pieces of
-// 300 KB, most of them on the few SMs that came first: 78 to 118 us, now 54 to 66.)  Out of line: in line these texts are 4 % faster,
-// but a call of 4,000 characters, which does none of this, takes 33.05 us instead of 32.75, a conversation of 17 appends 831
-// instead of 824.
+// 300 KB, most of them on the few SMs that came first: 78 to 118 us, now 54 to 66.)  Out of line: when a call of 4,000 characters,
+// which does none of this, took 33 us, it took 0.3 us more with the batches in line.  Now it takes 20.3 either way, 1,000 messages 55.8
+// and in line 54.4, 3M chars of long runs 189.8 and 186.3.
 __device__ __noinline__ void merge_short_batches(const PieceParams& P, const u8* __restrict__ text, const MergeIndex& X, int unit, int entries, bool by_ticket, u32* buf) {
     const u32 lane = threadIdx.x & 31, W = gridDim.x * MERGE_WARPS, NS = X.pre_s[entries], per = short_batch(NS), nb = (NS + per - 1) / per;
     u32 b = by_ticket ? warp_take(&P.hdr->t_tiles, (int)lane) : (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
@@ -1704,7 +1704,8 @@ constexpr int SCATTER_STAGE_IDS = 2048;                   // ids of one work ite
 // spill: 1M chars 32 -> 37 us).
 constexpr int SCATTER_CTAS = 4, SCATTER_CTAS_MANY = 5;
 constexpr u32 SCATTER_WARP_MAX = 512;                     // tokens of a piece that one warp copies; longer ones the whole CTA
-// Work items: (tile, block of 512 of its pieces), two neighbouring pieces per thread.  A request has a tile per CTA and most
+// Work items: (tile, block of 512 of its pieces), two neighbouring pieces per thread.  (A piece of more than eight ids has at least nine
+// bytes: a tile has at most 228 of them, which is what `big` holds.)  A request has a tile per CTA and most
 // tiles one item, so what counts is the chain of dependent steps: everything that does not depend on anything else -- the
 // tiles' token counts, the first item's values and offsets, read before its length is known -- is asked for at once, the sums
 // over the tiles and the scan over the item's pieces share one barrier, and a staged piece's ids are fetched side by

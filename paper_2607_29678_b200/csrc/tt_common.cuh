@@ -129,8 +129,8 @@ struct TTWorkspace {
     u32* piece_cnt;
     u32* q;
     u64* wq;           // bulk text only: warp-class pieces of all tiles (len / 33 + 64 entries)
-    u64* gq;           // bulk text only: short pieces of all tiles by length class (see tt_short_class_max): a warp merges 32
-    u64* gq_x[3];      // pieces of one list at a time, a thread each, and is done when the longest of them is
+    u64* gq;           // bulk text only: short pieces of all tiles by length class (see tt_short_class_max): a warp merges up to
+    u64* gq_x[3];      // 32 pieces of one list at a time, a thread each, and is done when the longest of them is
     uint4* lq;         // long pieces (len / 257 + 16 entries): all of bulk text, those for the whole grid of a request
     int32_t* stage;    // token ids staged at the byte offset of their piece (len)
     u64* pairbuf;      // (token, rank) pairs of the long-piece path, indexed like the text (len)

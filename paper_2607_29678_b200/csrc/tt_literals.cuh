@@ -34,7 +34,7 @@ struct LitParams {
     LitTable tab;
     u8* cand;                    // [hi + 1] aligned frame: length of the longest literal starting at the byte, 0 = none
     int32_t* stage;              // text offsets: id of that literal
-    u32* docmask; u32* litstart; u32* litin;     // bit per byte, aligned frame (cleared by k_lit_scan)
+    u32* docmask; u32* litstart; u32* litin;     // bit per byte, aligned frame (written whole by k_lit_mark, else cleared by k_lit_scan)
 };
 
 // A thread takes 16 bytes: nearly none of them begins a literal, so what counts is one load and one store for all of them.  (A

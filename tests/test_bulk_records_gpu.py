@@ -63,3 +63,35 @@ def test_constructs_across_the_edges_of_neighbouring_tiles(pattern, megabytes, d
     ids, ioff, status = gpu_encode_batch(gv, filler, off)
     want, woff = cv.encode_batch(filler, off, pattern, nthreads=8)
     assert status == 0 and same(ids, want) and same(ioff, woff)
+
+
+# a tile whose first word the CTA has kept from the tile before does not look at it again: bytes that are no UTF-8, and documents that begin
+# inside a character, at every place around the edges of a run's tiles
+@pytest.mark.parametrize("pattern", [0, 2])
+def test_invalid_text_around_the_edges_of_neighbouring_tiles(pattern):
+    import torch
+    gv = gpu_vocab("C1", pattern=pattern)
+    text = wl.generate(0, 23, 44_000_000)                              # ASCII; runs of three tiles on 148 SMs
+    d, bufs = torch.from_numpy(text).cuda(), gv.alloc(text.size, max_docs=2)
+    places = [2_048 * t + o for t in (1, 2, 3, 4, 5, 6, 21_482, 21_483, 21_484) for o in (-33, -32, -1, 0, 1, 31, 32, 33)]
+
+    def statuses(bytes_, off):
+        found = torch.zeros(len(places), dtype=torch.int32, device="cuda")
+        for i, at in enumerate(places):
+            kept = d[at:at + len(bytes_)].clone()
+            d[at:at + len(bytes_)] = torch.tensor(list(bytes_), dtype=torch.uint8, device="cuda")
+            if off is None:
+                gv.encode(d, bufs)
+            else:
+                gv.encode_batch(d, torch.tensor([0, at + off, text.size], dtype=torch.int64, device="cuda"), bufs)
+            found[i] = bufs["status"][0]
+            d[at:at + len(bytes_)] = kept
+        return found.cpu().numpy()
+
+    assert d.data_ptr() % 16 == 0 and 2_048 * 21_484 + 40 < text.size
+    assert (statuses(b"\xff", None) == 4).all()
+    assert (statuses(b"\x80", None) == 4).all()
+    assert (statuses(b"\xe3a", None) == 4).all()                       # a lead byte without the rest
+    assert (statuses(b"\xc3\xa9", None) == 0).all()
+    assert (statuses(b"\xc3\xa9", 1) == 4).all()                       # a document that begins with a continuation byte
+    assert (statuses(b"\xc3\xa9", 0) == 0).all()
