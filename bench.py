@@ -629,12 +629,12 @@ def csrc_hash() -> str:
 # captures.  They belong to the source state whose hash is recorded with them; with other sources they are not
 # printed as measurements (the keys are null and "capture_stale" is true).
 NCU_CAPTURE = {
-    "csrc": "7fea48fa5fb435cd",
+    "csrc": "ef846a6a15654c1b",
     # kernel -> dram__bytes_read.sum + dram__bytes_write.sum per launch, one cold C3 request (ncu --set full)
-    "c3_dram_bytes": {"front": 13650688, "merge": 9397248, "scatter": 2048512},
+    "c3_dram_bytes": {"front": 13650176, "merge": 9397760, "scatter": 2051072},
     # kernel -> smsp__inst_executed.sum per launch of the 256-request batch: captured on the first 32 documents of the same
     # batch (16,315,836 bytes) and scaled by text bytes to the full 132,689,913 (all work is per tile or per piece)
-    "batch_warp_inst": {"front": 279323000, "closing": 2480000, "merge_bulk": 89060000, "scatter_bulk": 83813000},
+    "batch_warp_inst": {"front": 278769000, "closing": 2481000, "merge_bulk": 89047000, "scatter_bulk": 83813000},
 }
 
 
